@@ -19,7 +19,7 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 // iteration count of a graph-driven run
 enum Word {
   W_NTILES = 0, W_BIGSEG, W_HEAD, W_NEXTBIG, W_BIGPTS, W_OFFUSED, W_MIDSEG,
-  W_SMALL, W_SMALLW, W_SMALLTOT, W_SMALLPTS,  // adjacent: written together by a tick
+  W_SMALL, W_SMALLW, W_SMALLTOT, W_SMALLPTS, W_SMALLOFF,  // adjacent: written together by a tick
   W_NC0, W_NC1, W_ITERS, W_COUNT
 };
 // a graph-driven run's iterations (two level steps each) before it gives up
@@ -128,7 +128,6 @@ TreePlan plan_tree(const kdt_params& p0, bool no_subtree) {
   for (int b = 0; b < 2; ++b) {
     t.xbuf[b] = take((size_t)p.d * n * 4);
     t.pbuf[b] = take(n * 4);
-    t.sbuf[b] = take(n * (size_t)t.sid_bytes);
   }
   t.terms = take(t.term_cap * sizeof(TermRec));
   t.root_off = take(((size_t)p.r + 1) * 4);
@@ -146,6 +145,9 @@ void StepNeeds::add(const kdt_params& p0, const TreePlan& tp) {
   maxB += tp.maxB;
   cap_small += tp.cap_small;
   nseg += tp.maxB * (uint64_t)p.r;
+  // rows of subset offsets of the small cells (explicit ids): as many words as
+  // two columns of the ids would take
+  if (tp.small_max > 0) small_off += tp.n * (uint64_t)tp.sid_bytes / 2;
   max_trees += 1;
   slice_cells = std::max<uint32_t>(slice_cells, (uint32_t)tp.small_max);
   widest = widest || p.key_rule == KDT_KEY_WIDEST_SPREAD;
@@ -163,6 +165,7 @@ StepPlan plan_step(const StepNeeds& needs) {
   s.max_tiles = (uint32_t)std::min<uint64_t>(needs.points / kTile + needs.maxB + 1, clamp);
   s.nseg_cap = (uint32_t)std::min<uint64_t>(needs.nseg, clamp);
   s.off_cap = (uint32_t)std::min<uint64_t>(needs.nseg + needs.maxB, clamp);
+  s.small_off_cap = (uint32_t)std::min<uint64_t>(needs.small_off, clamp);
   s.bigseg_cap = (uint32_t)std::min<uint64_t>(needs.points / (kSelWarpMin + 1) + 1, clamp);
   const int sms = device_sms();
   s.sms = (uint32_t)(sms > 0 ? sms : 148);
@@ -185,6 +188,7 @@ StepPlan plan_step(const StepNeeds& needs) {
   s.tile_base = take(((size_t)s.maxB + 1) * 4);
   s.seg_base = take(((size_t)s.maxB + 1) * 4);
   s.tiles = take((size_t)s.max_tiles * sizeof(uint2));
+  s.tile_seg = take((size_t)s.max_tiles * 4);
   s.tile_left = take((size_t)s.max_tiles * 4);
   s.tile_loff = take((size_t)s.max_tiles * 4);
   s.tile_mm = take(needs.widest || needs.fourier ? (size_t)s.max_tiles * 2 * kMaxDims * 2 * 4 : 0);
@@ -202,6 +206,7 @@ StepPlan plan_step(const StepNeeds& needs) {
     s.off[b] = take((size_t)s.off_cap * 4);
     s.obase[b] = take((size_t)s.maxB * 4);
   }
+  s.small_off = take((size_t)s.small_off_cap * 4);
   s.crow = take((size_t)s.maxB * 2 * sizeof(uint2));
   s.bytes = off;
   return s;
@@ -234,6 +239,7 @@ Engine::Engine(const StepPlan& plan, uint8_t* base, cudaStream_t st) : plan_(pla
   s_.bigseg_count = words_ + W_BIGSEG;
   s_.midseg = (uint32_t*)(base + plan.midseg);
   s_.midseg_count = words_ + W_MIDSEG;
+  s_.tile_seg = (uint32_t*)(base + plan.tile_seg);
   s_.tile_left = (uint32_t*)(base + plan.tile_left);
   s_.tile_loff = (uint32_t*)(base + plan.tile_loff);
   s_.next_big_count = words_ + W_NEXTBIG;
@@ -251,6 +257,9 @@ Engine::Engine(const StepPlan& plan, uint8_t* base, cudaStream_t st) : plan_(pla
   }
   s_.off_used = words_ + W_OFFUSED;
   s_.off_cap = plan.off_cap;
+  s_.small_off = (uint32_t*)(base + plan.small_off);
+  s_.small_off_used = words_ + W_SMALLOFF;
+  s_.small_off_cap = plan.small_off_cap;
   s_.bigseg_cap = plan.bigseg_cap;
   s_.midseg_cap = plan.nseg_cap;
   s_.crow = (uint2*)(base + plan.crow);
@@ -298,12 +307,12 @@ kdt_status Engine::admit(uint32_t slot, const float* points, const kdt_params& p
   h.sid_bytes = tp.sid_bytes;
   h.small_max = tp.small_max;
   h.presorted = tp.presorted ? 1 : 0;
+  h.contig_mul = p.n > 0 ? ((uint64_t)p.r << 32) / (uint64_t)p.n : 0;
   h.x_in = points;
   h.sid_in = p.subset_id16 ? (const void*)p.subset_id16 : (const void*)p.subset_id8;
   for (int b = 0; b < 2; ++b) {
     h.xbuf[b] = (float*)(tb + tp.xbuf[b]);
     h.pbuf[b] = (uint32_t*)(tb + tp.pbuf[b]);
-    h.sbuf[b] = (void*)(tb + tp.sbuf[b]);
   }
   h.root_off = (uint32_t*)(tb + tp.root_off);
   h.root_cur = (uint32_t*)(tb + tp.root_cur);
@@ -384,7 +393,7 @@ kdt_status Engine::tick() {
     pending_small_.clear();
     pending_small_w_.clear();
   }
-  const uint32_t sw[4] = {small_count_, small_count_w_, small_count_ + small_count_w_, (uint32_t)small_points_};
+  const uint32_t sw[5] = {small_count_, small_count_w_, small_count_ + small_count_w_, (uint32_t)small_points_, 0u};
   ENGINE_TRY(cudaMemcpyAsync(words_ + W_SMALL, sw, sizeof(sw), cudaMemcpyHostToDevice, st_));
 
   if (big_count_ > 0) {
@@ -454,19 +463,19 @@ void Engine::launch_small(bool from_device) {
   if (from_device) {
     // counts on the device (a recorded tick): the narrow front, then the wide
     // back walked from the end
-    launch_subtree(kSubNarrow, trees_, small_, cap, words_ + W_SMALL, false, words_ + W_HEAD, slices_,
+    launch_subtree(kSubNarrow, trees_, small_, cap, words_ + W_SMALL, false, s_.small_off, words_ + W_HEAD, slices_,
                    plan_.needs.slice_cells, gn, 0, st_);
-    launch_subtree(kSubWide, trees_, small_, cap, words_ + W_SMALLW, true, words_ + W_HEAD, slices_,
+    launch_subtree(kSubWide, trees_, small_, cap, words_ + W_SMALLW, true, s_.small_off, words_ + W_HEAD, slices_,
                    plan_.needs.slice_cells, gw, 0, st_);
     return;
   }
   const uint64_t pts = small_points_;
   if (small_count_ > 0)
-    launch_subtree(kSubNarrow, trees_, small_, small_count_, nullptr, false, words_ + W_HEAD, slices_,
+    launch_subtree(kSubNarrow, trees_, small_, small_count_, nullptr, false, s_.small_off, words_ + W_HEAD, slices_,
                    plan_.needs.slice_cells, std::min(gn, small_count_), pts, st_);  // the points of both
   if (small_count_w_ > 0)
     launch_subtree(kSubWide, trees_, small_ + cap - small_count_w_, small_count_w_, nullptr, false,
-                   words_ + W_HEAD, slices_, plan_.needs.slice_cells, std::min(gw, small_count_w_),
+                   s_.small_off, words_ + W_HEAD, slices_, plan_.needs.slice_cells, std::min(gw, small_count_w_),
                    small_count_ ? 0 : pts, st_);
 }
 
@@ -552,7 +561,7 @@ kdt_status Engine::record_tick(int p) {
   ENGINE_TRY(cudaMemsetAsync(words_ + W_NC0 + (p ^ 1), 0, 4, st_));
   ENGINE_TRY(cudaMemsetAsync(words_ + W_BIGPTS, 0, 4, st_));
   ENGINE_TRY(cudaMemsetAsync(words_ + W_OFFUSED, 0, 4, st_));
-  ENGINE_TRY(cudaMemsetAsync(words_ + W_SMALL, 0, 4 * (W_SMALLPTS - W_SMALL + 1), st_));
+  ENGINE_TRY(cudaMemsetAsync(words_ + W_SMALL, 0, 4 * (W_SMALLOFF - W_SMALL + 1), st_));
   StepDev sd = s_;
   sd.cells = big_[p];
   sd.ncells = plan_.maxB;  // a capacity: the count is the device word

@@ -37,7 +37,7 @@ struct TreePlan {
   uint64_t huge_cap = 0;  // terminal cells larger than one CTA's leaf sort
   uint64_t maxB = 0;      // big cells at one level
   uint64_t cap_small = 0; // small cells over the whole build
-  size_t xbuf[2] = {0, 0}, pbuf[2] = {0, 0}, sbuf[2] = {0, 0}, terms = 0, root_off = 0, root_cur = 0,
+  size_t xbuf[2] = {0, 0}, pbuf[2] = {0, 0}, terms = 0, root_off = 0, root_cur = 0,
          huge = 0, words = 0;
   size_t bytes = 0;
 };
@@ -48,7 +48,7 @@ TreePlan plan_tree(const kdt_params& p, bool no_subtree = false);
 // Capacities of the shared tables, accumulated over the trees they must serve
 // at the same time.
 struct StepNeeds {
-  uint64_t points = 0, maxB = 0, cap_small = 0, nseg = 0;
+  uint64_t points = 0, maxB = 0, cap_small = 0, nseg = 0, small_off = 0;
   uint32_t max_trees = 0, slice_cells = 32;
   bool widest = false;
   bool fourier = false;  // a tree splits by the Fourier-moment estimator
@@ -61,11 +61,12 @@ struct StepPlan {
   StepNeeds needs;
   // grid_step: the grid scale of the level step's kernels (two per SM);
   // sms: the device's SMs (the subtree kernel's grid is sms x its shape's CTAs)
-  uint32_t maxB = 0, cap_small = 0, max_tiles = 0, nseg_cap = 0, bigseg_cap = 0, grid_step = 0, sms = 0, off_cap = 0;
+  uint32_t maxB = 0, cap_small = 0, max_tiles = 0, nseg_cap = 0, bigseg_cap = 0, grid_step = 0, sms = 0, off_cap = 0,
+           small_off_cap = 0;
   size_t trees = 0, words = 0, slot_words = 0, slots_list = 0, big[2] = {0, 0}, small = 0, tile_base = 0,
-         seg_base = 0, tiles = 0, tile_left = 0, tile_loff = 0, tile_mm = 0, child_mm = 0, kdim = 0,
+         seg_base = 0, tiles = 0, tile_seg = 0, tile_left = 0, tile_loff = 0, tile_mm = 0, child_mm = 0, kdim = 0,
          mkey = 0, lcount = 0, seg_w = 0, seg_key = 0, seg_med = 0, bigseg = 0, midseg = 0, slices = 0,
-         off[2] = {0, 0}, obase[2] = {0, 0}, crow = 0;
+         off[2] = {0, 0}, obase[2] = {0, 0}, small_off = 0, crow = 0;
   size_t bytes = 0;
 };
 StepPlan plan_step(const StepNeeds& needs);

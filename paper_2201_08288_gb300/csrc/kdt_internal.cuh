@@ -68,11 +68,11 @@ struct TreeDev {
   int32_t sid_bytes;   // explicit mode: 1 or 2
   int32_t small_max;   // cells up to this size finish in the subtree kernel
   int32_t presorted;   // root reordered by subset into buf[1]; leaves sorted at the end
+  uint64_t contig_mul; // contiguous subsets: floor(2^32 r / n)
   const float* x_in;
   const void* sid_in;
   float* xbuf[2];
   uint32_t* pbuf[2];
-  void* sbuf[2];
   uint32_t* root_off;    // [r+1] subset offsets of the root (level 0)
   uint32_t* root_cur;    // [r] subset counts, then fill cursors of the presort
   uint32_t* huge;        // [huge_cap] terminal records too large for one CTA's leaf sort
@@ -94,6 +94,8 @@ struct TreeDev {
   int32_t* live;         // cells of this tree still waiting to be split (0: the tree is done)
 };
 
+constexpr uint32_t kNoRow = 0xffffffffu;
+
 // A cell of the tree: a contiguous position range [begin, begin+count) of its
 // tree's current order.
 struct Cell {
@@ -104,6 +106,8 @@ struct Cell {
   int8_t level;
   int8_t stall;   // consecutive splits on this path that left the right child empty
   int16_t dim;    // widest-spread key coordinate if already known, else -1
+  uint32_t row = kNoRow;  // cells queued for the subtree kernel: row of small_off with the cell's
+                          // subset offsets, or kNoRow
 };
 
 // A terminal cell (leaf of the real tree); finalize turns these into offsets
@@ -139,6 +143,7 @@ struct StepDev {
   uint32_t* bigseg_count; // device word
   uint32_t* midseg;       // [midseg_cap] segments of kSelTinyMax+1 .. kSelSmallMax points
   uint32_t* midseg_count; // device word
+  uint32_t* tile_seg;     // [ntiles] first subset offset of the cell at or after the tile's start
   uint32_t* tile_left;    // [ntiles]
   uint32_t* tile_loff;    // [ntiles]
   Cell* next_big;         // children that stay in the multi-CTA pipeline
@@ -161,6 +166,12 @@ struct StepDev {
   uint32_t* obase_next;       // [next_big_cap]
   uint32_t* off_used;         // device word: words of off_next handed out
   uint32_t off_cap;
+  // subset offsets of cells queued for the subtree kernel (explicit ids, while
+  // rows last; other modes follow from the original index, and so does a cell
+  // without a row)
+  uint32_t* small_off;
+  uint32_t* small_off_used;   // device word
+  uint32_t small_off_cap;
   uint32_t bigseg_cap;
   // select paths by segment size (kdt_tuning): one thread up to tiny_max keys,
   // a warp's bitonic network up to bitonic_max, a warp's radix select up to
@@ -179,8 +190,6 @@ struct StepDev {
   uint32_t* wcount;           // [ncells] points of the cell over all shards (the combine's weight)
   uint32_t* mm_tmp;           // [ncells][2][d][2] children's min / max over all shards
 };
-
-constexpr uint32_t kNoRow = 0xffffffffu;
 
 // ------------------------------------------------------------- key transform
 
@@ -208,47 +217,34 @@ __device__ __forceinline__ const float* src_cols(const TreeDev& t, int level) {
 __device__ __forceinline__ const uint32_t* src_perm(const TreeDev& t, int level) {
   return (level == 0 && !t.presorted) ? nullptr : t.pbuf[(level - 1) & 1];
 }
-__device__ __forceinline__ const void* src_sid(const TreeDev& t, int level) {
-  return (level == 0 && !t.presorted) ? t.sid_in : t.sbuf[(level - 1) & 1];
-}
 
 __device__ __forceinline__ void set_status(const TreeDev& t, int32_t code) {
   atomicCAS(t.status, ST_OK, code);
 }
 
-// Subset of the point at position pos whose original index is orig. An
-// explicit id >= r is reported as an invalid argument and replaced by 0 so
-// that no table is indexed out of range.
-__device__ __forceinline__ uint32_t subset_of(const TreeDev& t, const void* sidcol, uint32_t orig,
-                                              int64_t pos) {
+// Subset of a point from its original index (modes that define it so). For
+// contiguous subsets floor(orig r / n) comes from contig_mul = floor(2^32 r /
+// n): orig contig_mul / 2^32 falls short of orig r / n by less than 1 (orig <
+// 2^32), so its floor is the subset or one below it (a 64-bit division is
+// about a hundred instructions here).
+__device__ __forceinline__ uint32_t subset_from_orig(const TreeDev& t, uint32_t orig) {
   if (t.subset_mode == SUB_MOD) return orig % (uint32_t)t.r;
-  if (t.subset_mode == SUB_CONTIG)
-    return (uint32_t)(((uint64_t)orig * (uint64_t)t.r) / (uint64_t)t.n);
-  const uint32_t s = t.sid_bytes == 1 ? (uint32_t)((const uint8_t*)sidcol)[pos]
-                                      : (uint32_t)((const uint16_t*)sidcol)[pos];
+  const uint32_t lo = (uint32_t)(((uint64_t)orig * t.contig_mul) >> 32);
+  return lo + ((uint64_t)(lo + 1u) * (uint64_t)t.n <= (uint64_t)orig * (uint64_t)t.r ? 1u : 0u);
+}
+
+// Subset of the point with original index orig. An explicit id >= r is
+// reported as an invalid argument and replaced by 0 so that no table is
+// indexed out of range.
+__device__ __forceinline__ uint32_t subset_of(const TreeDev& t, uint32_t orig) {
+  if (t.subset_mode != SUB_EXPLICIT) return subset_from_orig(t, orig);
+  const uint32_t s = t.sid_bytes == 1 ? (uint32_t)__ldg((const uint8_t*)t.sid_in + orig)
+                                      : (uint32_t)__ldg((const uint16_t*)t.sid_in + orig);
   if (s >= (uint32_t)t.r) {
     set_status(t, ST_INVALID_ARG);
     return 0;
   }
   return s;
-}
-
-// Subset of a point from its original index (modes that define it so).
-__device__ __forceinline__ uint32_t subset_from_orig(const TreeDev& t, uint32_t orig) {
-  if (t.subset_mode == SUB_MOD) return orig % (uint32_t)t.r;
-  return (uint32_t)(((uint64_t)orig * (uint64_t)t.r) / (uint64_t)t.n);
-}
-
-// Subset of the point at position pos of the order level `level` reads
-// (explicit ids there are already checked and below r).
-__device__ __forceinline__ uint32_t subset_at(const TreeDev& t, int level, int64_t pos) {
-  if (t.subset_mode == SUB_EXPLICIT) {
-    const void* S = src_sid(t, level);
-    const uint32_t v = t.sid_bytes == 1 ? (uint32_t)((const uint8_t*)S)[pos] : (uint32_t)((const uint16_t*)S)[pos];
-    return min(v, (uint32_t)t.r - 1u);
-  }
-  const uint32_t* P = src_perm(t, level);
-  return subset_from_orig(t, P ? P[pos] : (uint32_t)pos);
 }
 
 // Terminal test for a cell about to be processed at `level` (reading R8 in

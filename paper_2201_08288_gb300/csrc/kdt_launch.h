@@ -100,13 +100,13 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
                      uint32_t max_bigseg, bool has_roots, bool need_root_dims, bool any_widest, int max_d, int uniform_d,
                      const SelectTuning& tune, uint64_t points, uint32_t sms, cudaStream_t st, bool fourier = false);
 
-// Dynamic shared memory of the staged scatter (two CTAs per SM).
+// Most dynamic shared memory of the staged scatter (two CTAs per SM).
 constexpr uint32_t kScatterSmemBytes = 100 * 1024;
 cudaError_t prepare_scatter_kernel();
 // uniform_d: the coordinate count of every tree of the step, 0 if they differ
 // (a kernel compiled for that d is used where there is one)
-void launch_scatter(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t grid_cap,
-                    uint64_t points, int uniform_d, cudaStream_t st);
+void launch_scatter(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t sms, uint64_t points,
+                    int uniform_d, bool any_widest, cudaStream_t st);
 
 // Sharded build (kdt_shard.cu): the per-level exchanges among the shards of
 // a step whose StepDev has shards > 0 (ncells_cap bounds the step's cells).
@@ -118,10 +118,11 @@ cudaError_t prepare_subtree_kernel();
 // One launch of the subtree kernel in the given shape over a queue of small
 // cells. count_dev: if set, the device word holding the queue's length
 // (count is then its cap). reversed: the queue is filled from the end of the
-// list (item j at list[count_cap - 1 - j], count_cap = count).
+// list (item j at list[count_cap - 1 - j], count_cap = count). small_off: the
+// cells' rows of subset offsets.
 void launch_subtree(const SubtreeShape& sh, const TreeDev* trees, const Cell* list, uint32_t count,
-                    const uint32_t* count_dev, bool reversed, uint32_t* head, LCell* slices, uint32_t slice_cells,
-                    uint32_t grid, uint64_t points, cudaStream_t st);
+                    const uint32_t* count_dev, bool reversed, const uint32_t* small_off, uint32_t* head,
+                    LCell* slices, uint32_t slice_cells, uint32_t grid, uint64_t points, cudaStream_t st);
 
 void launch_iota(uint32_t* out, uint32_t n, cudaStream_t st);
 

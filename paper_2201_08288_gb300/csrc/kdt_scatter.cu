@@ -7,10 +7,10 @@
 //     free ("empty" mbarrier), writes the sub-tile's metadata (output
 //     pointers, which children are terminal, what to compute), raises the
 //     buffer's expected byte count, starts bulk copies (cp.async.bulk) of
-//     the aligned middle of every coordinate column, of the permutation and
-//     of the subset ids, copies the ragged 16-byte edges (4-byte cp.async for
-//     word columns, plain loads for the ids) and arrives on the buffer's
-//     "full" mbarrier; the next tile's record is loaded one tile ahead;
+//     the aligned middle of every coordinate column and of the permutation,
+//     copies the ragged 16-byte edges (4-byte cp.async) and arrives on the
+//     buffer's "full" mbarrier; the next tile's record is loaded one tile
+//     ahead;
 //   consumer warps (0-7): wait for "full" (bounded), compute each point's
 //     left/right flag from its key and its rank by warp ballots in position
 //     order (so the partition is stable), store every value straight from
@@ -21,9 +21,15 @@
 // coordinate (per warp, then one shared-memory reduction per warp and
 // column, fire-and-forget). Points of a cell arrive in subset order
 // (contiguous segments), and a stable partition keeps that order in both
-// children; where the subset changes, the consumers write where each big
-// child's segments start (its left or right rank there), which is the
-// children's subset offset table.
+// children: a segment that starts at position p of the cell starts in the
+// left child at the number of left points before p, in the right child at p
+// minus that. So the children's subset offset tables come from the cell's own
+// table, one thread per segment start of the sub-tile, and no subset id moves
+// with the points. (Finding the starts by comparing neighbouring points'
+// subsets, ids staged and stored as one more column or computed from the
+// permutation by a division per point, took 33.1 instead of 26.8 ms per build
+// of 2^27 points with d = 8 and 256 explicit subsets; the bytes alone, 72
+// against 74 per point and level, are 25.9 ms at 6.8 TB/s.)
 #include <algorithm>
 
 #include "kdt_internal.cuh"
@@ -38,56 +44,69 @@ namespace {
 constexpr int kCW = 8;                // consumer warps
 constexpr int kCT = kCW * 32;         // consumer threads
 constexpr int kST = kCT + 32;         // + one producer warp
-constexpr int kMaxItems = 4;          // points per consumer thread in a sub-tile (T <= 1024)
-constexpr uint32_t kBufBytes = kScatterSmemBytes / 2;
 constexpr uint32_t kConsumerBar = 1;  // named barrier of the consumer warps
 
-// Largest power-of-two sub-tile whose ncols word columns (stride T + 4) and
-// an id column of sid_bytes per point (T + 32 entries) fit one buffer.
-__device__ __forceinline__ uint32_t sub_tile(int ncols, int sid_bytes) {
+// Words of one staged column of T points (room for the alignment phase).
+__host__ __device__ constexpr uint32_t col_stride(uint32_t T) { return T + 4u; }
+
+// Bytes of the two buffers for d coordinate columns and the permutation.
+__host__ __device__ constexpr uint32_t buf_bytes(int d, uint32_t T) { return (uint32_t)(d + 1) * col_stride(T) * 4u; }
+
+// Points of a sub-tile: a power of two, as many as two buffers of
+// kScatterSmemBytes in all hold, at most 1024.
+__host__ __device__ constexpr uint32_t sub_tile(int d) {
   uint32_t T = 1024;
-  while (T > 32 && (uint32_t)ncols * (T + 4) * 4u + (T + 32) * (uint32_t)sid_bytes > kBufBytes) T >>= 1;
+  while (T > 32 && 2u * buf_bytes(d, T) > kScatterSmemBytes) T >>= 1;
   return T;
+}
+
+// Resident CTAs per SM of an instance. A sub-tile costs its barriers, its scan
+// and a round trip to L2 whatever it holds, so what bounds a launch of few
+// columns is how many sub-tiles are in flight: at d = 3, 2^24 points and 14
+// levels the scatter took 2.62 ms per build with two CTAs, 1.42 with three and
+// 1.37 with four (0.18 per level at 6.8 TB/s would be 1.1). At d = 8 without
+// min / max two buffers of nine columns fit three times; with them the
+// accumulators take 94 registers, and three CTAs spill (28.0 against 26.8 ms
+// per build of 2^27 points).
+constexpr int scatter_ctas(int kD, bool kMM) {
+  return (kD == 2 || kD == 3) ? (kMM ? 3 : 4) : ((kD == 8 && !kMM) || kD == 16) ? 3 : 2;
 }
 
 // What the consumers need about the sub-tile in a buffer.
 struct SubMeta {
-  float* xout;         // coordinate columns of the next level
-  uint32_t* pout;      // permutation of the next level
-  void* sout;          // subset ids of the next level (explicit ids)
-  uint32_t* out_perm;  // final permutation (terminal children)
+  float* xout;           // coordinate columns of the next level
+  uint32_t* pout;        // permutation of the next level
+  uint32_t* out_perm;    // final permutation (terminal children)
+  const uint32_t* off;   // the cell's subset offsets
+  uint32_t* row[2];      // the children's subset offsets (null: none kept)
   int32_t* status;
   int64_t n;
-  uint32_t cell_begin, cell_count, cell_idx, tile, sub, mcnt, T, dim, mkey, L, loff, tile_start;
-  uint32_t row[2];     // rows of the children's subset offsets (kNoRow: not a big child)
-  uint32_t prev_sub;   // subset of the point before the CTA's first sub-tile (~0u at a cell's start)
-  uint32_t r, subset_mode, sid_bytes, sid_ph, tn;
+  uint32_t cell_begin, cell_count, cell_idx, sub, mcnt, T, dim, mkey, L, loff, tile_start;
+  uint32_t u0, u1;       // segment starts off[u0, u1) lie in this tile
   int32_t d;
   uint8_t term_left, term_right, want_mm, want_off, nan_check;
-  uint8_t run_more;  // this CTA's next tile is of the same cell (its min / max run goes on)
+  uint8_t run_more;      // this CTA's next tile is of the same cell (its min / max run goes on)
   uint8_t pad1, pad2;
   uint32_t ph[kMaxDims + 1];  // alignment phase of each staged word column
 };
 
-__device__ __forceinline__ uint32_t meta_subset(const SubMeta& m, uint32_t orig) {
-  if (m.subset_mode == SUB_MOD) return orig % m.r;
-  return (uint32_t)(((uint64_t)orig * (uint64_t)m.r) / (uint64_t)m.tn);
-}
-
 // kD > 0: compiled for trees of kD coordinates (the column loops unroll);
-// kD = 0: any d.
-template <int kD>
-__global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, StepDev s) {
+// kD = 0: any d. kMM: some tree of the step uses widest spread.
+template <int kD, bool kMM>
+__global__ void __launch_bounds__(kST, scatter_ctas(kD, kMM)) k_scatter_tma(const TreeDev* trees, StepDev s) {
+  constexpr int kMaxItems = kD > 0 ? (int)(sub_tile(kD > 0 ? kD : 1) / kCT) : 4;  // points per consumer thread
+  // words of a buffer (kD = 0: trees of several d may follow one another, so
+  // the halves are fixed)
+  constexpr uint32_t kBufWords =
+      (kD > 0 ? buf_bytes(kD > 0 ? kD : 1, (uint32_t)(kMaxItems * kCT)) : kScatterSmemBytes / 2) / 4;
   extern __shared__ __align__(128) uint32_t sm[];
   __shared__ __align__(8) uint64_t full[2], empty[2];
   __shared__ SubMeta meta[2];
   __shared__ uint32_t wcnt[kMaxItems][kCW];
-  __shared__ uint32_t sedge[kMaxItems][kCW];  // subset of each warp's last point per round
-  __shared__ unsigned wbal[kMaxItems][kCW];   // each (round, warp) block's left flags (explicit ids)
+  __shared__ unsigned wbal[kMaxItems][kCW];   // each (round, warp) block's left flags
   __shared__ uint32_t tmm[2][kMaxDims][2];    // this CTA's run of tiles of one cell: per child,
                                               // min / max key per coordinate
   __shared__ uint32_t s_fail;
-  __shared__ uint32_t s_carry;  // subset of the last point of the sub-tile the consumers finished last
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t ntiles = *s.ntiles_total;
   // this CTA's contiguous range of tiles: consecutive tiles mostly share a
@@ -122,18 +141,33 @@ __global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, St
       const bool run_more = tile + 1 < t_end && tl_next.x == tl.x;
       const TreeDev& tg = trees[c.tree];
       const int d = kD > 0 ? kD : tg.d, ncols = d + 1;
-      const bool expl = tg.subset_mode == SUB_EXPLICIT;
-      const int es = expl ? tg.sid_bytes : 0;
-      const uint32_t T = sub_tile(ncols, es), stride = T + 4;
+      const uint32_t T = kD > 0 ? (uint32_t)(kMaxItems * kCT) : sub_tile(d), stride = col_stride(T);
       const uint32_t tend = min(tl.y + (uint32_t)kTile, c.count);
       const float* X = src_cols(tg, c.level);
       const uint32_t* P = src_perm(tg, c.level);
-      const uint8_t* SID = (const uint8_t*)src_sid(tg, c.level);
       const uint32_t dim = s.kdim[tl.x], mkey = s.mkey[tl.x], L = s.lcount[tl.x], loff = s.tile_loff[tile];
       const uint2 cr0 = s.crow[2 * tl.x], cr1 = s.crow[2 * tl.x + 1];
       const int child_stall = (c.count == L) ? c.stall + 1 : 0;
       const bool term_left = is_terminal(tg, L, c.level + 1, child_stall);
       const bool term_right = is_terminal(tg, c.count - L, c.level + 1, child_stall);
+      // the children's rows of subset offsets: a big child's, or that of a
+      // small one that has one (the Fourier estimator reads no segments: its
+      // cells carry no offsets)
+      auto row_of = [&](uint2 cr) -> uint32_t* {
+        if (tg.fourier_j) return nullptr;
+        if (cr.x != kNoRow) return s.off_next + cr.y;
+        if (cr.y == kNoRow || tg.subset_mode != SUB_EXPLICIT) return nullptr;
+        const uint32_t row = s.small[cr.y].row;
+        return row == kNoRow ? nullptr : s.small_off + row;
+      };
+      uint32_t* const row0 = row_of(cr0);
+      uint32_t* const row1 = row_of(cr1);
+      const bool want_off = row0 || row1;
+      uint32_t u0 = 0, u1 = 0;
+      if (want_off) {
+        u0 = s.tile_seg[tile];
+        u1 = tl.y + (uint32_t)kTile < c.count ? min(s.tile_seg[tile + 1], (uint32_t)tg.r + 1u) : (uint32_t)tg.r + 1u;
+      }
       for (uint32_t sub = tl.y; sub < tend; sub += T, ++k) {
         const int b = k & 1;
         if (k >= 2) {
@@ -147,27 +181,17 @@ __global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, St
         const uint32_t mcnt = min(T, tend - sub);
         const uint32_t g0 = c.begin + sub;
         SubMeta& m = meta[b];
-        uint32_t* A = sm + (size_t)b * (kBufBytes / 4);
-        uint8_t* SA = (uint8_t*)(A + (size_t)ncols * stride);  // 16-byte aligned (stride * 4 is)
-        // id column: 16-byte phase in elements, aligned middle [sa0, sa1)
-        uint32_t sph = 0, sa0 = g0, sa1 = g0;
-        if (expl) {
-          const uint32_t per16 = 16u / (uint32_t)es;
-          sph = (uint32_t)(((uintptr_t)(SID + (size_t)g0 * es) / (uintptr_t)es) & (per16 - 1u));
-          sa0 = min(g0 + ((per16 - sph) & (per16 - 1u)), g0 + mcnt);
-          sa1 = sa0 + ((g0 + mcnt - sa0) & ~(per16 - 1u));
-        }
+        uint32_t* A = sm + (size_t)b * kBufWords;
         if (lane == 0) {
           m.xout = tg.xbuf[c.level & 1];
           m.pout = tg.pbuf[c.level & 1];
-          m.sout = tg.sbuf[c.level & 1];
           m.out_perm = tg.out_perm;
+          m.off = c.level == 0 ? tg.root_off : s.off_cur + s.obase_cur[tl.x];
           m.status = tg.status;
           m.n = tg.n;
           m.cell_begin = c.begin;
           m.cell_count = c.count;
           m.cell_idx = tl.x;
-          m.tile = tile;
           m.sub = sub;
           m.mcnt = mcnt;
           m.T = T;
@@ -176,24 +200,21 @@ __global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, St
           m.L = L;
           m.loff = loff;
           m.tile_start = tl.y;
-          m.row[0] = cr0.x == kNoRow ? kNoRow : cr0.y;
-          m.row[1] = cr1.x == kNoRow ? kNoRow : cr1.y;
-          m.r = (uint32_t)tg.r;
-          m.subset_mode = (uint32_t)tg.subset_mode;
-          m.sid_bytes = (uint32_t)es;
-          m.sid_ph = sph;
-          m.tn = (uint32_t)tg.n;
+          m.row[0] = row0;
+          m.row[1] = row1;
+          m.u0 = u0;
+          m.u1 = u1;
           m.d = d;
           m.term_left = term_left;
           m.term_right = term_right;
           m.want_mm = tg.key_rule == KEY_WIDEST && !(term_left && term_right);
-          m.want_off = cr0.x != kNoRow || cr1.x != kNoRow;
+          m.want_off = want_off;
           // the input's NaN check: the root's first pass over its columns (a
           // presorted root's presort checks them)
           m.nan_check = c.level == 0 && !tg.presorted;
           m.run_more = run_more;
         }
-        uint32_t total = expl ? (sa1 - sa0) * (uint32_t)es : 0u;
+        uint32_t total = 0u;
         for (int c0 = 0; c0 < ncols; c0 += 32) {
           const int col = c0 + lane;
           uint32_t bytes = 0;
@@ -224,30 +245,8 @@ __global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, St
           for (uint32_t idx = g0; idx < a0; ++idx) cp_async4(dst + ph + (idx - g0), src + idx);
           for (uint32_t idx = a1; idx < g0 + mcnt; ++idx) cp_async4(dst + ph + (idx - g0), src + idx);
         }
-        if (expl) {
-          if (lane == 0 && sa1 > sa0)
-            bulk_g2s(SA + (size_t)(sph + sa0 - g0) * es, SID + (size_t)sa0 * es, (sa1 - sa0) * (uint32_t)es,
-                     &full[b]);
-          // ragged ends of the id column: fewer than 16 bytes each, plain loads
-          const uint32_t nlo = sa0 - g0, nhi = g0 + mcnt - sa1;
-          if ((uint32_t)lane < nlo + nhi) {
-            const uint32_t idx = (uint32_t)lane < nlo ? g0 + lane : sa1 + (lane - nlo);
-            if (es == 1)
-              SA[sph + idx - g0] = SID[idx];
-            else
-              ((uint16_t*)SA)[sph + idx - g0] = ((const uint16_t*)SID)[idx];
-          }
-        }
         if (!P)
           for (uint32_t i = lane; i < mcnt; i += 32) A[(size_t)d * stride + i] = g0 + i;
-        // the subset of the point before the CTA's first sub-tile, if that is
-        // not a cell's start: one global load per CTA (each later sub-tile
-        // follows the one before it in the same cell, whose last subset the
-        // consumers keep)
-        if (lane == 0)
-          m.prev_sub = (k == 0 && sub > 0u && (cr0.x != kNoRow || cr1.x != kNoRow))
-                           ? subset_at(tg, c.level, (int64_t)g0 - 1)
-                           : 0xffffffffu;
         cp_async_mbar_arrive(&full[b]);  // this lane's edge copies count toward the phase
         __syncwarp();
         if (lane == 0) mbar_arrive(&full[b]);
@@ -265,7 +264,7 @@ __global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, St
   // points per coordinate and child over the whole run of the cell's tiles
   // (registers), reduced over the warp once at the run's end; otherwise the
   // warps reduce after every sub-tile.
-  constexpr bool kAcc = kD > 0 && kD <= 8;
+  constexpr bool kAcc = kMM && kD > 0 && kD <= 8;
   constexpr int kAD = kAcc ? kD : 1;
   const float inf = __int_as_float(0x7f800000);
   float acc[kAD][2][2];  // [coordinate][child][min, max]
@@ -290,32 +289,24 @@ __global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, St
       const SubMeta& m = meta[b];
       const int d = kD > 0 ? kD : m.d;
       const int64_t n = m.n;
-      const uint32_t T = m.T, stride = T + 4, mcnt = m.mcnt, L = m.L;
+      const uint32_t T = kD > 0 ? (uint32_t)(kMaxItems * kCT) : m.T, stride = col_stride(T);
+      const uint32_t mcnt = m.mcnt, L = m.L;
       const uint32_t cbeg = m.cell_begin, ccount = m.cell_count;
       const uint32_t tend = min(m.tile_start + (uint32_t)kTile, ccount);
       const bool term_left = m.term_left, term_right = m.term_right;
-      const bool want_mm = m.want_mm, want_off = m.want_off, nan_check = m.nan_check;
-      const bool explicit_sid = m.sid_bytes != 0;
-      // subset of the point before this sub-tile (~0u at the cell's start):
-      // the CTA's sub-tiles run in position order, so after its first one it
-      // is the last subset of the previous sub-tile (read here, before this
-      // sub-tile's second consumer barrier; rewritten after it)
-      const uint32_t prev_sub = m.sub == 0u ? 0xffffffffu : (k == 0 ? m.prev_sub : s_carry);
+      const bool want_mm = kMM && m.want_mm, want_off = m.want_off, nan_check = m.nan_check;
+      // this thread's first segment start of the tile, loaded ahead of its use
+      const uint32_t u_first = m.u0 + (uint32_t)tid;
+      uint32_t u_pos = want_off && u_first < m.u1 ? __ldg(m.off + u_first) : 0xffffffffu;
       if (m.sub == m.tile_start) {
         lnext = cbeg + m.loff;
         rnext = cbeg + L + (m.tile_start - m.loff);
       }
-      const uint32_t* A = sm + (size_t)b * (kBufBytes / 4);
-      const uint8_t* SA = (const uint8_t*)(A + (size_t)(d + 1) * stride) + (size_t)m.sid_ph * m.sid_bytes;
-      auto sid_of = [&](uint32_t i) -> uint32_t {
-        const uint32_t v = m.sid_bytes == 1 ? (uint32_t)SA[i] : (uint32_t)((const uint16_t*)SA)[i];
-        return min(v, m.r - 1u);
-      };
+      const uint32_t* A = sm + (size_t)b * kBufWords;
 
-      // ---- flags and ranks (position order); subsets where offsets are kept
+      // ---- flags and ranks (position order)
       bool left[kMaxItems];
       unsigned bal[kMaxItems];
-      uint32_t sv[kMaxItems];
       const uint32_t* keycol = A + (size_t)m.dim * stride + m.ph[m.dim];
       const uint32_t* pa = A + (size_t)d * stride + m.ph[d];
 #pragma unroll
@@ -323,33 +314,26 @@ __global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, St
         const uint32_t i = tid + q * kCT;
         left[q] = i < mcnt && ord_key(__uint_as_float(keycol[i])) <= m.mkey;
         bal[q] = __ballot_sync(0xffffffffu, left[q]);
-        if (lane == 0) wcnt[q][warp] = __popc(bal[q]);
-        sv[q] = 0;
-        if (want_off) {
-          if (explicit_sid) {
-            if (lane == 0) wbal[q][warp] = bal[q];
-          } else {
-            if (i < mcnt) sv[q] = meta_subset(m, pa[i]);
-            if (lane == 31) sedge[q][warp] = sv[q];
-          }
+        if (lane == 0) {
+          wcnt[q][warp] = __popc(bal[q]);
+          wbal[q][warp] = bal[q];
         }
       }
       named_sync(kConsumerBar, kCT);
-      // left points before each (round, warp) block: one scan over the
-      // kMaxItems * kCW = 32 block counts in position order
-      static_assert(kMaxItems * kCW == 32, "one lane per (round, warp) block");
-      const uint32_t wv = (&wcnt[0][0])[lane];
+      // left points before each (round, warp) block: one scan over the at
+      // most 32 block counts in position order
+      static_assert(kMaxItems >= 1 && kMaxItems * kCW <= 32, "one lane per (round, warp) block");
+      const uint32_t wv = lane < kMaxItems * kCW ? (&wcnt[0][0])[lane] : 0u;
       const uint32_t winc = warp_incl_scan(wv);
       const uint32_t wexc = winc - wv;
       const uint32_t nL = __shfl_sync(0xffffffffu, winc, 31);
-      uint32_t dst[kMaxItems], lrk[kMaxItems];
+      uint32_t dst[kMaxItems];
       bool keep[kMaxItems];  // the point's child is not terminal: its columns move
 #pragma unroll
       for (int q = 0; q < kMaxItems; ++q) {
         const uint32_t i = tid + q * kCT;
         const uint32_t lr = __shfl_sync(0xffffffffu, wexc, q * kCW + warp) + __popc(bal[q] & lt_mask);
         dst[q] = left[q] ? lnext + lr : rnext + (i - lr);
-        lrk[q] = lnext - cbeg + lr;  // points of the cell before this one that go left
         keep[q] = i < mcnt && !(left[q] ? term_left : term_right);
       }
 
@@ -449,74 +433,28 @@ __global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, St
           }
         }
       }
-      if (explicit_sid) {
-#pragma unroll
-        for (int q = 0; q < kMaxItems; ++q) {
-          const uint32_t i = tid + q * kCT;
-          if (!keep[q]) continue;
-          if (m.sid_bytes == 1)
-            ((uint8_t*)m.sout)[dst[q]] = SA[i];
-          else
-            ((uint16_t*)m.sout)[dst[q]] = ((const uint16_t*)SA)[i];
-        }
-      }
-      // ---- subset offsets of the big children, at the segment starts
-      // (each row holds r + 1 words below off_cap, checked when it was handed out)
-      if (want_off && explicit_sid) {
-        // thread tid checks positions 4 tid .. 4 tid + 3 against the one before
-        // each, reading the staged ids; only a warp holding a subset change or
-        // the cell's last point goes on, taking the left rank of a position
-        // from its block's count scan and left-flag ballot
-        const uint32_t r = m.r, i0 = 4u * (uint32_t)tid;
-        uint32_t v[5];
-        v[0] = i0 == 0u ? prev_sub : sid_of(i0 - 1u);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[j + 1] = i0 + j < mcnt ? sid_of(i0 + j) : v[j];
-        if (i0 < mcnt && i0 + 4u >= mcnt) s_carry = v[4];  // the sub-tile's last subset
-        bool any = false;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) any |= i0 + j < mcnt && (v[j] != v[j + 1] || m.sub + i0 + j + 1u == ccount);
-        if (__any_sync(0xffffffffu, any)) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t i = i0 + j;
-            const uint32_t blk = ((i / kCT) * kCW + ((i % kCT) >> 5)) & 31u;  // i < kMaxItems kCT
-            const uint32_t lr = __shfl_sync(0xffffffffu, wexc, blk) +
-                                __popc((&wbal[0][0])[blk] & ((1u << (i & 31u)) - 1u));
-            if (i >= mcnt) continue;
-            const uint32_t p = m.sub + i, lk = lnext - cbeg + lr;  // left points of the cell before i
-            for (int32_t u = (int32_t)v[j] + 1; u <= (int32_t)v[j + 1]; ++u) {
-              if (m.row[0] != kNoRow) s.off_next[m.row[0] + u] = lk;
-              if (m.row[1] != kNoRow) s.off_next[m.row[1] + u] = p - lk;
-            }
-            if (p + 1 == ccount)
-              for (uint32_t u = v[j + 1] + 1; u <= r; ++u) {
-                if (m.row[0] != kNoRow) s.off_next[m.row[0] + u] = L;
-                if (m.row[1] != kNoRow) s.off_next[m.row[1] + u] = ccount - L;
-              }
+      // ---- subset offsets of the children: each segment start off[u] = p of
+      // the cell that lies in this sub-tile (the cell's end in its last one)
+      // becomes the left child's start, the left points before p, and the
+      // right child's, p minus that (rows of r + 1 words, checked against
+      // their pool when they were handed out)
+      if (want_off) {
+        uint32_t* const row0 = m.row[0];
+        uint32_t* const row1 = m.row[1];
+        for (uint32_t ub = m.u0; ub < m.u1; ub += kCT) {
+          const uint32_t u = ub + (uint32_t)tid;
+          if (ub != m.u0) u_pos = u < m.u1 ? __ldg(m.off + u) : 0xffffffffu;
+          const uint32_t i = u_pos - m.sub;  // wraps for starts before the sub-tile
+          const bool end = u_pos == ccount && m.sub + mcnt == ccount;
+          const bool mine = u < m.u1 && u_pos >= m.sub && (i < mcnt || end);
+          if (!__any_sync(0xffffffffu, mine)) continue;
+          const uint32_t blk = min(i >> 5, 31u);  // i < 32 kMaxItems kCW where it counts
+          uint32_t lk = lnext - cbeg + __shfl_sync(0xffffffffu, wexc, blk);
+          if (mine) {
+            lk = end ? L : lk + (uint32_t)__popc((&wbal[0][0])[blk] & ((1u << (i & 31u)) - 1u));
+            if (row0) row0[u] = lk;
+            if (row1) row1[u] = u_pos - lk;
           }
-        }
-      } else if (want_off) {
-        const uint32_t r = m.r;
-#pragma unroll
-        for (int q = 0; q < kMaxItems; ++q) {
-          const uint32_t i = tid + q * kCT;
-          const uint32_t p = m.sub + i;  // position in the cell
-          int32_t sp = __shfl_up_sync(0xffffffffu, (int32_t)sv[q], 1);
-          if (lane == 0)
-            sp = (int32_t)(warp > 0 ? sedge[q][warp - 1] : (q > 0 ? sedge[q - 1][kCW - 1] : prev_sub));
-          if (i >= mcnt) continue;
-          if (i + 1 == mcnt) s_carry = sv[q];
-          if ((int32_t)sv[q] != sp)
-            for (uint32_t u = (uint32_t)(sp + 1); u <= sv[q]; ++u) {
-              if (m.row[0] != kNoRow) s.off_next[m.row[0] + u] = lrk[q];
-              if (m.row[1] != kNoRow) s.off_next[m.row[1] + u] = p - lrk[q];
-            }
-          if (p + 1 == ccount)
-            for (uint32_t u = sv[q] + 1; u <= r; ++u) {
-              if (m.row[0] != kNoRow) s.off_next[m.row[0] + u] = L;
-              if (m.row[1] != kNoRow) s.off_next[m.row[1] + u] = ccount - L;
-            }
         }
       }
       lnext += nL;
@@ -592,28 +530,55 @@ __global__ void __launch_bounds__(kST, 2) k_scatter_tma(const TreeDev* trees, St
 
 }  // namespace
 
-template <int kD>
+// Dynamic shared memory of an instance for trees of d coordinates (kD = 0:
+// the most a mix can need).
+constexpr uint32_t scatter_smem(int kD) { return kD > 0 ? 2u * buf_bytes(kD, sub_tile(kD)) : kScatterSmemBytes; }
+
+template <int kD, bool kMM>
 cudaError_t prepare_one() {
-  return cudaFuncSetAttribute(k_scatter_tma<kD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmemBytes);
+  return cudaFuncSetAttribute(k_scatter_tma<kD, kMM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)scatter_smem(kD));
 }
 
-cudaError_t prepare_scatter_kernel() {
-  for (cudaError_t e : {prepare_one<0>(), prepare_one<2>(), prepare_one<3>(), prepare_one<8>(), prepare_one<16>()})
+template <int kD, bool kMM>
+void launch_one(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t sms, cudaStream_t st) {
+  // two waves of resident CTAs, each taking a contiguous range of tiles
+  const uint32_t grid = std::max<uint32_t>(1, std::min(max_tiles, sms * 2u * (uint32_t)scatter_ctas(kD, kMM)));
+  k_scatter_tma<kD, kMM><<<grid, kST, scatter_smem(kD), st>>>(trees, s);
+}
+
+template <bool kMM>
+cudaError_t prepare_all() {
+  for (cudaError_t e : {prepare_one<0, kMM>(), prepare_one<2, kMM>(), prepare_one<3, kMM>(), prepare_one<8, kMM>(),
+                        prepare_one<16, kMM>()})
     if (e != cudaSuccess) return e;
   return cudaSuccess;
 }
 
-void launch_scatter(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t grid_cap,
-                    uint64_t points, int uniform_d, cudaStream_t st) {
-  TraceScope ts(K_PART_SCATTER, st, points);
-  const uint32_t grid = std::max<uint32_t>(1, std::min(max_tiles, grid_cap));
+template <bool kMM>
+void launch_d(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t sms, int uniform_d,
+              cudaStream_t st) {
   switch (uniform_d) {
-    case 2: k_scatter_tma<2><<<grid, kST, kScatterSmemBytes, st>>>(trees, s); break;
-    case 3: k_scatter_tma<3><<<grid, kST, kScatterSmemBytes, st>>>(trees, s); break;
-    case 8: k_scatter_tma<8><<<grid, kST, kScatterSmemBytes, st>>>(trees, s); break;
-    case 16: k_scatter_tma<16><<<grid, kST, kScatterSmemBytes, st>>>(trees, s); break;
-    default: k_scatter_tma<0><<<grid, kST, kScatterSmemBytes, st>>>(trees, s); break;
+    case 2: launch_one<2, kMM>(trees, s, max_tiles, sms, st); break;
+    case 3: launch_one<3, kMM>(trees, s, max_tiles, sms, st); break;
+    case 8: launch_one<8, kMM>(trees, s, max_tiles, sms, st); break;
+    case 16: launch_one<16, kMM>(trees, s, max_tiles, sms, st); break;
+    default: launch_one<0, kMM>(trees, s, max_tiles, sms, st); break;
   }
+}
+
+cudaError_t prepare_scatter_kernel() {
+  const cudaError_t e = prepare_all<false>();
+  return e != cudaSuccess ? e : prepare_all<true>();
+}
+
+void launch_scatter(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t sms, uint64_t points,
+                    int uniform_d, bool any_widest, cudaStream_t st) {
+  TraceScope ts(K_PART_SCATTER, st, points);
+  if (any_widest)
+    launch_d<true>(trees, s, max_tiles, sms, uniform_d, st);
+  else
+    launch_d<false>(trees, s, max_tiles, sms, uniform_d, st);
 }
 
 }  // namespace kdt

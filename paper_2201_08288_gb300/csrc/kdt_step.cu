@@ -17,9 +17,9 @@
 //   4. per cell: the count-weighted lower median of the segment medians;
 //   5. children sizes from per-tile counts and a per-cell scan of them; the
 //      children are classified (terminal / small / big) before the move;
-//   6. stable partition of all d columns, the permutation and the subset ids
-//      around the split (key <= split to the left); the scatter also writes
-//      the big children's subset offsets.
+//   6. stable partition of all d columns and the permutation around the split
+//      (key <= split to the left); the scatter also writes the big children's
+//      subset offsets.
 // Work is split into tiles of kTile points of one cell; a thread owns kItems
 // points of a tile (strided by the block size, so every load is coalesced)
 // and issues all of its loads before it uses any of them.
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kTileThreads) k_ps_count(const TreeDev* trees,
 #pragma unroll
     for (int q = 0; q < kItems; ++q) {
       const uint32_t i = tl.y + threadIdx.x + q * kTileThreads;
-      sub[q] = i < end ? subset_of(t, t.sid_in, 0u, (int64_t)i) : 0xffffffffu;
+      sub[q] = i < end ? subset_of(t, i) : 0xffffffffu;
     }
 #pragma unroll
     for (int q = 0; q < kItems; ++q)
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, St
 #pragma unroll
   for (int q = 0; q < kPsItems; ++q) {
     const uint32_t i = i0 + threadIdx.x + q * kPsThreads;
-    sub[q] = i < end ? (expl ? subset_of(t, t.sid_in, 0u, (int64_t)i) : i % r) : 0xffffffffu;
+    sub[q] = i < end ? subset_of(t, i) : 0xffffffffu;
   }
 #pragma unroll
   for (int q = 0; q < kPsItems; ++q) lp[q] = sub[q] != 0xffffffffu ? atomic_add_shared(&loff[sub[q]], 1u) : 0u;
@@ -363,13 +363,6 @@ __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, St
   }
   pass([&](int q) { return i0 + threadIdx.x + q * kPsThreads; },
        [&](uint32_t dst, uint32_t v) { t.pbuf[1][dst] = v; });
-  if (expl) {
-    if (t.sid_bytes == 1)
-      pass([&](int q) { return sub[q]; }, [&](uint32_t dst, uint32_t v) { ((uint8_t*)t.sbuf[1])[dst] = (uint8_t)v; });
-    else
-      pass([&](int q) { return sub[q]; },
-           [&](uint32_t dst, uint32_t v) { ((uint16_t*)t.sbuf[1])[dst] = (uint16_t)v; });
-  }
 }
 
 // ------------------------------------------------------- widest spread
@@ -520,9 +513,10 @@ __device__ __forceinline__ uint32_t kload(const uint32_t* p) { return ord_key(__
 
 // One CTA per cell (after its key coordinate is known): size and first key
 // of every (cell, subset) segment from the cell's subset offsets, and the
-// lists of segments for the warp and CTA selects. Offsets are clamped to the
-// cell, so a damaged table cannot send a later kernel outside it (it is
-// reported instead).
+// lists of segments for the warp and CTA selects; for each of the cell's
+// tiles, the first segment start in it (the scatter turns the starts in a
+// tile into the children's). Offsets are clamped to the cell, so a damaged
+// table cannot send a later kernel outside it (it is reported instead).
 __device__ __forceinline__ void segs_cell(const TreeDev* trees, const StepDev& s, uint32_t c) {
   const Cell cell = s.cells[c];
   const TreeDev& t = trees[cell.tree];
@@ -531,6 +525,19 @@ __device__ __forceinline__ void segs_cell(const TreeDev* trees, const StepDev& s
   const uint32_t g0 = s.seg_base[c];
   const uint32_t* kc = key_column(t, cell, s.kdim[c]) + cell.begin;
   if (threadIdx.x == 0 && (off[0] != 0u || off[r] != cell.count)) set_status(t, ST_INTERNAL);
+  // tiles that start in (off[j], off[j + 1]] have start j + 1 as their first
+  // (the first tile, at 0, has start 0); with fewer subsets than threads
+  // several threads share a segment's tiles
+  const uint32_t tb = s.tile_base[c], nt = s.tile_base[c + 1] - tb;
+  if (threadIdx.x == 0 && nt > 0u) s.tile_seg[tb] = 0;
+  if (nt > 1u) {
+    const uint32_t per = max(1u, blockDim.x / r);
+    for (uint32_t q = threadIdx.x; q < r * per; q += blockDim.x) {
+      const uint32_t j = q / per, a = min(off[j], cell.count), b = min(off[j + 1], cell.count);
+      for (uint32_t k = a / (uint32_t)kTile + 1u + q % per; k < nt && k * (uint32_t)kTile <= b; k += per)
+        s.tile_seg[tb + k] = j + 1u;
+    }
+  }
   for (uint32_t j = threadIdx.x; j < r; j += blockDim.x) {
     const uint32_t a = min(off[j], cell.count), b = min(off[j + 1], cell.count);
     if (b < a) set_status(t, ST_INTERNAL);
@@ -1389,12 +1396,19 @@ __device__ __forceinline__ void classify_cell(const TreeDev* trees, const StepDe
       set_status(t, ST_LEVEL_CAP);
     } else {
       ++live_delta;
-      const Cell child{cb[side], cc[side], heap, cell.tree, (int8_t)level, (int8_t)stall, (int16_t)-1};
+      Cell child{cb[side], cc[side], heap, cell.tree, (int8_t)level, (int8_t)stall, (int16_t)-1};
       if (cc[side] <= (uint32_t)t.small_max) {
         if (atomicAdd(s.small_total, 1u) < s.small_cap) {
           // the two ends of the queue never meet: at most small_cap cells get a slot
           const uint32_t slot = t.sub_wide ? s.small_cap - 1u - atomicAdd(s.small_count_w, 1u)
                                            : atomicAdd(s.small_count, 1u);
+          // explicit ids: a row of subset offsets where it is shorter than the
+          // cell and there is room
+          if (t.subset_mode == SUB_EXPLICIT && (uint32_t)t.r < cc[side]) {
+            const uint32_t words = (uint32_t)t.r + 1u;
+            const uint32_t row = atomicAdd(s.small_off_used, words);
+            if (row < s.small_off_cap && words <= s.small_off_cap - row) child.row = row;
+          }
           s.small[slot] = child;
           cr = make_uint2(kNoRow, slot);  // its widest coordinate is picked with the big children's
         } else {
@@ -1523,7 +1537,7 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
       k_part_scan<<<nc, 1024, 0, st>>>(s);
   }
   { TraceScope ts(K_CLASSIFY, st); k_classify<<<cells_grid(256, sms * 4u), 256, 0, st>>>(trees, s); }
-  launch_scatter(trees, s, max_tiles, 2 * sms, points, uniform_d, st);
+  launch_scatter(trees, s, max_tiles, sms / 2, points, uniform_d, any_widest, st);
   if (any_widest && s.shards) launch_shard_minmax(trees, s, nc, st);
   if (any_widest) {
     TraceScope ts(K_CHILD_DIMS, st);

@@ -219,7 +219,7 @@ __device__ __forceinline__ uint32_t warp_wsel_bits(uint32_t cnt, uint32_t rank, 
 template <bool kWide>
 __global__ void __launch_bounds__(T, (kWide ? kSubWide : kSubNarrow).ctas)
 k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t* count_dev, uint32_t reversed,
-          uint32_t* head, LCell* slices, uint32_t slice_cells, uint32_t probe_tries) {
+          const uint32_t* small_off, uint32_t* head, LCell* slices, uint32_t slice_cells, uint32_t probe_tries) {
   constexpr SubtreeShape kSh = kWide ? kSubWide : kSubNarrow;
   constexpr int kQ = kSh.q, kCells = kSh.cells;
   extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -337,34 +337,38 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
         if (ok) S.cols[(size_t)l * stride + ph + (idx - b0)] = src_of(l)[idx];
       }
       __syncthreads();
-      // explicit subset ids are read from global memory while the bulk copies
-      // run (neither touches the other's shared memory), eight loads in
-      // flight per thread
-      const void* SID = src_sid(t, c.level);
-      const bool expl = t.subset_mode == SUB_EXPLICIT;
-      for (uint32_t i0 = tid; i0 < N; i0 += 8 * T) {
-        uint32_t v[8];
-        if (expl) {
-#pragma unroll
+      // the points' subsets, while the bulk copies run (neither touches the
+      // other's shared memory): filled in from the cell's subset offsets if it
+      // has them (with fewer subsets than threads, several threads share a
+      // segment), else from the original indices, eight loads in flight per
+      // thread, explicit ids gathered from the caller's array (a 32-byte
+      // sector per id: for 2^27 points in cells of 1024 the gather cost 1.7 ms
+      // more than the rows)
+      if (c.row != kNoRow) {
+        const uint32_t* row = small_off + c.row;
+        const uint32_t per = max(1u, (uint32_t)T / (uint32_t)r);
+        for (uint32_t q = tid; q < (uint32_t)r * per; q += T) {
+          const uint32_t u = q / per, a = min(row[u], N), b = min(row[u + 1], N);
+          for (uint32_t i = a + q % per; i < b; i += per) S.sid[i] = (uint16_t)u;
+        }
+        for (uint32_t i = tid; i < N; i += T) S.cellid[i] = 0;
+      } else {
+        for (uint32_t i0 = tid; i0 < N; i0 += 8 * T) {
+          uint32_t v[8];
+  #pragma unroll
           for (int q = 0; q < 8; ++q) {
             const uint32_t i = i0 + (uint32_t)q * T;
-            v[q] = i >= N ? 0u
-                          : (t.sid_bytes == 1 ? (uint32_t)((const uint8_t*)SID)[(int64_t)b0 + i]
-                                              : (uint32_t)((const uint16_t*)SID)[(int64_t)b0 + i]);
+            v[q] = i < N ? (P ? P[b0 + i] : b0 + i) : 0u;
           }
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const uint32_t i = i0 + (uint32_t)q * T;
-          if (i >= N) break;
-          if (expl) {
-            if (v[q] >= (uint32_t)r) {  // an id outside [0, r): reported, replaced by 0
-              set_status(t, ST_INVALID_ARG);
-              v[q] = 0;
-            }
+  #pragma unroll
+          for (int q = 0; q < 8; ++q) v[q] = i0 + (uint32_t)q * T < N ? subset_of(t, v[q]) : 0u;
+  #pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const uint32_t i = i0 + (uint32_t)q * T;
+            if (i >= N) break;
             S.sid[i] = (uint16_t)v[q];
+            S.cellid[i] = 0;
           }
-          S.cellid[i] = 0;
         }
       }
       // one thread waits for the copies (a waiting thread keeps issuing
@@ -397,9 +401,6 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
         }
       }
       if (nan) set_status(t, ST_NAN_INPUT);
-      if (!expl)
-        for (uint32_t i = tid; i < N; i += T)
-          S.sid[i] = (uint16_t)subset_of(t, SID, P ? P[b0 + i] : b0 + i, (int64_t)b0 + i);
       // The root of a small tree arrives in index order: put it in subset
       // order (counting sort; order inside a subset is immaterial). Every
       // other cell is in subset order already.
@@ -908,8 +909,8 @@ void launch_iota(uint32_t* out, uint32_t n, cudaStream_t st) {
 }
 
 // The kernel instance of a shape.
-using SubtreeKernel = void (*)(const TreeDev*, const Cell*, uint32_t, const uint32_t*, uint32_t, uint32_t*, LCell*,
-                               uint32_t, uint32_t);
+using SubtreeKernel = void (*)(const TreeDev*, const Cell*, uint32_t, const uint32_t*, uint32_t, const uint32_t*,
+                               uint32_t*, LCell*, uint32_t, uint32_t);
 SubtreeKernel subtree_kernel(const SubtreeShape& sh) {
   return sh.q == kSubWide.q ? k_subtree<true> : k_subtree<false>;
 }
@@ -924,14 +925,14 @@ cudaError_t prepare_subtree_kernel() {
 }
 
 void launch_subtree(const SubtreeShape& sh, const TreeDev* trees, const Cell* list, uint32_t count,
-                    const uint32_t* count_dev, bool reversed, uint32_t* head, LCell* slices, uint32_t slice_cells,
-                    uint32_t grid, uint64_t points, cudaStream_t st) {
+                    const uint32_t* count_dev, bool reversed, const uint32_t* small_off, uint32_t* head,
+                    LCell* slices, uint32_t slice_cells, uint32_t grid, uint64_t points, cudaStream_t st) {
   if (count == 0 || grid == 0) return;
   cudaMemsetAsync(head, 0, sizeof(uint32_t), st);
   const uint32_t probe = fault_take(KDT_FAULT_WAIT) ? 1024u : 0u;
   TraceScope ts(K_SUBTREE, st, points);
-  subtree_kernel(sh)<<<grid, T, sh.smem, st>>>(trees, list, count, count_dev, reversed ? 1u : 0u, head, slices,
-                                               slice_cells, probe);
+  subtree_kernel(sh)<<<grid, T, sh.smem, st>>>(trees, list, count, count_dev, reversed ? 1u : 0u, small_off, head,
+                                               slices, slice_cells, probe);
 }
 
 void launch_finalize_many(const TreeDev* trees, const uint32_t* slots, uint32_t nslots, uint32_t max_records,
