@@ -25,7 +25,7 @@ enum Word {
 // a graph-driven run's iterations (two level steps each) before it gives up
 constexpr uint32_t kGraphIterMax = KDT_MAX_LEVELS + 4;
 // Per-slot words: [which][max_trees].
-enum SlotWord { S_TERM = 0, S_STATUS, S_LEVELS, S_LIVE, S_COUNT };
+enum SlotWord { S_TERM = 0, S_STATUS, S_LEVELS, S_LIVE, S_HUGE, S_COUNT };
 
 int device_sms() {
   int dev = 0, sms = 0;
@@ -133,7 +133,6 @@ TreePlan plan_tree(const kdt_params& p0, bool no_subtree) {
   t.root_off = take(((size_t)p.r + 1) * 4);
   t.root_cur = take((size_t)p.r * 4);
   t.huge = take(t.huge_cap * 4);
-  t.words = take(16);
   t.bytes = off;
   return t;
 }
@@ -181,7 +180,8 @@ StepPlan plan_step(const StepNeeds& needs) {
   s.trees = take((size_t)mt * sizeof(TreeDev));
   s.words = take(W_COUNT * 4);
   s.slot_words = take((size_t)S_COUNT * mt * 4);
-  s.slots_list = take((size_t)mt * 2 * 4);
+  s.slots_list = take(((size_t)mt * 2 + 1) * 4);  // SlotChunks
+  s.admits = take(mt > (uint32_t)kAdmitFew ? (size_t)mt * sizeof(AdmitRec) : 0);
   s.big[0] = take((size_t)s.maxB * sizeof(Cell));
   s.big[1] = take((size_t)s.maxB * sizeof(Cell));
   s.small = take((size_t)s.cap_small * sizeof(Cell));
@@ -265,26 +265,26 @@ Engine::Engine(const StepPlan& plan, uint8_t* base, cudaStream_t st) : plan_(pla
   s_.crow = (uint2*)(base + plan.crow);
   const uint32_t mt = std::max<uint32_t>(plan.needs.max_trees, 1);
   host_.assign(mt, TreeHost{});
-  leafsort_.assign(mt, 0);
-  wide_.assign(mt, 0);
+  recs_.assign(mt, 0);
+  sorts_.assign(mt, 0);
 }
 
 kdt_status Engine::reset() {
   ENGINE_TRY(prepare_subtree_kernel());
-  ENGINE_TRY(prepare_scatter_kernel());
+  ENGINE_TRY(prepare_scatter_kernel(uniform_d(), plan_.needs.widest));
   ENGINE_TRY(prepare_step_kernels());
   const uint32_t mt = std::max<uint32_t>(plan_.needs.max_trees, 1);
-  ENGINE_TRY(cudaMemsetAsync(words_, 0, W_COUNT * 4, st_));
-  ENGINE_TRY(cudaMemsetAsync(slot_words_, 0, (size_t)S_COUNT * mt * 4, st_));
+  // the engine words and, right behind them in the plan, the slots'
+  ENGINE_TRY(cudaMemsetAsync(words_, 0, plan_.slot_words - plan_.words + (size_t)S_COUNT * mt * 4, st_));
   cur_ = 0;
   big_count_ = small_count_ = small_count_w_ = 0;
   big_points_ = small_points_ = 0;
   root_dims_ = false;
-  pending_big_.clear();
-  pending_small_.clear();
-  pending_small_w_.clear();
+  pending_.clear();
   return KDT_OK;
 }
+
+int Engine::uniform_d() const { return plan_.needs.min_d == plan_.needs.max_d ? plan_.needs.max_d : 0; }
 
 kdt_status Engine::admit(uint32_t slot, const float* points, const kdt_params& p0, const TreePlan& tp,
                          uint8_t* tb, uint32_t* out_perm, float* out_vals, int8_t* out_dims, int64_t* out_offs) {
@@ -306,6 +306,7 @@ kdt_status Engine::admit(uint32_t slot, const float* points, const kdt_params& p
   h.stall_limit = p.key_rule == KDT_KEY_CYCLIC ? p.d : 1;
   h.sid_bytes = tp.sid_bytes;
   h.small_max = tp.small_max;
+  h.leafsort = tp.leafsort ? 1 : 0;
   h.presorted = tp.presorted ? 1 : 0;
   h.contig_mul = p.n > 0 ? ((uint64_t)p.r << 32) / (uint64_t)p.n : 0;
   h.x_in = points;
@@ -317,7 +318,7 @@ kdt_status Engine::admit(uint32_t slot, const float* points, const kdt_params& p
   h.root_off = (uint32_t*)(tb + tp.root_off);
   h.root_cur = (uint32_t*)(tb + tp.root_cur);
   h.huge = (uint32_t*)(tb + tp.huge);
-  h.huge_count = (uint32_t*)(tb + tp.words);
+  h.huge_count = slot_words_ + (size_t)S_HUGE * mt + slot;
   h.huge_cap = (uint32_t)std::min<uint64_t>(tp.huge_cap, 0xffffffffull);
   h.out_perm = out_perm;
   h.out_vals = out_vals;
@@ -329,77 +330,72 @@ kdt_status Engine::admit(uint32_t slot, const float* points, const kdt_params& p
   h.status = (int32_t*)(slot_words_ + (size_t)S_STATUS * mt + slot);
   h.levels = (int32_t*)(slot_words_ + (size_t)S_LEVELS * mt + slot);
   h.live = (int32_t*)(slot_words_ + (size_t)S_LIVE * mt + slot);
-  ENGINE_TRY(cudaMemcpyAsync(trees_ + slot, &h, sizeof(h), cudaMemcpyHostToDevice, st_));
-  for (int w = 0; w < S_COUNT; ++w)
-    ENGINE_TRY(cudaMemsetAsync(slot_words_ + (size_t)w * mt + slot, 0, 4, st_));
-  ENGINE_TRY(cudaMemsetAsync(h.huge_count, 0, 4, st_));
-  leafsort_[slot] = tp.leafsort ? 1 : 0;
-  wide_[slot] = tp.sub_wide ? 1 : 0;
   // after the build the tree's working buffers are free: the global leaf-sort
   // passes use pbuf[0] as their second buffer and xbuf[0] for tile tables
-  host_[slot] = TreeHost{(uint64_t)p.n, out_perm, h.pbuf[0], (void*)h.xbuf[0], (size_t)p.d * p.n * 4};
-
+  host_[slot] = TreeHost{(uint64_t)p.n, out_perm, h.pbuf[0], (void*)h.xbuf[0], (size_t)p.d * p.n * 4, h.huge,
+                         h.huge_cap, h.terms, h.term_cap};
   const uint64_t n = (uint64_t)p.n;
-  const Cell root{0u, (uint32_t)n, 0u, (int32_t)slot, 0, 0, -1};
   const bool root_terminal = p.depth > 0 ? (n == 0) : (n <= (uint64_t)p.leaf_size);
-  if (root_terminal) {
-    const TermRec tr{0u, (uint32_t)n, 0u, 0};
-    const uint32_t one = 1;
-    ENGINE_TRY(cudaMemcpyAsync(h.terms, &tr, sizeof(tr), cudaMemcpyHostToDevice, st_));
-    ENGINE_TRY(cudaMemcpyAsync(h.term_count, &one, 4, cudaMemcpyHostToDevice, st_));
-    launch_iota(out_perm, (uint32_t)n, st_);
-    ENGINE_TRY(cudaGetLastError());
-    return KDT_OK;
+  // terminal records to expect (sizes the launches that walk them; those take
+  // any number): a complete tree's leaves, or about two per leaf_size points
+  const uint64_t leaves = (uint64_t)1 << tp.L_cap;
+  recs_[slot] = (uint32_t)(p.depth > 0 ? leaves : std::min<uint64_t>(leaves, 2 * n / (uint64_t)p.leaf_size + 2));
+  sorts_[slot] = tp.leafsort ? 1 : 0;
+  Pending pe;
+  pe.rec = AdmitRec{h, slot, root_terminal ? 1u : 0u, nullptr};
+  pe.list = root_terminal ? kListNone
+            : !(n <= (uint64_t)tp.small_max && !tp.presorted) ? kListBig
+            : tp.sub_wide ? kListSmallWide : kListSmall;
+  if (pe.list == kListBig && p.key_rule == KDT_KEY_WIDEST_SPREAD) root_dims_ = true;
+  pending_.push_back(pe);
+  return KDT_OK;
+}
+
+// The admitted trees go to the device together: their records (one copy, or
+// none for a few), then one kernel that writes every table entry they need.
+kdt_status Engine::flush_admits(bool* has_big_roots) {
+  *has_big_roots = false;
+  if (pending_.empty()) return KDT_OK;
+  std::vector<AdmitRec>& recs = admitted_;  // kept: the copy below may still read it when this returns
+  recs.clear();
+  recs.reserve(pending_.size());
+  uint64_t big = 0, small = 0;
+  for (const Pending& pe : pending_) {
+    big += pe.list == kListBig;
+    small += pe.list == kListSmall || pe.list == kListSmallWide;
   }
-  const int32_t one = 1;
-  ENGINE_TRY(cudaMemcpyAsync(h.live, &one, 4, cudaMemcpyHostToDevice, st_));
-  if (n <= (uint64_t)tp.small_max && !tp.presorted) {
-    (tp.sub_wide ? pending_small_w_ : pending_small_).push_back(root);
-  } else {
-    pending_big_.push_back(root);
-    if (p.key_rule == KDT_KEY_WIDEST_SPREAD) root_dims_ = true;
+  if (big_count_ + big > plan_.maxB || (uint64_t)small_count_ + small_count_w_ + small > plan_.cap_small)
+    return KDT_ERR_CAPACITY;
+  for (Pending& pe : pending_) {
+    const uint64_t n = (uint64_t)pe.rec.tree.n;
+    if (pe.list == kListBig) {
+      pe.rec.root_dst = big_[cur_] + big_count_++;
+      big_points_ += n;
+    } else if (pe.list == kListSmall) {
+      pe.rec.root_dst = small_ + small_count_++;
+      small_points_ += n;
+    } else if (pe.list == kListSmallWide) {  // the back of the queue runs downwards
+      pe.rec.root_dst = small_ + plan_.cap_small - 1 - small_count_w_++;
+      small_points_ += n;
+    }
+    recs.push_back(pe.rec);
   }
+  *has_big_roots = big > 0;
+  pending_.clear();
+  ENGINE_TRY(launch_admit(recs, (AdmitRec*)(base_ + plan_.admits), trees_, st_));
   return KDT_OK;
 }
 
 kdt_status Engine::tick() {
   // new roots join the lists of this tick
-  const bool has_roots = !pending_big_.empty();
-  if (!pending_big_.empty()) {
-    if (big_count_ + pending_big_.size() > plan_.maxB) return KDT_ERR_CAPACITY;
-    ENGINE_TRY(cudaMemcpyAsync(big_[cur_] + big_count_, pending_big_.data(), pending_big_.size() * sizeof(Cell),
-                               cudaMemcpyHostToDevice, st_));
-    for (const Cell& c : pending_big_) big_points_ += c.count;
-    big_count_ += (uint32_t)pending_big_.size();
-    pending_big_.clear();
-  }
-  if (!pending_small_.empty() || !pending_small_w_.empty()) {
-    if ((uint64_t)small_count_ + small_count_w_ + pending_small_.size() + pending_small_w_.size() > plan_.cap_small)
-      return KDT_ERR_CAPACITY;
-    if (!pending_small_.empty())
-      ENGINE_TRY(cudaMemcpyAsync(small_ + small_count_, pending_small_.data(), pending_small_.size() * sizeof(Cell),
-                                 cudaMemcpyHostToDevice, st_));
-    if (!pending_small_w_.empty()) {
-      // the back of the queue runs downwards: entry j at small[cap - 1 - j]
-      std::reverse(pending_small_w_.begin(), pending_small_w_.end());
-      const size_t m = pending_small_w_.size();
-      ENGINE_TRY(cudaMemcpyAsync(small_ + plan_.cap_small - small_count_w_ - m, pending_small_w_.data(),
-                                 m * sizeof(Cell), cudaMemcpyHostToDevice, st_));
-    }
-    for (const Cell& c : pending_small_) small_points_ += c.count;
-    for (const Cell& c : pending_small_w_) small_points_ += c.count;
-    small_count_ += (uint32_t)pending_small_.size();
-    small_count_w_ += (uint32_t)pending_small_w_.size();
-    pending_small_.clear();
-    pending_small_w_.clear();
-  }
-  const uint32_t sw[5] = {small_count_, small_count_w_, small_count_ + small_count_w_, (uint32_t)small_points_, 0u};
-  ENGINE_TRY(cudaMemcpyAsync(words_ + W_SMALL, sw, sizeof(sw), cudaMemcpyHostToDevice, st_));
+  bool has_roots = false;
+  const kdt_status f = flush_admits(&has_roots);
+  if (f != KDT_OK) return f;
 
   if (big_count_ > 0) {
-    ENGINE_TRY(cudaMemsetAsync(words_ + W_NEXTBIG, 0, 4, st_));
-    ENGINE_TRY(cudaMemsetAsync(words_ + W_BIGPTS, 0, 4, st_));
-    ENGINE_TRY(cudaMemsetAsync(words_ + W_OFFUSED, 0, 4, st_));
+    s_.init_small = small_count_;
+    s_.init_small_w = small_count_w_;
+    s_.init_small_points = (uint32_t)small_points_;
     s_.cells = big_[cur_];
     s_.ncells = big_count_;
     s_.next_big = big_[cur_ ^ 1];
@@ -422,7 +418,7 @@ kdt_status Engine::tick() {
     s_.warp_max = tune.warp_max;
     launch_big_step(trees_, s_, tiles_bound, (uint32_t)nseg_bound, plan_.bigseg_cap, has_roots, root_dims_,
                     plan_.needs.widest, plan_.needs.max_d,
-                    plan_.needs.min_d == plan_.needs.max_d ? plan_.needs.max_d : 0, tune, big_points_,
+                    uniform_d(), tune, big_points_,
                     plan_.grid_step, st_, plan_.needs.fourier);
     ENGINE_TRY(cudaGetLastError());
     root_dims_ = false;
@@ -497,48 +493,45 @@ kdt_status Engine::finalize(const std::vector<uint32_t>& slots, std::vector<kdt_
   status->assign(slots.size(), KDT_OK);
   levels->assign(slots.size(), 0);
   if (slots.empty()) return KDT_OK;
-  // trees with an error get no finalize (their outputs are undefined)
-  std::vector<int32_t> st(mt), lv(mt);
-  std::vector<uint32_t> tc(mt);
-  ENGINE_TRY(cudaMemcpyAsync(tc.data(), slot_words_ + (size_t)S_TERM * mt, (size_t)mt * 4,
-                             cudaMemcpyDeviceToHost, st_));
-  ENGINE_TRY(cudaMemcpyAsync(st.data(), slot_words_ + (size_t)S_STATUS * mt, (size_t)mt * 4,
-                             cudaMemcpyDeviceToHost, st_));
-  ENGINE_TRY(cudaMemcpyAsync(lv.data(), slot_words_ + (size_t)S_LEVELS * mt, (size_t)mt * 4,
-                             cudaMemcpyDeviceToHost, st_));
-  ENGINE_TRY(cudaStreamSynchronize(st_));
-  std::vector<uint32_t> ok;
-  uint32_t max_rec = 0;
-  for (uint32_t s : slots)
-    if (st[s] == ST_OK) {
-      ok.push_back(s);
-      max_rec = std::max(max_rec, tc[s]);
+  bool has_roots = false;  // trees that were terminal from the start may not have met a tick
+  const kdt_status f = flush_admits(&has_roots);
+  if (f != KDT_OK) return f;
+  // offsets, sentinels and the leaves' order (trees with an error get none of
+  // it: their outputs are undefined); the kernels read the trees' statuses and
+  // record counts themselves, so nothing is waited for in between
+  SlotChunks sc{nullptr, (uint32_t)slots.size(), 0};
+  std::vector<uint32_t> list;
+  if (slots.size() == 1 && slots[0] == 0) {
+    sc.chunks = std::max<uint32_t>(1, std::min<uint32_t>((recs_[0] + 7) / 8, 8192));
+  } else {
+    list = slots;
+    for (uint32_t s : slots) {
+      list.push_back(sc.chunks);
+      sc.chunks += std::max<uint32_t>(1, std::min<uint32_t>((recs_[s] + kChunkRecords - 1) / kChunkRecords, 2048));
     }
-  std::vector<uint32_t> sorted;  // trees kept in subset order: their leaves need the leaf sort
-  for (uint32_t s : ok)
-    if (leafsort_[s]) sorted.push_back(s);
-  if (!ok.empty()) {
-    ENGINE_TRY(cudaMemcpyAsync(slots_list_, ok.data(), ok.size() * 4, cudaMemcpyHostToDevice, st_));
-    launch_finalize_many(trees_, slots_list_, (uint32_t)ok.size(), max_rec, st_);
-    ENGINE_TRY(cudaGetLastError());
-    if (!sorted.empty()) {
-      // the slot list is read by the finalize launch above: the sorted slots go after it
-      ENGINE_TRY(cudaMemcpyAsync(slots_list_ + ok.size(), sorted.data(), sorted.size() * 4,
-                                 cudaMemcpyHostToDevice, st_));
-      launch_leaf_sort(trees_, slots_list_ + ok.size(), (uint32_t)sorted.size(), max_rec, st_);
-      ENGINE_TRY(cudaGetLastError());
-    }
-    ENGINE_TRY(cudaStreamSynchronize(st_));
+    list.push_back(sc.chunks);
+    sc.slots = slots_list_;
+    ENGINE_TRY(cudaMemcpyAsync(slots_list_, list.data(), list.size() * 4, cudaMemcpyHostToDevice, st_));
   }
-  for (uint32_t s : sorted) {  // leaves too large for one CTA (shallow trees, cells that stop splitting)
-    TreeDev h;
-    uint32_t nh = 0;
-    ENGINE_TRY(cudaMemcpyAsync(&h, trees_ + s, sizeof(h), cudaMemcpyDeviceToHost, st_));
-    ENGINE_TRY(cudaStreamSynchronize(st_));
-    ENGINE_TRY(cudaMemcpyAsync(&nh, h.huge_count, 4, cudaMemcpyDeviceToHost, st_));
-    ENGINE_TRY(cudaStreamSynchronize(st_));
-    nh = std::min(nh, h.huge_cap);
-    if (nh == 0) continue;
+  launch_finalize_many(trees_, sc, st_);
+  ENGINE_TRY(cudaGetLastError());
+  bool any_sort = false;
+  for (uint32_t s : slots) any_sort = any_sort || sorts_[s];
+  if (any_sort) {
+    launch_leaf_sort(trees_, sc, st_);
+    ENGINE_TRY(cudaGetLastError());
+  }
+  std::vector<uint32_t> words((size_t)S_COUNT * mt);
+  ENGINE_TRY(cudaMemcpyAsync(words.data(), slot_words_, words.size() * 4, cudaMemcpyDeviceToHost, st_));
+  ENGINE_TRY(cudaStreamSynchronize(st_));
+  const uint32_t* tc = words.data() + (size_t)S_TERM * mt;
+  const int32_t* st = (const int32_t*)words.data() + (size_t)S_STATUS * mt;
+  const int32_t* lv = (const int32_t*)words.data() + (size_t)S_LEVELS * mt;
+  const uint32_t* huge = words.data() + (size_t)S_HUGE * mt;
+  for (uint32_t s : slots) {  // leaves too large for one CTA (shallow trees, cells that stop splitting)
+    const TreeHost& h = host_[s];
+    const uint32_t nh = std::min(huge[s], h.huge_cap);
+    if (nh == 0 || st[s] != ST_OK) continue;
     std::vector<uint32_t> idx(nh);
     std::vector<TermRec> all(std::min(tc[s], h.term_cap)), recs;
     ENGINE_TRY(cudaMemcpyAsync(idx.data(), h.huge, (size_t)nh * 4, cudaMemcpyDeviceToHost, st_));
@@ -546,7 +539,7 @@ kdt_status Engine::finalize(const std::vector<uint32_t>& slots, std::vector<kdt_
     ENGINE_TRY(cudaStreamSynchronize(st_));
     for (uint32_t k : idx)
       if (k < all.size()) recs.push_back(all[k]);
-    ENGINE_TRY(leaf_sort_huge(host_[s], recs, st_));
+    ENGINE_TRY(leaf_sort_huge(h, recs, st_));
     ENGINE_TRY(cudaStreamSynchronize(st_));
   }
   for (size_t i = 0; i < slots.size(); ++i) {
@@ -557,12 +550,8 @@ kdt_status Engine::finalize(const std::vector<uint32_t>& slots, std::vector<kdt_
 }
 
 kdt_status Engine::record_tick(int p) {
-  // the counters a step appends to start from zero
-  ENGINE_TRY(cudaMemsetAsync(words_ + W_NC0 + (p ^ 1), 0, 4, st_));
-  ENGINE_TRY(cudaMemsetAsync(words_ + W_BIGPTS, 0, 4, st_));
-  ENGINE_TRY(cudaMemsetAsync(words_ + W_OFFUSED, 0, 4, st_));
-  ENGINE_TRY(cudaMemsetAsync(words_ + W_SMALL, 0, 4 * (W_SMALLOFF - W_SMALL + 1), st_));
   StepDev sd = s_;
+  sd.init_small = sd.init_small_w = sd.init_small_points = 0;
   sd.cells = big_[p];
   sd.ncells = plan_.maxB;  // a capacity: the count is the device word
   sd.ncells_dev = words_ + W_NC0 + p;
@@ -577,7 +566,7 @@ kdt_status Engine::record_tick(int p) {
   sd.bitonic_max = tune.bitonic_max;
   sd.warp_max = tune.warp_max;
   launch_big_step(trees_, sd, plan_.max_tiles, plan_.nseg_cap, plan_.bigseg_cap, false, false, plan_.needs.widest,
-                  plan_.needs.max_d, plan_.needs.min_d == plan_.needs.max_d ? plan_.needs.max_d : 0, tune, 0,
+                  plan_.needs.max_d, uniform_d(), tune, 0,
                   plan_.grid_step, st_, plan_.needs.fourier);
   ENGINE_TRY(cudaGetLastError());
   launch_small(true);
@@ -587,7 +576,7 @@ kdt_status Engine::record_tick(int p) {
 
 kdt_status Engine::run_graph() {
   // the roots' step (presort, root dims) is sized and launched by the host
-  if (!pending_big_.empty() || !pending_small_.empty() || !pending_small_w_.empty()) {
+  if (!pending_.empty()) {
     const kdt_status s = tick();
     if (s != KDT_OK) return s;
   }
@@ -663,8 +652,7 @@ kdt_status Engine::run_graph() {
 }
 
 kdt_status Engine::run_to_completion() {
-  for (int guard = 0; busy() || !pending_big_.empty() || !pending_small_.empty() || !pending_small_w_.empty();
-       ++guard) {
+  for (int guard = 0; busy() || !pending_.empty(); ++guard) {
     if (guard > 2 * KDT_MAX_LEVELS + 4) return KDT_ERR_CUDA;
     const kdt_status s = tick();
     if (s != KDT_OK) return s;

@@ -38,7 +38,7 @@ struct TreePlan {
   uint64_t maxB = 0;      // big cells at one level
   uint64_t cap_small = 0; // small cells over the whole build
   size_t xbuf[2] = {0, 0}, pbuf[2] = {0, 0}, terms = 0, root_off = 0, root_cur = 0,
-         huge = 0, words = 0;
+         huge = 0;
   size_t bytes = 0;
 };
 // no_subtree: every cell stays in the multi-CTA pipeline (a sharded build's
@@ -63,7 +63,7 @@ struct StepPlan {
   // sms: the device's SMs (the subtree kernel's grid is sms x its shape's CTAs)
   uint32_t maxB = 0, cap_small = 0, max_tiles = 0, nseg_cap = 0, bigseg_cap = 0, grid_step = 0, sms = 0, off_cap = 0,
            small_off_cap = 0;
-  size_t trees = 0, words = 0, slot_words = 0, slots_list = 0, big[2] = {0, 0}, small = 0, tile_base = 0,
+  size_t trees = 0, words = 0, slot_words = 0, slots_list = 0, admits = 0, big[2] = {0, 0}, small = 0, tile_base = 0,
          seg_base = 0, tiles = 0, tile_seg = 0, tile_left = 0, tile_loff = 0, tile_mm = 0, child_mm = 0, kdim = 0,
          mkey = 0, lcount = 0, seg_w = 0, seg_key = 0, seg_med = 0, bigseg = 0, midseg = 0, slices = 0,
          off[2] = {0, 0}, obase[2] = {0, 0}, small_off = 0, crow = 0;
@@ -113,8 +113,8 @@ class Engine {
   cudaStream_t st_;
   TreeDev* trees_ = nullptr;      // device [max_trees]
   uint32_t* words_ = nullptr;     // device engine words
-  uint32_t* slot_words_ = nullptr;  // device [4][max_trees]: term_count, status, levels, live
-  uint32_t* slots_list_ = nullptr;  // device [max_trees]
+  uint32_t* slot_words_ = nullptr;  // device [5][max_trees]: term_count, status, levels, live, huge_count
+  uint32_t* slots_list_ = nullptr;  // device [2 max_trees + 1]: SlotChunks
   Cell* big_[2] = {nullptr, nullptr};
   uint32_t* off_[2] = {nullptr, nullptr};
   uint32_t* obase_[2] = {nullptr, nullptr};
@@ -132,10 +132,21 @@ class Engine {
   // The subtree kernel over the small-cell queue: the narrow shape over its
   // front, the wide one over its back (host counts, or the device's).
   void launch_small(bool from_device);
-  std::vector<Cell> pending_big_, pending_small_, pending_small_w_;
-  std::vector<TreeHost> host_;       // per slot: leaf-sort view of a presorted tree
-  std::vector<uint8_t> leafsort_;    // per slot
-  std::vector<uint8_t> wide_;        // per slot: the tree's small cells use the wide shape
+  // Admitted trees whose records are not on the device yet, and the list
+  // their root goes to.
+  enum List { kListNone, kListBig, kListSmall, kListSmallWide };
+  struct Pending {
+    AdmitRec rec;
+    List list;
+  };
+  kdt_status flush_admits(bool* has_big_roots);
+  // The coordinate count of every tree of the forest, 0 if they differ.
+  int uniform_d() const;
+  std::vector<Pending> pending_;
+  std::vector<AdmitRec> admitted_;  // the records of the last flush
+  std::vector<TreeHost> host_;   // per slot: what the global leaf-sort passes need
+  std::vector<uint32_t> recs_;   // per slot: terminal records to expect
+  std::vector<uint8_t> sorts_;   // per slot: the tree's leaves are sorted
 };
 
 }  // namespace kdt

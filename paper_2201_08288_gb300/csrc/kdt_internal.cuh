@@ -67,6 +67,7 @@ struct TreeDev {
   int32_t stall_limit; // d (cyclic) or 1 (widest)
   int32_t sid_bytes;   // explicit mode: 1 or 2
   int32_t small_max;   // cells up to this size finish in the subtree kernel
+  int32_t leafsort;    // subsets not in index order: leaves are sorted at the end
   int32_t presorted;   // root reordered by subset into buf[1]; leaves sorted at the end
   uint64_t contig_mul; // contiguous subsets: floor(2^32 r / n)
   const float* x_in;
@@ -155,6 +156,7 @@ struct StepDev {
   uint32_t* small_total;    // both (appends past small_cap fail)
   uint32_t next_big_cap;
   uint32_t small_cap;
+  uint32_t init_small, init_small_w, init_small_points;  // the queue's contents when the step starts
   uint32_t* next_big_points;  // points in next_big (for bandwidth accounting)
   uint32_t* small_points;     // points appended to small
   // subset offsets (relative to the cell's begin, r+1 per cell) of this

@@ -90,6 +90,22 @@ struct SelectTuning {
 };
 SelectTuning current_tuning();
 
+// A tree that joins the engine: what a kernel writes into its tables.
+struct AdmitRec {
+  TreeDev tree;
+  uint32_t slot;
+  uint32_t terminal;  // the root is a leaf
+  Cell* root_dst;     // else: its entry of a cell list
+};
+constexpr uint32_t kAdmitIota = 65536;  // larger terminal roots get their identity permutation from a launch of their own
+constexpr int kAdmitFew = 8;            // records that travel as launch parameters (below 4 KB)
+struct AdmitFew {
+  AdmitRec rec[kAdmitFew];
+};
+static_assert(sizeof(AdmitFew) <= 4000, "launch parameters");
+// staging: device memory for recs.size() records (more than kAdmitFew only)
+cudaError_t launch_admit(const std::vector<AdmitRec>& recs, AdmitRec* staging, TreeDev* trees, cudaStream_t st);
+
 cudaError_t prepare_step_kernels();
 // One thread: the loop condition of a graph whose body is a pair of level
 // steps (keep going while ncells_next > 0, at most `limit` iterations; the
@@ -102,7 +118,7 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
 
 // Most dynamic shared memory of the staged scatter (two CTAs per SM).
 constexpr uint32_t kScatterSmemBytes = 100 * 1024;
-cudaError_t prepare_scatter_kernel();
+cudaError_t prepare_scatter_kernel(int uniform_d, bool any_widest);
 // uniform_d: the coordinate count of every tree of the step, 0 if they differ
 // (a kernel compiled for that d is used where there is one)
 void launch_scatter(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t sms, uint64_t points,
@@ -126,22 +142,50 @@ void launch_subtree(const SubtreeShape& sh, const TreeDev* trees, const Cell* li
 
 void launch_iota(uint32_t* out, uint32_t n, cudaStream_t st);
 
+// CTAs of the kernels that walk the terminal records of several trees. One
+// tree (slots null: slot 0) has all of them; else slots[0, n) are the trees
+// and CTAs [first[i], first[i + 1]) work on the i-th, first = slots + n.
+constexpr uint32_t kChunkRecords = 32;  // records per CTA that the counts aim at
+struct SlotChunks {
+  const uint32_t* slots;
+  uint32_t nslots, chunks;
+};
+__device__ __forceinline__ uint32_t pick_chunk(const SlotChunks& sc, uint32_t* chunk, uint32_t* chunks) {
+  if (!sc.slots) {
+    *chunk = blockIdx.x;
+    *chunks = gridDim.x;
+    return 0;
+  }
+  const uint32_t* first = sc.slots + sc.nslots;
+  uint32_t lo = 0, hi = sc.nslots;
+  while (hi - lo > 1u) {
+    const uint32_t mid = (lo + hi) / 2u;
+    if (first[mid] <= blockIdx.x) lo = mid; else hi = mid;
+  }
+  *chunk = blockIdx.x - first[lo];
+  *chunks = first[lo + 1u] - first[lo];
+  return sc.slots[lo];
+}
+
 // Leaf sort (kdt_leafsort.cu): terminal cells up to kLeafWarpMax points are
 // sorted by one warp, up to kLeafBlockMax by one CTA; larger ones are listed
 // in the tree's `huge` table and sorted by leaf_sort_huge.
 constexpr int kLeafWarpMax = 256;
 constexpr int kLeafBlockMax = 4096;
-void launch_leaf_sort(const TreeDev* trees, const uint32_t* slots, uint32_t nslots, uint32_t max_records,
-                      cudaStream_t st);
+void launch_leaf_sort(const TreeDev* trees, const SlotChunks& sc, cudaStream_t st);
 // Host view of a finished tree for the global leaf-sort passes: the
 // permutation, a ping-pong buffer of n words and scratch for tile tables
 // (the tree's working buffers, free once its build is done).
 struct TreeHost {
-  uint64_t n;
-  uint32_t* out_perm;
-  uint32_t* keys;
-  void* scratch;
-  size_t scratch_bytes;
+  uint64_t n = 0;
+  uint32_t* out_perm = nullptr;
+  uint32_t* keys = nullptr;
+  void* scratch = nullptr;
+  size_t scratch_bytes = 0;
+  const uint32_t* huge = nullptr;   // device: the records listed for the global passes
+  uint32_t huge_cap = 0;
+  const TermRec* terms = nullptr;   // device
+  uint32_t term_cap = 0;
 };
 size_t leaf_huge_tiles_cap(uint64_t n);
 cudaError_t leaf_sort_huge(const TreeHost& th, const std::vector<TermRec>& recs, cudaStream_t st);
@@ -163,8 +207,6 @@ kdt_status build_in_workspace(const float* points, const kdt_params* p, void* wo
                               uint32_t* out_perm, float* out_split_vals, int8_t* out_split_dims,
                               int64_t* out_node_offsets, int32_t* out_levels, cudaStream_t st);
 
-void launch_finalize_many(const TreeDev* trees, const uint32_t* slots, uint32_t nslots, uint32_t max_records,
-                          cudaStream_t st);
-void launch_finalize(const TreeDev* tree, const uint32_t* term_count, uint32_t max_terms, cudaStream_t st);
+void launch_finalize_many(const TreeDev* trees, const SlotChunks& sc, cudaStream_t st);
 
 }  // namespace kdt

@@ -163,20 +163,19 @@ __device__ void block_sort_slice(uint32_t* a, uint32_t m, int digits, LsShared& 
   __syncthreads();
 }
 
-// Grid (chunks, trees). Warps sort the small terminal cells, CTAs the middle
+// A range of CTAs per tree (SlotChunks). Warps sort the small terminal cells, CTAs the middle
 // ones; the largest are listed for the global passes. Four CTAs per SM by a
 // register bound: the warps' networks, which sort nearly every leaf of a deep
 // tree, want the warps; the CTA path spills a few words.
-__global__ void __launch_bounds__(kLsThreads, 4) k_leaf_sort(const TreeDev* trees, const uint32_t* slots,
-                                                          uint32_t nslots) {
+__global__ void __launch_bounds__(kLsThreads, 4) k_leaf_sort(const TreeDev* trees, SlotChunks sc) {
   __shared__ LsShared S;
-  const uint32_t si = blockIdx.y;
-  if (si >= nslots) return;
-  const TreeDev& t = trees[slots[si]];
+  uint32_t chunk, chunks;
+  const TreeDev& t = trees[pick_chunk(sc, &chunk, &chunks)];
+  if (!t.leafsort || *t.status != ST_OK) return;
   const uint32_t nrec = min(*t.term_count, t.term_cap);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t wstride = gridDim.x * kLsWarps;
-  uint32_t rec = blockIdx.x * kLsWarps + warp;
+  const uint32_t wstride = chunks * kLsWarps;
+  uint32_t rec = chunk * kLsWarps + warp;
   TermRec trn = rec < nrec ? t.terms[rec] : TermRec{};
   for (; rec < nrec; rec += wstride) {
     const TermRec tr = trn;  // the next record is read before this cell is sorted
@@ -194,7 +193,7 @@ __global__ void __launch_bounds__(kLsThreads, 4) k_leaf_sort(const TreeDev* tree
   __shared__ uint32_t mids[kLsThreads];
   __shared__ uint32_t nmid;
   const int digits = index_digits((uint64_t)t.n);
-  for (uint32_t base = blockIdx.x * kLsThreads; base < nrec; base += gridDim.x * kLsThreads) {
+  for (uint32_t base = chunk * kLsThreads; base < nrec; base += chunks * kLsThreads) {
     if (threadIdx.x == 0) nmid = 0;
     __syncthreads();
     const uint32_t rec = base + threadIdx.x;
@@ -286,12 +285,9 @@ __global__ void k_leaf_copy(const uint32_t* src, uint32_t* dst, const LeafTile* 
 
 }  // namespace
 
-void launch_leaf_sort(const TreeDev* trees, const uint32_t* slots, uint32_t nslots, uint32_t max_records,
-                      cudaStream_t st) {
-  if (nslots == 0 || max_records == 0) return;
-  TraceScope ts(K_LEAF_SORT, st, max_records);
-  const uint32_t chunks = std::max<uint32_t>(1, std::min<uint32_t>((max_records + 63) / 64, 2048));
-  k_leaf_sort<<<dim3(chunks, nslots), kLsThreads, 0, st>>>(trees, slots, nslots);
+void launch_leaf_sort(const TreeDev* trees, const SlotChunks& sc, cudaStream_t st) {
+  TraceScope ts(K_LEAF_SORT, st);
+  k_leaf_sort<<<sc.chunks, kLsThreads, 0, st>>>(trees, sc);
 }
 
 size_t leaf_huge_tiles_cap(uint64_t n) { return (size_t)(2 * (n / kLeafBlockMax) + 2); }

@@ -548,11 +548,14 @@ void launch_one(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint
 }
 
 template <bool kMM>
-cudaError_t prepare_all() {
-  for (cudaError_t e : {prepare_one<0, kMM>(), prepare_one<2, kMM>(), prepare_one<3, kMM>(), prepare_one<8, kMM>(),
-                        prepare_one<16, kMM>()})
-    if (e != cudaSuccess) return e;
-  return cudaSuccess;
+cudaError_t prepare_d(int uniform_d) {
+  switch (uniform_d) {
+    case 2: return prepare_one<2, kMM>();
+    case 3: return prepare_one<3, kMM>();
+    case 8: return prepare_one<8, kMM>();
+    case 16: return prepare_one<16, kMM>();
+    default: return prepare_one<0, kMM>();
+  }
 }
 
 template <bool kMM>
@@ -567,9 +570,8 @@ void launch_d(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32
   }
 }
 
-cudaError_t prepare_scatter_kernel() {
-  const cudaError_t e = prepare_all<false>();
-  return e != cudaSuccess ? e : prepare_all<true>();
+cudaError_t prepare_scatter_kernel(int uniform_d, bool any_widest) {
+  return any_widest ? prepare_d<true>(uniform_d) : prepare_d<false>(uniform_d);
 }
 
 void launch_scatter(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t sms, uint64_t points,

@@ -469,7 +469,6 @@ kdt_status sharded_build(const float* points, const kdt_params& p, int32_t G, ui
   const size_t o_terms = take((size_t)nl * sizeof(TermRec));
   const size_t o_huge = take((size_t)nl * 4);
   const size_t o_td = take(sizeof(TreeDev));
-  const size_t o_slot = take(4);
   DevMem big;
   if (dev_malloc(&big.p, off) != cudaSuccess) {
     (void)cudaGetLastError();
@@ -558,13 +557,11 @@ kdt_status sharded_build(const float* points, const kdt_params& p, int32_t G, ui
   td.huge = (uint32_t*)(ws + o_huge);
   td.huge_count = (uint32_t*)(words + 3);
   td.huge_cap = nl;
+  td.leafsort = 1;
   td.status = words + 1;
   TreeDev* td_dev = (TreeDev*)(ws + o_td);
-  uint32_t* slot_dev = (uint32_t*)(ws + o_slot);
-  const uint32_t zero = 0;
   SH_TRY(cudaMemcpyAsync(td_dev, &td, sizeof td, cudaMemcpyHostToDevice, st));
-  SH_TRY(cudaMemcpyAsync(slot_dev, &zero, 4, cudaMemcpyHostToDevice, st));
-  launch_leaf_sort(td_dev, slot_dev, 1, nl, st);
+  launch_leaf_sort(td_dev, SlotChunks{nullptr, 1, std::min<uint32_t>((nl + 63) / 64, 2048u)}, st);
   SH_TRY(cudaGetLastError());
   uint32_t nh = 0;
   int32_t merge_status = 0;

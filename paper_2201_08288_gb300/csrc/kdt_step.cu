@@ -100,8 +100,17 @@ __global__ void k_prep(const TreeDev* trees, StepDev s) {
     s.tile_base[ncells] = tile_run;
     s.seg_base[ncells] = seg_run;
     *s.ntiles_total = tile_run;
+    // the counters that the step's later kernels append to
     *s.bigseg_count = 0;
     *s.midseg_count = 0;
+    *s.next_big_count = 0;
+    *s.next_big_points = 0;
+    *s.off_used = 0;
+    *s.small_count = s.init_small;
+    *s.small_count_w = s.init_small_w;
+    *s.small_total = s.init_small + s.init_small_w;
+    *s.small_points = s.init_small_points;
+    *s.small_off_used = 0;
   }
 }
 
@@ -1444,6 +1453,58 @@ __global__ void k_classify(const TreeDev* trees, StepDev s) {
 // ------------------------------------------------------------ launcher
 
 constexpr uint32_t kManyCells = 1024;  // from here on: a warp per cell in combine and scan
+
+namespace {
+
+// Trees that join the engine, a CTA each: their records, cleared words, the
+// root's cell in its list, or (a root that is terminal) its terminal record
+// and, up to kAdmitIota points, the identity permutation.
+__device__ __forceinline__ void admit_tree(const AdmitRec& a, TreeDev* trees) {
+  const TreeDev& t = a.tree;
+  if (a.terminal && t.n <= (int64_t)kAdmitIota)
+    for (uint32_t i = threadIdx.x; i < (uint32_t)t.n; i += blockDim.x) t.out_perm[i] = i;
+  if (threadIdx.x != 0) return;
+  trees[a.slot] = t;
+  *t.status = ST_OK;
+  *t.levels = 0;
+  *t.huge_count = 0;
+  *t.term_count = a.terminal ? 1u : 0u;
+  *t.live = a.terminal ? 0 : 1;
+  if (a.terminal)
+    t.terms[0] = TermRec{0u, (uint32_t)t.n, 0u, 0};
+  else
+    *a.root_dst = Cell{0u, (uint32_t)t.n, 0u, (int32_t)a.slot, 0, 0, -1};
+}
+
+__global__ void __launch_bounds__(256) k_admit(const AdmitRec* recs, TreeDev* trees) {
+  admit_tree(recs[blockIdx.x], trees);
+}
+
+// The same with the records among the launch's parameters (no copy before it).
+__global__ void __launch_bounds__(256) k_admit_few(const __grid_constant__ AdmitFew few, TreeDev* trees) {
+  admit_tree(few.rec[blockIdx.x], trees);
+}
+
+}  // namespace
+
+cudaError_t launch_admit(const std::vector<AdmitRec>& recs, AdmitRec* staging, TreeDev* trees, cudaStream_t st) {
+  if (recs.empty()) return cudaSuccess;
+  if (recs.size() <= (size_t)kAdmitFew) {
+    AdmitFew few{};
+    std::copy(recs.begin(), recs.end(), few.rec);
+    TraceScope ts(K_ADMIT, st);
+    k_admit_few<<<(unsigned)recs.size(), 256, 0, st>>>(few, trees);
+  } else {
+    const cudaError_t e =
+        cudaMemcpyAsync(staging, recs.data(), recs.size() * sizeof(AdmitRec), cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
+    TraceScope ts(K_ADMIT, st);
+    k_admit<<<(unsigned)recs.size(), 256, 0, st>>>(staging, trees);
+  }
+  for (const AdmitRec& a : recs)
+    if (a.terminal && a.tree.n > (int64_t)kAdmitIota) launch_iota(a.tree.out_perm, (uint32_t)a.tree.n, st);
+  return cudaGetLastError();
+}
 
 cudaError_t prepare_step_kernels() {
   return cudaFuncSetAttribute(k_ps_move, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemBytes);

@@ -242,11 +242,15 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
     s_fail = 0;
   }
   uint32_t phase = 0;
+  uint32_t own_item = blockIdx.x;  // no queue head: a CTA per cell
 
   for (;;) {
     fence_proxy_async_smem();  // earlier generic writes before the next bulk copies
     __syncthreads();
-    if (tid == 0) s_item = atomicAdd(head, 1u);
+    if (tid == 0) {
+      s_item = head ? atomicAdd(head, 1u) : own_item;
+      own_item = 0xffffffffu;
+    }
     __syncthreads();
     const uint32_t item = s_item;
     if (item >= count) break;
@@ -839,44 +843,17 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
 
 // One warp per terminal cell: offsets of the leaves at level L below it and
 // sentinels (dim -1, value +inf) on its own node and every node below it.
-__global__ void k_finalize(const TreeDev* tree, const uint32_t* term_count) {
-  const TreeDev& t = *tree;
-  const uint32_t nrec = min(*term_count, t.term_cap);
-  const int L = t.depth > 0 ? t.depth : *t.levels;
-  const int lane = threadIdx.x & 31;
-  const uint32_t rec = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (blockIdx.x == 0 && threadIdx.x == 0) t.out_offs[(int64_t)1 << L] = t.n;
-  if (rec >= nrec) return;
-  const TermRec tr = t.terms[rec];
-  const int lv = tr.level;
-  if (lv > L) return;
-  const int64_t k = (int64_t)tr.heap - (((int64_t)1 << lv) - 1);
-  const int64_t span = (int64_t)1 << (L - lv);
-  const int64_t leaf0 = k * span;
-  for (int64_t j = lane; j < span; j += 32)
-    t.out_offs[leaf0 + j] = (j == 0) ? (int64_t)tr.begin : (int64_t)tr.begin + tr.count;
-  for (int l2 = lv; l2 < L; ++l2) {
-    const int64_t width = (int64_t)1 << (l2 - lv);
-    const int64_t first = ((int64_t)tr.heap + 1) * width - 1;
-    for (int64_t j = lane; j < width; j += 32) {
-      t.out_dims[first + j] = -1;
-      t.out_vals[first + j] = __int_as_float(0x7f800000);
-    }
-  }
-}
-
-// Finalize of several trees: grid (chunks, trees); each warp takes terminal
-// records of its tree in turn (same per-record work as k_finalize).
-__global__ void k_finalize_many(const TreeDev* trees, const uint32_t* slots, uint32_t nslots) {
-  const uint32_t si = blockIdx.y;
-  if (si >= nslots) return;
-  const TreeDev& t = trees[slots[si]];
+// Trees that failed are left as they are.
+__global__ void k_finalize(const TreeDev* trees, SlotChunks sc) {
+  uint32_t chunk, chunks;
+  const TreeDev& t = trees[pick_chunk(sc, &chunk, &chunks)];
+  if (*t.status != ST_OK) return;
   const uint32_t nrec = min(*t.term_count, t.term_cap);
   const int L = t.depth > 0 ? t.depth : *t.levels;
   const int lane = threadIdx.x & 31;
   const uint32_t wpb = blockDim.x >> 5;
-  if (blockIdx.x == 0 && threadIdx.x == 0) t.out_offs[(int64_t)1 << L] = t.n;
-  for (uint32_t rec = blockIdx.x * wpb + (threadIdx.x >> 5); rec < nrec; rec += gridDim.x * wpb) {
+  if (chunk == 0 && threadIdx.x == 0) t.out_offs[(int64_t)1 << L] = t.n;
+  for (uint32_t rec = chunk * wpb + (threadIdx.x >> 5); rec < nrec; rec += chunks * wpb) {
     const TermRec tr = t.terms[rec];
     const int lv = tr.level;
     if (lv > L) continue;
@@ -928,25 +905,19 @@ void launch_subtree(const SubtreeShape& sh, const TreeDev* trees, const Cell* li
                     const uint32_t* count_dev, bool reversed, const uint32_t* small_off, uint32_t* head,
                     LCell* slices, uint32_t slice_cells, uint32_t grid, uint64_t points, cudaStream_t st) {
   if (count == 0 || grid == 0) return;
-  cudaMemsetAsync(head, 0, sizeof(uint32_t), st);
+  if (!count_dev && grid >= count)
+    head = nullptr;  // a CTA per cell: nothing to hand out
+  else
+    cudaMemsetAsync(head, 0, sizeof(uint32_t), st);
   const uint32_t probe = fault_take(KDT_FAULT_WAIT) ? 1024u : 0u;
   TraceScope ts(K_SUBTREE, st, points);
   subtree_kernel(sh)<<<grid, T, sh.smem, st>>>(trees, list, count, count_dev, reversed ? 1u : 0u, small_off, head,
                                                slices, slice_cells, probe);
 }
 
-void launch_finalize_many(const TreeDev* trees, const uint32_t* slots, uint32_t nslots, uint32_t max_records,
-                          cudaStream_t st) {
-  if (nslots == 0) return;
+void launch_finalize_many(const TreeDev* trees, const SlotChunks& sc, cudaStream_t st) {
   TraceScope ts(K_FINALIZE, st);
-  const uint32_t chunks = std::max<uint32_t>(1, std::min<uint32_t>((max_records + 7) / 8, 8192));
-  k_finalize_many<<<dim3(chunks, nslots), 256, 0, st>>>(trees, slots, nslots);
-}
-
-void launch_finalize(const TreeDev* tree, const uint32_t* term_count, uint32_t max_terms, cudaStream_t st) {
-  const uint32_t blocks = (max_terms + 7) / 8 + 1;
-  TraceScope ts(K_FINALIZE, st);
-  k_finalize<<<blocks, 256, 0, st>>>(tree, term_count);
+  k_finalize<<<sc.chunks, 256, 0, st>>>(trees, sc);
 }
 
 }  // namespace kdt

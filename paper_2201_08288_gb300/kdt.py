@@ -481,8 +481,9 @@ def kdt_build_batched(items, *, workspace=None, stream=None, outputs=None, descs
         n = descs[i].params.n
         m = (1 << L) - 1
         o = outs[i]
-        trees.append(Tree(o.perm[:n], o.split_vals[:m], o.split_dims[:m], o.node_offsets[:(1 << L) + 1], L))
-    return trees, [int(stats[i]) for i in range(num)]
+        perm = o.perm if o.perm.shape == (n,) else o.perm[:n]
+        trees.append(Tree(perm, o.split_vals[:m], o.split_dims[:m], o.node_offsets[:m + 2], L))
+    return trees, list(stats)
 
 
 def _tuning_dict(t: kdt_tuning) -> dict:
