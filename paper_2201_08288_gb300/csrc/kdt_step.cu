@@ -1133,109 +1133,152 @@ __global__ void __launch_bounds__(256, 2) k_fourier_moments(const TreeDev* trees
   }
 }
 
-// Per cell, one warp: the cell's sums C_j (its tiles' records added in tile
-// order; lane l holds terms l, l + 32, l + 64), its bounds (a, b) on its key
-// coordinate (the splits of its ancestors on that coordinate, (0,1) at the
-// root), and the root of Eq. (kd:eq:b) by 60 bisection steps in double on
-// (a, b) of F(m) = 1_J(a, m) - 1_J(m, b) = sum_j C_j (g_j(a, m) - g_j(m, b)),
-// with g_j of Lemma 1: the term of j = 0 is (1(b<1) - 1(a>0)) / 2, of
-// j = 2k-1 q (2 sin(Km) - 1(a>0) sin(Ka) - 1(b<1) sin(Kb)) and of j = 2k
-// q (1(a>0) cos(Ka) + 1(b<1) cos(Kb) - 2 cos(Km)), K = 2k-1, q = 2 / (pi K).
-// The lower end moves up while F < 0; the split is the last midpoint
-// rounded to float, and a point goes left when its coordinate is <= it. The
-// harmonics of the midpoint are evaluated in float (their error moves the
-// root by about 1e-7 of the cell's width), the sums in double.
-__global__ void __launch_bounds__(256) k_fourier_split(const TreeDev* trees, StepDev s, uint32_t mgrid) {
-  const int lane = threadIdx.x & 31;
+// Per cell, one CTA: the cell's sums C_j (its run records added in order,
+// thread j term j), its bounds (a, b) on its key coordinate (the splits of its
+// ancestors on that coordinate, (0,1) at the root), and the root of Eq.
+// (kd:eq:b) by 60 bisection steps in double on (a, b) of F(m) = 1_J(a, m) -
+// 1_J(m, b) = sum_j C_j (g_j(a, m) - g_j(m, b)), with g_j of Lemma 1: the term
+// of j = 0 is (1(b<1) - 1(a>0)) / 2, of j = 2k-1 q (2 sin(Km) - 1(a>0) sin(Ka)
+// - 1(b<1) sin(Kb)) and of j = 2k q (1(a>0) cos(Ka) + 1(b<1) cos(Kb) - 2
+// cos(Km)), K = 2k-1, q = 2 / (pi K). The lower end moves up while F < 0; the
+// split is the last midpoint rounded to float, and a point goes left when its
+// coordinate is <= it. The harmonics of the midpoint are evaluated in float
+// (their error moves the root by about 1e-7 of the cell's width), the sums in
+// double.
+// A step's chain of double operations takes over 2 us, and 60 of them in a
+// row, a warp per cell, were 165 us per level whatever the cells. So the CTA
+// takes three steps at once: warps 1..7 evaluate F at the seven midpoints that
+// the three can meet (warp w stands for the path that w's bits below its
+// highest one spell, 0 where F >= 0), and every warp then walks the path that
+// the signs give. (With more steps at once the double unit, not the chain,
+// bounds a level of many cells.) The sums per midpoint are those of the
+// one-warp form, lane for lane, so the splits are the same bits.
+constexpr int kFsSteps = 3, kFsWarps = 1 << kFsSteps;
+constexpr int kFsChunk = 32;  // run records staged at a time
+
+__global__ void __launch_bounds__(kFsWarps * 32) k_fourier_split(const TreeDev* trees, StepDev s, uint32_t mgrid) {
+  __shared__ double rec[kFsChunk][kFourierTerms];
+  __shared__ double s_base[96], s_slope[96];
+  __shared__ uint32_t s_neg[2];  // per parity of the round: bit w: F < 0 at warp w's midpoint
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t nc = ncells_of(s);
   const uint32_t ntiles = *s.ntiles_total;
   auto range_start = [&](uint32_t k) { return (uint32_t)(((uint64_t)k * ntiles) / mgrid); };
-  for (uint32_t c = blockIdx.x * 8u + (threadIdx.x >> 5); c < nc; c += gridDim.x * 8u) {
+  for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
     const Cell cell = s.cells[c];
     const TreeDev& t = trees[cell.tree];
     const int nt = 2 * t.fourier_j + 1;
     const uint32_t tb = s.tile_base[c], te = s.tile_base[c + 1];
-    // the moments kernel's runs of this cell start at tb and at every start
-    // of a CTA's tile range inside (tb, te)
-    uint64_t k0 = ((uint64_t)tb * mgrid) / (ntiles > 0u ? ntiles : 1u);
-    uint32_t k = (uint32_t)(k0 < (uint64_t)mgrid ? k0 : (uint64_t)(mgrid - 1u));
-    while (k > 0u && range_start(k) > tb) --k;
-    while (k + 1u < mgrid && range_start(k + 1u) <= tb) ++k;
-    double C[3] = {0.0, 0.0, 0.0};
-    uint32_t r0 = tb;
-    for (uint32_t kk = k + 1u;; ++kk) {
-      const double* rec = (const double*)(s.tile_mm + (size_t)r0 * kTileRecWords);
-#pragma unroll
-      for (int q = 0; q < 3; ++q)
-        if (lane + 32 * q < nt) C[q] += rec[lane + 32 * q];
-      uint32_t nxt = te;
-      while (kk < mgrid && (nxt = range_start(kk)) <= r0) ++kk;  // CTAs with empty ranges
-      if (kk >= mgrid || nxt >= te) break;
-      r0 = nxt;
+    // The moments kernel's runs of this cell start at tb and at every start of
+    // a CTA's tile range inside (tb, te): with at least as many tiles as CTAs
+    // the starts of ranges k0 + 1, k0 + 2, ... (k0: the range that holds tb),
+    // with fewer every tile.
+    uint32_t k0 = 0;
+    const bool dense = ntiles < mgrid;
+    if (!dense) {
+      const uint64_t kk = ((uint64_t)tb * mgrid) / (ntiles > 0u ? ntiles : 1u);
+      k0 = (uint32_t)(kk < (uint64_t)mgrid ? kk : (uint64_t)(mgrid - 1u));
+      while (k0 > 0u && range_start(k0) > tb) --k0;
+      while (k0 + 1u < mgrid && range_start(k0 + 1u) <= tb) ++k0;
     }
-    const uint32_t dim = s.kdim[c];
-    double a = 0.0, b = 1.0;
-    if (lane == 0)
-      for (uint32_t h = cell.heap; h > 0;) {
-        const uint32_t par = (h - 1u) / 2u;
-        const uint32_t plevel = 31u - (uint32_t)__clz(par + 1u);
-        if (plevel % (uint32_t)t.d == dim) {
-          const double v = (double)t.out_vals[par];
-          if (h == 2u * par + 1u)
-            b = fmin(b, v);
-          else
-            a = fmax(a, v);
-        }
-        h = par;
+    auto run_start = [&](uint32_t m) -> uint32_t {  // te: no such run
+      if (m == 0u) return tb;
+      if (dense) return tb + m;
+      return k0 + m < mgrid ? range_start(k0 + m) : te;
+    };
+    double C = 0.0;  // thread j: the sum of term j
+    for (uint32_t m0 = 0; run_start(m0) < te; m0 += kFsChunk) {
+      for (uint32_t i = tid; i < (uint32_t)(kFsChunk * nt); i += kFsWarps * 32) {
+        const uint32_t r0 = run_start(m0 + i / (uint32_t)nt);
+        if (r0 < te) rec[i / nt][i % nt] = ((const double*)(s.tile_mm + (size_t)r0 * kTileRecWords))[i % nt];
       }
-    a = __shfl_sync(0xffffffffu, a, 0);
-    b = __shfl_sync(0xffffffffu, b, 0);
+      __syncthreads();
+      if (tid < nt)
+        for (uint32_t m = 0; m < (uint32_t)kFsChunk && run_start(m0 + m) < te; ++m) C += rec[m][tid];
+      __syncthreads();
+    }
+    // bounds: lane i of every warp takes the i-th ancestor (splits are in
+    // [0, 1], where floats order like their bits)
+    const uint32_t dim = s.kdim[c];
+    uint32_t ba = 0u, bb = __float_as_uint(1.0f);
+    if (lane < (int)cell.level) {
+      const uint32_t par = ((cell.heap + 1u) >> (lane + 1)) - 1u;
+      const uint32_t child = ((cell.heap + 1u) >> lane) - 1u;
+      if (((uint32_t)cell.level - 1u - (uint32_t)lane) % (uint32_t)t.d == dim) {
+        const uint32_t v = __float_as_uint(t.out_vals[par]);
+        if (child == 2u * par + 1u) bb = v; else ba = v;
+      }
+    }
+    const double a = (double)__uint_as_float(__reduce_max_sync(0xffffffffu, ba));
+    const double b = (double)__uint_as_float(min(__reduce_min_sync(0xffffffffu, bb), __float_as_uint(1.0f)));
     const double ia = a > 0.0 ? 1.0 : 0.0, ib = b < 1.0 ? 1.0 : 0.0;
     // per term: F_j(m) = base + slope * (sin or cos)(K m)
+    if (tid < 96) {
+      double base = 0.0, slope = 0.0;
+      if (tid == 0) {
+        base = C * 0.5 * (ib - ia);
+      } else if (tid < nt) {
+        const double k = (double)(2 * ((tid + 1) / 2) - 1);
+        const double qk = 2.0 / (3.14159265358979323846 * k);
+        if (tid & 1) {
+          base = -C * qk * (ia * sin(k * a) + ib * sin(k * b));
+          slope = 2.0 * C * qk;
+        } else {
+          base = C * qk * (ia * cos(k * a) + ib * cos(k * b));
+          slope = -2.0 * C * qk;
+        }
+      }
+      s_base[tid] = base;
+      s_slope[tid] = slope;
+    }
+    if (tid < 2) s_neg[tid] = 0u;
+    __syncthreads();
     double base[3], slope[3], K[3];
-    bool use_sin[3];
+    bool use[3], wave[3], use_sin[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       const int j = lane + 32 * q;
-      base[q] = slope[q] = 0.0;
-      K[q] = 0.0;
-      use_sin[q] = true;
-      if (j >= nt) continue;
-      if (j == 0) {
-        base[q] = C[q] * 0.5 * (ib - ia);
-        continue;
-      }
-      const double k = (double)(2 * ((j + 1) / 2) - 1);
-      const double qk = 2.0 / (3.14159265358979323846 * k);
-      K[q] = k;
-      if (j & 1) {
-        base[q] = -C[q] * qk * (ia * sin(k * a) + ib * sin(k * b));
-        slope[q] = 2.0 * C[q] * qk;
-      } else {
-        base[q] = C[q] * qk * (ia * cos(k * a) + ib * cos(k * b));
-        slope[q] = -2.0 * C[q] * qk;
-        use_sin[q] = false;
-      }
+      base[q] = s_base[j];
+      slope[q] = s_slope[j];
+      K[q] = (double)(2 * ((j + 1) / 2) - 1);
+      wave[q] = slope[q] != 0.0;
+      use[q] = wave[q] || base[q] != 0.0;
+      use_sin[q] = (j & 1) != 0;
     }
     double lo = a, hi = b;
-    for (int it = 0; it < 60; ++it) {
-      const double mid = 0.5 * (lo + hi);
-      double f = 0.0;
+    for (int it = 0; it < 60 / kFsSteps; ++it) {
+      if (warp > 0) {
+        double l = lo, h = hi, mid = 0.5 * (lo + hi);
+        for (int bit = 30 - __clz(warp); bit >= 0; --bit) {
+          if ((warp >> bit) & 1) l = mid; else h = mid;
+          mid = 0.5 * (l + h);
+        }
+        double f = 0.0;
 #pragma unroll
-      for (int q = 0; q < 3; ++q)
-        if (slope[q] != 0.0 || base[q] != 0.0)
-          f += base[q] + (slope[q] != 0.0
-                              ? slope[q] * (double)(use_sin[q] ? sinf((float)(K[q] * mid)) : cosf((float)(K[q] * mid)))
-                              : 0.0);
+        for (int q = 0; q < 3; ++q)
+          if (use[q])
+            f += base[q] + (wave[q] ? slope[q] * (double)(use_sin[q] ? sinf((float)(K[q] * mid)) : cosf((float)(K[q] * mid)))
+                                    : 0.0);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) f += __shfl_down_sync(0xffffffffu, f, o);
-      f = __shfl_sync(0xffffffffu, f, 0);  // lane 0's sum decides for the warp
-      if (f < 0.0)
-        lo = mid;
-      else
-        hi = mid;
+        for (int o = 16; o > 0; o >>= 1) f += __shfl_down_sync(0xffffffffu, f, o);
+        if (lane == 0 && f < 0.0) atomicOr(&s_neg[it & 1], 1u << warp);  // lane 0's sum decides
+      }
+      __syncthreads();
+      const uint32_t neg = s_neg[it & 1];
+      uint32_t w = 1;
+#pragma unroll
+      for (int st = 0; st < kFsSteps; ++st) {
+        const double mid = 0.5 * (lo + hi);
+        const uint32_t up = (neg >> w) & 1u;
+        if (up) lo = mid; else hi = mid;
+        w = 2u * w + up;
+      }
+      // the next round collects in the other word; this one is cleared for the
+      // round after it, once all have read it
+      __syncthreads();
+      if (tid == 0) s_neg[it & 1] = 0u;
     }
-    if (lane == 0) {
+    if (tid == 0) {
       const float m32 = (float)(0.5 * (lo + hi));
       s.mkey[c] = ord_key(m32);
       t.out_vals[cell.heap] = m32;
@@ -1548,7 +1591,7 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
       TraceScope ts(K_FOURIER_MOMENTS, st, points);
       k_fourier_moments<<<mgrid, 256, 0, st>>>(trees, s);
     }
-    { TraceScope ts(K_FOURIER_SPLIT, st); k_fourier_split<<<cells_grid(8, sms * 8u), 256, 0, st>>>(trees, s, mgrid); }
+    { TraceScope ts(K_FOURIER_SPLIT, st); k_fourier_split<<<cells_grid(1, sms * 4u), kFsWarps * 32, 0, st>>>(trees, s, mgrid); }
   } else {
     { TraceScope ts(K_SEGS, st); k_segs<<<cells_grid(1, sms * 8u), 256, 0, st>>>(trees, s); }
     {
