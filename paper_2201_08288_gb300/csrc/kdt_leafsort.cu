@@ -10,9 +10,13 @@
 //   - up to kLeafWarpMax points: one warp, bitonic network in registers;
 //   - up to kLeafBlockMax points: one CTA, LSD radix sort (8-bit digits) in
 //     shared memory, stable ranks from warp match masks;
-//   - larger: the same LSD passes over global memory, tiles of kLeafBlockMax
-//     points, per-(tile, digit) counts scanned per leaf (host-driven; only
-//     shallow trees or cells that stop splitting produce such leaves).
+//   - up to kBucketPoints: one CTA, one pass into buckets by the leading bits
+//     where the leaf's indices differ, then a warp's network per bucket;
+//   - larger, or with a bucket too full for a warp: LSD passes over global
+//     memory, tiles of kLeafBlockMax points, per-(tile, digit) counts scanned
+//     per leaf.
+// The last two are host-driven; only shallow trees or cells that stop
+// splitting produce such leaves.
 // Original indices are distinct, so the result does not depend on stability
 // across equal keys; stability is what makes the LSD passes correct.
 #include <algorithm>
@@ -42,7 +46,7 @@ __host__ __device__ inline int index_digits(uint64_t n) {
 // -------------------------------------------------------- one warp, <= 32K
 
 template <int K>
-__device__ void warp_sort_slice(uint32_t* a, uint32_t m) {
+__device__ void warp_sort_slice(const uint32_t* a, uint32_t* out, uint32_t m) {
   const int lane = threadIdx.x & 31;
   uint32_t v[K];
 #pragma unroll
@@ -77,15 +81,16 @@ __device__ void warp_sort_slice(uint32_t* a, uint32_t m) {
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const uint32_t e = (uint32_t)(k * 32 + lane);
-    if (e < m) a[e] = v[k];
+    if (e < m) out[e] = v[k];
   }
 }
 
-__device__ void warp_sort_any(uint32_t* a, uint32_t m) {
-  if (m <= 32) warp_sort_slice<1>(a, m);
-  else if (m <= 64) warp_sort_slice<2>(a, m);
-  else if (m <= 128) warp_sort_slice<4>(a, m);
-  else warp_sort_slice<8>(a, m);
+// One warp: a[0..m) ascending into out (which may be a), m <= kLeafWarpMax.
+__device__ void warp_sort_any(const uint32_t* a, uint32_t* out, uint32_t m) {
+  if (m <= 32) warp_sort_slice<1>(a, out, m);
+  else if (m <= 64) warp_sort_slice<2>(a, out, m);
+  else if (m <= 128) warp_sort_slice<4>(a, out, m);
+  else warp_sort_slice<8>(a, out, m);
 }
 
 // ------------------------------------------------------ block ranking
@@ -182,7 +187,7 @@ __global__ void __launch_bounds__(kLsThreads, 4) k_leaf_sort(const TreeDev* tree
     if (rec + wstride < nrec) trn = t.terms[rec + wstride];
     if (tr.count <= 1u) continue;
     if (tr.count <= (uint32_t)kLeafWarpMax) {
-      warp_sort_any(t.out_perm + tr.begin, tr.count);
+      warp_sort_any(t.out_perm + tr.begin, t.out_perm + tr.begin, tr.count);
     } else if (tr.count > (uint32_t)kLeafBlockMax && lane == 0) {
       const uint32_t k = atomicAdd(t.huge_count, 1u);
       if (k < t.huge_cap) t.huge[k] = rec; else set_status(t, ST_CAPACITY);
@@ -209,7 +214,90 @@ __global__ void __launch_bounds__(kLsThreads, 4) k_leaf_sort(const TreeDev* tree
   }
 }
 
-// --------------------------------------------- global passes (large leaves)
+// ------------------------------------------------- one CTA, buckets (large leaves)
+
+// Leaves of kLeafBlockMax + 1 .. kBucketPoints points, a CTA each: the indices
+// are counted by bucket (bits above `shift`, the smallest that leaves at most
+// kBuckets of them between the leaf's least and largest index, so 512 to 1024
+// when they are spread evenly), moved into shared memory bucket by bucket, and
+// each bucket is sorted by a warp in registers straight into the leaf's place.
+// A leaf with a bucket above kLeafWarpMax is left as it is and its flag set
+// (the caller sorts it by the global passes).
+// What bounds it: the shared-memory atomics and the networks; the leaf is read
+// three times, twice of them from L2. For 1024 leaves of 48,800 points it took
+// 0.42 ms where the four global LSD passes took 2.03.
+constexpr int kBucketThreads = 1024;
+constexpr int kBuckets = 1024;
+constexpr uint32_t kBucketPoints = 54272;
+constexpr size_t kBucketSmem = (size_t)kBucketPoints * 4;
+
+__global__ void __launch_bounds__(kBucketThreads) k_leaf_buckets(uint32_t* perm, const uint2* leaves, uint32_t nleaves,
+                                                                 uint32_t* failed) {
+  extern __shared__ __align__(16) uint32_t keys[];
+  __shared__ uint32_t start[kBuckets + 1];
+  __shared__ uint32_t cursor[kBuckets];
+  __shared__ uint32_t tmp[33];
+  __shared__ uint32_t s_lo, s_hi, s_most;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (uint32_t lf = blockIdx.x; lf < nleaves; lf += gridDim.x) {
+    const uint32_t m = leaves[lf].y;
+    uint32_t* a = perm + leaves[lf].x;
+    if (tid == 0) {
+      s_lo = 0xffffffffu;
+      s_hi = 0u;
+      s_most = 0u;
+    }
+    cursor[tid] = 0;
+    __syncthreads();
+    uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll 8
+    for (uint32_t i = tid; i < m; i += kBucketThreads) {
+      const uint32_t v = a[i];
+      lo = min(lo, v);
+      hi = max(hi, v);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+      atomicMin(&s_lo, lo);
+      atomicMax(&s_hi, hi);
+    }
+    __syncthreads();
+    lo = s_lo;
+    const uint32_t span = s_hi - lo;
+    const int shift = max(0, 32 - __clz(span) - 10);  // span >> shift < 1024
+#pragma unroll 8
+    for (uint32_t i = tid; i < m; i += kBucketThreads) atomicAdd(&cursor[(a[i] - lo) >> shift], 1u);
+    __syncthreads();
+    const uint32_t cnt = cursor[tid];
+    const uint32_t most = __reduce_max_sync(0xffffffffu, cnt);
+    if (lane == 0) atomicMax(&s_most, most);
+    uint32_t tot;
+    const uint32_t ex = block_excl_scan(cnt, tmp, &tot);
+    start[tid] = ex;
+    cursor[tid] = ex;
+    if (tid == 0) start[kBuckets] = m;
+    __syncthreads();
+    if (s_most > (uint32_t)kLeafWarpMax) {
+      if (tid == 0) failed[lf] = 1u;
+      __syncthreads();  // s_most is read by all before the next leaf resets it
+      continue;
+    }
+#pragma unroll 8
+    for (uint32_t i = tid; i < m; i += kBucketThreads) {
+      const uint32_t v = a[i];
+      keys[atomicAdd(&cursor[(v - lo) >> shift], 1u)] = v;
+    }
+    __syncthreads();
+    for (int b = warp; b < kBuckets; b += kBucketThreads / 32) {
+      const uint32_t s0 = start[b], w = start[b + 1] - s0;
+      if (w) warp_sort_any(keys + s0, a + s0, w);
+    }
+    __syncthreads();
+  }
+}
+
+// --------------------------------------------- global passes (larger leaves)
 
 // Tile of a large leaf: absolute begin of the leaf, its size, the tile's
 // offset inside it.
@@ -292,14 +380,59 @@ void launch_leaf_sort(const TreeDev* trees, const SlotChunks& sc, cudaStream_t s
 
 size_t leaf_huge_tiles_cap(uint64_t n) { return (size_t)(2 * (n / kLeafBlockMax) + 2); }
 
-cudaError_t leaf_sort_huge(const TreeHost& th, const std::vector<TermRec>& recs, cudaStream_t st) {
+namespace {
+
+// Leaves of at most kBucketPoints points; those it could not sort go to *rest.
+cudaError_t leaf_sort_buckets(const TreeHost& th, const std::vector<uint2>& leaves, std::vector<uint2>* rest,
+                              cudaStream_t st) {
+  const size_t nl = leaves.size();
+  const size_t flags_at = (nl * sizeof(uint2) + 255) & ~(size_t)255;
+  if (flags_at + nl * 4 > th.scratch_bytes) {
+    rest->insert(rest->end(), leaves.begin(), leaves.end());
+    return cudaSuccess;
+  }
+  uint2* d_leaves = (uint2*)th.scratch;
+  uint32_t* d_failed = (uint32_t*)((uint8_t*)th.scratch + flags_at);
+  int dev = 0, sms = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(k_leaf_buckets, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBucketSmem)) !=
+          cudaSuccess ||
+      (e = cudaMemcpyAsync(d_leaves, leaves.data(), nl * sizeof(uint2), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
+      (e = cudaMemsetAsync(d_failed, 0, nl * 4, st)) != cudaSuccess)
+    return e;
+  {
+    TraceScope ts(K_LEAF_BUCKETS, st);
+    k_leaf_buckets<<<(unsigned)std::min<size_t>(nl, (size_t)sms), kBucketThreads, kBucketSmem, st>>>(
+        th.out_perm, d_leaves, (uint32_t)nl, d_failed);
+  }
+  std::vector<uint32_t> failed(nl);
+  if ((e = cudaGetLastError()) != cudaSuccess ||
+      (e = cudaMemcpyAsync(failed.data(), d_failed, nl * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+      (e = cudaStreamSynchronize(st)) != cudaSuccess)
+    return e;
+  for (size_t i = 0; i < nl; ++i)
+    if (failed[i]) rest->push_back(leaves[i]);
+  return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t leaf_sort_huge(const TreeHost& th, const std::vector<TermRec>& all, cudaStream_t st) {
+  std::vector<uint2> recs, fit;  // begin and count of the leaves
+  for (const TermRec& r : all) (r.count <= kBucketPoints ? fit : recs).push_back(make_uint2(r.begin, r.count));
+  if (!fit.empty()) {
+    const cudaError_t e = leaf_sort_buckets(th, fit, &recs, st);
+    if (e != cudaSuccess) return e;
+  }
   if (recs.empty()) return cudaSuccess;
   std::vector<LeafTile> tiles;
   std::vector<uint32_t> first, ntiles;
-  for (const TermRec& r : recs) {
+  for (const uint2& r : recs) {
     first.push_back((uint32_t)tiles.size());
     uint32_t k = 0;
-    for (uint32_t off = 0; off < r.count; off += kLeafBlockMax, ++k) tiles.push_back(LeafTile{r.begin, r.count, off, 0});
+    for (uint32_t off = 0; off < r.y; off += kLeafBlockMax, ++k) tiles.push_back(LeafTile{r.x, r.y, off, 0});
     ntiles.push_back(k);
   }
   const size_t nt = tiles.size(), nr = recs.size();
