@@ -417,7 +417,7 @@ kdt_status Engine::tick() {
     s_.bitonic_max = tune.bitonic_max;
     s_.warp_max = tune.warp_max;
     launch_big_step(trees_, s_, tiles_bound, (uint32_t)nseg_bound, plan_.bigseg_cap, has_roots, root_dims_,
-                    plan_.needs.widest, plan_.needs.max_d,
+                    plan_.needs.widest, plan_.needs.max_r,
                     uniform_d(), tune, big_points_,
                     plan_.grid_step, st_, plan_.needs.fourier);
     ENGINE_TRY(cudaGetLastError());
@@ -566,7 +566,7 @@ kdt_status Engine::record_tick(int p) {
   sd.bitonic_max = tune.bitonic_max;
   sd.warp_max = tune.warp_max;
   launch_big_step(trees_, sd, plan_.max_tiles, plan_.nseg_cap, plan_.bigseg_cap, false, false, plan_.needs.widest,
-                  plan_.needs.max_d, uniform_d(), tune, 0,
+                  plan_.needs.max_r, uniform_d(), tune, 0,
                   plan_.grid_step, st_, plan_.needs.fourier);
   ENGINE_TRY(cudaGetLastError());
   launch_small(true);

@@ -113,7 +113,7 @@ cudaError_t prepare_step_kernels();
 void launch_loop_cond(cudaGraphConditionalHandle h, const uint32_t* ncells_next, uint32_t* iters, uint32_t limit,
                       cudaStream_t st);
 void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t nseg,
-                     uint32_t max_bigseg, bool has_roots, bool need_root_dims, bool any_widest, int max_d, int uniform_d,
+                     uint32_t max_bigseg, bool has_roots, bool need_root_dims, bool any_widest, int max_r, int uniform_d,
                      const SelectTuning& tune, uint64_t points, uint32_t sms, cudaStream_t st, bool fourier = false);
 
 // Most dynamic shared memory of the staged scatter (two CTAs per SM).

@@ -240,6 +240,7 @@ kdt_status kdt_server_create(size_t mem_budget_bytes, int32_t max_trees_in_fligh
   cap.slice_cells = 8192;
   cap.widest = true;
   cap.max_d = KDT_MAX_DIMS;
+  cap.max_r = KDT_MAX_SUBSETS;
   sv->step = kdt::plan_step(cap);
   sv->tree_base = align_up(sv->step.bytes);
   if (sv->tree_base + ((size_t)16 << 20) > mem_budget_bytes) {

@@ -40,7 +40,12 @@ constexpr int kPsGroup = 2;                       // tiles per block of the root
 constexpr int kPsPoints = kPsGroup * kTile;
 constexpr int kPsThreads = 512;
 constexpr int kPsItems = kPsPoints / kPsThreads;
-constexpr size_t kPsSmemBytes = (size_t)kPsPoints * 6;  // one word and one u16 subset per point
+constexpr uint32_t kPsHole = 0xffffu;             // a place of the sorted group that holds no point
+// Places of a group sorted by r subsets (at most one empty place per subset of
+// two or more points), and its shared memory (a word and a u16 subset per
+// place).
+__host__ __device__ constexpr uint32_t ps_places(uint32_t r) { return kPsPoints + (r < kPsPoints / 2u ? r : kPsPoints / 2u); }
+constexpr size_t ps_smem_bytes(uint32_t r) { return (size_t)((ps_places(r) + 7u) & ~7u) * 6; }
 
 __device__ __forceinline__ bool tile_of(const StepDev& s, uint32_t tile, uint2* out) {
   if (tile >= *s.ntiles_total) return false;
@@ -243,7 +248,14 @@ __global__ void k_ps_offsets(const TreeDev* trees, StepDev s) {
 // kdt_internal.cuh), each subset of the group reserves a run of its place in
 // subset order (explicit ids: from the fill cursors; index mod r: closed
 // form), and every column passes through shared memory in subset order so
-// that the stores are contiguous runs of about kPsPoints / r points.
+// that the stores are contiguous runs of about kPsPoints / r points. With
+// subsets by index mod r a warp's 32 points go to 32 consecutive subsets, and
+// at an even distance of kPsPoints / r places they share banks (64 subsets:
+// all 32 in one), so there a subset takes an odd number of places (one is left
+// empty where its count is even): 50,000,021 points in 3 coordinates, 64
+// subsets, 0.50 ms against 1.16. Explicit ids spread over the banks by
+// themselves; the empty places only cost (2^27 points in 8: 3.25 ms against
+// 2.91).
 __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, StepDev s) {
   uint2 tl;
   Cell cell;
@@ -259,14 +271,13 @@ __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, St
         s.tile_mm[((size_t)blockIdx.x * 2 * kMaxDims + j / 2) * 2 + (j & 1)] = (j & 1) ? 0u : 0xffffffffu;
     return;
   }
-  extern __shared__ __align__(16) uint32_t ps_buf[];  // kPsPoints words, then kPsPoints u16 subsets
-  uint16_t* lsub = (uint16_t*)(ps_buf + kPsPoints);
+  extern __shared__ __align__(16) uint32_t ps_buf[];  // a word per place, then a u16 subset per place
+  uint16_t* lsub = (uint16_t*)(ps_buf + ((ps_places((uint32_t)t.r) + 7u) & ~7u));
   __shared__ uint32_t loff[kMaxSubsets];   // counts, then local offsets
   __shared__ uint32_t gbase[kMaxSubsets];  // global start of each subset's run
   __shared__ uint32_t tmp[33];
   __shared__ uint32_t gmm[kMaxDims][2];
   const uint32_t r = (uint32_t)t.r, i0 = tl.y, end = min(i0 + (uint32_t)kPsPoints, cell.count);
-  const uint32_t m = end - i0;
   const bool expl = t.subset_mode == SUB_EXPLICIT;
   for (uint32_t j = threadIdx.x; j < r; j += kPsThreads) loff[j] = 0;
   for (int j = threadIdx.x; j < 2 * t.d; j += kPsThreads) gmm[j / 2][j & 1] = (j & 1) ? 0u : 0xffffffffu;
@@ -291,10 +302,15 @@ __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, St
         gbase[j] = t.root_off[j] + i0 / r + (j < i0 % r ? 1u : 0u);
     }
     uint32_t tot;
-    const uint32_t ex = block_excl_scan(c, tmp, &tot);
-    if (j < r) loff[j] = run + ex;
+    const uint32_t odd = c + (!expl && c != 0u && (c & 1u) == 0u ? 1u : 0u);
+    const uint32_t ex = block_excl_scan(odd, tmp, &tot);
+    if (j < r) {
+      loff[j] = run + ex;
+      if (odd != c) lsub[run + ex + c] = (uint16_t)kPsHole;
+    }
     run += tot;
   }
+  const uint32_t m = run;  // places in use
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < kPsItems; ++q)
@@ -311,6 +327,7 @@ __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, St
     __syncthreads();
     for (uint32_t j = threadIdx.x; j < m; j += kPsThreads) {
       const uint32_t sj = lsub[j];
+      if (sj == kPsHole) continue;
       const uint32_t dst = gbase[sj] + (j - loff[sj]);
       if (dst < cell.count) store(dst, ps_buf[j]); else set_status(t, ST_INTERNAL);
     }
@@ -1552,11 +1569,12 @@ cudaError_t launch_admit(const std::vector<AdmitRec>& recs, AdmitRec* staging, T
 }
 
 cudaError_t prepare_step_kernels() {
-  return cudaFuncSetAttribute(k_ps_move, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemBytes);
+  return cudaFuncSetAttribute(k_ps_move, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)ps_smem_bytes(kMaxSubsets));
 }
 
 void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t nseg,
-                     uint32_t max_bigseg, bool has_roots, bool need_root_dims, bool any_widest, int max_d, int uniform_d,
+                     uint32_t max_bigseg, bool has_roots, bool need_root_dims, bool any_widest, int max_r, int uniform_d,
                      const SelectTuning& tune, uint64_t points, uint32_t sms, cudaStream_t st, bool fourier) {
   // s.ncells: the step's cells, or (s.ncells_dev set: a step inside a graph)
   // their capacity; per-cell kernels stride over the cells, so their grids
@@ -1577,7 +1595,7 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
       k_ps_count<<<std::max<uint32_t>(1, std::min(max_tiles, sms * 4u)), kTileThreads, 0, st>>>(trees, s);
     }
     { TraceScope ts(K_PS_OFFSETS, st); k_ps_offsets<<<nc, 1024, 0, st>>>(trees, s); }
-    { TraceScope ts(K_PS_MOVE, st, points); k_ps_move<<<max_tiles, kPsThreads, kPsSmemBytes, st>>>(trees, s); }
+    { TraceScope ts(K_PS_MOVE, st, points); k_ps_move<<<max_tiles, kPsThreads, ps_smem_bytes((uint32_t)max_r), st>>>(trees, s); }
   }
   if (need_root_dims) {
     { TraceScope ts(K_MINMAX, st, points); k_minmax<<<max_tiles, kTileThreads, 0, st>>>(trees, s); }
