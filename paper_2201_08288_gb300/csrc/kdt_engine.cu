@@ -15,12 +15,13 @@ constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 
 // Engine words.
-// W_NC0, W_NC1, W_ITERS (adjacent): the cell counts of the two lists and the
-// iteration count of a graph-driven run
+// Per cell list (parity p): W_BIG + 2p its cells and, next to it, their
+// segments; W_TILE + 2p their tiles and points; W_BIGSEG + p, W_MIDSEG + p the
+// segment lists of the step over it. W_SMALL, W_SMALL + 1: the subtree queue's
+// front and back. W_ITERS: the iterations of a graph-driven run.
 enum Word {
-  W_NTILES = 0, W_BIGSEG, W_HEAD, W_NEXTBIG, W_BIGPTS, W_OFFUSED, W_MIDSEG,
-  W_SMALL, W_SMALLW, W_SMALLTOT, W_SMALLPTS, W_SMALLOFF,  // adjacent: written together by a tick
-  W_NC0, W_NC1, W_ITERS, W_COUNT
+  W_BIG = 0, W_TILE = 4, W_SMALL = 8, W_SMALLPTS = 10, W_SMALLOFF, W_BIGSEG = 12, W_MIDSEG = 14, W_HEAD = 16, W_ITERS,
+  W_COUNT
 };
 // a graph-driven run's iterations (two level steps each) before it gives up
 constexpr uint32_t kGraphIterMax = KDT_MAX_LEVELS + 4;
@@ -185,8 +186,6 @@ StepPlan plan_step(const StepNeeds& needs) {
   s.big[0] = take((size_t)s.maxB * sizeof(Cell));
   s.big[1] = take((size_t)s.maxB * sizeof(Cell));
   s.small = take((size_t)s.cap_small * sizeof(Cell));
-  s.tile_base = take(((size_t)s.maxB + 1) * 4);
-  s.seg_base = take(((size_t)s.maxB + 1) * 4);
   s.tiles = take((size_t)s.max_tiles * sizeof(uint2));
   s.tile_seg = take((size_t)s.max_tiles * 4);
   s.tile_left = take((size_t)s.max_tiles * 4);
@@ -223,10 +222,9 @@ Engine::Engine(const StepPlan& plan, uint8_t* base, cudaStream_t st) : plan_(pla
   big_[1] = (Cell*)(base + plan.big[1]);
   small_ = (Cell*)(base + plan.small);
   slices_ = (LCell*)(base + plan.slices);
-  s_.tile_base = (uint32_t*)(base + plan.tile_base);
-  s_.seg_base = (uint32_t*)(base + plan.seg_base);
   s_.tiles = (uint2*)(base + plan.tiles);
-  s_.ntiles_total = words_ + W_NTILES;
+  s_.tiles_cap = plan.max_tiles;
+  s_.nseg_cap = plan.nseg_cap;
   s_.kdim = (uint32_t*)(base + plan.kdim);
   s_.mkey = (uint32_t*)(base + plan.mkey);
   s_.lcount = (uint32_t*)(base + plan.lcount);
@@ -236,26 +234,19 @@ Engine::Engine(const StepPlan& plan, uint8_t* base, cudaStream_t st) : plan_(pla
   s_.seg_key = (const uint32_t**)(base + plan.seg_key);
   s_.seg_med = (uint32_t*)(base + plan.seg_med);
   s_.bigseg = (uint32_t*)(base + plan.bigseg);
-  s_.bigseg_count = words_ + W_BIGSEG;
   s_.midseg = (uint32_t*)(base + plan.midseg);
-  s_.midseg_count = words_ + W_MIDSEG;
   s_.tile_seg = (uint32_t*)(base + plan.tile_seg);
   s_.tile_left = (uint32_t*)(base + plan.tile_left);
   s_.tile_loff = (uint32_t*)(base + plan.tile_loff);
-  s_.next_big_count = words_ + W_NEXTBIG;
   s_.small = small_;
-  s_.small_count = words_ + W_SMALL;
-  s_.small_count_w = words_ + W_SMALLW;
-  s_.small_total = words_ + W_SMALLTOT;
+  s_.small_ctr = (unsigned long long*)(words_ + W_SMALL);
   s_.small_cap = plan.cap_small;
   s_.next_big_cap = plan.maxB;
-  s_.next_big_points = words_ + W_BIGPTS;
   s_.small_points = words_ + W_SMALLPTS;
   for (int b = 0; b < 2; ++b) {
     off_[b] = (uint32_t*)(base + plan.off[b]);
     obase_[b] = (uint32_t*)(base + plan.obase[b]);
   }
-  s_.off_used = words_ + W_OFFUSED;
   s_.off_cap = plan.off_cap;
   s_.small_off = (uint32_t*)(base + plan.small_off);
   s_.small_off_used = words_ + W_SMALLOFF;
@@ -278,10 +269,27 @@ kdt_status Engine::reset() {
   ENGINE_TRY(cudaMemsetAsync(words_, 0, plan_.slot_words - plan_.words + (size_t)S_COUNT * mt * 4, st_));
   cur_ = 0;
   big_count_ = small_count_ = small_count_w_ = 0;
+  big_tiles_ = big_segs_ = 0;
   big_points_ = small_points_ = 0;
   root_dims_ = false;
   pending_.clear();
   return KDT_OK;
+}
+
+// Point a step's tables at cell list p and the other one.
+void Engine::use_lists(StepDev* s, int p) {
+  s->cells = big_[p];
+  s->next_big = big_[p ^ 1];
+  s->next_big_ctr = (unsigned long long*)(words_ + W_BIG + 2 * (p ^ 1));
+  s->next_tile_ctr = (unsigned long long*)(words_ + W_TILE + 2 * (p ^ 1));
+  s->bigseg_count = words_ + W_BIGSEG + p;
+  s->bigseg_count_next = words_ + W_BIGSEG + (p ^ 1);
+  s->midseg_count = words_ + W_MIDSEG + p;
+  s->midseg_count_next = words_ + W_MIDSEG + (p ^ 1);
+  s->off_cur = off_[p];
+  s->obase_cur = obase_[p];
+  s->off_next = off_[p ^ 1];
+  s->obase_next = obase_[p ^ 1];
 }
 
 int Engine::uniform_d() const { return plan_.needs.min_d == plan_.needs.max_d ? plan_.needs.max_d : 0; }
@@ -342,7 +350,7 @@ kdt_status Engine::admit(uint32_t slot, const float* points, const kdt_params& p
   recs_[slot] = (uint32_t)(p.depth > 0 ? leaves : std::min<uint64_t>(leaves, 2 * n / (uint64_t)p.leaf_size + 2));
   sorts_[slot] = tp.leafsort ? 1 : 0;
   Pending pe;
-  pe.rec = AdmitRec{h, slot, root_terminal ? 1u : 0u, nullptr};
+  pe.rec = AdmitRec{h, slot, root_terminal ? 1u : 0u, nullptr, 0, 0};
   pe.list = root_terminal ? kListNone
             : !(n <= (uint64_t)tp.small_max && !tp.presorted) ? kListBig
             : tp.sub_wide ? kListSmallWide : kListSmall;
@@ -370,6 +378,10 @@ kdt_status Engine::flush_admits(bool* has_big_roots) {
     const uint64_t n = (uint64_t)pe.rec.tree.n;
     if (pe.list == kListBig) {
       pe.rec.root_dst = big_[cur_] + big_count_++;
+      pe.rec.tile0 = big_tiles_;
+      pe.rec.seg0 = big_segs_;
+      big_tiles_ += tiles_of((uint32_t)n);
+      big_segs_ += (uint32_t)pe.rec.tree.r;
       big_points_ += n;
     } else if (pe.list == kListSmall) {
       pe.rec.root_dst = small_ + small_count_++;
@@ -396,29 +408,17 @@ kdt_status Engine::tick() {
     s_.init_small = small_count_;
     s_.init_small_w = small_count_w_;
     s_.init_small_points = (uint32_t)small_points_;
-    s_.cells = big_[cur_];
+    use_lists(&s_, cur_);
     s_.ncells = big_count_;
-    s_.next_big = big_[cur_ ^ 1];
-    s_.off_cur = off_[cur_];
-    s_.obase_cur = obase_[cur_];
-    s_.off_next = off_[cur_ ^ 1];
-    s_.obase_next = obase_[cur_ ^ 1];
-    const uint64_t nseg_bound = std::min<uint64_t>((uint64_t)big_count_ * (uint64_t)plan_.needs.max_r, plan_.nseg_cap);
-    // tiles of this step: at most one per kTile points plus one per cell (a
-    // tight launch size; the plan's max_tiles is the capacity of a full forest)
-    // (the point counter is one device word: trust it only while it cannot wrap)
-    const uint32_t tiles_bound =
-        plan_.needs.points > 0xffffffffull
-            ? plan_.max_tiles
-            : (uint32_t)std::min<uint64_t>(big_points_ / (uint64_t)kTile + (uint64_t)big_count_ + 1,
-                                           (uint64_t)plan_.max_tiles);
+    s_.ntiles = std::min(big_tiles_, plan_.max_tiles);
+    s_.nseg = std::min(big_segs_, plan_.nseg_cap);
+    s_.few_segs = step_selects_all(s_.nseg, big_points_, plan_.sms) ? 1u : 0u;
     const SelectTuning tune = current_tuning();
     s_.tiny_max = tune.tiny_max;
     s_.bitonic_max = tune.bitonic_max;
     s_.warp_max = tune.warp_max;
-    launch_big_step(trees_, s_, tiles_bound, (uint32_t)nseg_bound, plan_.bigseg_cap, has_roots, root_dims_,
-                    plan_.needs.widest, plan_.needs.max_r,
-                    uniform_d(), tune, big_points_,
+    launch_big_step(trees_, s_, s_.ntiles, s_.nseg, plan_.bigseg_cap, has_roots, root_dims_, plan_.needs.widest,
+                    plan_.needs.max_r, uniform_d(), tune, big_points_,
                     plan_.grid_step, st_, plan_.needs.fourier);
     ENGINE_TRY(cudaGetLastError());
     root_dims_ = false;
@@ -429,20 +429,21 @@ kdt_status Engine::tick() {
       const uint32_t mt = std::max<uint32_t>(plan_.needs.max_trees, 1);
       std::vector<int32_t> stv(mt);
       ENGINE_TRY(cudaMemcpy(stv.data(), slot_words_ + (size_t)S_STATUS * mt, (size_t)mt * 4, cudaMemcpyDeviceToHost));
-      std::fprintf(stderr, "kdt tick: big %u -> %u, small %u + %u\n", big_count_, w[W_NEXTBIG], w[W_SMALL],
-                   w[W_SMALLW]);
+      std::fprintf(stderr, "kdt tick: big %u -> %u, small %u + %u\n", big_count_, w[W_BIG + 2 * (cur_ ^ 1)], w[W_SMALL],
+                   w[W_SMALL + 1]);
       for (uint32_t k = 0; k < mt; ++k)
         if (stv[k]) std::fprintf(stderr, "kdt tick: slot %u status %d\n", k, stv[k]);
     }
-    big_count_ = std::min(w[W_NEXTBIG], plan_.maxB);
+    const uint32_t* wb = w + W_BIG + 2 * (cur_ ^ 1);
+    const uint32_t* wt = w + W_TILE + 2 * (cur_ ^ 1);
+    big_count_ = std::min(wb[0], plan_.maxB);
+    big_segs_ = std::min(wb[1], plan_.nseg_cap);
+    big_tiles_ = std::min(wt[0], plan_.max_tiles);
+    big_points_ = wt[1];
     small_count_ = std::min(w[W_SMALL], plan_.cap_small);
-    small_count_w_ = std::min(w[W_SMALLW], plan_.cap_small - small_count_);
-    big_points_ = w[W_BIGPTS];
+    small_count_w_ = std::min(w[W_SMALL + 1], plan_.cap_small - small_count_);
     small_points_ = w[W_SMALLPTS];
     cur_ ^= 1;
-  } else {
-    big_count_ = 0;
-    big_points_ = 0;
   }
   if (small_count_ > 0 || small_count_w_ > 0) {
     launch_small(false);
@@ -461,7 +462,7 @@ void Engine::launch_small(bool from_device) {
     // back walked from the end
     launch_subtree(kSubNarrow, trees_, small_, cap, words_ + W_SMALL, false, s_.small_off, words_ + W_HEAD, slices_,
                    plan_.needs.slice_cells, gn, 0, st_);
-    launch_subtree(kSubWide, trees_, small_, cap, words_ + W_SMALLW, true, s_.small_off, words_ + W_HEAD, slices_,
+    launch_subtree(kSubWide, trees_, small_, cap, words_ + W_SMALL + 1, true, s_.small_off, words_ + W_HEAD, slices_,
                    plan_.needs.slice_cells, gw, 0, st_);
     return;
   }
@@ -552,15 +553,12 @@ kdt_status Engine::finalize(const std::vector<uint32_t>& slots, std::vector<kdt_
 kdt_status Engine::record_tick(int p) {
   StepDev sd = s_;
   sd.init_small = sd.init_small_w = sd.init_small_points = 0;
-  sd.cells = big_[p];
-  sd.ncells = plan_.maxB;  // a capacity: the count is the device word
-  sd.ncells_dev = words_ + W_NC0 + p;
-  sd.next_big = big_[p ^ 1];
-  sd.next_big_count = words_ + W_NC0 + (p ^ 1);
-  sd.off_cur = off_[p];
-  sd.obase_cur = obase_[p];
-  sd.off_next = off_[p ^ 1];
-  sd.obase_next = obase_[p ^ 1];
+  use_lists(&sd, p);
+  sd.ncells = plan_.maxB;  // capacities: the counts are the device words
+  sd.ncells_dev = words_ + W_BIG + 2 * p;
+  sd.nseg_dev = words_ + W_BIG + 2 * p + 1;
+  sd.ntiles_dev = words_ + W_TILE + 2 * p;
+  sd.few_segs = 0;
   const SelectTuning tune = current_tuning();
   sd.tiny_max = tune.tiny_max;
   sd.bitonic_max = tune.bitonic_max;
@@ -586,10 +584,8 @@ kdt_status Engine::run_graph() {
   // from the device, until a step leaves no cell (the tick above has
   // launched the subtree kernel over its queue, so that queue is empty)
   const int p0 = cur_;
-  uint32_t init[3] = {0u, 0u, 0u};  // W_NC0, W_NC1, W_ITERS
-  init[p0] = big_count_;
-  ENGINE_TRY(cudaMemcpyAsync(words_ + W_NC0, init, sizeof(init), cudaMemcpyHostToDevice, st_));
-  ENGINE_TRY(cudaStreamSynchronize(st_));
+  // (the tick above left the list's counts in their device words)
+  ENGINE_TRY(cudaMemsetAsync(words_ + W_ITERS, 0, 4, st_));
   // the steps are recorded on a private stream (the caller's may be the
   // legacy default stream, which cannot be captured); the graph runs on the
   // caller's stream
@@ -630,7 +626,7 @@ kdt_status Engine::run_graph() {
   const uint64_t l0 = kdt_launch_count();
   kdt_status rec = record_tick(p0);
   if (rec == KDT_OK) rec = record_tick(p0 ^ 1);
-  if (rec == KDT_OK) launch_loop_cond(h, words_ + W_NC0 + p0, words_ + W_ITERS, kGraphIterMax, st_);
+  if (rec == KDT_OK) launch_loop_cond(h, words_ + W_BIG + 2 * p0, words_ + W_ITERS, kGraphIterMax, st_);
   const uint64_t per_iter = kdt_launch_count() - l0;
   st_ = caller;
   cudaGraph_t captured = nullptr;
@@ -640,12 +636,13 @@ kdt_status Engine::run_graph() {
   if ((e = cudaGetLastError()) != cudaSuccess) return fail("recording", e);
   if ((e = cudaGraphInstantiate(&gr.ex, gr.g, 0)) != cudaSuccess) return fail("instantiate", e);
   if ((e = cudaGraphLaunch(gr.ex, st_)) != cudaSuccess) return fail("launch", e);
-  uint32_t fin[3];
-  ENGINE_TRY(cudaMemcpyAsync(fin, words_ + W_NC0, sizeof(fin), cudaMemcpyDeviceToHost, st_));
+  uint32_t fin[W_COUNT];
+  ENGINE_TRY(cudaMemcpyAsync(fin, words_, sizeof(fin), cudaMemcpyDeviceToHost, st_));
   ENGINE_TRY(cudaStreamSynchronize(st_));
-  if (fin[2] > 1) trace_add_launches((uint64_t)(fin[2] - 1) * per_iter);  // replays beyond the recorded one
-  graph_iters_ = fin[2];
-  if (fin[p0] != 0) return KDT_ERR_CUDA;  // stopped at the iteration cap with cells left
+  const uint32_t iters = fin[W_ITERS];
+  if (iters > 1) trace_add_launches((uint64_t)(iters - 1) * per_iter);  // replays beyond the recorded one
+  graph_iters_ = iters;
+  if (fin[W_BIG + 2 * p0] != 0) return KDT_ERR_CUDA;  // stopped at the iteration cap with cells left
   big_count_ = small_count_ = small_count_w_ = 0;
   big_points_ = small_points_ = 0;
   return KDT_OK;

@@ -63,8 +63,7 @@ struct StepPlan {
   // sms: the device's SMs (the subtree kernel's grid is sms x its shape's CTAs)
   uint32_t maxB = 0, cap_small = 0, max_tiles = 0, nseg_cap = 0, bigseg_cap = 0, grid_step = 0, sms = 0, off_cap = 0,
            small_off_cap = 0;
-  size_t trees = 0, words = 0, slot_words = 0, slots_list = 0, admits = 0, big[2] = {0, 0}, small = 0, tile_base = 0,
-         seg_base = 0, tiles = 0, tile_seg = 0, tile_left = 0, tile_loff = 0, tile_mm = 0, child_mm = 0, kdim = 0,
+  size_t trees = 0, words = 0, slot_words = 0, slots_list = 0, admits = 0, big[2] = {0, 0}, small = 0, tiles = 0, tile_seg = 0, tile_left = 0, tile_loff = 0, tile_mm = 0, child_mm = 0, kdim = 0,
          mkey = 0, lcount = 0, seg_w = 0, seg_key = 0, seg_med = 0, bigseg = 0, midseg = 0, slices = 0,
          off[2] = {0, 0}, obase[2] = {0, 0}, small_off = 0, crow = 0;
   size_t bytes = 0;
@@ -123,6 +122,7 @@ class Engine {
   StepDev s_{};
   int cur_ = 0;
   uint32_t big_count_ = 0, small_count_ = 0, small_count_w_ = 0;  // small: front (narrow), back (wide)
+  uint32_t big_tiles_ = 0, big_segs_ = 0;  // of the big cells
   uint64_t big_points_ = 0, small_points_ = 0;
   bool root_dims_ = false;
   bool debug_ = false;
@@ -140,6 +140,7 @@ class Engine {
     List list;
   };
   kdt_status flush_admits(bool* has_big_roots);
+  void use_lists(StepDev* s, int p);
   // The coordinate count of every tree of the forest, 0 if they differ.
   int uniform_d() const;
   std::vector<Pending> pending_;

@@ -99,7 +99,7 @@ constexpr uint32_t kNoRow = 0xffffffffu;
 
 // A cell of the tree: a contiguous position range [begin, begin+count) of its
 // tree's current order.
-struct Cell {
+struct alignas(16) Cell {
   uint32_t begin;
   uint32_t count;
   uint32_t heap;
@@ -109,6 +109,8 @@ struct Cell {
   int16_t dim;    // widest-spread key coordinate if already known, else -1
   uint32_t row = kNoRow;  // cells queued for the subtree kernel: row of small_off with the cell's
                           // subset offsets, or kNoRow
+  uint32_t tile0 = 0;     // big cells: first of the cell's tiles and segments in the step's tables
+  uint32_t seg0 = 0;
 };
 
 // A terminal cell (leaf of the real tree); finalize turns these into offsets
@@ -126,11 +128,11 @@ struct StepDev {
   const Cell* cells;      // big cells of this step
   uint32_t ncells;              // cells of this step (steps driven by the host)
   const uint32_t* ncells_dev;   // if set: the device word that holds it (steps inside a graph)
-  uint32_t pad;
-  uint32_t* tile_base;    // [ncells+1] first tile of each cell (exclusive scan)
-  uint32_t* seg_base;     // [ncells+1] first segment of each cell
+  uint32_t ntiles, nseg;        // tiles and segments of this step, or the device words:
+  const uint32_t* ntiles_dev;
+  const uint32_t* nseg_dev;
+  uint32_t tiles_cap, nseg_cap;
   uint2* tiles;           // [ntiles] (cell, offset within cell)
-  uint32_t* ntiles_total; // device word
   uint32_t* kdim;         // [ncells] key coordinate
   uint32_t* mkey;         // [ncells] split key
   uint32_t* lcount;       // [ncells] left child size
@@ -142,22 +144,24 @@ struct StepDev {
   uint32_t* seg_med;      // [nseg] lower median key
   uint32_t* bigseg;       // [bigseg_cap] segments larger than kSelSmallMax
   uint32_t* bigseg_count; // device word
+  uint32_t* bigseg_count_next;  // the next step's, cleared by this one
   uint32_t* midseg;       // [midseg_cap] segments of kSelTinyMax+1 .. kSelSmallMax points
   uint32_t* midseg_count; // device word
+  uint32_t* midseg_count_next;
+  uint32_t few_segs;      // every segment gets a CTA: no lists
   uint32_t* tile_seg;     // [ntiles] first subset offset of the cell at or after the tile's start
   uint32_t* tile_left;    // [ntiles]
   uint32_t* tile_loff;    // [ntiles]
   Cell* next_big;         // children that stay in the multi-CTA pipeline
-  uint32_t* next_big_count;
+  unsigned long long* next_big_ctr;   // device: their number (low word) and their segments (high)
+  unsigned long long* next_tile_ctr;  // device: their tiles (low) and points (high)
   Cell* small;            // children that finish in the subtree kernel: cells of narrow-shape
                           // trees from the front, of wide-shape trees from the back
-  uint32_t* small_count;  // cells at the front
-  uint32_t* small_count_w;  // cells at the back (small[small_cap - 1 - j])
-  uint32_t* small_total;    // both (appends past small_cap fail)
+  unsigned long long* small_ctr;  // device: cells at the front (low word) and at the back (high:
+                                  // small[small_cap - 1 - j])
   uint32_t next_big_cap;
   uint32_t small_cap;
   uint32_t init_small, init_small_w, init_small_points;  // the queue's contents when the step starts
-  uint32_t* next_big_points;  // points in next_big (for bandwidth accounting)
   uint32_t* small_points;     // points appended to small
   // subset offsets (relative to the cell's begin, r+1 per cell) of this
   // step's cells: rows of off_cur at obase_cur[c]; level-0 cells use their
@@ -166,7 +170,6 @@ struct StepDev {
   const uint32_t* obase_cur;  // [ncells]
   uint32_t* off_next;
   uint32_t* obase_next;       // [next_big_cap]
-  uint32_t* off_used;         // device word: words of off_next handed out
   uint32_t off_cap;
   // subset offsets of cells queued for the subtree kernel (explicit ids, while
   // rows last; other modes follow from the original index, and so does a cell
@@ -255,6 +258,16 @@ __device__ __forceinline__ uint32_t subset_of(const TreeDev& t, uint32_t orig) {
 // reads (clamped to the capacity of the cell lists).
 __device__ __forceinline__ uint32_t ncells_of(const StepDev& s) {
   return s.ncells_dev ? min(*s.ncells_dev, s.next_big_cap) : s.ncells;
+}
+
+__device__ __forceinline__ uint32_t ntiles_of(const StepDev& s) {
+  return s.ntiles_dev ? min(*s.ntiles_dev, s.tiles_cap) : s.ntiles;
+}
+__device__ __forceinline__ uint32_t nseg_of(const StepDev& s) {
+  return s.nseg_dev ? min(*s.nseg_dev, s.nseg_cap) : s.nseg;
+}
+__host__ __device__ __forceinline__ uint32_t tiles_of(uint32_t count) {
+  return count / (uint32_t)kTile + (count % (uint32_t)kTile != 0u ? 1u : 0u);
 }
 
 // Points of step cell c whose split is being combined: its own count, or in a

@@ -96,6 +96,7 @@ struct AdmitRec {
   uint32_t slot;
   uint32_t terminal;  // the root is a leaf
   Cell* root_dst;     // else: its entry of a cell list
+  uint32_t tile0, seg0;  // and where a big root's tiles and segments start
 };
 constexpr uint32_t kAdmitIota = 65536;  // larger terminal roots get their identity permutation from a launch of their own
 constexpr int kAdmitFew = 8;            // records that travel as launch parameters (below 4 KB)
@@ -107,6 +108,8 @@ static_assert(sizeof(AdmitFew) <= 4000, "launch parameters");
 cudaError_t launch_admit(const std::vector<AdmitRec>& recs, AdmitRec* staging, TreeDev* trees, cudaStream_t st);
 
 cudaError_t prepare_step_kernels();
+// Whether a step of nseg segments of so many points gets a CTA for each (StepDev::few_segs).
+bool step_selects_all(uint32_t nseg, uint64_t points, uint32_t sms);
 // One thread: the loop condition of a graph whose body is a pair of level
 // steps (keep going while ncells_next > 0, at most `limit` iterations; the
 // count of iterations is kept in *iters).

@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kST, scatter_ctas(kD, kMM)) k_scatter_tma(cons
                                               // min / max key per coordinate
   __shared__ uint32_t s_fail;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t ntiles = *s.ntiles_total;
+  const uint32_t ntiles = ntiles_of(s);
   // this CTA's contiguous range of tiles: consecutive tiles mostly share a
   // cell, so the per-cell min / max stay in the CTA for long runs
   const uint32_t t_begin = (uint32_t)(((uint64_t)blockIdx.x * ntiles) / gridDim.x);

@@ -66,15 +66,15 @@ __global__ void k_shard_medians(const TreeDev* trees, StepDev s) {
     }
     w = warp_sum(w);
     if (lane == 0) s.wcount[c] = w;
-    const uint32_t g0 = s.seg_base[c];
+    const uint32_t g0 = cell.seg0;
     for (uint32_t j = lane; j < r; j += 32) {
       const uint32_t o = j % G;
       if (o == g) continue;  // this shard's own subset
       const uint32_t co = row[(size_t)o * s.shard_span];
       uint32_t med = 0, wj = 0;
       if (co != kNoRow) {
-        med = s.seg_med[s.seg_base[co] + j];
-        wj = s.seg_w[s.seg_base[co] + j];
+        med = s.seg_med[s.cells[co].seg0 + j];
+        wj = s.seg_w[s.cells[co].seg0 + j];
       }
       s.seg_med[g0 + j] = med;
       s.seg_w[g0 + j] = wj;

@@ -48,94 +48,29 @@ __host__ __device__ constexpr uint32_t ps_places(uint32_t r) { return kPsPoints 
 constexpr size_t ps_smem_bytes(uint32_t r) { return (size_t)((ps_places(r) + 7u) & ~7u) * 6; }
 
 __device__ __forceinline__ bool tile_of(const StepDev& s, uint32_t tile, uint2* out) {
-  if (tile >= *s.ntiles_total) return false;
+  if (tile >= ntiles_of(s)) return false;
   *out = s.tiles[tile];
   return true;
 }
 
-// ---------------------------------------------------------------- prep
+// ---------------------------------------------------------------- roots
 
-// Single CTA: per-cell tile and segment counts, exclusive scans, key dims
-// that are already known. Each thread takes kPrepItems consecutive cells per
-// round, so a deep level's many cells cost few block scans.
-constexpr int kPrepItems = 4;
-
-__global__ void k_prep(const TreeDev* trees, StepDev s) {
-  __shared__ uint32_t tmp[33];
-  uint32_t tile_run = 0, seg_run = 0;
-  const uint32_t ncells = ncells_of(s);
-  for (uint32_t c0 = 0; c0 < ncells; c0 += blockDim.x * kPrepItems) {
-    const uint32_t cb = c0 + threadIdx.x * kPrepItems;
-    uint32_t nt[kPrepItems], ns[kPrepItems], st = 0, ss = 0;
-#pragma unroll
-    for (int q = 0; q < kPrepItems; ++q) {
-      const uint32_t c = cb + q;
-      nt[q] = 0;
-      ns[q] = 0;
-      if (c < ncells) {
-        const Cell cell = s.cells[c];
-        const TreeDev& t = trees[cell.tree];
-        nt[q] = (cell.count + kTile - 1) / kTile;
-        ns[q] = (uint32_t)t.r;
-        if (t.key_rule == KEY_CYCLIC)
-          s.kdim[c] = (uint32_t)(cell.level % t.d);
-        else if (cell.dim >= 0)
-          s.kdim[c] = (uint32_t)cell.dim;
-      }
-      st += nt[q];
-      ss += ns[q];
-    }
-    uint32_t tot_t, tot_s;
-    uint32_t et = block_excl_scan(st, tmp, &tot_t);
-    uint32_t es = block_excl_scan(ss, tmp, &tot_s);
-#pragma unroll
-    for (int q = 0; q < kPrepItems; ++q) {
-      const uint32_t c = cb + q;
-      if (c < ncells) {
-        s.tile_base[c] = tile_run + et;
-        s.seg_base[c] = seg_run + es;
-      }
-      et += nt[q];
-      es += ns[q];
-    }
-    tile_run += tot_t;
-    seg_run += tot_s;
-  }
-  if (threadIdx.x == 0) {
-    s.tile_base[ncells] = tile_run;
-    s.seg_base[ncells] = seg_run;
-    *s.ntiles_total = tile_run;
-    // the counters that the step's later kernels append to
-    *s.bigseg_count = 0;
-    *s.midseg_count = 0;
-    *s.next_big_count = 0;
-    *s.next_big_points = 0;
-    *s.off_used = 0;
-    *s.small_count = s.init_small;
-    *s.small_count_w = s.init_small_w;
-    *s.small_total = s.init_small + s.init_small_w;
-    *s.small_points = s.init_small_points;
-    *s.small_off_used = 0;
-  }
-}
-
-// One warp per cell: tile list entries; zeroed subset counts of a presorted
-// root, and (widest spread, coordinate not known yet) the identities in its
-// first tile's min / max record, which the presort's groups reduce into.
-// (Most cells of a deep level have one to three tiles.)
+// One warp per cell of a step with roots, before their presort: tile list
+// entries (the presort's kernels walk all tiles); zeroed subset counts of a
+// presorted root, and (widest spread, coordinate not known yet) the identities
+// in its first tile's min / max record, which the presort's groups reduce into.
 __device__ __forceinline__ void tiles_cell(const TreeDev* trees, const StepDev& s, uint32_t c) {
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t tb = s.tile_base[c], te = s.tile_base[c + 1];
-  for (uint32_t j = tb + lane; j < te; j += 32u) s.tiles[j] = make_uint2(c, (j - tb) * (uint32_t)kTile);
   const Cell cell = s.cells[c];
-  if (cell.level == 0) {
-    const TreeDev& t = trees[cell.tree];
-    if (t.presorted) {
-      for (uint32_t j = lane; j < (uint32_t)t.r; j += 32u) t.root_cur[j] = 0;
-      if (t.key_rule == KEY_WIDEST && cell.dim < 0 && tb < te)
-        for (uint32_t j = lane; j < 2u * (uint32_t)t.d; j += 32u)
-          s.tile_mm[((size_t)tb * 2 * kMaxDims + j / 2) * 2 + (j & 1)] = (j & 1) ? 0u : 0xffffffffu;
-    }
+  const uint32_t tb = cell.tile0, nt = tiles_of(cell.count);
+  for (uint32_t j = lane; j < nt; j += 32u) s.tiles[tb + j] = make_uint2(c, j * (uint32_t)kTile);
+  if (cell.level != 0) return;
+  const TreeDev& t = trees[cell.tree];
+  if (t.presorted) {
+    for (uint32_t j = lane; j < (uint32_t)t.r; j += 32u) t.root_cur[j] = 0;
+    if (t.key_rule == KEY_WIDEST && cell.dim < 0 && nt > 0u)
+      for (uint32_t j = lane; j < 2u * (uint32_t)t.d; j += 32u)
+        s.tile_mm[((size_t)tb * 2 * kMaxDims + j / 2) * 2 + (j & 1)] = (j & 1) ? 0u : 0xffffffffu;
   }
 }
 
@@ -160,7 +95,7 @@ __device__ __forceinline__ bool presort_tile(const TreeDev* trees, const StepDev
 // its end.
 __global__ void __launch_bounds__(kTileThreads) k_ps_count(const TreeDev* trees, StepDev s) {
   __shared__ uint32_t hist[kMaxSubsets];
-  const uint32_t ntiles = *s.ntiles_total;
+  const uint32_t ntiles = ntiles_of(s);
   const uint32_t t_begin = (uint32_t)(((uint64_t)blockIdx.x * ntiles) / gridDim.x);
   const uint32_t t_end = (uint32_t)(((uint64_t)(blockIdx.x + 1) * ntiles) / gridDim.x);
   int32_t cur = -1;  // tree whose counts hist holds
@@ -379,7 +314,7 @@ __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, St
   if (want_mm) {  // the passes' barriers order the shared-memory reductions before this
     // into the root's first tile record (identities set by k_tiles); this
     // tile's own record, if another, holds the identities
-    const uint32_t tb = s.tile_base[tl.x];
+    const uint32_t tb = cell.tile0;
     for (int j = threadIdx.x; j < 2 * t.d; j += kPsThreads) {
       uint32_t* acc = &s.tile_mm[((size_t)tb * 2 * kMaxDims + j / 2) * 2 + (j & 1)];
       if (j & 1) atomicMax(acc, gmm[j / 2][1]); else atomicMin(acc, gmm[j / 2][0]);
@@ -467,10 +402,10 @@ __device__ __forceinline__ void pick_dim_cell(const TreeDev* trees, const StepDe
   __syncthreads();
   // the roots of a sharded build's shards are parts of one root: every one
   // of them reduces the tiles of all
-  const uint32_t tb = s.shards ? 0u : s.tile_base[c];
+  const uint32_t tb = s.shards ? 0u : cell.tile0;
   // a presorted root's presort gathered its min / max in its first tile's
   // record; other roots' are spread over their tiles
-  const uint32_t te = s.shards ? s.tile_base[ncells_of(s)] : (t.presorted ? tb + 1u : s.tile_base[c + 1]);
+  const uint32_t te = s.shards ? ntiles_of(s) : tb + (t.presorted ? 1u : tiles_of(cell.count));
   const int lane = threadIdx.x & 31;
   for (int c0 = 0; c0 < t.d; c0 += 8) {
     const int nc = min(8, t.d - c0);
@@ -537,39 +472,52 @@ __device__ __forceinline__ const uint32_t* key_column(const TreeDev& t, const Ce
 __device__ __forceinline__ uint32_t kload(const uint32_t* p) { return ord_key(__uint_as_float(__ldg(p))); }
 
 
-// One CTA per cell (after its key coordinate is known): size and first key
-// of every (cell, subset) segment from the cell's subset offsets, and the
+// A group of `gt` threads per cell (after a root's presort and key
+// coordinate): the cell's tile list entries and key coordinate; size and first
+// key of every (cell, subset) segment from the cell's subset offsets, and the
 // lists of segments for the warp and CTA selects; for each of the cell's
-// tiles, the first segment start in it (the scatter turns the starts in a
-// tile into the children's). Offsets are clamped to the cell, so a damaged
-// table cannot send a later kernel outside it (it is reported instead).
-__device__ __forceinline__ void segs_cell(const TreeDev* trees, const StepDev& s, uint32_t c) {
+// tiles, the first segment start in it (the scatter turns the starts in a tile
+// into the children's). Offsets are clamped to the cell, so a damaged table
+// cannot send a later kernel outside it (it is reported instead). Where a
+// cell's tiles and segments start in the step's tables was settled when its
+// parent was classified, so no scan over the cells is needed.
+__device__ __forceinline__ void open_cell(const TreeDev* trees, const StepDev& s, uint32_t c, uint32_t tid,
+                                          uint32_t gt) {
   const Cell cell = s.cells[c];
   const TreeDev& t = trees[cell.tree];
+  const uint32_t tb = cell.tile0, nt = tiles_of(cell.count);
+  for (uint32_t k = tid; k < nt; k += gt) s.tiles[tb + k] = make_uint2(c, k * (uint32_t)kTile);
+  uint32_t dim;
+  if (t.key_rule == KEY_CYCLIC)
+    dim = (uint32_t)(cell.level % t.d);
+  else
+    dim = cell.dim >= 0 ? (uint32_t)cell.dim : s.kdim[c];  // (a widest root's was picked before)
+  if (tid == 0) s.kdim[c] = dim;
+  if (t.fourier_j) return;  // no segments
   const uint32_t r = (uint32_t)t.r;
   const uint32_t* off = cell.level == 0 ? t.root_off : s.off_cur + s.obase_cur[c];
-  const uint32_t g0 = s.seg_base[c];
-  const uint32_t* kc = key_column(t, cell, s.kdim[c]) + cell.begin;
-  if (threadIdx.x == 0 && (off[0] != 0u || off[r] != cell.count)) set_status(t, ST_INTERNAL);
+  const uint32_t g0 = cell.seg0;
+  const uint32_t* kc = key_column(t, cell, dim) + cell.begin;
+  if (tid == 0 && (off[0] != 0u || off[r] != cell.count)) set_status(t, ST_INTERNAL);
   // tiles that start in (off[j], off[j + 1]] have start j + 1 as their first
   // (the first tile, at 0, has start 0); with fewer subsets than threads
   // several threads share a segment's tiles
-  const uint32_t tb = s.tile_base[c], nt = s.tile_base[c + 1] - tb;
-  if (threadIdx.x == 0 && nt > 0u) s.tile_seg[tb] = 0;
+  if (tid == 0 && nt > 0u) s.tile_seg[tb] = 0;
   if (nt > 1u) {
-    const uint32_t per = max(1u, blockDim.x / r);
-    for (uint32_t q = threadIdx.x; q < r * per; q += blockDim.x) {
+    const uint32_t per = max(1u, gt / r);
+    for (uint32_t q = tid; q < r * per; q += gt) {
       const uint32_t j = q / per, a = min(off[j], cell.count), b = min(off[j + 1], cell.count);
       for (uint32_t k = a / (uint32_t)kTile + 1u + q % per; k < nt && k * (uint32_t)kTile <= b; k += per)
         s.tile_seg[tb + k] = j + 1u;
     }
   }
-  for (uint32_t j = threadIdx.x; j < r; j += blockDim.x) {
+  for (uint32_t j = tid; j < r; j += gt) {
     const uint32_t a = min(off[j], cell.count), b = min(off[j + 1], cell.count);
     if (b < a) set_status(t, ST_INTERNAL);
     const uint32_t w = b >= a ? b - a : 0u;
     s.seg_key[g0 + j] = kc + a;
     s.seg_w[g0 + j] = w;
+    if (s.few_segs) continue;
     if (w > s.warp_max) {
       const uint32_t k = atomicAdd(s.bigseg_count, 1u);
       if (k < s.bigseg_cap) s.bigseg[k] = g0 + j; else set_status(t, ST_INTERNAL);
@@ -580,12 +528,24 @@ __device__ __forceinline__ void segs_cell(const TreeDev* trees, const StepDev& s
   }
 }
 
-__global__ void k_segs(const TreeDev* trees, StepDev s) {
-  const uint32_t nc = ncells_of(s);
-  for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
-    segs_cell(trees, s, c);
-    __syncthreads();  // the cell's shared memory is free for the next one
+// The first kernel over a step's cells; `gt` divides the CTA. It also sets the
+// counters that the step's later kernels, and the next step's first, append to.
+// (Scanning the cells' tiles and segments first took two more launches, one of
+// them a single CTA: 135 us for the six steps of a build of 65,536 points, 50
+// now.)
+__global__ void __launch_bounds__(256) k_cells(const TreeDev* trees, StepDev s, uint32_t gt) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *s.next_big_ctr = 0ull;
+    *s.next_tile_ctr = 0ull;
+    *s.small_ctr = (unsigned long long)s.init_small | ((unsigned long long)s.init_small_w << 32);
+    *s.small_points = s.init_small_points;
+    *s.small_off_used = 0;
+    *s.bigseg_count_next = 0;
+    *s.midseg_count_next = 0;
   }
+  const uint32_t nc = ncells_of(s);
+  const uint32_t per = blockDim.x / gt, sub = threadIdx.x / gt, tid = threadIdx.x % gt;
+  for (uint32_t c = blockIdx.x * per + sub; c < nc; c += gridDim.x * per) open_cell(trees, s, c, tid, gt);
 }
 
 // ------------------------------------------------------------ selection
@@ -644,7 +604,7 @@ __device__ __forceinline__ uint32_t thread_lower_median(const uint32_t* keys, ui
 // networks in registers does (they spill about 300 bytes per thread to local
 // memory; measured faster than four or six CTAs per SM).
 __global__ void __launch_bounds__(256, 5) k_select_tiny(const TreeDev* trees, StepDev s) {
-  const uint32_t nseg = s.seg_base[ncells_of(s)];
+  const uint32_t nseg = nseg_of(s);
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t g0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); g0 < nseg; g0 += stride) {
@@ -836,14 +796,14 @@ __global__ void __launch_bounds__(256) k_select_small(const TreeDev* trees, Step
   }
 }
 
-// CTAs of kThreads stride over the listed segments above the warp-select
-// size: MSD radix select with kBits-bit digits (8: four passes, one histogram
+// Lower median of w >= 1 keys by a CTA of kThreads: MSD radix select with
+// kBits-bit digits (8: four passes, one histogram
 // per warp, which suits the few bins that the top digits of clustered data
 // fall into; 11: three passes over a CTA-wide 2048-bin histogram), keys read
 // from global memory 16 bytes at a time (the unaligned head and tail of the
 // segment by single words).
 template <int kThreads, int kBits>
-__global__ void __launch_bounds__(kThreads) k_select_big(const TreeDev* trees, StepDev s) {
+__device__ __forceinline__ uint32_t cta_lower_median(const uint32_t* keys, uint32_t w) {
   constexpr int kW = kThreads / 32;
   constexpr bool kWarpHist = kBits == 8;
   constexpr int kBins = 1 << kBits;
@@ -855,86 +815,103 @@ __global__ void __launch_bounds__(kThreads) k_select_big(const TreeDev* trees, S
   __shared__ uint32_t bcast[2];
   const int warp = threadIdx.x >> 5;
   uint32_t* tot = kWarpHist ? tot_w : hist;
+  const uint32_t head = min(w, (4u - (uint32_t)(((uintptr_t)keys >> 2) & 3u)) & 3u);
+  const uint4* kv = (const uint4*)(keys + head);  // 16-byte aligned
+  const uint32_t nv = (w - head) >> 2, tail0 = head + nv * 4u;
+  uint32_t rank = (w - 1) / 2, prefix = 0;
+  for (int top = 32; top > 0;) {  // bits [top, 32) are known
+    const int bits = top < kBits ? top : kBits, shift = top - bits;
+    const uint32_t mask = top == 32 ? 0u : ~((1u << top) - 1u), nb = 1u << bits;
+    for (int i = threadIdx.x; i < kHist; i += kThreads) hist[i] = 0;
+    __syncthreads();
+    uint32_t* wh = kWarpHist ? hist + warp * kBins : hist;
+    auto add = [&](uint32_t u) {
+      const uint32_t k = ord_key(__uint_as_float(u));
+      if ((k & mask) == prefix) atomicAdd(&wh[(k >> shift) & (nb - 1u)], 1u);
+    };
+    uint32_t v = threadIdx.x;
+    for (; v + 3 * kThreads < nv; v += 4 * kThreads) {
+      uint4 q[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) q[u] = __ldg(kv + v + u * kThreads);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        add(q[u].x);
+        add(q[u].y);
+        add(q[u].z);
+        add(q[u].w);
+      }
+    }
+    for (; v < nv; v += kThreads) {
+      const uint4 q = __ldg(kv + v);
+      add(q.x);
+      add(q.y);
+      add(q.z);
+      add(q.w);
+    }
+    if (threadIdx.x < head) add(__ldg(keys + threadIdx.x));
+    if (threadIdx.x < w - tail0) add(__ldg(keys + tail0 + threadIdx.x));
+    __syncthreads();
+    if (kWarpHist) {
+      for (int b = threadIdx.x; b < kBins; b += kThreads) {
+        uint32_t sum = 0;
+#pragma unroll
+        for (int q = 0; q < kW; ++q) sum += hist[q * kBins + b];
+        tot[b] = sum;
+      }
+      __syncthreads();
+    }
+    // the bin holding `rank`: each thread scans kPer consecutive bins
+    const uint32_t first = (uint32_t)threadIdx.x * kPer;
+    uint32_t loc[kPer], sum = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      loc[q] = first + q < nb ? tot[first + q] : 0u;
+      sum += loc[q];
+    }
+    uint32_t all;
+    const uint32_t ex = block_excl_scan(sum, tmp, &all);
+    if (rank >= ex && rank < ex + sum) {
+      uint32_t acc = ex;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        if (rank < acc + loc[q]) {
+          bcast[0] = first + q;
+          bcast[1] = acc;
+          break;
+        }
+        acc += loc[q];
+      }
+    }
+    __syncthreads();
+    rank -= bcast[1];
+    prefix |= bcast[0] << shift;
+    top = shift;
+    __syncthreads();
+  }
+  return prefix;
+}
+
+// CTAs stride over the listed segments above the warp-select size.
+template <int kThreads, int kBits>
+__global__ void __launch_bounds__(kThreads) k_select_big(const TreeDev* trees, StepDev s) {
   const uint32_t cnt = min(*s.bigseg_count, s.bigseg_cap);
   for (uint32_t jb = blockIdx.x; jb < cnt; jb += gridDim.x) {
     const uint32_t g = s.bigseg[jb];
+    const uint32_t med = cta_lower_median<kThreads, kBits>(s.seg_key[g], s.seg_w[g]);
+    if (threadIdx.x == 0) s.seg_med[g] = med;
+  }
+}
+
+// Steps of few segments: a CTA for every one of them, whatever its size, in
+// one launch instead of three.
+__global__ void __launch_bounds__(256) k_select_all(const TreeDev* trees, StepDev s) {
+  const uint32_t nseg = nseg_of(s);
+  for (uint32_t g = blockIdx.x; g < nseg; g += gridDim.x) {
     const uint32_t w = s.seg_w[g];
-    const uint32_t* keys = s.seg_key[g];
-    const uint32_t head = min(w, (4u - (uint32_t)(((uintptr_t)keys >> 2) & 3u)) & 3u);
-    const uint4* kv = (const uint4*)(keys + head);  // 16-byte aligned
-    const uint32_t nv = (w - head) >> 2, tail0 = head + nv * 4u;
-    uint32_t rank = (w - 1) / 2, prefix = 0;
-    for (int top = 32; top > 0;) {  // bits [top, 32) are known
-      const int bits = top < kBits ? top : kBits, shift = top - bits;
-      const uint32_t mask = top == 32 ? 0u : ~((1u << top) - 1u), nb = 1u << bits;
-      for (int i = threadIdx.x; i < kHist; i += kThreads) hist[i] = 0;
-      __syncthreads();
-      uint32_t* wh = kWarpHist ? hist + warp * kBins : hist;
-      auto add = [&](uint32_t u) {
-        const uint32_t k = ord_key(__uint_as_float(u));
-        if ((k & mask) == prefix) atomicAdd(&wh[(k >> shift) & (nb - 1u)], 1u);
-      };
-      uint32_t v = threadIdx.x;
-      for (; v + 3 * kThreads < nv; v += 4 * kThreads) {
-        uint4 q[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) q[u] = __ldg(kv + v + u * kThreads);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          add(q[u].x);
-          add(q[u].y);
-          add(q[u].z);
-          add(q[u].w);
-        }
-      }
-      for (; v < nv; v += kThreads) {
-        const uint4 q = __ldg(kv + v);
-        add(q.x);
-        add(q.y);
-        add(q.z);
-        add(q.w);
-      }
-      if (threadIdx.x < head) add(__ldg(keys + threadIdx.x));
-      if (threadIdx.x < w - tail0) add(__ldg(keys + tail0 + threadIdx.x));
-      __syncthreads();
-      if (kWarpHist) {
-        for (int b = threadIdx.x; b < kBins; b += kThreads) {
-          uint32_t sum = 0;
-#pragma unroll
-          for (int q = 0; q < kW; ++q) sum += hist[q * kBins + b];
-          tot[b] = sum;
-        }
-        __syncthreads();
-      }
-      // the bin holding `rank`: each thread scans kPer consecutive bins
-      const uint32_t first = (uint32_t)threadIdx.x * kPer;
-      uint32_t loc[kPer], sum = 0;
-#pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        loc[q] = first + q < nb ? tot[first + q] : 0u;
-        sum += loc[q];
-      }
-      uint32_t all;
-      const uint32_t ex = block_excl_scan(sum, tmp, &all);
-      if (rank >= ex && rank < ex + sum) {
-        uint32_t acc = ex;
-#pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-          if (rank < acc + loc[q]) {
-            bcast[0] = first + q;
-            bcast[1] = acc;
-            break;
-          }
-          acc += loc[q];
-        }
-      }
-      __syncthreads();
-      rank -= bcast[1];
-      prefix |= bcast[0] << shift;
-      top = shift;
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) s.seg_med[g] = prefix;
+    if (w == 0u) continue;
+    const uint32_t med = cta_lower_median<256, 11>(s.seg_key[g], w);
+    if (threadIdx.x == 0) s.seg_med[g] = med;
   }
 }
 
@@ -947,7 +924,7 @@ __device__ __forceinline__ void combine_cell(const TreeDev* trees, const StepDev
   const Cell cell = s.cells[c];
   const TreeDev& t = trees[cell.tree];
   const int r = t.r;
-  const uint32_t g0 = s.seg_base[c];
+  const uint32_t g0 = cell.seg0;
   const bool unit = t.combine_rule == 1;  // every non-empty subset counts once
   uint32_t rank = (cell_weight(s, c, cell) - 1) / 2, prefix = 0, mask = 0;
   if (unit) {  // rank (m - 1) / 2 among the m non-empty segments
@@ -1008,7 +985,7 @@ __device__ __forceinline__ void combine_warp_cell(const TreeDev* trees, const St
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Cell cell = s.cells[c];
   const TreeDev& t = trees[cell.tree];
-  const uint32_t g0 = s.seg_base[c];
+  const uint32_t g0 = cell.seg0;
   const uint32_t* med = s.seg_med + g0;
   const uint32_t* wt = s.seg_w + g0;
   const bool unit = t.combine_rule == 1;  // every non-empty subset counts once
@@ -1056,7 +1033,7 @@ __global__ void __launch_bounds__(256, 2) k_fourier_moments(const TreeDev* trees
   constexpr int kPer = kTile / 256;
   __shared__ float red[8][kFourierTerms];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t ntiles = *s.ntiles_total;
+  const uint32_t ntiles = ntiles_of(s);
   const uint32_t t_begin = (uint32_t)(((uint64_t)blockIdx.x * ntiles) / gridDim.x);
   const uint32_t t_end = (uint32_t)(((uint64_t)(blockIdx.x + 1) * ntiles) / gridDim.x);
   // a tile's record, cell and this thread's points (loaded one tile ahead)
@@ -1181,13 +1158,13 @@ __global__ void __launch_bounds__(kFsWarps * 32) k_fourier_split(const TreeDev* 
   __shared__ uint32_t s_neg[2];  // per parity of the round: bit w: F < 0 at warp w's midpoint
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t nc = ncells_of(s);
-  const uint32_t ntiles = *s.ntiles_total;
+  const uint32_t ntiles = ntiles_of(s);
   auto range_start = [&](uint32_t k) { return (uint32_t)(((uint64_t)k * ntiles) / mgrid); };
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
     const Cell cell = s.cells[c];
     const TreeDev& t = trees[cell.tree];
     const int nt = 2 * t.fourier_j + 1;
-    const uint32_t tb = s.tile_base[c], te = s.tile_base[c + 1];
+    const uint32_t tb = cell.tile0, te = tb + tiles_of(cell.count);
     // The moments kernel's runs of this cell start at tb and at every start of
     // a CTA's tile range inside (tb, te): with at least as many tiles as CTAs
     // the starts of ranges k0 + 1, k0 + 2, ... (k0: the range that holds tb),
@@ -1343,15 +1320,15 @@ __device__ __forceinline__ void part_count_tile(const TreeDev* trees, const Step
 // registers: a lane's sixteen 16-byte loads still fit, with a few words of
 // spill).
 __global__ void __launch_bounds__(256, 3) k_part_count(const TreeDev* trees, StepDev s) {
-  const uint32_t ntiles = *s.ntiles_total;
+  const uint32_t ntiles = ntiles_of(s);
   for (uint32_t tile = blockIdx.x * 8u + (threadIdx.x >> 5); tile < ntiles; tile += gridDim.x * 8u)
     part_count_tile(trees, s, tile, s.tiles[tile]);
 }
 
 // One CTA per cell: exclusive scan of its tiles' left counts.
-__device__ __forceinline__ void part_scan_cell(const StepDev& s, uint32_t c) {
+__device__ __forceinline__ void part_scan_cell(const StepDev& s, uint32_t c, const Cell& cell) {
   __shared__ uint32_t tmp[33];
-  const uint32_t tb = s.tile_base[c], te = s.tile_base[c + 1];
+  const uint32_t tb = cell.tile0, te = tb + tiles_of(cell.count);
   uint32_t run = 0;
   for (uint32_t j0 = tb; j0 < te; j0 += blockDim.x) {
     const uint32_t j = j0 + threadIdx.x;
@@ -1367,29 +1344,9 @@ __device__ __forceinline__ void part_scan_cell(const StepDev& s, uint32_t c) {
 __global__ void k_part_scan(StepDev s) {
   const uint32_t nc = ncells_of(s);
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
-    part_scan_cell(s, c);
+    part_scan_cell(s, c, s.cells[c]);
     __syncthreads();  // the cell's shared memory is free for the next one
   }
-}
-
-// One warp per cell (steps with many cells, few tiles each).
-__device__ __forceinline__ void part_scan_warp_cell(const StepDev& s, uint32_t c) {
-  const int lane = threadIdx.x & 31;
-  const uint32_t tb = s.tile_base[c], te = s.tile_base[c + 1];
-  uint32_t run = 0;
-  for (uint32_t j0 = tb; j0 < te; j0 += 32) {
-    const uint32_t j = j0 + (uint32_t)lane;
-    const uint32_t v = j < te ? s.tile_left[j] : 0u;
-    const uint32_t inc = warp_incl_scan(v);
-    if (j < te) s.tile_loff[j] = run + inc - v;
-    run += __shfl_sync(0xffffffffu, inc, 31);
-  }
-  if (lane == 0) s.lcount[c] = run;
-}
-
-__global__ void __launch_bounds__(256) k_part_scan_warp(StepDev s) {
-  const uint32_t nc = ncells_of(s);
-  for (uint32_t c = blockIdx.x * 8u + (threadIdx.x >> 5); c < nc; c += gridDim.x * 8u) part_scan_warp_cell(s, c);
 }
 
 // One warp per cell (widest spread): the key coordinate of each big child,
@@ -1440,81 +1397,239 @@ __global__ void __launch_bounds__(256, 1) k_child_dims(const TreeDev* trees, Ste
 
 // ------------------------------------------------------------- children
 
-// One thread per cell, after the children's sizes are known and before the
-// move: terminal children are recorded, small ones queued for the subtree
-// kernel, big ones get a slot of the next step and a row of its subset
-// offsets (which the scatter fills).
-__device__ __forceinline__ void classify_cell(const TreeDev* trees, const StepDev& s, uint32_t c) {
-  const Cell cell = s.cells[c];
+// Exclusive prefix of v over the warp's lanes; *total for all.
+__device__ __forceinline__ uint32_t warp_excl(uint32_t v, uint32_t* total) {
+  const uint32_t inc = warp_incl_scan(v);
+  *total = __shfl_sync(0xffffffffu, inc, 31);
+  return inc - v;
+}
+
+// The cells of a warp's active lanes, one each, after the children's sizes are
+// known and before the move: terminal children are recorded, small ones queued
+// for the subtree kernel, big ones get a slot of the next step, their tiles,
+// their segments and a row of subset offsets (which the scatter fills). The
+// warp's children reserve together, an atomic per counter (each counter is one
+// address for all cells of a step); every row of offsets is one word longer
+// than the child's segments, so the big children's slots and segments, counted
+// in one 64-bit word, give its place too.
+__device__ __forceinline__ void classify_lanes(const TreeDev* trees, const StepDev& s, uint32_t c, bool active) {
+  const int lane = threadIdx.x & 31;
+  Cell cell{};
+  uint32_t L = 0;
+  if (active) {
+    cell = s.cells[c];
+    L = s.lcount[c];
+  }
   const TreeDev& t = trees[cell.tree];
-  const uint32_t L = s.lcount[c], R = cell.count - L;
+  const uint32_t R = cell.count - L;
   const int level = cell.level + 1;
   const int stall = (R == 0) ? cell.stall + 1 : 0;
   const uint32_t cb[2] = {cell.begin, cell.begin + L};
   const uint32_t cc[2] = {L, R};
   int live_delta = -1;  // this cell is done; each child that still needs splitting adds one
-  if (t.key_rule == KEY_WIDEST)  // identities for the scatter's min / max reductions
-    for (int j = 0; j < 4 * t.d; ++j) {
-      const int side = j / (2 * t.d), l = (j / 2) % t.d, which = j & 1;
-      s.child_mm[(((size_t)c * 2 + side) * kMaxDims + l) * 2 + which] = which ? 0u : 0xffffffffu;
-    }
+  bool big[2] = {false, false}, small[2] = {false, false};
+  uint32_t row_words[2] = {0u, 0u};
+#pragma unroll
   for (int side = 0; side < 2; ++side) {
-    uint2 cr = make_uint2(kNoRow, kNoRow);
-    const uint32_t heap = 2u * cell.heap + 1u + (uint32_t)side;
+    if (!active) continue;
     if (is_terminal(t, cc[side], level, stall)) {
-      record_terminal(t, cb[side], cc[side], heap, level);
+      record_terminal(t, cb[side], cc[side], 2u * cell.heap + 1u + (uint32_t)side, level);
     } else if (t.depth == 0 && level >= t.max_levels) {
       set_status(t, ST_LEVEL_CAP);
     } else {
       ++live_delta;
-      Cell child{cb[side], cc[side], heap, cell.tree, (int8_t)level, (int8_t)stall, (int16_t)-1};
-      if (cc[side] <= (uint32_t)t.small_max) {
-        if (atomicAdd(s.small_total, 1u) < s.small_cap) {
-          // the two ends of the queue never meet: at most small_cap cells get a slot
-          const uint32_t slot = t.sub_wide ? s.small_cap - 1u - atomicAdd(s.small_count_w, 1u)
-                                           : atomicAdd(s.small_count, 1u);
-          // explicit ids: a row of subset offsets where it is shorter than the
-          // cell and there is room
-          if (t.subset_mode == SUB_EXPLICIT && (uint32_t)t.r < cc[side]) {
-            const uint32_t words = (uint32_t)t.r + 1u;
-            const uint32_t row = atomicAdd(s.small_off_used, words);
-            if (row < s.small_off_cap && words <= s.small_off_cap - row) child.row = row;
-          }
-          s.small[slot] = child;
-          cr = make_uint2(kNoRow, slot);  // its widest coordinate is picked with the big children's
-        } else {
-          set_status(t, ST_CAPACITY);
-        }
-        atomicAdd(s.small_points, cc[side]);
+      small[side] = cc[side] <= (uint32_t)t.small_max;
+      big[side] = !small[side];
+      // explicit ids: a row of subset offsets where it is shorter than the cell
+      if (small[side] && t.subset_mode == SUB_EXPLICIT && (uint32_t)t.r < cc[side])
+        row_words[side] = (uint32_t)t.r + 1u;
+    }
+  }
+  const uint32_t nb = (uint32_t)big[0] + (uint32_t)big[1], ns = (uint32_t)small[0] + (uint32_t)small[1];
+  const bool wide = active && t.sub_wide != 0;
+  const uint32_t tl[2] = {big[0] ? tiles_of(cc[0]) : 0u, big[1] ? tiles_of(cc[1]) : 0u};
+  const uint32_t segs = active ? nb * (uint32_t)t.r : 0u;
+  uint32_t nb_all, segs_all, tl_all, bp_all, nn_all, nw_all, sp_all, rw_all;
+  const uint32_t nb_ex = warp_excl(nb, &nb_all);
+  const uint32_t segs_ex = warp_excl(segs, &segs_all);
+  const uint32_t tl_ex = warp_excl(tl[0] + tl[1], &tl_all);
+  const uint32_t nn_ex = warp_excl(wide ? 0u : ns, &nn_all);
+  const uint32_t nw_ex = warp_excl(wide ? ns : 0u, &nw_all);
+  const uint32_t rw_ex = warp_excl(row_words[0] + row_words[1], &rw_all);
+  bp_all = warp_sum((big[0] ? cc[0] : 0u) + (big[1] ? cc[1] : 0u));
+  sp_all = warp_sum((small[0] ? cc[0] : 0u) + (small[1] ? cc[1] : 0u));
+  unsigned long long b0 = 0, t0 = 0, s0 = 0;
+  uint32_t w0 = 0;
+  if (lane == 0) {
+    if (nb_all) {
+      b0 = atomicAdd(s.next_big_ctr, (unsigned long long)nb_all | ((unsigned long long)segs_all << 32));
+      t0 = atomicAdd(s.next_tile_ctr, (unsigned long long)tl_all | ((unsigned long long)bp_all << 32));
+    }
+    if (nn_all | nw_all) {
+      s0 = atomicAdd(s.small_ctr, (unsigned long long)nn_all | ((unsigned long long)nw_all << 32));
+      atomicAdd(s.small_points, sp_all);
+    }
+    if (rw_all) w0 = atomicAdd(s.small_off_used, rw_all);
+  }
+  b0 = __shfl_sync(0xffffffffu, b0, 0);
+  t0 = __shfl_sync(0xffffffffu, t0, 0);
+  s0 = __shfl_sync(0xffffffffu, s0, 0);
+  w0 = __shfl_sync(0xffffffffu, w0, 0);
+  if (!active) return;
+  // the two ends of the queue never meet while their counts sum to small_cap at most
+  const bool room = (uint64_t)(uint32_t)s0 + (uint32_t)(s0 >> 32) + nn_all + nw_all <= (uint64_t)s.small_cap;
+  uint32_t slot_b = (uint32_t)b0 + nb_ex, seg = (uint32_t)(b0 >> 32) + segs_ex, tile = (uint32_t)t0 + tl_ex;
+  uint32_t slot_n = (uint32_t)s0 + nn_ex, slot_w = (uint32_t)(s0 >> 32) + nw_ex, rw = w0 + rw_ex;
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    uint2 cr = make_uint2(kNoRow, kNoRow);
+    Cell child{cb[side], cc[side], 2u * cell.heap + 1u + (uint32_t)side, cell.tree, (int8_t)level, (int8_t)stall,
+               (int16_t)-1};
+    if (small[side]) {
+      if (room) {
+        const uint32_t slot = wide ? s.small_cap - 1u - slot_w++ : slot_n++;
+        const uint32_t words = row_words[side];
+        if (words && rw < s.small_off_cap && words <= s.small_off_cap - rw) child.row = rw;
+        rw += words;
+        s.small[slot] = child;
+        cr = make_uint2(kNoRow, slot);  // its widest coordinate is picked with the big children's
       } else {
-        const uint32_t slot = atomicAdd(s.next_big_count, 1u);
-        const uint32_t row = atomicAdd(s.off_used, (uint32_t)t.r + 1u);
-        if (slot < s.next_big_cap && row <= s.off_cap - ((uint32_t)t.r + 1u)) {
-          s.next_big[slot] = child;
-          s.obase_next[slot] = row;
-          cr = make_uint2(slot, row);
-        } else {
-          set_status(t, ST_CAPACITY);
-        }
-        atomicAdd(s.next_big_points, cc[side]);
+        set_status(t, ST_CAPACITY);
       }
+    } else if (big[side]) {
+      const uint32_t r = (uint32_t)t.r, row = seg + slot_b;
+      if (slot_b < s.next_big_cap && row <= s.off_cap - (r + 1u) && seg + r <= s.nseg_cap &&
+          tile + tl[side] <= s.tiles_cap) {
+        child.tile0 = tile;
+        child.seg0 = seg;
+        s.next_big[slot_b] = child;
+        s.obase_next[slot_b] = row;
+        cr = make_uint2(slot_b, row);
+      } else {
+        set_status(t, ST_CAPACITY);
+      }
+      ++slot_b;
+      seg += r;
+      tile += tl[side];
     }
     s.crow[2 * c + side] = cr;
   }
   if (live_delta) atomicAdd(t.live, live_delta);
 }
 
-__global__ void k_classify(const TreeDev* trees, StepDev s) {
+// Identities for the scatter's min / max reductions of the cell's children.
+__device__ __forceinline__ void clear_child_mm(const TreeDev* trees, const StepDev& s, uint32_t c, uint32_t tid,
+                                               uint32_t threads) {
+  const TreeDev& t = trees[s.cells[c].tree];
+  if (t.key_rule != KEY_WIDEST) return;
+  for (uint32_t j = tid; j < 4u * (uint32_t)t.d; j += threads) {
+    const uint32_t side = j / (2u * (uint32_t)t.d), l = (j / 2u) % (uint32_t)t.d, which = j & 1u;
+    s.child_mm[(((size_t)c * 2 + side) * kMaxDims + l) * 2 + which] = which ? 0u : 0xffffffffu;
+  }
+}
+
+// 32 cells per CTA: the left counts of each cell's tiles are scanned by a warp
+// (unless k_part_scan did), then one warp classifies the 32 together.
+__global__ void __launch_bounds__(256) k_classify(const TreeDev* trees, StepDev s, bool scanned) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t nc = ncells_of(s);
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x)
-    classify_cell(trees, s, c);
+  for (uint32_t c0 = blockIdx.x * 32u; c0 < nc; c0 += gridDim.x * 32u) {
+    for (uint32_t c = c0 + warp; c < min(c0 + 32u, nc); c += 8u) {
+      clear_child_mm(trees, s, c, lane, 32u);
+      if (scanned) continue;
+      const Cell cell = s.cells[c];
+      const uint32_t tb = cell.tile0, te = tb + tiles_of(cell.count);
+      uint32_t run = 0;
+      for (uint32_t j0 = tb; j0 < te; j0 += 32) {
+        const uint32_t j = j0 + (uint32_t)lane;
+        const uint32_t v = j < te ? s.tile_left[j] : 0u;
+        const uint32_t inc = warp_incl_scan(v);
+        if (j < te) s.tile_loff[j] = run + inc - v;
+        run += __shfl_sync(0xffffffffu, inc, 31);
+      }
+      if (lane == 0) s.lcount[c] = run;
+    }
+    __syncthreads();
+    if (warp == 0) classify_lanes(trees, s, c0 + lane, c0 + lane < nc);
+    __syncthreads();
+  }
+}
+
+// Steps of few cells of few tiles: one CTA per cell does what k_combine,
+// k_part_count, k_part_scan and k_classify do in four launches (65,536 points, 8
+// subsets: 75 us for the six steps of a build, 183 in four launches each).
+constexpr int kSplitThreads = 512;
+__global__ void __launch_bounds__(kSplitThreads) k_split(const TreeDev* trees, StepDev s) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t nc = ncells_of(s);
+  for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
+    const Cell cell = s.cells[c];
+    clear_child_mm(trees, s, c, threadIdx.x, kSplitThreads);
+    combine_cell(trees, s, c);
+    __syncthreads();  // the split key is written
+    const uint32_t nt = tiles_of(cell.count);
+    for (uint32_t k = warp; k < nt; k += kSplitThreads / 32)
+      part_count_tile(trees, s, cell.tile0 + k, make_uint2(c, k * (uint32_t)kTile));
+    __syncthreads();
+    part_scan_cell(s, c, cell);
+    __syncthreads();
+    if (warp == 0) classify_lanes(trees, s, c, lane == 0);
+    __syncthreads();  // shared memory is free for the next cell
+  }
 }
 
 }  // namespace
 
 // ------------------------------------------------------------ launcher
 
-constexpr uint32_t kManyCells = 1024;  // from here on: a warp per cell in combine and scan
+constexpr uint32_t kManyCells = 1024;  // from here on: a warp per cell in combine
+
+// Steps whose launches weigh more than their work: while all segments fit the
+// SMs at once (8 CTAs of 256 threads each) and are of at most 8192 keys on
+// average, every one gets such a CTA, in one launch (65,536 points, 8 subsets:
+// 68 us for the six steps of a build, 229 in three launches a step). Larger ones
+// get the 512 threads of the listed path (64 segments of 780,000 keys and the
+// four levels below them: 1.33 ms here, 0.84 there).
+bool step_selects_all(uint32_t nseg, uint64_t points, uint32_t sms) {
+  return nseg <= 8u * sms && points <= 8192ull * nseg;
+}
+
+// One CTA per cell combines, counts, scans and classifies: while the cells'
+// CTAs fit the SMs at once (4 each) and a cell has at most 64 tiles on average
+// (a warp reads 4).
+static bool step_splits(const StepDev& s, uint32_t sms2) {
+  return !s.ncells_dev && s.ncells <= 2u * sms2 && s.ntiles <= 64u * s.ncells;
+}
+
+// The selects by segment size: one thread, one warp, one CTA per segment.
+static void launch_listed_selects(const TreeDev* trees, const StepDev& s, uint32_t nseg, uint32_t max_bigseg,
+                                  const SelectTuning& tune, uint64_t points, uint32_t sms, cudaStream_t st) {
+  {
+    TraceScope ts(K_SELECT_TINY, st, points);
+    k_select_tiny<<<std::max<uint32_t>(1, std::min<uint32_t>((nseg + 255) / 256, sms * 16u)), 256, 0, st>>>(trees, s);
+  }
+  {
+    TraceScope ts(K_SELECT_SMALL, st, points);
+    k_select_small<<<std::max<uint32_t>(1, std::min<uint32_t>((nseg + 7) / 8, sms * 8u)), 256, 0, st>>>(trees, s);
+  }
+  if (max_bigseg == 0) return;
+  TraceScope ts(K_SELECT_BIG, st);
+  // nseg bounds the big segments too; with few of them (the first levels
+  // of a large tree) a CTA's loads in flight set the rate, so they take
+  // 512 threads whatever the tuning
+  const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>(std::min(max_bigseg, nseg), sms * 4u));
+  if (tune.cta_threads == 512 || nseg <= sms * 4u) {
+    if (tune.digit_bits == 8)
+      k_select_big<512, 8><<<grid, 512, 0, st>>>(trees, s);
+    else
+      k_select_big<512, 11><<<grid, 512, 0, st>>>(trees, s);
+  } else {
+    if (tune.digit_bits == 8)
+      k_select_big<256, 8><<<grid, 256, 0, st>>>(trees, s);
+    else
+      k_select_big<256, 11><<<grid, 256, 0, st>>>(trees, s);
+  }
+}
 
 namespace {
 
@@ -1535,7 +1650,7 @@ __device__ __forceinline__ void admit_tree(const AdmitRec& a, TreeDev* trees) {
   if (a.terminal)
     t.terms[0] = TermRec{0u, (uint32_t)t.n, 0u, 0};
   else
-    *a.root_dst = Cell{0u, (uint32_t)t.n, 0u, (int32_t)a.slot, 0, 0, -1};
+    *a.root_dst = Cell{0u, (uint32_t)t.n, 0u, (int32_t)a.slot, 0, 0, -1, kNoRow, a.tile0, a.seg0};
 }
 
 __global__ void __launch_bounds__(256) k_admit(const AdmitRec* recs, TreeDev* trees) {
@@ -1586,10 +1701,9 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
     const uint32_t g = (nc + per_block - 1) / per_block;
     return std::max<uint32_t>(1, dev ? std::min(g, cap) : g);
   };
-  { TraceScope ts(K_PREP, st); k_prep<<<1, 1024, 0, st>>>(trees, s); }
-  { TraceScope ts(K_TILES, st); k_tiles<<<cells_grid(8, sms * 8u), 256, 0, st>>>(trees, s); }
   if (s.shards) launch_shard_index(s, nc, st);
   if (has_roots) {
+    { TraceScope ts(K_TILES, st); k_tiles<<<cells_grid(8, sms * 8u), 256, 0, st>>>(trees, s); }
     {
       TraceScope ts(K_PS_COUNT, st, points);
       k_ps_count<<<std::max<uint32_t>(1, std::min(max_tiles, sms * 4u)), kTileThreads, 0, st>>>(trees, s);
@@ -1601,10 +1715,19 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
     { TraceScope ts(K_MINMAX, st, points); k_minmax<<<max_tiles, kTileThreads, 0, st>>>(trees, s); }
     { TraceScope ts(K_PICK_DIM, st); k_pick_dim<<<nc, 1024, 0, st>>>(trees, s); }
   }
+  {
+    // threads per cell: enough for its segments
+    uint32_t gt = 32;
+    while (gt < 256u && gt < (uint32_t)max_r) gt *= 2;
+    if (!dev && nc < sms) gt = 256;  // few cells: their tiles count
+    TraceScope ts(K_CELLS, st);
+    k_cells<<<cells_grid(256u / gt, sms * 8u), 256, 0, st>>>(trees, s, gt);
+  }
   // a CTA per cell while cells are few (large subset counts, deep scans),
   // a warp per cell once they are many (and in a graph, where the count is
   // not known when the launch is recorded)
   const bool many = dev || nc >= kManyCells;
+  const bool split = step_splits(s, sms) && !fourier;
   if (fourier) {  // the paper's estimator: per-run sums, then the root per cell
     const uint32_t mgrid = std::max<uint32_t>(1, std::min(max_tiles, sms * 2u));
     {
@@ -1613,35 +1736,14 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
     }
     { TraceScope ts(K_FOURIER_SPLIT, st); k_fourier_split<<<cells_grid(1, sms * 4u), kFsWarps * 32, 0, st>>>(trees, s, mgrid); }
   } else {
-    { TraceScope ts(K_SEGS, st); k_segs<<<cells_grid(1, sms * 8u), 256, 0, st>>>(trees, s); }
-    {
-      TraceScope ts(K_SELECT_TINY, st, points);
-      k_select_tiny<<<std::max<uint32_t>(1, std::min<uint32_t>((nseg + 255) / 256, sms * 16u)), 256, 0, st>>>(trees, s);
-    }
-    {
-      TraceScope ts(K_SELECT_SMALL, st, points);
-      k_select_small<<<std::max<uint32_t>(1, std::min<uint32_t>((nseg + 7) / 8, sms * 8u)), 256, 0, st>>>(trees, s);
-    }
-    if (max_bigseg) {
-      TraceScope ts(K_SELECT_BIG, st);
-      // nseg bounds the big segments too; with few of them (the first levels
-      // of a large tree) a CTA's loads in flight set the rate, so they take
-      // 512 threads whatever the tuning
-      const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>(std::min(max_bigseg, nseg), sms * 4u));
-      if (tune.cta_threads == 512 || nseg <= sms * 4u) {
-        if (tune.digit_bits == 8)
-          k_select_big<512, 8><<<grid, 512, 0, st>>>(trees, s);
-        else
-          k_select_big<512, 11><<<grid, 512, 0, st>>>(trees, s);
-      } else {
-        if (tune.digit_bits == 8)
-          k_select_big<256, 8><<<grid, 256, 0, st>>>(trees, s);
-        else
-          k_select_big<256, 11><<<grid, 256, 0, st>>>(trees, s);
-      }
+    if (s.few_segs) {
+      TraceScope ts(K_SELECT_ALL, st, points);
+      k_select_all<<<std::max<uint32_t>(1, nseg), 256, 0, st>>>(trees, s);
+    } else {
+      launch_listed_selects(trees, s, nseg, max_bigseg, tune, points, sms, st);
     }
     if (s.shards) launch_shard_medians(trees, s, nc, st);  // the all-gather of the segment statistics
-    {
+    if (!split) {
       TraceScope ts(K_COMBINE, st);
       if (many)
         k_combine_warp<<<cells_grid(8, sms * 8u), 256, 0, st>>>(trees, s);
@@ -1649,18 +1751,22 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
         k_combine<<<nc, 256, 0, st>>>(trees, s);
     }
   }
-  {
-    TraceScope ts(K_PART_COUNT, st, points);
-    k_part_count<<<std::max<uint32_t>(1, std::min((max_tiles + 7) / 8, sms * 16u)), 256, 0, st>>>(trees, s);
-  }
-  {
-    TraceScope ts(K_PART_SCAN, st);
-    if (many)
-      k_part_scan_warp<<<cells_grid(8, sms * 8u), 256, 0, st>>>(s);
-    else
+  if (split) {
+    TraceScope ts(K_SPLIT, st, points);
+    k_split<<<nc, kSplitThreads, 0, st>>>(trees, s);
+  } else {
+    {
+      TraceScope ts(K_PART_COUNT, st, points);
+      k_part_count<<<std::max<uint32_t>(1, std::min((max_tiles + 7) / 8, sms * 16u)), 256, 0, st>>>(trees, s);
+    }
+    // a cell of very many tiles: a CTA scans them, not a warp
+    const bool scanned = !dev && max_tiles / nc > 64u;
+    if (scanned) {
+      TraceScope ts(K_PART_SCAN, st);
       k_part_scan<<<nc, 1024, 0, st>>>(s);
+    }
+    { TraceScope ts(K_CLASSIFY, st); k_classify<<<cells_grid(32, sms * 4u), 256, 0, st>>>(trees, s, scanned); }
   }
-  { TraceScope ts(K_CLASSIFY, st); k_classify<<<cells_grid(256, sms * 4u), 256, 0, st>>>(trees, s); }
   launch_scatter(trees, s, max_tiles, sms / 2, points, uniform_d, any_widest, st);
   if (any_widest && s.shards) launch_shard_minmax(trees, s, nc, st);
   if (any_widest) {

@@ -12,12 +12,12 @@ namespace kdt {
 namespace {
 
 const char* const kNames[K_NUM] = {
-    "k_prep",       "k_tiles",      "k_ps_count",   "k_ps_offsets",  "k_ps_move",     "k_segs",
+    "k_cells",       "k_tiles",      "k_ps_count",   "k_ps_offsets",  "k_ps_move",     "k_select_all",
     "k_minmax",     "k_pick_dim",   "k_select_tiny", "k_select_small", "k_select_big", "k_combine",    "k_part_count",
     "k_part_scan",  "k_classify",   "k_part_scatter", "k_child_dims",  "k_subtree",
     "k_finalize",   "k_iota",       "k_leaf_sort",  "k_leaf_hist",   "k_leaf_scan",   "k_leaf_scatter",
     "k_leaf_copy",  "k_fourier_moments", "k_fourier_split", "k_shard_exchange", "k_shard_split",
-    "k_shard_merge", "k_query",     "k_admit", "k_leaf_buckets"};
+    "k_shard_merge", "k_query",     "k_admit", "k_leaf_buckets", "k_split"};
 
 struct Pending {
   KernelId id;

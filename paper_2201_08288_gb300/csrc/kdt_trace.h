@@ -11,11 +11,11 @@
 namespace kdt {
 
 enum KernelId {
-  K_PREP, K_TILES, K_PS_COUNT, K_PS_OFFSETS, K_PS_MOVE, K_SEGS, K_MINMAX, K_PICK_DIM,
+  K_CELLS, K_TILES, K_PS_COUNT, K_PS_OFFSETS, K_PS_MOVE, K_SELECT_ALL, K_MINMAX, K_PICK_DIM,
   K_SELECT_TINY, K_SELECT_SMALL, K_SELECT_BIG, K_COMBINE, K_PART_COUNT, K_PART_SCAN, K_CLASSIFY, K_PART_SCATTER,
   K_CHILD_DIMS, K_SUBTREE, K_FINALIZE, K_IOTA, K_LEAF_SORT, K_LEAF_HIST, K_LEAF_SCAN,
   K_LEAF_SCATTER, K_LEAF_COPY, K_FOURIER_MOMENTS, K_FOURIER_SPLIT, K_SHARD_EXCHANGE, K_SHARD_SPLIT,
-  K_SHARD_MERGE, K_QUERY, K_ADMIT, K_LEAF_BUCKETS, K_NUM
+  K_SHARD_MERGE, K_QUERY, K_ADMIT, K_LEAF_BUCKETS, K_SPLIT, K_NUM
 };
 
 // Launches replayed by a graph beyond the ones counted while it was captured.
