@@ -95,6 +95,8 @@ kdt_params effective_params(const kdt_params& p) {
     e.subset_id8 = nullptr;
     e.subset_id16 = nullptr;
   }
+  // one subset by index is one block: index order is subset order
+  if (e.subset_mode == KDT_SUBSET_MOD && e.r == 1) e.subset_mode = KDT_SUBSET_CONTIGUOUS;
   return e;
 }
 
@@ -413,6 +415,8 @@ kdt_status Engine::tick() {
     s_.ntiles = std::min(big_tiles_, plan_.max_tiles);
     s_.nseg = std::min(big_segs_, plan_.nseg_cap);
     s_.few_segs = step_selects_all(s_.nseg, big_points_, plan_.sms) ? 1u : 0u;
+    // (not for shards: one segment of a shard's cell is a part of the cell's)
+    s_.wide_segs = !s_.shards && step_selects_wide(s_.nseg, big_points_) ? 1u : 0u;
     const SelectTuning tune = current_tuning();
     s_.tiny_max = tune.tiny_max;
     s_.bitonic_max = tune.bitonic_max;
@@ -558,7 +562,7 @@ kdt_status Engine::record_tick(int p) {
   sd.ncells_dev = words_ + W_BIG + 2 * p;
   sd.nseg_dev = words_ + W_BIG + 2 * p + 1;
   sd.ntiles_dev = words_ + W_TILE + 2 * p;
-  sd.few_segs = 0;
+  sd.few_segs = sd.wide_segs = 0;
   const SelectTuning tune = current_tuning();
   sd.tiny_max = tune.tiny_max;
   sd.bitonic_max = tune.bitonic_max;

@@ -149,6 +149,7 @@ struct StepDev {
   uint32_t* midseg_count; // device word
   uint32_t* midseg_count_next;
   uint32_t few_segs;      // every segment gets a CTA: no lists
+  uint32_t wide_segs;     // segments above warp_max get several CTAs (where their cell has room, wide_cell)
   uint32_t* tile_seg;     // [ntiles] first subset offset of the cell at or after the tile's start
   uint32_t* tile_left;    // [ntiles]
   uint32_t* tile_loff;    // [ntiles]

@@ -110,6 +110,8 @@ cudaError_t launch_admit(const std::vector<AdmitRec>& recs, AdmitRec* staging, T
 cudaError_t prepare_step_kernels();
 // Whether a step of nseg segments of so many points gets a CTA for each (StepDev::few_segs).
 bool step_selects_all(uint32_t nseg, uint64_t points, uint32_t sms);
+// ... or several CTAs for its large segments (StepDev::wide_segs).
+bool step_selects_wide(uint32_t nseg, uint64_t points);
 // One thread: the loop condition of a graph whose body is a pair of level
 // steps (keep going while ncells_next > 0, at most `limit` iterations; the
 // count of iterations is kept in *iters).

@@ -472,6 +472,19 @@ __device__ __forceinline__ const uint32_t* key_column(const TreeDev& t, const Ce
 __device__ __forceinline__ uint32_t kload(const uint32_t* p) { return ord_key(__uint_as_float(__ldg(p))); }
 
 
+// Words that a segment of several CTAs keeps while its median is sought: a
+// histogram, then its state (key bits found, rank left, CTAs that are done).
+// They lie in the part of the next level's first column that the cell's
+// scatter will overwrite, so a cell has room for them or takes one CTA per
+// segment.
+constexpr uint32_t kWideBins = 2048, kWideWords = kWideBins + 4;
+__device__ __forceinline__ bool wide_cell(const TreeDev& t, const Cell& cell) {
+  return (uint64_t)t.r * kWideWords <= (uint64_t)cell.count;
+}
+__device__ __forceinline__ uint32_t* wide_words(const TreeDev& t, const Cell& cell, uint32_t j) {
+  return (uint32_t*)t.xbuf[cell.level & 1] + cell.begin + (size_t)j * kWideWords;
+}
+
 // A group of `gt` threads per cell (after a root's presort and key
 // coordinate): the cell's tile list entries and key coordinate; size and first
 // key of every (cell, subset) segment from the cell's subset offsets, and the
@@ -511,13 +524,14 @@ __device__ __forceinline__ void open_cell(const TreeDev* trees, const StepDev& s
         s.tile_seg[tb + k] = j + 1u;
     }
   }
+  const bool wide = s.wide_segs && wide_cell(t, cell);
   for (uint32_t j = tid; j < r; j += gt) {
     const uint32_t a = min(off[j], cell.count), b = min(off[j + 1], cell.count);
     if (b < a) set_status(t, ST_INTERNAL);
     const uint32_t w = b >= a ? b - a : 0u;
     s.seg_key[g0 + j] = kc + a;
     s.seg_w[g0 + j] = w;
-    if (s.few_segs) continue;
+    if (s.few_segs || (wide && w > s.warp_max)) continue;
     if (w > s.warp_max) {
       const uint32_t k = atomicAdd(s.bigseg_count, 1u);
       if (k < s.bigseg_cap) s.bigseg[k] = g0 + j; else set_status(t, ST_INTERNAL);
@@ -796,6 +810,37 @@ __global__ void __launch_bounds__(256) k_select_small(const TreeDev* trees, Step
   }
 }
 
+// add(raw bits) for each of w keys by a CTA: 16 bytes at a time, four loads of
+// a thread in flight (the unaligned head and tail by single words).
+template <int kThreads, class Add>
+__device__ __forceinline__ void cta_for_keys(const uint32_t* keys, uint32_t w, Add add) {
+  const uint32_t head = min(w, (4u - (uint32_t)(((uintptr_t)keys >> 2) & 3u)) & 3u);
+  const uint4* kv = (const uint4*)(keys + head);  // 16-byte aligned
+  const uint32_t nv = (w - head) >> 2, tail0 = head + nv * 4u;
+  uint32_t v = threadIdx.x;
+  for (; v + 3 * kThreads < nv; v += 4 * kThreads) {
+    uint4 q[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) q[u] = __ldg(kv + v + u * kThreads);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      add(q[u].x);
+      add(q[u].y);
+      add(q[u].z);
+      add(q[u].w);
+    }
+  }
+  for (; v < nv; v += kThreads) {
+    const uint4 q = __ldg(kv + v);
+    add(q.x);
+    add(q.y);
+    add(q.z);
+    add(q.w);
+  }
+  if (threadIdx.x < head) add(__ldg(keys + threadIdx.x));
+  if (threadIdx.x < w - tail0) add(__ldg(keys + tail0 + threadIdx.x));
+}
+
 // Lower median of w >= 1 keys by a CTA of kThreads: MSD radix select with
 // kBits-bit digits (8: four passes, one histogram
 // per warp, which suits the few bins that the top digits of clustered data
@@ -815,9 +860,6 @@ __device__ __forceinline__ uint32_t cta_lower_median(const uint32_t* keys, uint3
   __shared__ uint32_t bcast[2];
   const int warp = threadIdx.x >> 5;
   uint32_t* tot = kWarpHist ? tot_w : hist;
-  const uint32_t head = min(w, (4u - (uint32_t)(((uintptr_t)keys >> 2) & 3u)) & 3u);
-  const uint4* kv = (const uint4*)(keys + head);  // 16-byte aligned
-  const uint32_t nv = (w - head) >> 2, tail0 = head + nv * 4u;
   uint32_t rank = (w - 1) / 2, prefix = 0;
   for (int top = 32; top > 0;) {  // bits [top, 32) are known
     const int bits = top < kBits ? top : kBits, shift = top - bits;
@@ -829,28 +871,7 @@ __device__ __forceinline__ uint32_t cta_lower_median(const uint32_t* keys, uint3
       const uint32_t k = ord_key(__uint_as_float(u));
       if ((k & mask) == prefix) atomicAdd(&wh[(k >> shift) & (nb - 1u)], 1u);
     };
-    uint32_t v = threadIdx.x;
-    for (; v + 3 * kThreads < nv; v += 4 * kThreads) {
-      uint4 q[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) q[u] = __ldg(kv + v + u * kThreads);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        add(q[u].x);
-        add(q[u].y);
-        add(q[u].z);
-        add(q[u].w);
-      }
-    }
-    for (; v < nv; v += kThreads) {
-      const uint4 q = __ldg(kv + v);
-      add(q.x);
-      add(q.y);
-      add(q.z);
-      add(q.w);
-    }
-    if (threadIdx.x < head) add(__ldg(keys + threadIdx.x));
-    if (threadIdx.x < w - tail0) add(__ldg(keys + tail0 + threadIdx.x));
+    cta_for_keys<kThreads>(keys, w, add);
     __syncthreads();
     if (kWarpHist) {
       for (int b = threadIdx.x; b < kBins; b += kThreads) {
@@ -913,6 +934,87 @@ __global__ void __launch_bounds__(256) k_select_all(const TreeDev* trees, StepDe
     const uint32_t med = cta_lower_median<256, 11>(s.seg_key[g], w);
     if (threadIdx.x == 0) s.seg_med[g] = med;
   }
+}
+
+// Steps of few, large segments (the first levels, and every tree of few
+// subsets): a segment's keys are spread over gridDim.x CTAs. Three launches,
+// 11 key bits each (10 in the last): every CTA counts the digits of its part
+// in shared memory and adds them to the segment's histogram; the last one to
+// finish finds the digit that holds the rank and clears the histogram for the
+// next launch. One segment of 20,000,003 keys (a tree of one subset, depth 10):
+// kdt_build 18.6 -> 2.7 ms, where one CTA had read it three times.
+constexpr int kWideThreads = 512;
+
+__device__ __forceinline__ bool wide_segment(const TreeDev* trees, const StepDev& s, uint32_t* g, uint32_t* w,
+                                             uint32_t** words) {
+  const Cell cell = s.cells[blockIdx.z];
+  const TreeDev& t = trees[cell.tree];
+  if (blockIdx.y >= (uint32_t)t.r || !wide_cell(t, cell)) return false;
+  *g = cell.seg0 + blockIdx.y;
+  *w = s.seg_w[*g];
+  *words = wide_words(t, cell, blockIdx.y);
+  return *w > s.warp_max;
+}
+
+__global__ void __launch_bounds__(kWideThreads) k_wide_clear(const TreeDev* trees, StepDev s) {
+  uint32_t g, w, *H;
+  if (!wide_segment(trees, s, &g, &w, &H)) return;
+  for (uint32_t i = threadIdx.x; i < kWideWords; i += kWideThreads) H[i] = i == kWideBins + 1u ? (w - 1u) / 2u : 0u;
+}
+
+__global__ void __launch_bounds__(kWideThreads) k_wide_pass(const TreeDev* trees, StepDev s, int top) {
+  __shared__ uint32_t hist[kWideBins];
+  __shared__ uint32_t tmp[33];
+  __shared__ bool last;
+  constexpr int kPer = kWideBins / kWideThreads;
+  uint32_t g, w, *H;
+  if (!wide_segment(trees, s, &g, &w, &H)) return;
+  uint32_t* state = H + kWideBins;
+  const int bits = min(top, 11), shift = top - bits;
+  const uint32_t mask = top == 32 ? 0u : ~((1u << top) - 1u), nb = 1u << bits;
+  const uint32_t prefix = state[0];
+  for (int i = threadIdx.x; i < (int)kWideBins; i += kWideThreads) hist[i] = 0;
+  __syncthreads();
+  const uint32_t a = (uint32_t)(((uint64_t)w * blockIdx.x) / gridDim.x);
+  const uint32_t b = (uint32_t)(((uint64_t)w * (blockIdx.x + 1u)) / gridDim.x);
+  cta_for_keys<kWideThreads>(s.seg_key[g] + a, b - a, [&](uint32_t u) {
+    const uint32_t k = ord_key(__uint_as_float(u));
+    if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & (nb - 1u)], 1u);
+  });
+  __syncthreads();
+  for (int i = threadIdx.x; i < (int)kWideBins; i += kWideThreads)
+    if (hist[i]) atomicAdd(&H[i], hist[i]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&state[2], 1u) == gridDim.x - 1u;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const uint32_t rank = state[1];  // written before this launch
+  uint32_t loc[kPer], sum = 0;
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    const uint32_t i = threadIdx.x * kPer + q;
+    loc[q] = __ldcg(H + i);
+    H[i] = 0u;
+    sum += loc[q];
+  }
+  uint32_t all;
+  uint32_t acc = block_excl_scan(sum, tmp, &all);
+  if (rank >= acc && rank < acc + sum) {  // one thread
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      if (rank < acc + loc[q]) {
+        const uint32_t key = prefix | ((threadIdx.x * kPer + q) << shift);
+        state[0] = key;
+        state[1] = rank - acc;
+        if (shift == 0) s.seg_med[g] = key;
+        break;
+      }
+      acc += loc[q];
+    }
+  }
+  if (threadIdx.x == 0) state[2] = 0u;
 }
 
 // One CTA per cell: count-weighted lower median of the segment medians: the
@@ -1594,6 +1696,12 @@ bool step_selects_all(uint32_t nseg, uint64_t points, uint32_t sms) {
   return nseg <= 8u * sms && points <= 8192ull * nseg;
 }
 
+// Few, large segments: several CTAs each. One CTA takes about 0.25 ns a key,
+// the four launches 40 us and 4 ps a key of the step (64 segments of 262,144
+// keys: 66 us with a CTA each, 108 here), so the line lies where 262,144 keys
+// of each of 32 segments cost the same.
+bool step_selects_wide(uint32_t nseg, uint64_t points) { return nseg <= 32u && points >= 262144ull * nseg; }
+
 // One CTA per cell combines, counts, scans and classifies: while the cells'
 // CTAs fit the SMs at once (4 each) and a cell has at most 64 tiles on average
 // (a warp reads 4).
@@ -1602,8 +1710,9 @@ static bool step_splits(const StepDev& s, uint32_t sms2) {
 }
 
 // The selects by segment size: one thread, one warp, one CTA per segment.
-static void launch_listed_selects(const TreeDev* trees, const StepDev& s, uint32_t nseg, uint32_t max_bigseg,
-                                  const SelectTuning& tune, uint64_t points, uint32_t sms, cudaStream_t st) {
+static void launch_listed_selects(const TreeDev* trees, const StepDev& s, uint32_t nseg, uint32_t max_r,
+                                  uint32_t max_bigseg, const SelectTuning& tune, uint64_t points, uint32_t sms,
+                                  cudaStream_t st) {
   {
     TraceScope ts(K_SELECT_TINY, st, points);
     k_select_tiny<<<std::max<uint32_t>(1, std::min<uint32_t>((nseg + 255) / 256, sms * 16u)), 256, 0, st>>>(trees, s);
@@ -1613,6 +1722,17 @@ static void launch_listed_selects(const TreeDev* trees, const StepDev& s, uint32
     k_select_small<<<std::max<uint32_t>(1, std::min<uint32_t>((nseg + 7) / 8, sms * 8u)), 256, 0, st>>>(trees, s);
   }
   if (max_bigseg == 0) return;
+  if (s.wide_segs) {
+    // CTAs per segment: four per SM in all, of at least 8192 keys each
+    const uint32_t x = std::max<uint32_t>(
+        1, (uint32_t)std::min<uint64_t>(2u * sms / std::max(1u, nseg), points / std::max(1u, nseg) / 8192u));
+    const uint32_t y = std::min(max_r, nseg - std::min(nseg, s.ncells) + 1u);  // every cell has a segment
+    { TraceScope ts(K_SELECT_WIDE, st); k_wide_clear<<<dim3(1, y, s.ncells), kWideThreads, 0, st>>>(trees, s); }
+    for (int top = 32; top > 0; top -= 11) {
+      TraceScope ts(K_SELECT_WIDE, st, points);
+      k_wide_pass<<<dim3(x, y, s.ncells), kWideThreads, 0, st>>>(trees, s, top);
+    }
+  }
   TraceScope ts(K_SELECT_BIG, st);
   // nseg bounds the big segments too; with few of them (the first levels
   // of a large tree) a CTA's loads in flight set the rate, so they take
@@ -1740,7 +1860,7 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
       TraceScope ts(K_SELECT_ALL, st, points);
       k_select_all<<<std::max<uint32_t>(1, nseg), 256, 0, st>>>(trees, s);
     } else {
-      launch_listed_selects(trees, s, nseg, max_bigseg, tune, points, sms, st);
+      launch_listed_selects(trees, s, nseg, (uint32_t)max_r, max_bigseg, tune, points, sms, st);
     }
     if (s.shards) launch_shard_medians(trees, s, nc, st);  // the all-gather of the segment statistics
     if (!split) {

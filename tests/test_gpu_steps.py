@@ -71,3 +71,43 @@ def test_step_forms_in_one_batch():
     assert status == [0] * len(CASES)
     for t, x, c in zip(trees, xs, CASES):
         _same(t, oracle.build_tree(x, **c[3]), str(c))
+
+
+WIDE = [
+    (300_007, 3, "uniform", dict(r=1, leaf_size=40, max_levels=20)),
+    (800_007, 2, "student", dict(r=3, depth=8)),
+    (1_048_576, 3, "student", dict(r=4, depth=7)),          # 262,144 keys a segment
+    (1_048_575, 3, "student", dict(r=4, depth=7)),          # just below
+    (600_001, 1, "ties", dict(r=2, depth=5)),
+    (900_001, 5, "student", dict(r=3, depth=6, key_rule=1)),
+    (2_900, 2, "uniform", dict(r=2, depth=3)),              # beside large trees: no room for a histogram per segment
+]
+
+
+@pytest.mark.parametrize("case", range(len(WIDE)))
+def test_several_ctas_per_segment(case):
+    from paper_2201_08288_gb300 import kdt
+    n, d, kind, kw = WIDE[case]
+    x = _points(n, d, kind, 50 + case)
+    _same(kdt.kdt_build(torch.from_numpy(x).cuda(), **kw), oracle.build_tree(x, **kw), str(WIDE[case]))
+
+
+def test_several_ctas_per_segment_in_one_batch():
+    from paper_2201_08288_gb300 import kdt
+    xs = [_points(n, d, kind, 50 + i) for i, (n, d, kind, _) in enumerate(WIDE)]
+    trees, status = kdt.kdt_build_batched([dict(points=torch.from_numpy(x).cuda(), **c[3]) for x, c in zip(xs, WIDE)])
+    assert status == [0] * len(WIDE)
+    for t, x, c in zip(trees, xs, WIDE):
+        _same(t, oracle.build_tree(x, **c[3]), str(c))
+
+
+def test_several_ctas_for_unequal_subsets():
+    """Explicit ids, one subset nearly empty: its segment takes the path by size."""
+    from paper_2201_08288_gb300 import kdt
+    n = 1_100_007
+    x = _points(n, 3, "student", 90)
+    sid = (np.random.default_rng(1).random(n) < 0.5).astype(np.uint8)
+    sid[::3001] = 2
+    kw = dict(r=4, subset_mode=2, depth=8)  # subset 3 is empty
+    g = kdt.kdt_build(torch.from_numpy(x).cuda(), sid=torch.from_numpy(sid).cuda(), **kw)
+    _same(g, oracle.build_tree(x, sid=sid, **kw), "unequal")
