@@ -507,7 +507,9 @@ kdt_status Engine::finalize(const std::vector<uint32_t>& slots, std::vector<kdt_
   SlotChunks sc{nullptr, (uint32_t)slots.size(), 0};
   std::vector<uint32_t> list;
   if (slots.size() == 1 && slots[0] == 0) {
-    sc.chunks = std::max<uint32_t>(1, std::min<uint32_t>((recs_[0] + 7) / 8, 8192));
+    // a warp per record, or a CTA where the leaves are larger than a warp sorts
+    const uint32_t per = host_[0].n > (uint64_t)kLeafWarpMax * recs_[0] ? 1u : 8u;
+    sc.chunks = std::max<uint32_t>(1, std::min<uint32_t>((recs_[0] + per - 1) / per, 8192));
   } else {
     list = slots;
     for (uint32_t s : slots) {
