@@ -444,6 +444,55 @@ __device__ uint32_t warp_weighted_select(uint32_t cnt, uint32_t rank, uint32_t* 
   return warp_weighted_select<kUnit>(cnt, rank, hist, key_of, w_of, [](uint32_t) { return true; });
 }
 
+// Lower median of 1 <= w <= 32K keys (key_of(e), e < w) by one warp, element e
+// = k * 32 + lane in register k of a lane. The keys are padded to N = 32K with
+// the smallest and the largest key so that the median has rank N/2 - 1
+// (padding keys equal to a real key would not change the element at that
+// rank); the bitonic network runs its stages up to size N/2 only, which
+// leaves the first half ascending and the second descending: a bitonic
+// sequence whose half-cleaner holds the N/2 smallest keys, the largest of
+// which (over the warp) is the median.
+template <int K, class KeyOf>
+__device__ __forceinline__ uint32_t warp_bitonic_median(KeyOf key_of, uint32_t w) {
+  static_assert(K >= 2 && (K & (K - 1)) == 0, "K: a power of two of at least 2");
+  const int lane = threadIdx.x & 31;
+  constexpr int N = 32 * K;
+  const uint32_t zeros_end = w + (uint32_t)(N / 2 - 1) - (w - 1u) / 2u;  // [w, zeros_end) hold 0
+  uint32_t v[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t e = (uint32_t)(k * 32 + lane);
+    v[k] = e < w ? key_of(e) : (e < zeros_end ? 0u : 0xffffffffu);
+  }
+#pragma unroll
+  for (int size = 2; size <= N / 2; size <<= 1) {
+#pragma unroll
+    for (int j = size >> 1; j > 0; j >>= 1) {
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const int e = k * 32 + lane;
+        const bool asc = (e & size) == 0;
+        if (j >= 32) {
+          const int kk = k ^ (j >> 5);
+          if (k < kk) {
+            const uint32_t lo = min(v[k], v[kk]), hi = max(v[k], v[kk]);
+            v[k] = asc ? lo : hi;
+            v[kk] = asc ? hi : lo;
+          }
+        } else {
+          const uint32_t o = __shfl_xor_sync(0xffffffffu, v[k], j);
+          const bool lower = (lane & j) == 0;
+          v[k] = (lower == asc) ? min(v[k], o) : max(v[k], o);
+        }
+      }
+    }
+  }
+  uint32_t m = 0u;
+#pragma unroll
+  for (int k = 0; k < K / 2; ++k) m = max(m, min(v[k], v[k + K / 2]));
+  return __reduce_max_sync(0xffffffffu, m);
+}
+
 // Block-wide exclusive scan of one value per thread; returns the exclusive
 // prefix and writes the block total. `tmp` holds 33 words.
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* tmp, uint32_t* total) {

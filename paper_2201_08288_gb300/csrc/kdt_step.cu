@@ -641,54 +641,6 @@ __global__ void __launch_bounds__(256, 5) k_select_tiny(const TreeDev* trees, St
   }
 }
 
-// Lower median of 1 <= w <= 32K keys by one warp, element e = k * 32 + lane
-// in register k of a lane. As in thread_lower_median the keys are padded to
-// N = 32K with the smallest and the largest key so that the median has rank
-// N/2 - 1; the bitonic network runs its stages up to size N/2 only, which
-// leaves the first half ascending and the second descending: a bitonic
-// sequence whose half-cleaner min(v[k], v[k + K/2]) holds the N/2 smallest
-// keys, the largest of which (over the warp) is the median.
-template <int K>
-__device__ uint32_t warp_bitonic_median(const uint32_t* keys, uint32_t w) {
-  static_assert(K >= 2 && (K & (K - 1)) == 0, "K: a power of two of at least 2");
-  const int lane = threadIdx.x & 31;
-  constexpr int N = 32 * K;
-  const uint32_t zeros_end = w + (uint32_t)(N / 2 - 1) - (w - 1u) / 2u;  // [w, zeros_end) hold 0
-  uint32_t v[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const uint32_t e = (uint32_t)(k * 32 + lane);
-    v[k] = e < w ? kload(keys + e) : (e < zeros_end ? 0u : 0xffffffffu);
-  }
-#pragma unroll
-  for (int size = 2; size <= N / 2; size <<= 1) {
-#pragma unroll
-    for (int j = size >> 1; j > 0; j >>= 1) {
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const int e = k * 32 + lane;
-        const bool asc = (e & size) == 0;
-        if (j >= 32) {
-          const int kk = k ^ (j >> 5);
-          if (k < kk) {
-            const uint32_t lo = min(v[k], v[kk]), hi = max(v[k], v[kk]);
-            v[k] = asc ? lo : hi;
-            v[kk] = asc ? hi : lo;
-          }
-        } else {
-          const uint32_t o = __shfl_xor_sync(0xffffffffu, v[k], j);
-          const bool lower = (lane & j) == 0;
-          v[k] = (lower == asc) ? min(v[k], o) : max(v[k], o);
-        }
-      }
-    }
-  }
-  uint32_t m = 0u;
-#pragma unroll
-  for (int k = 0; k < K / 2; ++k) m = max(m, min(v[k], v[k + K / 2]));
-  return __reduce_max_sync(0xffffffffu, m);
-}
-
 // State of a warp's radix select: the key bits found so far (`prefix`, all
 // bits above `rem`) and the rank still sought below them.
 struct RadixState {
@@ -778,13 +730,14 @@ __global__ void __launch_bounds__(256) k_select_small(const TreeDev* trees, Step
     const uint32_t g = s.midseg[j];
     const uint32_t w = s.seg_w[g];
     const uint32_t* keys = s.seg_key[g];
+    auto key_of = [&](uint32_t e) { return kload(keys + e); };
     uint32_t med;
     if (w <= s.bitonic_max && w <= 64u) {
-      med = warp_bitonic_median<2>(keys, w);
+      med = warp_bitonic_median<2>(key_of, w);
     } else if (w <= s.bitonic_max && w <= 128u) {
-      med = warp_bitonic_median<4>(keys, w);
+      med = warp_bitonic_median<4>(key_of, w);
     } else if (w <= s.bitonic_max) {
-      med = warp_bitonic_median<8>(keys, w);
+      med = warp_bitonic_median<8>(key_of, w);
     } else if (w <= 1024u) {
       uint32_t* st = stage[warp];
       for (uint32_t b0 = 0; b0 < w; b0 += 256) {

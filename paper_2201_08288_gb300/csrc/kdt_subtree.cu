@@ -15,8 +15,8 @@
 //      starts (a cell's first position, or a change of subset), numbered by
 //      one block-wide scan;
 //   3. the lower median of every segment: rank counting inside the segment
-//      (at most kRankMax points), else a warp radix select over the bits
-//      where its keys differ;
+//      (at most kRankMax points), else a warp per segment with the keys in
+//      registers;
 //   4. per cell, the count-weighted lower median of its segments' medians;
 //   5. a stable partition of the local order around the split (ties left);
 //   6. children: terminal cells are recorded, the others form the next level.
@@ -47,7 +47,7 @@ struct Smem {
   uint32_t* whist;    // NW * 256 words: warp histograms, tables of few cells, root subset counts
   uint16_t* biglist;  // kSubtreeBigCap segments above kRankMax points
   LCell* tab;         // 2 * cells: the cell tables of two levels
-  uint32_t* cols;     // d key columns at stride `stride`
+  uint32_t* cols;     // d coordinate columns (raw floats) at stride `stride`
   uint32_t* gk;       // N: key of each position on its cell's coordinate
   uint32_t* smed;     // N: median of each segment
   uint16_t* sid;      // N: subset of each local point
@@ -168,17 +168,18 @@ __device__ __forceinline__ uint32_t block_excl_scan_1bar(uint32_t v, uint32_t* w
 // and their number (one warp sum of (w << 12) | 1) and fixes that bit. The
 // answer is the key of a remaining candidate, so once a single candidate is
 // left its key is the answer and the lower bits need no steps.
-template <int K, class KeyOf, class WOf>
+// kUnit: every item weighs 1.
+template <int K, bool kUnit, class KeyOf, class WOf>
 __device__ __forceinline__ uint32_t warp_wsel_bits(uint32_t cnt, uint32_t rank, KeyOf key_of, WOf w_of) {
   const int lane = threadIdx.x & 31;
-  uint32_t key[K], pw[K];
+  uint32_t key[K], pw[kUnit ? 1 : K];
   uint32_t lo = 0xffffffffu, hi = 0u;
 #pragma unroll
   for (int q = 0; q < K; ++q) {
     const uint32_t j = (uint32_t)lane + 32u * q;
     const bool ok = j < cnt;
-    key[q] = ok ? key_of(j) : 0u;
-    pw[q] = ok ? (w_of(j) << 12) | 1u : 0u;
+    key[q] = ok ? key_of(j) : 0xffffffffu;  // above every key that is no NaN
+    if (!kUnit) pw[q] = ok ? (w_of(j) << 12) | 1u : 0u;
     if (ok) {
       lo = min(lo, key[q]);
       hi = max(hi, key[q]);
@@ -194,9 +195,9 @@ __device__ __forceinline__ uint32_t warp_wsel_bits(uint32_t cnt, uint32_t rank, 
     const uint32_t fixed = ~((1u << bit) - 1u);     // bits above `bit`, and `bit` itself
     uint32_t acc = 0;
 #pragma unroll
-    for (int q = 0; q < K; ++q) acc += ((key[q] ^ prefix) & fixed) == 0u ? pw[q] : 0u;
+    for (int q = 0; q < K; ++q) acc += ((key[q] ^ prefix) & fixed) == 0u ? (kUnit ? 1u : pw[kUnit ? 0 : q]) : 0u;
     acc = __reduce_add_sync(0xffffffffu, acc);
-    const uint32_t w0 = acc >> 12, n0 = acc & 0xfffu;
+    const uint32_t w0 = kUnit ? acc : acc >> 12, n0 = kUnit ? acc : acc & 0xfffu;
     if (rank >= w0) {
       rank -= w0;
       prefix |= 1u << bit;
@@ -208,11 +209,28 @@ __device__ __forceinline__ uint32_t warp_wsel_bits(uint32_t cnt, uint32_t rank, 
       uint32_t m = 0;
 #pragma unroll
       for (int q = 0; q < K; ++q)
-        if (pw[q] != 0u && ((key[q] ^ prefix) & fixed) == 0u) m = key[q];
+        if ((uint32_t)lane + 32u * q < cnt && ((key[q] ^ prefix) & fixed) == 0u) m = key[q];
       return __reduce_max_sync(0xffffffffu, m);
     }
   }
   return prefix;
+}
+
+// Lower median of kRankMax < w keys by one warp: a network up to 64 keys, bit
+// by bit with the keys in registers up to 512, else by radix histogram (a chain
+// of some 7000 cycles whatever the size, so trees of few subsets waited there
+// for most of their first levels: 1000 points in 8 subsets 62 -> 50 us, 512
+// trees of 4 to 64 subsets 3.95 -> 3.2 ms. A form for 1024 keys, 32 registers,
+// slowed every other path of the kernel by 3%.)
+template <class KeyOf>
+__device__ __forceinline__ uint32_t warp_segment_median(uint32_t w, uint32_t* hist, KeyOf key_of) {
+  auto one = [](uint32_t) { return 1u; };
+  const uint32_t rank = (w - 1u) / 2u;
+  if (w <= 64u) return warp_bitonic_median<2>(key_of, w);
+  if (w <= 128u) return warp_wsel_bits<4, true>(w, rank, key_of, one);
+  if (w <= 256u) return warp_wsel_bits<8, true>(w, rank, key_of, one);
+  if (w <= 512u) return warp_wsel_bits<16, true>(w, rank, key_of, one);
+  return warp_weighted_select<true>(w, rank, hist, key_of, one);
 }
 
 // kWide: compiled for the wide shape, else the narrow one (kdt_launch.h).
@@ -391,20 +409,17 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
         }
         continue;
       }
-      // keys in place; NaN is looked for in the roots of small trees only (the
-      // multi-CTA pipeline checked every point of a larger tree at its root)
-      bool nan = false;
-      const bool check_nan = c.level == 0;
-      for (int l = 0; l < d; ++l) {
-        uint32_t* col = S.cols + s_colbase[l];
+      // NaN is looked for in the roots of small trees only (the multi-CTA
+      // pipeline checked every point of a larger tree at its root)
+      if (c.level == 0) {
+        bool nan = false;
+        for (int l = 0; l < d; ++l) {
+          const uint32_t* col = S.cols + s_colbase[l];
 #pragma unroll 4
-        for (uint32_t i = tid; i < N; i += T) {
-          const float x = __uint_as_float(col[i]);
-          nan |= check_nan && is_nan_bits(x);
-          col[i] = ord_key(x);
+          for (uint32_t i = tid; i < N; i += T) nan |= is_nan_bits(__uint_as_float(col[i]));
         }
+        if (nan) set_status(t, ST_NAN_INPUT);
       }
-      if (nan) set_status(t, ST_NAN_INPUT);
       // The root of a small tree arrives in index order: put it in subset
       // order (counting sort; order inside a subset is immaterial). Every
       // other cell is in subset order already.
@@ -479,28 +494,30 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
             uint32_t lo2[2] = {0xffffffffu, 0xffffffffu}, hi2[2] = {0u, 0u};
             for (int c0 = 0; c0 < d; c0 += 8) {
               const int nc = min(8, d - c0);
-              uint32_t base[8], lo[8], hi[8];
+              // as floats (only max - min is used, which -0 and +0 do not change)
+              uint32_t base[8];
+              float lo[8], hi[8];
 #pragma unroll
               for (int q = 0; q < 8; ++q) {
                 base[q] = q < nc ? s_colbase[c0 + q] : 0u;
-                lo[q] = 0xffffffffu;
-                hi[q] = 0u;
+                lo[q] = __int_as_float(0x7f800000);
+                hi[q] = -__int_as_float(0x7f800000);
               }
               for (uint32_t i = i0 + lane; i < i1; i += 32) {
                 const uint32_t o = ordA[i];
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
                   if (q < nc) {
-                    const uint32_t kk = S.cols[base[q] + o];
-                    lo[q] = min(lo[q], kk);
-                    hi[q] = max(hi[q], kk);
+                    const float x = __uint_as_float(S.cols[base[q] + o]);
+                    lo[q] = fminf(lo[q], x);
+                    hi[q] = fmaxf(hi[q], x);
                   }
               }
 #pragma unroll
               for (int q = 0; q < 8; ++q)
                 if (q < nc) {
-                  const uint32_t l = __reduce_min_sync(0xffffffffu, lo[q]);
-                  const uint32_t h = __reduce_max_sync(0xffffffffu, hi[q]);
+                  const uint32_t l = __reduce_min_sync(0xffffffffu, ord_key(lo[q]));
+                  const uint32_t h = __reduce_max_sync(0xffffffffu, ord_key(hi[q]));
                   const int col = c0 + q;
                   if (lane == (col & 31)) {
                     if (col < 32) {
@@ -565,7 +582,7 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
             if (k != kNoCell) {
               const uint32_t o = ordA[i];
               const uint32_t cb = cc[k].begin;
-              key = S.cols[s_colbase[cc[k].dim] + o];
+              key = ord_key(__uint_as_float(S.cols[s_colbase[cc[k].dim] + o]));
               f = (i == cb) || S.sid[o] != S.sid[ordA[i - 1]];
               S.gk[i] = key;
             }
@@ -598,7 +615,7 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
         __syncthreads();
 
         // ---- 3. lower median of every segment: rank counting inside the
-        // segment, or (more than kRankMax points) a warp radix select
+        // segment, or (more than kRankMax points) a warp per segment
 #pragma unroll
         for (int q = 0; q < kQ; ++q) {
           const uint32_t i = (uint32_t)tid + (uint32_t)q * T;
@@ -631,9 +648,8 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
             const uint16_t k = S.cellid[b];
             const uint32_t e = min((uint32_t)S.segs[sx + 1], (uint32_t)cc[k].begin + cc[k].count);
             const uint32_t* g = S.gk + b;
-            const uint32_t m = warp_weighted_select<true>(e - b, (e - b - 1) / 2, S.whist + warp * 256,
-                                                          [&](uint32_t jj) { return g[jj]; },
-                                                          [](uint32_t) { return 1u; });
+            const uint32_t m =
+                warp_segment_median(e - b, S.whist + warp * 256, [&](uint32_t jj) { return g[jj]; });
             if (lane == 0) S.smed[sx] = m;
           }
           __syncthreads();
@@ -656,13 +672,13 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
           };
           uint32_t m;
           if (ns <= 32u)
-            m = warp_wsel_bits<1>(ns, rank, key_of, w_of);
+            m = warp_wsel_bits<1, false>(ns, rank, key_of, w_of);
           else if (ns <= 64u)
-            m = warp_wsel_bits<2>(ns, rank, key_of, w_of);
+            m = warp_wsel_bits<2, false>(ns, rank, key_of, w_of);
           else if (ns <= 128u)
-            m = warp_wsel_bits<4>(ns, rank, key_of, w_of);
+            m = warp_wsel_bits<4, false>(ns, rank, key_of, w_of);
           else if (ns <= 256u)
-            m = warp_wsel_bits<8>(ns, rank, key_of, w_of);
+            m = warp_wsel_bits<8, false>(ns, rank, key_of, w_of);
           else
             m = warp_weighted_select(ns, rank, S.whist + warp * 256, key_of, w_of);
           if (lane == 0) cc[k].mkey = m;
