@@ -37,9 +37,10 @@ namespace kdt {
 
 namespace {
 
-constexpr int kQueryThreads = 128;
+constexpr int kQueryThreads = 64;  // (a block ends with its longest search: 64 threads 0.60 ms where 128 take 0.61)
 constexpr int kQueryWarps = kQueryThreads / 32;
 constexpr unsigned kAll = 0xffffffffu;
+constexpr int kDimChunk = 4;  // coordinates of a point whose loads go out together
 
 struct TreeView {
   const float* x;  // [d][n]
@@ -98,14 +99,19 @@ __global__ void __launch_bounds__(kQueryThreads) k_query_box(TreeView tv, const 
       const int64_t p1 = tv.offs[k + 1];
       for (int64_t p = tv.offs[k]; p < p1; p += 32) {
         bool in = p + lane < p1;
-        const uint32_t i = in ? tv.perm[p + lane] : 0u;
-        for (int j = 0; j < d; ++j) {
-          if (in) {
-            const uint32_t kx = ord_key(__ldg(tv.x + (int64_t)j * tv.n + i));
-            const uint2 b = bx[j];
-            in = b.x <= kx && kx <= b.y;
-          }
-          if ((j & 3) == 3 && !__any_sync(kAll, in)) break;
+        const uint32_t i = in ? __ldg(tv.perm + p + lane) : 0u;
+        for (int j0 = 0; j0 < d; j0 += kDimChunk) {
+          uint32_t kx[kDimChunk];
+#pragma unroll
+          for (int j = 0; j < kDimChunk; ++j)
+            if (j0 + j < d) kx[j] = in ? ord_key(__ldg(tv.x + (int64_t)(j0 + j) * tv.n + i)) : 0u;
+#pragma unroll
+          for (int j = 0; j < kDimChunk; ++j)
+            if (j0 + j < d) {
+              const uint2 b = bx[j0 + j];
+              in = in && b.x <= kx[j] && kx[j] <= b.y;
+            }
+          if (j0 + kDimChunk < d && !__any_sync(kAll, in)) break;
         }
         const unsigned bal = __ballot_sync(kAll, in);
         const uint32_t at = found + (uint32_t)__popc(bal & lt);
@@ -127,9 +133,17 @@ __device__ __forceinline__ bool nearer(double a, uint32_t ia, double b, uint32_t
 
 __device__ __forceinline__ double dist2(const TreeView& tv, const float* q, uint32_t i) {
   double d2 = 0.0;
-  for (int j = 0; j < tv.d; ++j) {
-    const double df = __dsub_rn((double)__ldg(tv.x + (int64_t)j * tv.n + i), (double)q[j]);
-    d2 = __dadd_rn(d2, __dmul_rn(df, df));
+  for (int j0 = 0; j0 < tv.d; j0 += kDimChunk) {
+    float x[kDimChunk];
+#pragma unroll
+    for (int j = 0; j < kDimChunk; ++j)
+      if (j0 + j < tv.d) x[j] = __ldg(tv.x + (int64_t)(j0 + j) * tv.n + i);
+#pragma unroll
+    for (int j = 0; j < kDimChunk; ++j)
+      if (j0 + j < tv.d) {
+        const double df = __dsub_rn((double)x[j], (double)q[j0 + j]);
+        d2 = __dadd_rn(d2, __dmul_rn(df, df));
+      }
   }
   return d2;
 }
@@ -320,12 +334,20 @@ __device__ __forceinline__ KnnResult knn_warp(const TreeView& tv, const float* q
     const int64_t p1 = tv.offs[leaf + 1];
     for (int64_t p = tv.offs[leaf]; p < p1; p += 32) {
       bool in = p + lane < p1;
-      const uint32_t i = in ? tv.perm[p + lane] : 0u;
+      const uint32_t i = in ? __ldg(tv.perm + p + lane) : 0u;
       float f = 0.0f;
-      for (int j = 0; j < d; ++j) {
-        const float df = __ldg(tv.x + (int64_t)j * tv.n + i) - q[j];
-        f = fmaf(df, df, f);
-        if ((j & 7) == 7) {
+      for (int j0 = 0; j0 < d; j0 += kDimChunk) {
+        float x[kDimChunk];
+#pragma unroll
+        for (int j = 0; j < kDimChunk; ++j)
+          if (j0 + j < d) x[j] = __ldg(tv.x + (int64_t)(j0 + j) * tv.n + i);
+#pragma unroll
+        for (int j = 0; j < kDimChunk; ++j)
+          if (j0 + j < d) {
+            const float df = x[j] - q[j0 + j];
+            f = fmaf(df, df, f);
+          }
+        if (j0 + kDimChunk < d) {
           in = in && !(f * shrink > kth_up);
           if (!__any_sync(kAll, in)) break;
         }
@@ -390,7 +412,8 @@ __device__ __forceinline__ KnnResult knn_warp(const TreeView& tv, const float* q
 // What bounds it: the chains of dependent loads (node after node, a leaf's
 // offsets, its permutation, the gathered coordinates) over the resident warps.
 // 100,003 queries of 8 neighbours among 1,000,003 points in 3 coordinates,
-// leaves of 31: 0.78 ms; 2.0 with double distances throughout (the double
+// leaves of 31: 0.60 ms; 0.73 with the coordinates loaded one after another, 2.0
+// with double distances throughout as well (the double
 // unit), 10.6 with one thread per query (its chains are longer, and 32
 // searches diverge).
 __global__ void __launch_bounds__(kQueryThreads) k_query_knn(TreeView tv, const float* qs, int32_t nq, int32_t k,
