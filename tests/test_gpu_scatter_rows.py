@@ -53,3 +53,12 @@ def test_explicit_ids(n, d, r, skew, rule):
 def test_ids_from_the_index(n, r, mode):
     pts = workloads.gaussian_mixture(n, 3, 16, 0.05, seed=r)
     _check(pts, None, None, r=r, subset_mode=mode, leaf_size=24, max_levels=22)
+
+
+@pytest.mark.parametrize("rule", [0, 1])
+@pytest.mark.parametrize("d", [1, 4, 6, 7, 9, 12, 13])
+def test_coordinate_counts(d, rule):
+    n = 30_000 + 77 * d
+    pts = workloads.student_t_snapped(n, d, 3.0, 0.1, 256, seed=d)
+    sid = np.random.default_rng(d).integers(0, 40, n).astype(np.uint8)
+    _check(pts, torch.from_numpy(sid).cuda(), sid, r=40, subset_mode=2, leaf_size=16, max_levels=20, key_rule=rule)
