@@ -121,8 +121,9 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
                      uint32_t max_bigseg, bool has_roots, bool need_root_dims, bool any_widest, int max_r, int uniform_d,
                      const SelectTuning& tune, uint64_t points, uint32_t sms, cudaStream_t st, bool fourier = false);
 
-// Most dynamic shared memory of the staged scatter (two CTAs per SM).
-constexpr uint32_t kScatterSmemBytes = 100 * 1024;
+// Most dynamic shared memory of the staged scatter: three CTAs per SM with
+// their static part and the kilobyte that each one reserves.
+constexpr uint32_t kScatterSmemBytes = 74240;
 cudaError_t prepare_scatter_kernel(int uniform_d, bool any_widest);
 // uniform_d: the coordinate count of every tree of the step, 0 if they differ
 // (a kernel compiled for that d is used where there is one)

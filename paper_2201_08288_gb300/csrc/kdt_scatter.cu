@@ -68,9 +68,11 @@ __host__ __device__ constexpr uint32_t sub_tile(int d) {
 // 1.37 with four (0.18 per level at 6.8 TB/s would be 1.1). At d = 8 without
 // min / max two buffers of nine columns fit three times; with them the
 // accumulators take 94 registers, and three CTAs spill (28.0 against 26.8 ms
-// per build of 2^27 points).
+// per build of 2^27 points). The instance for any d (forests of mixed d) takes
+// 72 registers, so three CTAs too: a forest of 512 trees spent 2.38 ms in it
+// with two CTAs of 100 KB each, 1.81 with three of 72.5.
 constexpr int scatter_ctas(int kD, bool kMM) {
-  if (kD == 0 || ((kD == 7 || kD == 8) && kMM)) return 2;
+  if ((kD == 7 || kD == 8) && kMM) return 2;
   return kD >= 2 && kD <= 5 && !kMM ? 4 : 3;
 }
 
