@@ -31,7 +31,7 @@ struct PlainPlan {
 
 PlainPlan plan_plain(const kdt_params& p) {
   PlainPlan pp;
-  pp.tree = plan_tree(p);
+  pp.tree = plan_tree(p, false, /*alone=*/true);
   StepNeeds needs;
   needs.add(p, pp.tree);
   pp.step = plan_step(needs);

@@ -41,6 +41,12 @@ int device_sms() {
   return sms;
 }
 
+// The SMs that plans are made for.
+int plan_sms() {
+  const int sms = device_sms();
+  return sms > 0 ? sms : 148;
+}
+
 kdt_status map_status(int32_t st) {
   switch (st) {
     case ST_OK: return KDT_OK;
@@ -100,7 +106,7 @@ kdt_params effective_params(const kdt_params& p) {
   return e;
 }
 
-TreePlan plan_tree(const kdt_params& p0, bool no_subtree) {
+TreePlan plan_tree(const kdt_params& p0, bool no_subtree, bool alone) {
   const kdt_params p = effective_params(p0);
   TreePlan t;
   const uint64_t n = (uint64_t)p.n;
@@ -111,6 +117,20 @@ TreePlan plan_tree(const kdt_params& p0, bool no_subtree) {
   const bool fourier = p.fourier_j > 0;
   t.small_max = (fourier || no_subtree) ? 0 : subtree_capacity(p.d);
   t.sub_wide = &subtree_shape(p.d) == &kSubWide;
+  if (t.small_max > 0 && alone && n > (uint64_t)t.small_max) {
+    // the tall shape while its cells, of half its capacity to all of it, are no
+    // more than the SMs (a single cell that the other shapes hold finishes sooner
+    // there: 1000 points 50 us, 61 in the tall shape)
+    const int tall = subtree_capacity(p.d, kSubTall);
+    const uint64_t sms = (uint64_t)plan_sms();
+    uint64_t cells = 1;
+    while (cells <= sms && cells * (uint64_t)tall < n) cells *= 2;
+    if (cells <= sms && tall > t.small_max) {
+      t.small_max = tall;
+      t.sub_wide = false;
+      t.sub_tall = (int)std::min<uint64_t>(sms, cells + cells / 4 + 1);
+    }
+  }
   t.sid_bytes = p.subset_mode == KDT_SUBSET_EXPLICIT ? (p.subset_id16 ? 2 : 1) : 0;
   const bool root_terminal = p.depth > 0 ? (n == 0) : (n <= (uint64_t)p.leaf_size);
   t.leafsort = !root_terminal && p.subset_mode != KDT_SUBSET_CONTIGUOUS && !fourier;
@@ -152,6 +172,7 @@ void StepNeeds::add(const kdt_params& p0, const TreePlan& tp) {
   if (tp.small_max > 0) small_off += tp.n * (uint64_t)tp.sid_bytes / 2;
   max_trees += 1;
   slice_cells = std::max<uint32_t>(slice_cells, (uint32_t)tp.small_max);
+  sub_tall = tp.sub_tall;
   widest = widest || p.key_rule == KDT_KEY_WIDEST_SPREAD;
   max_d = std::max(max_d, (int)p.d);
   max_r = std::max(max_r, (int)p.r);
@@ -169,10 +190,10 @@ StepPlan plan_step(const StepNeeds& needs) {
   s.off_cap = (uint32_t)std::min<uint64_t>(needs.nseg + needs.maxB, clamp);
   s.small_off_cap = (uint32_t)std::min<uint64_t>(needs.small_off, clamp);
   s.bigseg_cap = (uint32_t)std::min<uint64_t>(needs.points / (kSelWarpMin + 1) + 1, clamp);
-  const int sms = device_sms();
-  s.sms = (uint32_t)(sms > 0 ? sms : 148);
+  s.sms = (uint32_t)plan_sms();
   s.grid_step = s.sms * 2u;
-  const uint32_t grid_sub_max = s.sms * (uint32_t)std::max(kSubNarrow.ctas, kSubWide.ctas);
+  const uint32_t grid_sub_max =
+      needs.sub_tall ? (uint32_t)needs.sub_tall : s.sms * (uint32_t)std::max(kSubNarrow.ctas, kSubWide.ctas);
   const uint32_t mt = std::max<uint32_t>(needs.max_trees, 1);
   size_t off = 0;
   auto take = [&](size_t b) {
@@ -460,11 +481,13 @@ kdt_status Engine::tick() {
 
 void Engine::launch_small(bool from_device) {
   const uint32_t cap = plan_.cap_small;
-  const uint32_t gn = plan_.sms * (uint32_t)kSubNarrow.ctas, gw = plan_.sms * (uint32_t)kSubWide.ctas;
+  const SubtreeShape& front = plan_.needs.sub_tall ? kSubTall : kSubNarrow;
+  const uint32_t gn = plan_.needs.sub_tall ? (uint32_t)plan_.needs.sub_tall : plan_.sms * (uint32_t)front.ctas;
+  const uint32_t gw = plan_.sms * (uint32_t)kSubWide.ctas;
   if (from_device) {
     // counts on the device (a recorded tick): the narrow front, then the wide
     // back walked from the end
-    launch_subtree(kSubNarrow, trees_, small_, cap, words_ + W_SMALL, false, s_.small_off, words_ + W_HEAD, slices_,
+    launch_subtree(front, trees_, small_, cap, words_ + W_SMALL, false, s_.small_off, words_ + W_HEAD, slices_,
                    plan_.needs.slice_cells, gn, 0, st_);
     launch_subtree(kSubWide, trees_, small_, cap, words_ + W_SMALL + 1, true, s_.small_off, words_ + W_HEAD, slices_,
                    plan_.needs.slice_cells, gw, 0, st_);
@@ -472,7 +495,7 @@ void Engine::launch_small(bool from_device) {
   }
   const uint64_t pts = small_points_;
   if (small_count_ > 0)
-    launch_subtree(kSubNarrow, trees_, small_, small_count_, nullptr, false, s_.small_off, words_ + W_HEAD, slices_,
+    launch_subtree(front, trees_, small_, small_count_, nullptr, false, s_.small_off, words_ + W_HEAD, slices_,
                    plan_.needs.slice_cells, std::min(gn, small_count_), pts, st_);  // the points of both
   if (small_count_w_ > 0)
     launch_subtree(kSubWide, trees_, small_ + cap - small_count_w_, small_count_w_, nullptr, false,

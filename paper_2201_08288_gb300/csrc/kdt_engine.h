@@ -30,6 +30,7 @@ struct TreePlan {
   int small_max = 0;
   int sid_bytes = 0;
   bool sub_wide = false;   // small cells run in the subtree kernel's wide shape
+  int sub_tall = 0;        // > 0: in its tall shape, by at most this many CTAs
   bool presorted = false;  // root split by the pipeline, reordered by subset first
   bool leafsort = false;   // subsets not in index order: leaves are sorted at the end
   uint64_t n = 0;
@@ -42,14 +43,16 @@ struct TreePlan {
   size_t bytes = 0;
 };
 // no_subtree: every cell stays in the multi-CTA pipeline (a sharded build's
-// trees, whose splits are exchanged level by level).
-TreePlan plan_tree(const kdt_params& p, bool no_subtree = false);
+// trees, whose splits are exchanged level by level). alone: no other tree is
+// built with this one.
+TreePlan plan_tree(const kdt_params& p, bool no_subtree = false, bool alone = false);
 
 // Capacities of the shared tables, accumulated over the trees they must serve
 // at the same time.
 struct StepNeeds {
   uint64_t points = 0, maxB = 0, cap_small = 0, nseg = 0, small_off = 0;
   uint32_t max_trees = 0, slice_cells = 32;
+  int sub_tall = 0;  // the forest's one tree uses the subtree kernel's tall shape
   bool widest = false;
   bool fourier = false;  // a tree splits by the Fourier-moment estimator
   int max_d = 1, min_d = 1 << 30;  // min_d == max_d: every tree has the same d
@@ -60,7 +63,8 @@ struct StepNeeds {
 struct StepPlan {
   StepNeeds needs;
   // grid_step: the grid scale of the level step's kernels (two per SM);
-  // sms: the device's SMs (the subtree kernel's grid is sms x its shape's CTAs)
+  // sms: the device's SMs (the subtree kernel's grid is sms x its shape's CTAs,
+  // or sub_tall)
   uint32_t maxB = 0, cap_small = 0, max_tiles = 0, nseg_cap = 0, bigseg_cap = 0, grid_step = 0, sms = 0, off_cap = 0,
            small_off_cap = 0;
   size_t trees = 0, words = 0, slot_words = 0, slots_list = 0, admits = 0, big[2] = {0, 0}, small = 0, tiles = 0, tile_seg = 0, tile_left = 0, tile_loff = 0, tile_mm = 0, child_mm = 0, kdim = 0,

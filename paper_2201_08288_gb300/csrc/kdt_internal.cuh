@@ -32,8 +32,6 @@ constexpr int kTileThreads = 256;     // threads of the tile kernels
 constexpr int kSelTinyMax = 64;       // segments up to this size: one thread per segment
 constexpr int kSelSmallMax = 4096;    // largest warp-select segment (kdt_tuning warp_max)
 constexpr int kSelWarpMin = 1024;     // smallest warp_max: sizes the list of CTA-select segments
-constexpr int kSubtreeThreads = 256;  // threads of a CTA of the in-shared-memory subtree kernel
-constexpr int kSubtreeWarps = kSubtreeThreads / 32;
 
 // status codes (mirror include/kdt.h)
 enum : int32_t {

@@ -23,28 +23,38 @@ struct LCell {
 };
 static_assert(sizeof(LCell) == 16, "LCell is 16 bytes");
 
-// The subtree kernel comes in two shapes (kSubtreeThreads threads per CTA in
-// both); each tree uses one, by its coordinate count:
-//   narrow (d <= kSubtreeNarrowMaxD): at most 5 positions per thread (1280
+// The subtree kernel comes in three shapes:
+//   narrow (d <= kSubtreeNarrowMaxD): 256 threads of at most 5 positions (1280
 //     points), three CTAs per SM in 74 KB of dynamic shared memory each, cell
 //     tables of 128 cells;
-//   wide (larger d): at most 8 positions per thread (2048 points), two CTAs
-//     per SM in 112 KB each, cell tables of 256 cells.
-// Several CTAs share an SM, each finishing its own cell, so that one CTA's
-// barriers and copies overlap the others' work.
+//   wide (larger d): 256 threads of at most 8 positions (2048 points), two CTAs
+//     per SM in 112 KB each, cell tables of 256 cells;
+//   tall (trees built alone whose cells of that size are no more than the SMs):
+//     1024 threads of at most 5 positions (5120 points), one CTA per SM in 220
+//     KB, cell tables of 256 cells.
+// In the first two several CTAs share an SM, each finishing its own cell, so
+// that one CTA's barriers and copies overlap the others' work: that is best
+// while there are more cells than CTAs. With fewer, what a build waits for is
+// the levels above, a chain of launches each (about 35 us a level with its
+// wait), so the tall shape takes cells two levels larger. (65,536 points, d = 3:
+// 427 us in the narrow shape, 382 in the tall one; 300,007 points, d = 16: 829
+// in the wide shape, 675 in the tall one.)
 struct SubtreeShape {
+  int threads;
   int q;        // positions per thread
   int ctas;     // CTAs per SM
   size_t smem;  // dynamic shared memory per CTA
   int cells;    // cells of one level's table in shared memory
+  int bigs;     // segments above the rank-counting size (32): points / 33 at most
 };
-constexpr SubtreeShape kSubNarrow{5, 3, 74 * 1024, 128};
-constexpr SubtreeShape kSubWide{8, 2, 112 * 1024, 256};
+constexpr SubtreeShape kSubNarrow{256, 5, 3, 74 * 1024, 128, 64};
+constexpr SubtreeShape kSubWide{256, 8, 2, 112 * 1024, 256, 64};
+constexpr SubtreeShape kSubTall{1024, 5, 1, 220 * 1024, 256, 160};
 constexpr int kSubtreeNarrowMaxD = 8;
-constexpr int kSubtreeBigCap = 64;           // segments above the rank-counting size (32): N / 33 < 64
-constexpr int kSubtreeHistWords = kSubtreeWarps * 256;  // warp histograms; also the root's subset counts
-__host__ __device__ constexpr size_t subtree_fixed_bytes(int cells) {
-  return (size_t)kSubtreeHistWords * 4 + (size_t)kSubtreeBigCap * 2 + 2 * (size_t)cells * sizeof(LCell);
+constexpr int kSubtreeHists = 8;                       // warps that may use a radix histogram at a time
+constexpr int kSubtreeHistWords = kSubtreeHists * 256;  // their histograms; also the root's subset counts
+__host__ __device__ constexpr size_t subtree_fixed_bytes(const SubtreeShape& sh) {
+  return (size_t)kSubtreeHistWords * 4 + (size_t)sh.bigs * 2 + 2 * (size_t)sh.cells * sizeof(LCell);
 }
 inline const SubtreeShape& subtree_shape(int d) { return d <= kSubtreeNarrowMaxD ? kSubNarrow : kSubWide; }
 
@@ -62,20 +72,20 @@ __host__ __device__ inline size_t subtree_point_bytes(uint32_t N, int d) {
          6 * ((((size_t)N + 1) * 2 + 15) & ~(size_t)15);
 }
 
-// Largest cell (points) the subtree kernel holds for d coordinates in the
-// shape that trees of d coordinates use.
-inline int subtree_capacity(int d) {
+// Largest cell (points) that a shape of the subtree kernel holds for d
+// coordinates.
+inline int subtree_capacity(int d, const SubtreeShape& sh) {
   if (d < 1) return 0;
-  const SubtreeShape& sh = subtree_shape(d);
-  const size_t fixed = subtree_fixed_bytes(sh.cells);
+  const size_t fixed = subtree_fixed_bytes(sh);
   int lo = 32, hi = 8192;
   if (fixed + subtree_point_bytes(lo, d) > sh.smem) return 0;
   while (lo < hi) {
     const int mid = (lo + hi + 1) / 2;
     if (fixed + subtree_point_bytes(mid, d) <= sh.smem) lo = mid; else hi = mid - 1;
   }
-  return std::min(lo & ~31, sh.q * kSubtreeThreads);
+  return std::min(lo & ~31, sh.q * sh.threads);
 }
+inline int subtree_capacity(int d) { return subtree_capacity(d, subtree_shape(d)); }
 
 // Subset counts of a small root (put in subset order by the subtree kernel)
 // live in the warp histograms: trees with more subsets presort their root in

@@ -36,16 +36,14 @@ namespace kdt {
 
 namespace {
 
-constexpr int T = kSubtreeThreads;
-constexpr int NW = kSubtreeWarps;
 constexpr uint16_t kNoCell = 0xffff;
 constexpr uint32_t kRankMax = 32;
 
 // -------------------------------------------------------- shared layout
 
 struct Smem {
-  uint32_t* whist;    // NW * 256 words: warp histograms, tables of few cells, root subset counts
-  uint16_t* biglist;  // kSubtreeBigCap segments above kRankMax points
+  uint32_t* whist;    // kSubtreeHistWords: warp histograms, tables of few cells, root subset counts
+  uint16_t* biglist;  // segments above kRankMax points (SubtreeShape::bigs)
   LCell* tab;         // 2 * cells: the cell tables of two levels
   uint32_t* cols;     // d coordinate columns (raw floats) at stride `stride`
   uint32_t* gk;       // N: key of each position on its cell's coordinate
@@ -63,13 +61,13 @@ __device__ __forceinline__ uint32_t al16(uint32_t off) { return (off + 15u) & ~1
 // Carve the dynamic shared memory with plain byte offsets from its base (no
 // pointer is stored through another pointer), so that the compiler keeps
 // every array in the shared address space.
-__device__ __forceinline__ Smem carve(uint8_t* base, uint32_t N, int d, int cells) {
+__device__ __forceinline__ Smem carve(uint8_t* base, uint32_t N, int d, int cells, int bigs) {
   Smem s;
   uint32_t off = 0;
   s.whist = (uint32_t*)(base + off);
-  off += (uint32_t)NW * 256u * 4u;
+  off += (uint32_t)kSubtreeHistWords * 4u;
   s.biglist = (uint16_t*)(base + off);
-  off += (uint32_t)kSubtreeBigCap * 2u;
+  off += (uint32_t)bigs * 2u;
   s.tab = (LCell*)(base + off);
   off += 2u * (uint32_t)cells * (uint32_t)sizeof(LCell);
   s.cols = (uint32_t*)(base + off);
@@ -122,29 +120,32 @@ __device__ __forceinline__ int warp_pick_widest(const uint32_t (&lo)[2], const u
 }
 
 // Exclusive prefix, over all positions, of the flags whose warp ballots are
-// bal[q] (position tid + q T, block q NW + warp), given the popcount of every
-// block in cnt[kQ NW] (block order = position order; at most 64 blocks);
-// *total is the sum.
-template <int kQ>
+// bal[q] (position tid + q T of T = 32 NW threads, block q NW + warp), given the
+// popcount of every block in cnt[kQ NW] (block order = position order); *total
+// is the sum.
+template <int kQ, int NW>
 __device__ __forceinline__ void block_counts_scan(const unsigned (&bal)[kQ], const uint32_t* cnt, int lane,
                                                   int warp, uint32_t (&excl)[kQ], uint32_t* total) {
-  static_assert(kQ * NW <= 64, "two block counts per lane at most");
-  const uint32_t c0 = lane < kQ * NW ? cnt[lane] : 0u, c1 = lane + 32 < kQ * NW ? cnt[lane + 32] : 0u;
-  const uint32_t i0 = warp_incl_scan(c0);
-  const uint32_t i1 = warp_incl_scan(c1) + __shfl_sync(0xffffffffu, i0, 31);
-  *total = __shfl_sync(0xffffffffu, i1, 31);
-  const uint32_t e0 = i0 - c0, e1 = i1 - c1;
+  static_assert(32 % NW == 0, "a thread's blocks lie in one row of 32 each");
+  constexpr int R = (kQ * NW + 31) / 32;  // rows of 32 block counts
+  uint32_t e[R], run = 0;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const uint32_t c = lane + 32 * r < kQ * NW ? cnt[lane + 32 * r] : 0u;
+    const uint32_t i = warp_incl_scan(c);
+    e[r] = run + i - c;
+    run += __shfl_sync(0xffffffffu, i, 31);
+  }
+  *total = run;
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
-  for (int q = 0; q < kQ; ++q) {
-    const int src = (q * NW + warp) & 31;
-    const uint32_t v0 = __shfl_sync(0xffffffffu, e0, src), v1 = __shfl_sync(0xffffffffu, e1, src);
-    excl[q] = (q * NW < 32 ? v0 : v1) + (uint32_t)__popc(bal[q] & lt);
-  }
+  for (int q = 0; q < kQ; ++q)
+    excl[q] = __shfl_sync(0xffffffffu, e[(q * NW) / 32], (q * NW + warp) & 31) + (uint32_t)__popc(bal[q] & lt);
 }
 
 // Block-wide exclusive scan of one value per thread with one barrier; wtot
 // (NW words) must not be reused before the next barrier.
+template <int NW>
 __device__ __forceinline__ uint32_t block_excl_scan_1bar(uint32_t v, uint32_t* wtot, int lane, int warp,
                                                          uint32_t* total) {
   const uint32_t incl = warp_incl_scan(v);
@@ -216,35 +217,37 @@ __device__ __forceinline__ uint32_t warp_wsel_bits(uint32_t cnt, uint32_t rank, 
   return prefix;
 }
 
-// Lower median of kRankMax < w keys by one warp: a network up to 64 keys, bit
-// by bit with the keys in registers up to 512, else by radix histogram (a chain
-// of some 7000 cycles whatever the size, so trees of few subsets waited there
-// for most of their first levels: 1000 points in 8 subsets 62 -> 50 us, 512
-// trees of 4 to 64 subsets 3.95 -> 3.2 ms. A form for 1024 keys, 32 registers,
-// slowed every other path of the kernel by 3%.)
+// Lower median of kRankMax < w <= kBitsMax keys by one warp: a network up to 64
+// keys, then bit by bit with the keys in registers. (A radix histogram, which
+// larger segments take, is a chain of some 7000 cycles whatever the size, so
+// trees of few subsets waited there for most of their first levels: 1000 points
+// in 8 subsets 62 -> 50 us, 512 trees of 4 to 64 subsets 3.95 -> 3.2 ms. A form
+// for 1024 keys, 32 registers, slowed every other path of the kernel by 3%.)
+constexpr uint32_t kBitsMax = 512;
 template <class KeyOf>
-__device__ __forceinline__ uint32_t warp_segment_median(uint32_t w, uint32_t* hist, KeyOf key_of) {
+__device__ __forceinline__ uint32_t warp_segment_median(uint32_t w, KeyOf key_of) {
   auto one = [](uint32_t) { return 1u; };
   const uint32_t rank = (w - 1u) / 2u;
   if (w <= 64u) return warp_bitonic_median<2>(key_of, w);
   if (w <= 128u) return warp_wsel_bits<4, true>(w, rank, key_of, one);
   if (w <= 256u) return warp_wsel_bits<8, true>(w, rank, key_of, one);
-  if (w <= 512u) return warp_wsel_bits<16, true>(w, rank, key_of, one);
-  return warp_weighted_select<true>(w, rank, hist, key_of, one);
+  return warp_wsel_bits<16, true>(w, rank, key_of, one);
 }
 
-// kWide: compiled for the wide shape, else the narrow one (kdt_launch.h).
-template <bool kWide>
-__global__ void __launch_bounds__(T, (kWide ? kSubWide : kSubNarrow).ctas)
+// The shapes of kdt_launch.h.
+constexpr SubtreeShape kShapes[3] = {kSubNarrow, kSubWide, kSubTall};
+
+template <int kShape>
+__global__ void __launch_bounds__(kShapes[kShape].threads, kShapes[kShape].ctas)
 k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t* count_dev, uint32_t reversed,
           const uint32_t* small_off, uint32_t* head, LCell* slices, uint32_t slice_cells, uint32_t probe_tries) {
-  constexpr SubtreeShape kSh = kWide ? kSubWide : kSubNarrow;
-  constexpr int kQ = kSh.q, kCells = kSh.cells;
+  constexpr SubtreeShape kSh = kShapes[kShape];
+  constexpr int T = kSh.threads, NW = T / 32, kQ = kSh.q, kCells = kSh.cells;
   extern __shared__ __align__(128) uint8_t smem_raw[];
   const uint32_t count_cap = count;
   if (count_dev) count = min(*count_dev, count);  // a graph-driven step: the queue's length, capped
   __shared__ uint32_t tmp[33];
-  __shared__ uint32_t s_item, s_ncur, s_nbig, s_where, s_fail;
+  __shared__ uint32_t s_item, s_ncur, s_nbig, s_nhist, s_where, s_fail;
   __shared__ __align__(8) uint64_t s_bar;
   __shared__ uint32_t s_colbase[kMaxDims];
   __shared__ uint32_t s_bcnt[kQ * NW];  // per-block counts of a level's position flags
@@ -299,7 +302,7 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
     const uint32_t N = c.count;
     const int d = t.d, r = t.r;
     const int64_t n = t.n;
-    if (N > (uint32_t)(kQ * T) || subtree_fixed_bytes(kCells) + subtree_point_bytes(N, d) > kSh.smem) {
+    if (N > (uint32_t)(kQ * T) || subtree_fixed_bytes(kSh) + subtree_point_bytes(N, d) > kSh.smem) {
       // a queue holds only cells within its shape's capacity
       if (tid == 0) {
         set_status(t, ST_INTERNAL);
@@ -308,7 +311,7 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
       continue;
     }
     const uint32_t stride = subtree_stride(N);
-    Smem S = carve(smem_raw, N, d, kCells);
+    Smem S = carve(smem_raw, N, d, kCells, kSh.bigs);
     // Column l of the cell sits at S.cols + s_colbase[l]. Each column's
     // offset absorbs the 16-byte alignment phase of its global source so that
     // the bulk copies are aligned on both sides.
@@ -478,7 +481,9 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
         } else {
           // per (cell, part): min and max key of every coordinate, coordinate l
           // ending in lane l % 32; G warps share a cell when there are few cells
-          const uint32_t G = ncur >= (uint32_t)NW ? 1u : (uint32_t)NW / ncur;
+          const uint32_t G = ncur >= (uint32_t)NW || 2u * ncur * (uint32_t)d > (uint32_t)kSubtreeHistWords
+                                 ? 1u
+                                 : (uint32_t)NW / ncur;
           uint32_t* tab = S.whist;  // few cells: [ncur][d][2]
           if (G > 1) {
             for (uint32_t j = tid; j < ncur * (uint32_t)d; j += T) {
@@ -592,11 +597,11 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
           balq[q] = __ballot_sync(0xffffffffu, f);
           if (lane == 0) s_bcnt[q * NW + warp] = (uint32_t)__popc(balq[q]);
         }
-        if (tid == 0) s_nbig = 0;
+        if (tid == 0) s_nbig = s_nhist = 0;
         __syncthreads();
         {
           uint32_t total;
-          block_counts_scan(balq, s_bcnt, lane, warp, segq, &total);
+          block_counts_scan<kQ, NW>(balq, s_bcnt, lane, warp, segq, &total);
 #pragma unroll
           for (int q = 0; q < kQ; ++q) {
             const uint32_t i = (uint32_t)tid + (uint32_t)q * T;
@@ -627,7 +632,8 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
           if (w > kRankMax) {
             if (i == b) {
               const uint32_t slot = atomicAdd(&s_nbig, 1u);
-              if (slot < (uint32_t)kSubtreeBigCap) S.biglist[slot] = (uint16_t)sx; else set_status(t, ST_INTERNAL);
+              if (slot < (uint32_t)kSh.bigs) S.biglist[slot] = (uint16_t)sx; else set_status(t, ST_INTERNAL);
+              if (w > kBitsMax) s_nhist = 1;
             }
             continue;
           }
@@ -641,17 +647,30 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
         }
         __syncthreads();
         if (s_nbig) {
-          const uint32_t nbig = min(s_nbig, (uint32_t)kSubtreeBigCap);
-          for (uint32_t j = warp; j < nbig; j += NW) {
-            const uint32_t sx = S.biglist[j];
-            const uint32_t b = S.segs[sx];
+          const uint32_t nbig = min(s_nbig, (uint32_t)kSh.bigs);
+          auto segment = [&](uint32_t j, uint32_t* sx, uint32_t* w) -> const uint32_t* {
+            *sx = S.biglist[j];
+            const uint32_t b = S.segs[*sx];
             const uint16_t k = S.cellid[b];
-            const uint32_t e = min((uint32_t)S.segs[sx + 1], (uint32_t)cc[k].begin + cc[k].count);
-            const uint32_t* g = S.gk + b;
-            const uint32_t m =
-                warp_segment_median(e - b, S.whist + warp * 256, [&](uint32_t jj) { return g[jj]; });
+            *w = min((uint32_t)S.segs[*sx + 1], (uint32_t)cc[k].begin + cc[k].count) - b;
+            return S.gk + b;
+          };
+          uint32_t sx, w;
+          for (uint32_t j = warp; j < nbig; j += NW) {
+            const uint32_t* g = segment(j, &sx, &w);
+            if (w > kBitsMax) continue;
+            const uint32_t m = warp_segment_median(w, [&](uint32_t jj) { return g[jj]; });
             if (lane == 0) S.smed[sx] = m;
           }
+          if (s_nhist && warp < kSubtreeHists)  // a histogram each
+            for (uint32_t j = warp; j < nbig; j += kSubtreeHists) {
+              const uint32_t* g = segment(j, &sx, &w);
+              if (w <= kBitsMax) continue;
+              const uint32_t m = warp_weighted_select<true>(w, (w - 1u) / 2u, S.whist + warp * 256,
+                                                            [&](uint32_t jj) { return g[jj]; },
+                                                            [](uint32_t) { return 1u; });
+              if (lane == 0) S.smed[sx] = m;
+            }
           __syncthreads();
         }
 
@@ -661,9 +680,12 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
         // pre[end]). One warp per cell, no block barrier: up to 256 segments
         // are held in registers and the key is settled one bit per step by a
         // warp sum; more segments go through the warp's radix histogram.
-        for (uint32_t k = warp; k < ncur; k += NW) {
+        // (the histograms are fewer than the warps of the tall shape: its cells of
+        // more segments follow in a second round of that many warps)
+        auto combine = [&](uint32_t k, bool hist_round) {
           const uint32_t b = cc[k].begin, e = b + cc[k].count;
           const uint32_t s0 = S.pre[b], s1 = S.pre[e], ns = s1 - s0;
+          if (NW > kSubtreeHists && (ns > 256u) != hist_round) return;
           const bool unit = t.combine_rule == 1;  // every subset counts once (segments are non-empty)
           const uint32_t rank = unit ? (ns - 1u) / 2u : (cc[k].count - 1u) / 2u;
           auto key_of = [&](uint32_t j) { return S.smed[s0 + j]; };
@@ -682,7 +704,10 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
           else
             m = warp_weighted_select(ns, rank, S.whist + warp * 256, key_of, w_of);
           if (lane == 0) cc[k].mkey = m;
-        }
+        };
+        for (uint32_t k = warp; k < ncur; k += NW) combine(k, false);
+        if (NW > kSubtreeHists && r > 256 && warp < kSubtreeHists)
+          for (uint32_t k = warp; k < ncur; k += kSubtreeHists) combine(k, true);
         __syncthreads();
         for (uint32_t k = tid; k < ncur; k += T) {
           t.out_vals[cc[k].heap] = key_float(cc[k].mkey);
@@ -703,7 +728,7 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
           }
           __syncthreads();
           uint32_t lpre[kQ], tot;
-          block_counts_scan(lbq, s_bcnt, lane, warp, lpre, &tot);
+          block_counts_scan<kQ, NW>(lbq, s_bcnt, lane, warp, lpre, &tot);
 #pragma unroll
           for (int q = 0; q < kQ; ++q) {
             const uint32_t i = (uint32_t)tid + (uint32_t)q * T;
@@ -769,7 +794,7 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
             }
           }
           const uint32_t nlive = (uint32_t)live[0] + (uint32_t)live[1];
-          const uint32_t ex = block_excl_scan_1bar(nlive, s_wtot, lane, warp, &run_out);
+          const uint32_t ex = block_excl_scan_1bar<NW>(nlive, s_wtot, lane, warp, &run_out);
           nwhere = run_out <= (uint32_t)kCells ? 0 : 1;
           LCell* nc = nwhere ? gslice + (size_t)(which ^ 1) * slice_cells : S.tab + (which ^ 1) * kCells;
           if (k < ncur) {
@@ -905,11 +930,11 @@ void launch_iota(uint32_t* out, uint32_t n, cudaStream_t st) {
 using SubtreeKernel = void (*)(const TreeDev*, const Cell*, uint32_t, const uint32_t*, uint32_t, const uint32_t*,
                                uint32_t*, LCell*, uint32_t, uint32_t);
 SubtreeKernel subtree_kernel(const SubtreeShape& sh) {
-  return sh.q == kSubWide.q ? k_subtree<true> : k_subtree<false>;
+  return sh.threads == kSubTall.threads ? k_subtree<2> : sh.q == kSubWide.q ? k_subtree<1> : k_subtree<0>;
 }
 
 cudaError_t prepare_subtree_kernel() {
-  for (const SubtreeShape* sh : {&kSubNarrow, &kSubWide}) {
+  for (const SubtreeShape* sh : {&kSubNarrow, &kSubWide, &kSubTall}) {
     const cudaError_t e = cudaFuncSetAttribute(subtree_kernel(*sh), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)sh->smem);
     if (e != cudaSuccess) return e;
@@ -927,8 +952,8 @@ void launch_subtree(const SubtreeShape& sh, const TreeDev* trees, const Cell* li
     cudaMemsetAsync(head, 0, sizeof(uint32_t), st);
   const uint32_t probe = fault_take(KDT_FAULT_WAIT) ? 1024u : 0u;
   TraceScope ts(K_SUBTREE, st, points);
-  subtree_kernel(sh)<<<grid, T, sh.smem, st>>>(trees, list, count, count_dev, reversed ? 1u : 0u, small_off, head,
-                                               slices, slice_cells, probe);
+  subtree_kernel(sh)<<<grid, sh.threads, sh.smem, st>>>(trees, list, count, count_dev, reversed ? 1u : 0u, small_off,
+                                               head, slices, slice_cells, probe);
 }
 
 void launch_finalize_many(const TreeDev* trees, const SlotChunks& sc, cudaStream_t st) {

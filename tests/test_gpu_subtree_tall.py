@@ -1,0 +1,59 @@
+"""GPU: trees built alone that end in the subtree kernel's tall shape: sizes
+around one such cell and a few, every column count class (its capacity falls
+with d), segments above 512 keys, more subsets than a cell has points, cells
+that ties leave unequal (more of them than the splits by halves give), both key
+rules, each kind of subset. Bit for bit against the oracle."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import require_gpu
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    require_gpu()
+
+
+def _check(x, gsid, sid, **kw):
+    from paper_2201_08288_gb300 import kdt
+    try:
+        o = oracle.build_tree(x, sid=sid, **kw)
+    except oracle.OracleError:  # ties beyond the level cap: refused here too
+        with pytest.raises(kdt.KdtError):
+            kdt.kdt_build(torch.from_numpy(x).cuda(), sid=gsid, **kw)
+        return
+    g = kdt.kdt_build(torch.from_numpy(x).cuda(), sid=gsid, **kw)
+    assert g.levels == o.levels
+    assert np.array_equal(g.perm.cpu().numpy().view(np.uint32), o.perm)
+    assert np.array_equal(g.split_vals.cpu().numpy().view(np.uint32), o.split_vals.view(np.uint32))
+    assert np.array_equal(g.split_dims.cpu().numpy(), o.split_dims)
+    assert np.array_equal(g.node_offsets.cpu().numpy(), o.node_offsets)
+
+
+@pytest.mark.parametrize("n", [1281, 2049, 4093, 5120, 5121, 20_479, 50_001])
+@pytest.mark.parametrize("d,rule", [(1, 0), (2, 1), (3, 0), (8, 1), (9, 0), (16, 1), (33, 0)])
+@pytest.mark.parametrize("r,mode", [(1, 0), (3, 0), (40, 2), (700, 1), (5000, 2)])
+def test_sizes(n, d, rule, r, mode):
+    rng = np.random.default_rng(n + d + r)
+    x = rng.standard_normal((d, n)).astype(np.float32)
+    if r != 40:  # ties in the first columns: cells of unequal sizes, some with an empty side
+        x[: max(1, d - 1)] = np.where(rng.random((max(1, d - 1), n)) < 0.6, np.float32(0.25), np.round(x[: max(1, d - 1)] * 4) / 4)
+    r = min(r, 4096)
+    sid = gsid = None
+    if mode == 2:
+        sid = (rng.random(n) ** 2 * r).astype(np.uint8 if r <= 256 else np.uint16)
+        gsid = torch.from_numpy(sid if r <= 256 else sid.view(np.int16)).cuda()
+    _check(x, gsid, sid, r=r, subset_mode=mode, leaf_size=9, max_levels=22, key_rule=rule)
+
+
+@pytest.mark.parametrize("d", [2, 7, 24])
+def test_fixed_depth(d):
+    x = np.random.default_rng(d).standard_normal((d, 6001)).astype(np.float32)
+    for depth in (1, 2, 5, 13):
+        _check(x, None, None, r=6, subset_mode=0, depth=depth)
