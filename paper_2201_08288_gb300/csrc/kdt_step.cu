@@ -1194,31 +1194,82 @@ __global__ void __launch_bounds__(256, 2) k_fourier_moments(const TreeDev* trees
 // coordinate is <= it. The harmonics of the midpoint are evaluated in float
 // (their error moves the root by about 1e-7 of the cell's width), the sums in
 // double.
-// A step's chain of double operations takes over 2 us, and 60 of them in a
-// row, a warp per cell, were 165 us per level whatever the cells. So the CTA
-// takes three steps at once: warps 1..7 evaluate F at the seven midpoints that
-// the three can meet (warp w stands for the path that w's bits below its
-// highest one spell, 0 where F >= 0), and every warp then walks the path that
-// the signs give. (With more steps at once the double unit, not the chain,
-// bounds a level of many cells.) 4,000,037 points, J = 16, ten levels: 1.06 ms
-// per build; 1.86 with a warp per cell whose root added its 304 run records one
-// load at a time. The sums per midpoint are those of the
-// one-warp form, lane for lane, so the splits are the same bits.
-constexpr int kFsSteps = 3, kFsWarps = 1 << kFsSteps;
+// Double arithmetic bounds this: an SM's quarter finishes one warp-wide double
+// operation in 64 cycles and starts the next after about as many (conversions
+// to and from double too), and a step is a chain of a product, two sums per
+// term, a tree of five sums and a midpoint. A warp per cell that took the 60
+// steps one by one, each lane with its own terms and its own conversions, was
+// 165 us per level whatever the cells. So the CTA takes three steps at once:
+//   the seven midpoints that the three can meet (candidate w stands for the
+//     path that w's bits below its highest one spell, 0 where F >= 0) were
+//     formed during the round before, for each of its eight outcomes, by warps
+//     without terms of their own;
+//   a thread per candidate and harmonic evaluates both of its terms; what can
+//     be had exactly from integers (K m rounded to float, the waves widened to
+//     double) is;
+//   half a warp per candidate adds its terms, in the order and tree of the
+//     one-warp form, so the splits are the same bits; the signs are the round's
+//     outcome.
+// The start of every run record comes from a 64-bit division: formed once per
+// chunk of them, by a lane each (a thread that formed its own spent 347,000
+// cycles on the root's 304). 4,000,037 points, J = 16, ten levels: 0.60 ms per
+// build; 1.86 with a warp per cell.
+constexpr int kFsSteps = 3, kFsCand = 1 << kFsSteps;  // candidates 1 .. kFsCand - 1
+constexpr int kFsThreads = 256;
 constexpr int kFsChunk = 32;  // run records staged at a time
+static_assert((kFsCand - 1) * KDT_FOURIER_MAX_J <= kFsThreads, "a thread per candidate and harmonic");
+static_assert((kFsCand - 1) * 16 <= kFsThreads && 4 * KDT_FOURIER_MAX_J <= kFsThreads, "threads for the other parts");
 
-__global__ void __launch_bounds__(kFsWarps * 32) k_fourier_split(const TreeDev* trees, StepDev s, uint32_t mgrid) {
+// (float)(k * x) for 0 < x < 4 and an odd k below 64, k * x rounded to double
+// first: the product of x's 53 bits and k's 6 in 64, rounded to nearest even
+// twice.
+__device__ __forceinline__ float product_float(uint32_t k, double x) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(u >> 52);
+  if (ex < 1023 - 96) return (float)((double)k * x);  // (zero, or near the float's smallest numbers)
+  unsigned long long p = ((u & 0xfffffffffffffull) | 0x10000000000000ull) * k;  // below 2^59
+  auto round_off = [&](int n) {  // p / 2^n to nearest even, n >= 1
+    const unsigned long long half = 1ull << (n - 1), rest = p & ((1ull << n) - 1ull);
+    p >>= n;
+    p += rest > half || (rest == half && (p & 1ull)) ? 1ull : 0ull;
+  };
+  int e = ex - 1075;  // the value is p 2^e
+  const int over = 64 - __clzll((long long)p) - 53;
+  if (over > 0) {
+    round_off(over);
+    e += over;
+  }
+  const int more = 64 - __clzll((long long)p) - 24;  // p has 53 or 54 bits
+  round_off(more);
+  e += more;
+  return __int2float_rn((int)p) * __int_as_float((e + 127) << 23);  // both exact: at most 25 bits, a power of two
+}
+
+// (double)x from its bits where x is a normal float.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), e = (u >> 23) & 255u;
+  if (e == 0u || e == 255u) return (double)x;
+  return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu)), (int)(u << 29));
+}
+
+__global__ void __launch_bounds__(kFsThreads) k_fourier_split(const TreeDev* trees, StepDev s, uint32_t mgrid) {
   __shared__ double rec[kFsChunk][kFourierTerms];
-  __shared__ double s_base[96], s_slope[96];
-  __shared__ uint32_t s_neg[2];  // per parity of the round: bit w: F < 0 at warp w's midpoint
+  __shared__ double s_base[kFourierTerms], s_slope[kFourierTerms];
+  __shared__ double s_wave[4][KDT_FOURIER_MAX_J];  // sin K a, sin K b, cos K a, cos K b
+  __shared__ double s_mid[2][kFsCand][kFsCand];  // by round's parity, outcome of the round before, candidate
+  __shared__ double s_end[2][kFsCand][2];        // and each outcome's (lo, hi)
+  __shared__ double s_term[kFsCand][96];
+  __shared__ uint32_t s_neg[2];  // by round's parity; bit w: F < 0 at candidate w's midpoint
+  __shared__ uint32_t s_run[kFsChunk], s_nrun;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t nc = ncells_of(s);
   const uint32_t ntiles = ntiles_of(s);
   auto range_start = [&](uint32_t k) { return (uint32_t)(((uint64_t)k * ntiles) / mgrid); };
+  for (int i = tid; i < kFsCand * 96; i += kFsThreads) (&s_term[0][0])[i] = 0.0;  // terms that no tree here has
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
     const Cell cell = s.cells[c];
     const TreeDev& t = trees[cell.tree];
-    const int nt = 2 * t.fourier_j + 1;
+    const int J = t.fourier_j, nt = 2 * J + 1;
     const uint32_t tb = cell.tile0, te = tb + tiles_of(cell.count);
     // The moments kernel's runs of this cell start at tb and at every start of
     // a CTA's tile range inside (tb, te): with at least as many tiles as CTAs
@@ -1234,19 +1285,27 @@ __global__ void __launch_bounds__(kFsWarps * 32) k_fourier_split(const TreeDev* 
     }
     auto run_start = [&](uint32_t m) -> uint32_t {  // te: no such run
       if (m == 0u) return tb;
-      if (dense) return tb + m;
-      return k0 + m < mgrid ? range_start(k0 + m) : te;
+      if (dense) return min(tb + m, te);
+      return k0 + m < mgrid ? min(range_start(k0 + m), te) : te;
     };
     double C = 0.0;  // thread j: the sum of term j
-    for (uint32_t m0 = 0; run_start(m0) < te; m0 += kFsChunk) {
-      for (uint32_t i = tid; i < (uint32_t)(kFsChunk * nt); i += kFsWarps * 32) {
-        const uint32_t r0 = run_start(m0 + i / (uint32_t)nt);
-        if (r0 < te) rec[i / nt][i % nt] = ((const double*)(s.tile_mm + (size_t)r0 * kTileRecWords))[i % nt];
+    for (uint32_t m0 = 0;; m0 += kFsChunk) {
+      if (warp == 0) {
+        const uint32_t r0 = run_start(m0 + (uint32_t)lane);
+        s_run[lane] = r0;
+        const unsigned some = __ballot_sync(0xffffffffu, r0 < te);
+        if (lane == 0) s_nrun = (uint32_t)__popc(some);
       }
       __syncthreads();
-      if (tid < nt)
-        for (uint32_t m = 0; m < (uint32_t)kFsChunk && run_start(m0 + m) < te; ++m) C += rec[m][tid];
+      const uint32_t nrun = s_nrun;
+      for (uint32_t m = warp; m < nrun; m += kFsThreads / 32)
+        for (int j = lane; j < nt; j += 32)
+          rec[m][j] = ((const double*)(s.tile_mm + (size_t)s_run[m] * kTileRecWords))[j];
       __syncthreads();
+      if (tid < nt)
+        for (uint32_t m = 0; m < nrun; ++m) C += rec[m][tid];
+      __syncthreads();
+      if (nrun < (uint32_t)kFsChunk) break;
     }
     // bounds: lane i of every warp takes the i-th ancestor (splits are in
     // [0, 1], where floats order like their bits)
@@ -1262,79 +1321,131 @@ __global__ void __launch_bounds__(kFsWarps * 32) k_fourier_split(const TreeDev* 
     }
     const double a = (double)__uint_as_float(__reduce_max_sync(0xffffffffu, ba));
     const double b = (double)__uint_as_float(min(__reduce_min_sync(0xffffffffu, bb), __float_as_uint(1.0f)));
-    const double ia = a > 0.0 ? 1.0 : 0.0, ib = b < 1.0 ? 1.0 : 0.0;
+    // the bounds' waves, a thread each (a bound at the interval's end has
+    // weight 0: its waves are not needed)
+    {
+      const int which = tid / KDT_FOURIER_MAX_J, j = tid % KDT_FOURIER_MAX_J;
+      if (which < 4 && j < J) {
+        const double x = (double)(2 * j + 1) * ((which & 1) ? b : a);
+        const bool needed = (which & 1) ? b < 1.0 : a > 0.0;
+        s_wave[which][j] = !needed ? 0.0 : which < 2 ? sin(x) : cos(x);
+      }
+    }
+    __syncthreads();
     // per term: F_j(m) = base + slope * (sin or cos)(K m)
-    if (tid < 96) {
-      double base = 0.0, slope = 0.0;
+    const double ia = a > 0.0 ? 1.0 : 0.0, ib = b < 1.0 ? 1.0 : 0.0;
+    if (tid < nt) {
+      double base, slope = 0.0;
       if (tid == 0) {
         base = C * 0.5 * (ib - ia);
-      } else if (tid < nt) {
-        const double k = (double)(2 * ((tid + 1) / 2) - 1);
-        const double qk = 2.0 / (3.14159265358979323846 * k);
+      } else {
+        const int j = (tid - 1) / 2;
+        const double qk = 2.0 / (3.14159265358979323846 * (double)(2 * j + 1));
         if (tid & 1) {
-          base = -C * qk * (ia * sin(k * a) + ib * sin(k * b));
+          base = -C * qk * (ia * s_wave[0][j] + ib * s_wave[1][j]);
           slope = 2.0 * C * qk;
         } else {
-          base = C * qk * (ia * cos(k * a) + ib * cos(k * b));
+          base = C * qk * (ia * s_wave[2][j] + ib * s_wave[3][j]);
           slope = -2.0 * C * qk;
         }
       }
       s_base[tid] = base;
       s_slope[tid] = slope;
     }
-    if (tid < 2) s_neg[tid] = 0u;
     __syncthreads();
-    double base[3], slope[3], K[3];
-    bool use[3], wave[3], use_sin[3];
+    // this thread's candidate and harmonic, and the half warp's candidate
+    const int cand = 1 + tid / J, k = 1 + tid % J;
+    const bool waves = cand < kFsCand;
+    const double base_s = waves ? s_base[2 * k - 1] : 0.0, slope_s = waves ? s_slope[2 * k - 1] : 0.0;
+    const double base_c = waves ? s_base[2 * k] : 0.0, slope_c = waves ? s_slope[2 * k] : 0.0;
+    const int sum_cand = 1 + tid / 16, l = tid & 15;
+    const bool sums = sum_cand < kFsCand;
+    if (tid < kFsCand) s_term[tid][0] = s_base[0];
+    const bool wave_s = slope_s != 0.0, wave_c = slope_c != 0.0;
+    // half of a sum of bounds: its exponent less one (0 only for the cell [0, 0])
+    auto half = [](double x) {
+      const int h = __double2hiint(x), g = __double2loint(x);
+      return (h | g) == 0 ? 0.0 : __hiloint2double(h - 0x00100000, g);
+    };
+    // thread (outcome, candidate): the midpoint of the candidate after that
+    // outcome of a round whose midpoints are `mids`, its bounds to `end`
+    auto form = [&](int i, double x, double y, const double* mids, double (*next)[kFsCand], double (*end)[2]) {
+      const int out = i / kFsCand, cnd = i % kFsCand, top = 31 - __clz(cnd);
+      if (mids) {
+        uint32_t w = 1;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const int j = lane + 32 * q;
-      base[q] = s_base[j];
-      slope[q] = s_slope[j];
-      K[q] = (double)(2 * ((j + 1) / 2) - 1);
-      wave[q] = slope[q] != 0.0;
-      use[q] = wave[q] || base[q] != 0.0;
-      use_sin[q] = (j & 1) != 0;
-    }
-    double lo = a, hi = b;
-    for (int it = 0; it < 60 / kFsSteps; ++it) {
-      if (warp > 0) {
-        double l = lo, h = hi, mid = 0.5 * (lo + hi);
-        for (int bit = 30 - __clz(warp); bit >= 0; --bit) {
-          if ((warp >> bit) & 1) l = mid; else h = mid;
-          mid = 0.5 * (l + h);
+        for (int st = 0; st < kFsSteps; ++st) {
+          const uint32_t up = ((uint32_t)out >> (kFsSteps - 1 - st)) & 1u;
+          if (up) x = mids[w]; else y = mids[w];
+          w = 2u * w + up;
         }
+      }
+      if (cnd == 0) {
+        end[out][0] = x;
+        end[out][1] = y;
+        return;
+      }
+      double mid = half(x + y);
+#pragma unroll
+      for (int st = 0; st < kFsSteps - 1; ++st)
+        if (top > st) {
+          if ((cnd >> (top - 1 - st)) & 1) x = mid; else y = mid;
+          mid = half(x + y);
+        }
+      next[out][cnd] = mid;
+    };
+    if (tid < kFsCand) form(tid, a, b, nullptr, s_mid[0], s_end[0]);  // the first round: outcome 0 of none
+    if (tid == 0) s_neg[0] = 0u;
+    uint32_t out = 0;
+    __syncthreads();
+    for (int it = 0; it < 60 / kFsSteps; ++it) {
+      const double* mids = s_mid[it & 1][out];
+      if (waves) {
+        const float arg = product_float((uint32_t)(2 * k - 1), mids[cand]);
+        float sn, cs;
+        sincosf(arg, &sn, &cs);
+        s_term[cand][2 * k - 1] = wave_s ? __dadd_rn(base_s, __dmul_rn(slope_s, widen(sn))) : base_s;
+        s_term[cand][2 * k] = wave_c ? __dadd_rn(base_c, __dmul_rn(slope_c, widen(cs))) : base_c;
+      }
+      if (tid >= kFsThreads - kFsCand * kFsCand)  // the last two warps (with terms of their own only for J > 27)
+        form(tid - (kFsThreads - kFsCand * kFsCand), s_end[it & 1][out][0], s_end[it & 1][out][1], mids,
+             s_mid[(it + 1) & 1], s_end[(it + 1) & 1]);
+      __syncthreads();
+      if (tid == 0) s_neg[(it + 1) & 1] = 0u;  // (read by all before this barrier, written after the next)
+      {
         double f = 0.0;
+        if (sums) {
+          const double* p = s_term[sum_cand];
+          double u = p[l], v = p[l + 16];
+          if (l + 32 < nt) u = __dadd_rn(u, p[l + 32]);
+          if (l + 48 < nt) v = __dadd_rn(v, p[l + 48]);
+          if (l + 64 < nt) u = __dadd_rn(u, p[l + 64]);
+          f = __dadd_rn(u, v);
+        }
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
-          if (use[q])
-            f += base[q] + (wave[q] ? slope[q] * (double)(use_sin[q] ? sinf((float)(K[q] * mid)) : cosf((float)(K[q] * mid)))
-                                    : 0.0);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) f += __shfl_down_sync(0xffffffffu, f, o);
-        if (lane == 0 && f < 0.0) atomicOr(&s_neg[it & 1], 1u << warp);  // lane 0's sum decides
+        for (int o = 8; o > 0; o >>= 1) f += __shfl_down_sync(0xffffffffu, f, o, 16);
+        // F < 0: the sign, unless it is zero
+        const int h = __double2hiint(f);
+        if (sums && l == 0 && h < 0 && (((uint32_t)h << 1) | (uint32_t)__double2loint(f)) != 0u)
+          atomicOr(&s_neg[it & 1], 1u << sum_cand);
       }
       __syncthreads();
       const uint32_t neg = s_neg[it & 1];
       uint32_t w = 1;
 #pragma unroll
-      for (int st = 0; st < kFsSteps; ++st) {
-        const double mid = 0.5 * (lo + hi);
-        const uint32_t up = (neg >> w) & 1u;
-        if (up) lo = mid; else hi = mid;
-        w = 2u * w + up;
-      }
-      // the next round collects in the other word; this one is cleared for the
-      // round after it, once all have read it
-      __syncthreads();
-      if (tid == 0) s_neg[it & 1] = 0u;
+      for (int st = 0; st < kFsSteps; ++st) w = 2u * w + ((neg >> w) & 1u);
+      out = w - (uint32_t)kFsCand;
     }
+    const double lo = s_end[0][out][0], hi = s_end[0][out][1];
     if (tid == 0) {
       const float m32 = (float)(0.5 * (lo + hi));
       s.mkey[c] = ord_key(m32);
       t.out_vals[cell.heap] = m32;
       t.out_dims[cell.heap] = (int8_t)dim;
     }
+    __syncthreads();  // shared memory is free for the next cell
+    if (c + gridDim.x < nc)  // (another tree may have fewer terms)
+      for (int i = tid; i < kFsCand * 96; i += kFsThreads) (&s_term[0][0])[i] = 0.0;
   }
 }
 
@@ -1807,7 +1918,7 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
       TraceScope ts(K_FOURIER_MOMENTS, st, points);
       k_fourier_moments<<<mgrid, 256, 0, st>>>(trees, s);
     }
-    { TraceScope ts(K_FOURIER_SPLIT, st); k_fourier_split<<<cells_grid(1, sms * 4u), kFsWarps * 32, 0, st>>>(trees, s, mgrid); }
+    { TraceScope ts(K_FOURIER_SPLIT, st); k_fourier_split<<<cells_grid(1, sms * 4u), kFsThreads, 0, st>>>(trees, s, mgrid); }
   } else {
     if (s.few_segs) {
       TraceScope ts(K_SELECT_ALL, st, points);
