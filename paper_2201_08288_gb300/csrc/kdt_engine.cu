@@ -137,6 +137,10 @@ TreePlan plan_tree(const kdt_params& p0, bool no_subtree, bool alone) {
   // a small root is put in subset order by the subtree kernel itself, which
   // counts at most kSubtreeHistWords subsets
   t.presorted = t.leafsort && (n > (uint64_t)t.small_max || !subtree_sorts_root(p.r));
+  // a level of 2^k cells of the n points has one of ceil(n / 2^k) or more
+  const uint64_t ends = std::max<uint64_t>(t.small_max, p.depth > 0 ? 0 : (uint64_t)p.leaf_size);
+  if (!root_terminal && (t.presorted || n > (uint64_t)t.small_max)) t.steps = 1;
+  while (t.steps > 0 && t.steps < t.L_cap && ((n - 1) >> t.steps) + 1 > ends) ++t.steps;
   t.huge_cap = t.leafsort ? n / (uint64_t)(kLeafBlockMax + 1) + 1 : 0;
   const uint64_t leaves = (uint64_t)1 << t.L_cap;
   t.maxB = std::min<uint64_t>(n / (uint64_t)(t.small_max + 1) + 1, leaves);
@@ -294,7 +298,8 @@ kdt_status Engine::reset() {
   big_count_ = small_count_ = small_count_w_ = 0;
   big_tiles_ = big_segs_ = 0;
   big_points_ = small_points_ = 0;
-  root_dims_ = false;
+  root_dims_ = unsure_ = false;
+  ahead_ = 0;
   pending_.clear();
   return KDT_OK;
 }
@@ -378,6 +383,10 @@ kdt_status Engine::admit(uint32_t slot, const float* points, const kdt_params& p
             : !(n <= (uint64_t)tp.small_max && !tp.presorted) ? kListBig
             : tp.sub_wide ? kListSmallWide : kListSmall;
   if (pe.list == kListBig && p.key_rule == KDT_KEY_WIDEST_SPREAD) root_dims_ = true;
+  if (mt == 1 && !s_.shards) {
+    ahead_ = pe.list == kListBig ? tp.steps : 0;
+    ahead_wide_ = tp.sub_wide;
+  }
   pending_.push_back(pe);
   return KDT_OK;
 }
@@ -421,6 +430,68 @@ kdt_status Engine::flush_admits(bool* has_big_roots) {
   return KDT_OK;
 }
 
+void Engine::launch_step(bool has_roots) {
+  s_.few_segs = step_selects_all(s_.nseg, big_points_, plan_.sms) ? 1u : 0u;
+  // (not for shards: one segment of a shard's cell is a part of the cell's)
+  s_.wide_segs = !s_.shards && step_selects_wide(s_.nseg, big_points_) ? 1u : 0u;
+  const SelectTuning tune = current_tuning();
+  s_.tiny_max = tune.tiny_max;
+  s_.bitonic_max = tune.bitonic_max;
+  s_.warp_max = tune.warp_max;
+  launch_big_step(trees_, s_, s_.ntiles, s_.nseg, plan_.bigseg_cap, has_roots, root_dims_, plan_.needs.widest,
+                  plan_.needs.max_r, uniform_d(), tune, big_points_,
+                  plan_.grid_step, st_, plan_.needs.fourier);
+  root_dims_ = false;
+}
+
+void Engine::read_big(const uint32_t* w) {
+  const uint32_t* wb = w + W_BIG + 2 * cur_;
+  const uint32_t* wt = w + W_TILE + 2 * cur_;
+  big_count_ = std::min(wb[0], plan_.maxB);
+  big_segs_ = std::min(wb[1], plan_.nseg_cap);
+  big_tiles_ = std::min(wt[0], plan_.max_tiles);
+  big_points_ = wt[1];
+}
+
+// The steps of a tree built alone that have cells whatever its points are, and
+// then the subtree kernel, without a wait: a step's grids are sized for the
+// cells that halving gives at most, and its kernels read how many there are.
+// (Waiting for the counts of each level and launching the next left the GPU idle
+// for 10 to 17 us a level.)
+kdt_status Engine::run_ahead() {
+  bool has_roots = false;
+  const kdt_status f = flush_admits(&has_roots);
+  if (f != KDT_OK) return f;
+  s_.init_small = s_.init_small_w = s_.init_small_points = 0;
+  uint64_t cells = 1;  // of the step, at most
+  for (int k = 0; k < ahead_; ++k) {
+    use_lists(&s_, cur_);
+    if (k > 0) {
+      s_.ncells_dev = words_ + W_BIG + 2 * cur_;
+      s_.nseg_dev = words_ + W_BIG + 2 * cur_ + 1;
+      s_.ntiles_dev = words_ + W_TILE + 2 * cur_;
+      s_.bounded = s_.keep_small = 1;
+    }
+    s_.ncells = (uint32_t)cells;
+    s_.ntiles = (uint32_t)std::min<uint64_t>(k == 0 ? big_tiles_ : big_points_ / kTile + cells, plan_.max_tiles);
+    s_.nseg = (uint32_t)std::min<uint64_t>(cells * (uint64_t)plan_.needs.max_r, plan_.nseg_cap);
+    launch_step(has_roots && k == 0);
+    ENGINE_TRY(cudaGetLastError());
+    cur_ ^= 1;
+    cells = std::min<uint64_t>(2 * cells, plan_.maxB);
+  }
+  s_.ncells_dev = s_.nseg_dev = s_.ntiles_dev = nullptr;
+  s_.bounded = s_.keep_small = 0;
+  // small cells: disjoint, none deeper than the steps
+  const uint32_t most = (uint32_t)std::min<uint64_t>((uint64_t)1 << ahead_, plan_.cap_small);
+  if (!plan_.needs.fourier) launch_small_dev(ahead_wide_ ? 1 : 0, most);
+  ENGINE_TRY(cudaGetLastError());
+  big_count_ = 0;
+  unsure_ = true;
+  ahead_ = 0;
+  return KDT_OK;
+}
+
 kdt_status Engine::tick() {
   // new roots join the lists of this tick
   bool has_roots = false;
@@ -435,18 +506,8 @@ kdt_status Engine::tick() {
     s_.ncells = big_count_;
     s_.ntiles = std::min(big_tiles_, plan_.max_tiles);
     s_.nseg = std::min(big_segs_, plan_.nseg_cap);
-    s_.few_segs = step_selects_all(s_.nseg, big_points_, plan_.sms) ? 1u : 0u;
-    // (not for shards: one segment of a shard's cell is a part of the cell's)
-    s_.wide_segs = !s_.shards && step_selects_wide(s_.nseg, big_points_) ? 1u : 0u;
-    const SelectTuning tune = current_tuning();
-    s_.tiny_max = tune.tiny_max;
-    s_.bitonic_max = tune.bitonic_max;
-    s_.warp_max = tune.warp_max;
-    launch_big_step(trees_, s_, s_.ntiles, s_.nseg, plan_.bigseg_cap, has_roots, root_dims_, plan_.needs.widest,
-                    plan_.needs.max_r, uniform_d(), tune, big_points_,
-                    plan_.grid_step, st_, plan_.needs.fourier);
+    launch_step(has_roots);
     ENGINE_TRY(cudaGetLastError());
-    root_dims_ = false;
     uint32_t w[W_COUNT];
     ENGINE_TRY(cudaMemcpyAsync(w, words_, sizeof(w), cudaMemcpyDeviceToHost, st_));
     ENGINE_TRY(cudaStreamSynchronize(st_));
@@ -459,19 +520,14 @@ kdt_status Engine::tick() {
       for (uint32_t k = 0; k < mt; ++k)
         if (stv[k]) std::fprintf(stderr, "kdt tick: slot %u status %d\n", k, stv[k]);
     }
-    const uint32_t* wb = w + W_BIG + 2 * (cur_ ^ 1);
-    const uint32_t* wt = w + W_TILE + 2 * (cur_ ^ 1);
-    big_count_ = std::min(wb[0], plan_.maxB);
-    big_segs_ = std::min(wb[1], plan_.nseg_cap);
-    big_tiles_ = std::min(wt[0], plan_.max_tiles);
-    big_points_ = wt[1];
+    cur_ ^= 1;
+    read_big(w);
     small_count_ = std::min(w[W_SMALL], plan_.cap_small);
     small_count_w_ = std::min(w[W_SMALL + 1], plan_.cap_small - small_count_);
     small_points_ = w[W_SMALLPTS];
-    cur_ ^= 1;
   }
   if (small_count_ > 0 || small_count_w_ > 0) {
-    launch_small(false);
+    launch_small();
     ENGINE_TRY(cudaGetLastError());
     small_count_ = small_count_w_ = 0;
     small_points_ = 0;
@@ -479,20 +535,20 @@ kdt_status Engine::tick() {
   return KDT_OK;
 }
 
-void Engine::launch_small(bool from_device) {
+// The queue with its counts on the device: the narrow (or tall) front, or the
+// wide back walked from the end; it holds at most `most` cells.
+void Engine::launch_small_dev(int wide, uint32_t most) {
+  const SubtreeShape& sh = wide ? kSubWide : plan_.needs.sub_tall ? kSubTall : kSubNarrow;
+  const uint32_t g = !wide && plan_.needs.sub_tall ? (uint32_t)plan_.needs.sub_tall : plan_.sms * (uint32_t)sh.ctas;
+  launch_subtree(sh, trees_, wide ? small_ + (plan_.cap_small - most) : small_, most, words_ + W_SMALL + wide, wide != 0,
+                 s_.small_off, words_ + W_HEAD, slices_, plan_.needs.slice_cells, std::min(g, most), 0, st_);
+}
+
+void Engine::launch_small() {
   const uint32_t cap = plan_.cap_small;
   const SubtreeShape& front = plan_.needs.sub_tall ? kSubTall : kSubNarrow;
   const uint32_t gn = plan_.needs.sub_tall ? (uint32_t)plan_.needs.sub_tall : plan_.sms * (uint32_t)front.ctas;
   const uint32_t gw = plan_.sms * (uint32_t)kSubWide.ctas;
-  if (from_device) {
-    // counts on the device (a recorded tick): the narrow front, then the wide
-    // back walked from the end
-    launch_subtree(front, trees_, small_, cap, words_ + W_SMALL, false, s_.small_off, words_ + W_HEAD, slices_,
-                   plan_.needs.slice_cells, gn, 0, st_);
-    launch_subtree(kSubWide, trees_, small_, cap, words_ + W_SMALL + 1, true, s_.small_off, words_ + W_HEAD, slices_,
-                   plan_.needs.slice_cells, gw, 0, st_);
-    return;
-  }
   const uint64_t pts = small_points_;
   if (small_count_ > 0)
     launch_subtree(front, trees_, small_, small_count_, nullptr, false, s_.small_off, words_ + W_HEAD, slices_,
@@ -543,21 +599,33 @@ kdt_status Engine::finalize(const std::vector<uint32_t>& slots, std::vector<kdt_
     sc.slots = slots_list_;
     ENGINE_TRY(cudaMemcpyAsync(slots_list_, list.data(), list.size() * 4, cudaMemcpyHostToDevice, st_));
   }
-  launch_finalize_many(trees_, sc, st_);
-  ENGINE_TRY(cudaGetLastError());
   bool any_sort = false;
   for (uint32_t s : slots) any_sort = any_sort || sorts_[s];
-  if (any_sort) {
-    launch_leaf_sort(trees_, sc, st_);
+  // the engine's words and, behind them in the plan, the slots'
+  const size_t lead = unsure_ ? (plan_.slot_words - plan_.words) / 4 : 0;
+  std::vector<uint32_t> words(lead + (size_t)S_COUNT * mt);
+  for (;;) {
+    launch_finalize_many(trees_, sc, st_);
     ENGINE_TRY(cudaGetLastError());
+    if (any_sort) {
+      launch_leaf_sort(trees_, sc, st_);
+      ENGINE_TRY(cudaGetLastError());
+    }
+    ENGINE_TRY(cudaMemcpyAsync(words.data(), slot_words_ - lead, words.size() * 4, cudaMemcpyDeviceToHost, st_));
+    ENGINE_TRY(cudaStreamSynchronize(st_));
+    if (!unsure_) break;
+    unsure_ = false;
+    read_big(words.data());
+    if (big_count_ == 0) break;
+    // cells are left (unequal halves): the kernels above did nothing yet
+    const kdt_status r = run_to_completion();
+    if (r != KDT_OK) return r;
   }
-  std::vector<uint32_t> words((size_t)S_COUNT * mt);
-  ENGINE_TRY(cudaMemcpyAsync(words.data(), slot_words_, words.size() * 4, cudaMemcpyDeviceToHost, st_));
-  ENGINE_TRY(cudaStreamSynchronize(st_));
-  const uint32_t* tc = words.data() + (size_t)S_TERM * mt;
-  const int32_t* st = (const int32_t*)words.data() + (size_t)S_STATUS * mt;
-  const int32_t* lv = (const int32_t*)words.data() + (size_t)S_LEVELS * mt;
-  const uint32_t* huge = words.data() + (size_t)S_HUGE * mt;
+  const uint32_t* sw = words.data() + lead;
+  const uint32_t* tc = sw + (size_t)S_TERM * mt;
+  const int32_t* st = (const int32_t*)sw + (size_t)S_STATUS * mt;
+  const int32_t* lv = (const int32_t*)sw + (size_t)S_LEVELS * mt;
+  const uint32_t* huge = sw + (size_t)S_HUGE * mt;
   for (uint32_t s : slots) {  // leaves too large for one CTA (shallow trees, cells that stop splitting)
     const TreeHost& h = host_[s];
     const uint32_t nh = std::min(huge[s], h.huge_cap);
@@ -596,7 +664,8 @@ kdt_status Engine::record_tick(int p) {
                   plan_.needs.max_r, uniform_d(), tune, 0,
                   plan_.grid_step, st_, plan_.needs.fourier);
   ENGINE_TRY(cudaGetLastError());
-  launch_small(true);
+  launch_small_dev(0, plan_.cap_small);
+  launch_small_dev(1, plan_.cap_small);
   ENGINE_TRY(cudaGetLastError());
   return KDT_OK;
 }
@@ -678,6 +747,7 @@ kdt_status Engine::run_graph() {
 }
 
 kdt_status Engine::run_to_completion() {
+  if (ahead_ > 0) return run_ahead();
   for (int guard = 0; busy() || !pending_.empty(); ++guard) {
     if (guard > 2 * KDT_MAX_LEVELS + 4) return KDT_ERR_CUDA;
     const kdt_status s = tick();

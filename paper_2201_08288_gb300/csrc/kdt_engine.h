@@ -31,6 +31,7 @@ struct TreePlan {
   int sid_bytes = 0;
   bool sub_wide = false;   // small cells run in the subtree kernel's wide shape
   int sub_tall = 0;        // > 0: in its tall shape, by at most this many CTAs
+  int steps = 0;           // level steps that have cells whatever the points are
   bool presorted = false;  // root split by the pipeline, reordered by subset first
   bool leafsort = false;   // subsets not in index order: leaves are sorted at the end
   uint64_t n = 0;
@@ -101,7 +102,9 @@ class Engine {
   // Offsets and sentinels of finished trees, then their status and L.
   kdt_status finalize(const std::vector<uint32_t>& slots, std::vector<kdt_status>* status,
                       std::vector<int32_t>* levels);
-  // Run ticks until nothing is left in flight.
+  // Run ticks until nothing is left in flight. (Of a forest of one tree, the
+  // steps that are sure to have cells are launched without waiting for any;
+  // finalize() looks whether they were all.)
   kdt_status run_to_completion();
   // The same with one graph launch: the first tick (new roots) from the
   // host, then every later tick inside a CUDA graph whose conditional while
@@ -131,11 +134,20 @@ class Engine {
   bool root_dims_ = false;
   bool debug_ = false;
   uint32_t graph_iters_ = 0;
+  int ahead_ = 0;            // the one tree's steps to launch without waiting
+  bool ahead_wide_ = false;  // its small cells run in the wide shape
+  bool unsure_ = false;      // launched so; cells may be left
+  // The launches of a step over the current list; s_ holds its counts.
+  void launch_step(bool has_roots);
+  kdt_status run_ahead();
+  // What the device's words say of the current list.
+  void read_big(const uint32_t* words);
   // Record a tick over cell list p into the stream's capture (counts on the device).
   kdt_status record_tick(int p);
-  // The subtree kernel over the small-cell queue: the narrow shape over its
-  // front, the wide one over its back (host counts, or the device's).
-  void launch_small(bool from_device);
+  // The subtree kernel over the small-cell queue: the narrow (or tall) shape
+  // over its front, the wide one over its back (host counts, or the device's).
+  void launch_small();
+  void launch_small_dev(int wide, uint32_t most);
   // Admitted trees whose records are not on the device yet, and the list
   // their root goes to.
   enum List { kListNone, kListBig, kListSmall, kListSmallWide };

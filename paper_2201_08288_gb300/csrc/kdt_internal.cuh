@@ -125,10 +125,11 @@ struct TermRec {
 struct StepDev {
   const Cell* cells;      // big cells of this step
   uint32_t ncells;              // cells of this step (steps driven by the host)
-  const uint32_t* ncells_dev;   // if set: the device word that holds it (steps inside a graph)
+  const uint32_t* ncells_dev;   // if set: the device word that holds it (steps inside a graph, steps ahead)
   uint32_t ntiles, nseg;        // tiles and segments of this step, or the device words:
   const uint32_t* ntiles_dev;
   const uint32_t* nseg_dev;
+  uint32_t bounded;             // the words' values are at most ncells, ntiles and nseg, and seldom much less
   uint32_t tiles_cap, nseg_cap;
   uint2* tiles;           // [ntiles] (cell, offset within cell)
   uint32_t* kdim;         // [ncells] key coordinate
@@ -161,6 +162,7 @@ struct StepDev {
   uint32_t next_big_cap;
   uint32_t small_cap;
   uint32_t init_small, init_small_w, init_small_points;  // the queue's contents when the step starts
+  uint32_t keep_small;        // or what the step before left in it
   uint32_t* small_points;     // points appended to small
   // subset offsets (relative to the cell's begin, r+1 per cell) of this
   // step's cells: rows of off_cur at obase_cur[c]; level-0 cells use their

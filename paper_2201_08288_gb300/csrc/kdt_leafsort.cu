@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kLsThreads, 5) k_leaf_sort(const TreeDev* tree
   __shared__ LsShared S;
   uint32_t chunk, chunks;
   const TreeDev& t = trees[pick_chunk(sc, &chunk, &chunks)];
-  if (!t.leafsort || *t.status != ST_OK) return;
+  if (!t.leafsort || *t.status != ST_OK || *t.live > 0) return;
   const uint32_t nrec = min(*t.term_count, t.term_cap);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t wstride = chunks * kLsWarps;

@@ -386,8 +386,8 @@ kdt_status sharded_build(const float* points, const kdt_params& p, int32_t G, ui
   off += sh_align((size_t)G * 4);
   const size_t o_base = off;
   off += sh_align((size_t)G * 4);
-  const size_t o_words = off;  // split status, merge status, term count, huge count
-  off += sh_align(16);
+  const size_t o_words = off;  // split status, merge status, term count, huge count, the merged tree's cells left (0)
+  off += sh_align(20);
   DevMem small;
   if (dev_malloc(&small.p, off) != cudaSuccess) {
     (void)cudaGetLastError();
@@ -411,7 +411,7 @@ kdt_status sharded_build(const float* points, const kdt_params& p, int32_t G, ui
   a.ntot = (uint32_t*)(sm + o_ntot);
   a.base = (const uint32_t*)(sm + o_base);
   a.status = words;
-  SH_TRY(cudaMemsetAsync(words, 0, 16, st));
+  SH_TRY(cudaMemsetAsync(words, 0, 20, st));
   SH_TRY(cudaMemsetAsync(a.ntot, 0, (size_t)G * 4, st));
   if (ntiles) {
     TraceScope ts(K_SHARD_SPLIT, st, (uint64_t)n);
@@ -559,6 +559,7 @@ kdt_status sharded_build(const float* points, const kdt_params& p, int32_t G, ui
   td.huge_cap = nl;
   td.leafsort = 1;
   td.status = words + 1;
+  td.live = words + 4;
   TreeDev* td_dev = (TreeDev*)(ws + o_td);
   SH_TRY(cudaMemcpyAsync(td_dev, &td, sizeof td, cudaMemcpyHostToDevice, st));
   launch_leaf_sort(td_dev, SlotChunks{nullptr, 1, std::min<uint32_t>((nl + 63) / 64, 2048u)}, st);

@@ -551,9 +551,11 @@ __global__ void __launch_bounds__(256) k_cells(const TreeDev* trees, StepDev s, 
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *s.next_big_ctr = 0ull;
     *s.next_tile_ctr = 0ull;
-    *s.small_ctr = (unsigned long long)s.init_small | ((unsigned long long)s.init_small_w << 32);
-    *s.small_points = s.init_small_points;
-    *s.small_off_used = 0;
+    if (!s.keep_small) {
+      *s.small_ctr = (unsigned long long)s.init_small | ((unsigned long long)s.init_small_w << 32);
+      *s.small_points = s.init_small_points;
+      *s.small_off_used = 0;
+    }
     *s.bigseg_count_next = 0;
     *s.midseg_count_next = 0;
   }
@@ -900,6 +902,7 @@ constexpr int kWideThreads = 512;
 
 __device__ __forceinline__ bool wide_segment(const TreeDev* trees, const StepDev& s, uint32_t* g, uint32_t* w,
                                              uint32_t** words) {
+  if (blockIdx.z >= ncells_of(s)) return false;  // a step ahead: fewer cells than its launches allow for
   const Cell cell = s.cells[blockIdx.z];
   const TreeDev& t = trees[cell.tree];
   if (blockIdx.y >= (uint32_t)t.r || !wide_cell(t, cell)) return false;
@@ -1770,7 +1773,7 @@ bool step_selects_wide(uint32_t nseg, uint64_t points) { return nseg <= 32u && p
 // CTAs fit the SMs at once (4 each) and a cell has at most 64 tiles on average
 // (a warp reads 4).
 static bool step_splits(const StepDev& s, uint32_t sms2) {
-  return !s.ncells_dev && s.ncells <= 2u * sms2 && s.ntiles <= 64u * s.ncells;
+  return (!s.ncells_dev || s.bounded) && s.ncells <= 2u * sms2 && s.ntiles <= 64u * s.ncells;
 }
 
 // The selects by segment size: one thread, one warp, one CTA per segment.
@@ -1875,12 +1878,12 @@ cudaError_t prepare_step_kernels() {
 void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t nseg,
                      uint32_t max_bigseg, bool has_roots, bool need_root_dims, bool any_widest, int max_r, int uniform_d,
                      const SelectTuning& tune, uint64_t points, uint32_t sms, cudaStream_t st, bool fourier) {
-  // s.ncells: the step's cells, or (s.ncells_dev set: a step inside a graph)
-  // their capacity; per-cell kernels stride over the cells, so their grids
-  // cover the cells exactly here and are capped there
+  // s.ncells: the step's cells, or at most so many (s.bounded), or (a step inside
+  // a graph) their capacity; per-cell kernels stride over the cells, so their
+  // grids cover the cells exactly in the first two and are capped in the last
   const uint32_t nc = s.ncells;
   if (nc == 0) return;
-  const bool dev = s.ncells_dev != nullptr;
+  const bool dev = s.ncells_dev != nullptr && !s.bounded;
   auto cells_grid = [&](uint32_t per_block, uint32_t cap) {
     const uint32_t g = (nc + per_block - 1) / per_block;
     return std::max<uint32_t>(1, dev ? std::min(g, cap) : g);

@@ -884,11 +884,12 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
 
 // One warp per terminal cell: offsets of the leaves at level L below it and
 // sentinels (dim -1, value +inf) on its own node and every node below it.
-// Trees that failed are left as they are.
+// Trees that failed, or have cells left (their steps were launched ahead and
+// were too few), are left as they are.
 __global__ void k_finalize(const TreeDev* trees, SlotChunks sc) {
   uint32_t chunk, chunks;
   const TreeDev& t = trees[pick_chunk(sc, &chunk, &chunks)];
-  if (*t.status != ST_OK) return;
+  if (*t.status != ST_OK || *t.live > 0) return;
   const uint32_t nrec = min(*t.term_count, t.term_cap);
   const int L = t.depth > 0 ? t.depth : *t.levels;
   const int lane = threadIdx.x & 31;
@@ -946,7 +947,7 @@ void launch_subtree(const SubtreeShape& sh, const TreeDev* trees, const Cell* li
                     const uint32_t* count_dev, bool reversed, const uint32_t* small_off, uint32_t* head,
                     LCell* slices, uint32_t slice_cells, uint32_t grid, uint64_t points, cudaStream_t st) {
   if (count == 0 || grid == 0) return;
-  if (!count_dev && grid >= count)
+  if (grid >= count)
     head = nullptr;  // a CTA per cell: nothing to hand out
   else
     cudaMemsetAsync(head, 0, sizeof(uint32_t), st);
