@@ -253,6 +253,13 @@ __device__ __forceinline__ uint32_t subset_of(const TreeDev& t, uint32_t orig) {
   return s;
 }
 
+// The first statement of a kernel that launch_chained launches: every thread
+// waits until the kernel before it in the stream has ended and its writes are
+// visible.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Terminal test for a cell about to be processed at `level` (reading R8 in
 // leaf mode; empty cells and the last level in depth mode).
 // Cells of a step: the host's count, or the device word a graph-driven step

@@ -230,6 +230,7 @@ __device__ __noinline__ bool block_bucket_slice(uint32_t* a, uint32_t m, LsShare
 // tree, want the warps; the CTA paths, calls, spill (2^20 leaves of 128 points:
 // 0.75 ms; 0.78 with the bucket path inlined).
 __global__ void __launch_bounds__(kLsThreads, 5) k_leaf_sort(const TreeDev* trees, SlotChunks sc) {
+  chain_wait();
   __shared__ LsShared S;
   uint32_t chunk, chunks;
   const TreeDev& t = trees[pick_chunk(sc, &chunk, &chunks)];
@@ -437,7 +438,7 @@ __global__ void k_leaf_copy(const uint32_t* src, uint32_t* dst, const LeafTile* 
 
 void launch_leaf_sort(const TreeDev* trees, const SlotChunks& sc, cudaStream_t st) {
   TraceScope ts(K_LEAF_SORT, st);
-  k_leaf_sort<<<sc.chunks, kLsThreads, 0, st>>>(trees, sc);
+  launch_chained(k_leaf_sort, sc.chunks, kLsThreads, 0, st, trees, sc);
 }
 
 size_t leaf_huge_tiles_cap(uint64_t n) { return (size_t)(2 * (n / kLeafBlockMax) + 2); }

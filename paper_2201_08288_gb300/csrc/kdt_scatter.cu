@@ -98,6 +98,7 @@ struct SubMeta {
 // kD = 0: any d. kMM: some tree of the step uses widest spread.
 template <int kD, bool kMM>
 __global__ void __launch_bounds__(kST, scatter_ctas(kD, kMM)) k_scatter_tma(const TreeDev* trees, StepDev s) {
+  chain_wait();
   constexpr int kMaxItems = kD > 0 ? (int)(sub_tile(kD > 0 ? kD : 1) / kCT) : 4;  // points per consumer thread
   // words of a buffer (kD = 0: trees of several d may follow one another, so
   // the halves are fixed)
@@ -548,7 +549,7 @@ template <int kD, bool kMM>
 void launch_one(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint32_t sms, cudaStream_t st) {
   // two waves of resident CTAs, each taking a contiguous range of tiles
   const uint32_t grid = std::max<uint32_t>(1, std::min(max_tiles, sms * 2u * (uint32_t)scatter_ctas(kD, kMM)));
-  k_scatter_tma<kD, kMM><<<grid, kST, scatter_smem(kD), st>>>(trees, s);
+  launch_chained(k_scatter_tma<kD, kMM>, grid, kST, scatter_smem(kD), st, trees, s);
 }
 
 // f(instance) for the trees' coordinate count: compiled for 1 to 8, 12 and 16.

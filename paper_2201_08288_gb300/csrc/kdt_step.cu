@@ -75,6 +75,7 @@ __device__ __forceinline__ void tiles_cell(const TreeDev* trees, const StepDev& 
 }
 
 __global__ void k_tiles(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t nc = ncells_of(s);
   const uint32_t wpb = blockDim.x >> 5;
   for (uint32_t c = blockIdx.x * wpb + (threadIdx.x >> 5); c < nc; c += gridDim.x * wpb) tiles_cell(trees, s, c);
@@ -94,6 +95,7 @@ __device__ __forceinline__ bool presort_tile(const TreeDev* trees, const StepDev
 // to the root's totals (root_cur) when the range moves to another tree and at
 // its end.
 __global__ void __launch_bounds__(kTileThreads) k_ps_count(const TreeDev* trees, StepDev s) {
+  chain_wait();
   __shared__ uint32_t hist[kMaxSubsets];
   const uint32_t ntiles = ntiles_of(s);
   const uint32_t t_begin = (uint32_t)(((uint64_t)blockIdx.x * ntiles) / gridDim.x);
@@ -170,6 +172,7 @@ __device__ __forceinline__ void ps_offsets_cell(const TreeDev* trees, const Step
 }
 
 __global__ void k_ps_offsets(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t nc = ncells_of(s);
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
     ps_offsets_cell(trees, s, c);
@@ -192,6 +195,7 @@ __global__ void k_ps_offsets(const TreeDev* trees, StepDev s) {
 // themselves; the empty places only cost (2^27 points in 8: 3.25 ms against
 // 2.91).
 __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, StepDev s) {
+  chain_wait();
   uint2 tl;
   Cell cell;
   if (!presort_tile(trees, s, blockIdx.x, &tl, &cell)) return;
@@ -331,6 +335,7 @@ __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, St
 // Per tile and coordinate of a cell whose key coordinate is not known yet
 // (the root): min and max key, reduced per cell by k_pick_dim.
 __global__ void __launch_bounds__(kTileThreads) k_minmax(const TreeDev* trees, StepDev s) {
+  chain_wait();
   uint2 tl;
   if (!tile_of(s, blockIdx.x, &tl)) return;
   const Cell cell = s.cells[tl.x];
@@ -455,6 +460,7 @@ __device__ __forceinline__ void pick_dim_cell(const TreeDev* trees, const StepDe
 }
 
 __global__ void __launch_bounds__(1024) k_pick_dim(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t nc = ncells_of(s);
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
     pick_dim_cell(trees, s, c);
@@ -548,6 +554,7 @@ __device__ __forceinline__ void open_cell(const TreeDev* trees, const StepDev& s
 // them a single CTA: 135 us for the six steps of a build of 65,536 points, 50
 // now.)
 __global__ void __launch_bounds__(256) k_cells(const TreeDev* trees, StepDev s, uint32_t gt) {
+  chain_wait();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *s.next_big_ctr = 0ull;
     *s.next_tile_ctr = 0ull;
@@ -620,6 +627,7 @@ __device__ __forceinline__ uint32_t thread_lower_median(const uint32_t* keys, ui
 // networks in registers does (they spill about 300 bytes per thread to local
 // memory; measured faster than four or six CTAs per SM).
 __global__ void __launch_bounds__(256, 5) k_select_tiny(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t nseg = nseg_of(s);
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t stride = gridDim.x * blockDim.x;
@@ -724,6 +732,7 @@ __device__ uint32_t warp_select_stream(const uint32_t* keys, uint32_t w, uint32_
 // memory for a radix select; larger segments read from global memory on every
 // pass.
 __global__ void __launch_bounds__(256) k_select_small(const TreeDev* trees, StepDev s) {
+  chain_wait();
   __shared__ uint32_t hist[8][256];
   __shared__ uint32_t stage[8][1024];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -871,6 +880,7 @@ __device__ __forceinline__ uint32_t cta_lower_median(const uint32_t* keys, uint3
 // CTAs stride over the listed segments above the warp-select size.
 template <int kThreads, int kBits>
 __global__ void __launch_bounds__(kThreads) k_select_big(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t cnt = min(*s.bigseg_count, s.bigseg_cap);
   for (uint32_t jb = blockIdx.x; jb < cnt; jb += gridDim.x) {
     const uint32_t g = s.bigseg[jb];
@@ -882,6 +892,7 @@ __global__ void __launch_bounds__(kThreads) k_select_big(const TreeDev* trees, S
 // Steps of few segments: a CTA for every one of them, whatever its size, in
 // one launch instead of three.
 __global__ void __launch_bounds__(256) k_select_all(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t nseg = nseg_of(s);
   for (uint32_t g = blockIdx.x; g < nseg; g += gridDim.x) {
     const uint32_t w = s.seg_w[g];
@@ -913,12 +924,14 @@ __device__ __forceinline__ bool wide_segment(const TreeDev* trees, const StepDev
 }
 
 __global__ void __launch_bounds__(kWideThreads) k_wide_clear(const TreeDev* trees, StepDev s) {
+  chain_wait();
   uint32_t g, w, *H;
   if (!wide_segment(trees, s, &g, &w, &H)) return;
   for (uint32_t i = threadIdx.x; i < kWideWords; i += kWideThreads) H[i] = i == kWideBins + 1u ? (w - 1u) / 2u : 0u;
 }
 
 __global__ void __launch_bounds__(kWideThreads) k_wide_pass(const TreeDev* trees, StepDev s, int top) {
+  chain_wait();
   __shared__ uint32_t hist[kWideBins];
   __shared__ uint32_t tmp[33];
   __shared__ bool last;
@@ -1028,6 +1041,7 @@ __device__ __forceinline__ void combine_cell(const TreeDev* trees, const StepDev
 }
 
 __global__ void __launch_bounds__(256) k_combine(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t nc = ncells_of(s);
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
     combine_cell(trees, s, c);
@@ -1064,6 +1078,7 @@ __device__ __forceinline__ void combine_warp_cell(const TreeDev* trees, const St
 }
 
 __global__ void __launch_bounds__(256, 1) k_combine_warp(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t nc = ncells_of(s);
   for (uint32_t c = blockIdx.x * 8u + (threadIdx.x >> 5); c < nc; c += gridDim.x * 8u) combine_warp_cell(trees, s, c);
 }
@@ -1088,6 +1103,7 @@ static_assert(kFourierTerms * 2 <= kTileRecWords, "a tile's sums fit its record"
 // records in order, so the result does not depend on scheduling. A
 // coordinate outside (0,1) is reported.
 __global__ void __launch_bounds__(256, 2) k_fourier_moments(const TreeDev* trees, StepDev s) {
+  chain_wait();
   constexpr int kPer = kTile / 256;
   __shared__ float red[8][kFourierTerms];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1256,6 +1272,7 @@ __device__ __forceinline__ double widen(float x) {
 }
 
 __global__ void __launch_bounds__(kFsThreads) k_fourier_split(const TreeDev* trees, StepDev s, uint32_t mgrid) {
+  chain_wait();
   __shared__ double rec[kFsChunk][kFourierTerms];
   __shared__ double s_base[kFourierTerms], s_slope[kFourierTerms];
   __shared__ double s_wave[4][KDT_FOURIER_MAX_J];  // sin K a, sin K b, cos K a, cos K b
@@ -1489,6 +1506,7 @@ __device__ __forceinline__ void part_count_tile(const TreeDev* trees, const Step
 // registers: a lane's sixteen 16-byte loads still fit, with a few words of
 // spill).
 __global__ void __launch_bounds__(256, 3) k_part_count(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t ntiles = ntiles_of(s);
   for (uint32_t tile = blockIdx.x * 8u + (threadIdx.x >> 5); tile < ntiles; tile += gridDim.x * 8u)
     part_count_tile(trees, s, tile, s.tiles[tile]);
@@ -1511,6 +1529,7 @@ __device__ __forceinline__ void part_scan_cell(const StepDev& s, uint32_t c, con
 }
 
 __global__ void k_part_scan(StepDev s) {
+  chain_wait();
   const uint32_t nc = ncells_of(s);
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
     part_scan_cell(s, c, s.cells[c]);
@@ -1560,6 +1579,7 @@ __device__ __forceinline__ void child_dims_cell(const TreeDev* trees, const Step
 }
 
 __global__ void __launch_bounds__(256, 1) k_child_dims(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const uint32_t nc = ncells_of(s);
   for (uint32_t c = blockIdx.x * 8u + (threadIdx.x >> 5); c < nc; c += gridDim.x * 8u) child_dims_cell(trees, s, c);
 }
@@ -1700,6 +1720,7 @@ __device__ __forceinline__ void clear_child_mm(const TreeDev* trees, const StepD
 // 32 cells per CTA: the left counts of each cell's tiles are scanned by a warp
 // (unless k_part_scan did), then one warp classifies the 32 together.
 __global__ void __launch_bounds__(256) k_classify(const TreeDev* trees, StepDev s, bool scanned) {
+  chain_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t nc = ncells_of(s);
   for (uint32_t c0 = blockIdx.x * 32u; c0 < nc; c0 += gridDim.x * 32u) {
@@ -1729,6 +1750,7 @@ __global__ void __launch_bounds__(256) k_classify(const TreeDev* trees, StepDev 
 // subsets: 75 us for the six steps of a build, 183 in four launches each).
 constexpr int kSplitThreads = 512;
 __global__ void __launch_bounds__(kSplitThreads) k_split(const TreeDev* trees, StepDev s) {
+  chain_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t nc = ncells_of(s);
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
@@ -1782,11 +1804,13 @@ static void launch_listed_selects(const TreeDev* trees, const StepDev& s, uint32
                                   cudaStream_t st) {
   {
     TraceScope ts(K_SELECT_TINY, st, points);
-    k_select_tiny<<<std::max<uint32_t>(1, std::min<uint32_t>((nseg + 255) / 256, sms * 16u)), 256, 0, st>>>(trees, s);
+    launch_chained(k_select_tiny, std::max<uint32_t>(1, std::min<uint32_t>((nseg + 255) / 256, sms * 16u)), 256, 0, st,
+                   trees, s);
   }
   {
     TraceScope ts(K_SELECT_SMALL, st, points);
-    k_select_small<<<std::max<uint32_t>(1, std::min<uint32_t>((nseg + 7) / 8, sms * 8u)), 256, 0, st>>>(trees, s);
+    launch_chained(k_select_small, std::max<uint32_t>(1, std::min<uint32_t>((nseg + 7) / 8, sms * 8u)), 256, 0, st,
+                   trees, s);
   }
   if (max_bigseg == 0) return;
   if (s.wide_segs) {
@@ -1794,10 +1818,13 @@ static void launch_listed_selects(const TreeDev* trees, const StepDev& s, uint32
     const uint32_t x = std::max<uint32_t>(
         1, (uint32_t)std::min<uint64_t>(2u * sms / std::max(1u, nseg), points / std::max(1u, nseg) / 8192u));
     const uint32_t y = std::min(max_r, nseg - std::min(nseg, s.ncells) + 1u);  // every cell has a segment
-    { TraceScope ts(K_SELECT_WIDE, st); k_wide_clear<<<dim3(1, y, s.ncells), kWideThreads, 0, st>>>(trees, s); }
+    {
+      TraceScope ts(K_SELECT_WIDE, st);
+      launch_chained(k_wide_clear, dim3(1, y, s.ncells), kWideThreads, 0, st, trees, s);
+    }
     for (int top = 32; top > 0; top -= 11) {
       TraceScope ts(K_SELECT_WIDE, st, points);
-      k_wide_pass<<<dim3(x, y, s.ncells), kWideThreads, 0, st>>>(trees, s, top);
+      launch_chained(k_wide_pass, dim3(x, y, s.ncells), kWideThreads, 0, st, trees, s, top);
     }
   }
   TraceScope ts(K_SELECT_BIG, st);
@@ -1807,14 +1834,14 @@ static void launch_listed_selects(const TreeDev* trees, const StepDev& s, uint32
   const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>(std::min(max_bigseg, nseg), sms * 4u));
   if (tune.cta_threads == 512 || nseg <= sms * 4u) {
     if (tune.digit_bits == 8)
-      k_select_big<512, 8><<<grid, 512, 0, st>>>(trees, s);
+      launch_chained(k_select_big<512, 8>, grid, 512, 0, st, trees, s);
     else
-      k_select_big<512, 11><<<grid, 512, 0, st>>>(trees, s);
+      launch_chained(k_select_big<512, 11>, grid, 512, 0, st, trees, s);
   } else {
     if (tune.digit_bits == 8)
-      k_select_big<256, 8><<<grid, 256, 0, st>>>(trees, s);
+      launch_chained(k_select_big<256, 8>, grid, 256, 0, st, trees, s);
     else
-      k_select_big<256, 11><<<grid, 256, 0, st>>>(trees, s);
+      launch_chained(k_select_big<256, 11>, grid, 256, 0, st, trees, s);
   }
 }
 
@@ -1841,11 +1868,13 @@ __device__ __forceinline__ void admit_tree(const AdmitRec& a, TreeDev* trees) {
 }
 
 __global__ void __launch_bounds__(256) k_admit(const AdmitRec* recs, TreeDev* trees) {
+  chain_wait();
   admit_tree(recs[blockIdx.x], trees);
 }
 
 // The same with the records among the launch's parameters (no copy before it).
 __global__ void __launch_bounds__(256) k_admit_few(const __grid_constant__ AdmitFew few, TreeDev* trees) {
+  chain_wait();
   admit_tree(few.rec[blockIdx.x], trees);
 }
 
@@ -1857,13 +1886,13 @@ cudaError_t launch_admit(const std::vector<AdmitRec>& recs, AdmitRec* staging, T
     AdmitFew few{};
     std::copy(recs.begin(), recs.end(), few.rec);
     TraceScope ts(K_ADMIT, st);
-    k_admit_few<<<(unsigned)recs.size(), 256, 0, st>>>(few, trees);
+    launch_chained(k_admit_few, (unsigned)recs.size(), 256, 0, st, few, trees);
   } else {
     const cudaError_t e =
         cudaMemcpyAsync(staging, recs.data(), recs.size() * sizeof(AdmitRec), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
     TraceScope ts(K_ADMIT, st);
-    k_admit<<<(unsigned)recs.size(), 256, 0, st>>>(staging, trees);
+    launch_chained(k_admit, (unsigned)recs.size(), 256, 0, st, staging, trees);
   }
   for (const AdmitRec& a : recs)
     if (a.terminal && a.tree.n > (int64_t)kAdmitIota) launch_iota(a.tree.out_perm, (uint32_t)a.tree.n, st);
@@ -1890,17 +1919,20 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
   };
   if (s.shards) launch_shard_index(s, nc, st);
   if (has_roots) {
-    { TraceScope ts(K_TILES, st); k_tiles<<<cells_grid(8, sms * 8u), 256, 0, st>>>(trees, s); }
+    { TraceScope ts(K_TILES, st); launch_chained(k_tiles, cells_grid(8, sms * 8u), 256, 0, st, trees, s); }
     {
       TraceScope ts(K_PS_COUNT, st, points);
-      k_ps_count<<<std::max<uint32_t>(1, std::min(max_tiles, sms * 4u)), kTileThreads, 0, st>>>(trees, s);
+      launch_chained(k_ps_count, std::max<uint32_t>(1, std::min(max_tiles, sms * 4u)), kTileThreads, 0, st, trees, s);
     }
-    { TraceScope ts(K_PS_OFFSETS, st); k_ps_offsets<<<nc, 1024, 0, st>>>(trees, s); }
-    { TraceScope ts(K_PS_MOVE, st, points); k_ps_move<<<max_tiles, kPsThreads, ps_smem_bytes((uint32_t)max_r), st>>>(trees, s); }
+    { TraceScope ts(K_PS_OFFSETS, st); launch_chained(k_ps_offsets, nc, 1024, 0, st, trees, s); }
+    {
+      TraceScope ts(K_PS_MOVE, st, points);
+      launch_chained(k_ps_move, max_tiles, kPsThreads, ps_smem_bytes((uint32_t)max_r), st, trees, s);
+    }
   }
   if (need_root_dims) {
-    { TraceScope ts(K_MINMAX, st, points); k_minmax<<<max_tiles, kTileThreads, 0, st>>>(trees, s); }
-    { TraceScope ts(K_PICK_DIM, st); k_pick_dim<<<nc, 1024, 0, st>>>(trees, s); }
+    { TraceScope ts(K_MINMAX, st, points); launch_chained(k_minmax, max_tiles, kTileThreads, 0, st, trees, s); }
+    { TraceScope ts(K_PICK_DIM, st); launch_chained(k_pick_dim, nc, 1024, 0, st, trees, s); }
   }
   {
     // threads per cell: enough for its segments
@@ -1908,7 +1940,7 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
     while (gt < 256u && gt < (uint32_t)max_r) gt *= 2;
     if (!dev && nc < sms) gt = 256;  // few cells: their tiles count
     TraceScope ts(K_CELLS, st);
-    k_cells<<<cells_grid(256u / gt, sms * 8u), 256, 0, st>>>(trees, s, gt);
+    launch_chained(k_cells, cells_grid(256u / gt, sms * 8u), 256, 0, st, trees, s, gt);
   }
   // a CTA per cell while cells are few (large subset counts, deep scans),
   // a warp per cell once they are many (and in a graph, where the count is
@@ -1919,13 +1951,16 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
     const uint32_t mgrid = std::max<uint32_t>(1, std::min(max_tiles, sms * 2u));
     {
       TraceScope ts(K_FOURIER_MOMENTS, st, points);
-      k_fourier_moments<<<mgrid, 256, 0, st>>>(trees, s);
+      launch_chained(k_fourier_moments, mgrid, 256, 0, st, trees, s);
     }
-    { TraceScope ts(K_FOURIER_SPLIT, st); k_fourier_split<<<cells_grid(1, sms * 4u), kFsThreads, 0, st>>>(trees, s, mgrid); }
+    {
+      TraceScope ts(K_FOURIER_SPLIT, st);
+      launch_chained(k_fourier_split, cells_grid(1, sms * 4u), kFsThreads, 0, st, trees, s, mgrid);
+    }
   } else {
     if (s.few_segs) {
       TraceScope ts(K_SELECT_ALL, st, points);
-      k_select_all<<<std::max<uint32_t>(1, nseg), 256, 0, st>>>(trees, s);
+      launch_chained(k_select_all, std::max<uint32_t>(1, nseg), 256, 0, st, trees, s);
     } else {
       launch_listed_selects(trees, s, nseg, (uint32_t)max_r, max_bigseg, tune, points, sms, st);
     }
@@ -1933,32 +1968,36 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
     if (!split) {
       TraceScope ts(K_COMBINE, st);
       if (many)
-        k_combine_warp<<<cells_grid(8, sms * 8u), 256, 0, st>>>(trees, s);
+        launch_chained(k_combine_warp, cells_grid(8, sms * 8u), 256, 0, st, trees, s);
       else
-        k_combine<<<nc, 256, 0, st>>>(trees, s);
+        launch_chained(k_combine, nc, 256, 0, st, trees, s);
     }
   }
   if (split) {
     TraceScope ts(K_SPLIT, st, points);
-    k_split<<<nc, kSplitThreads, 0, st>>>(trees, s);
+    launch_chained(k_split, nc, kSplitThreads, 0, st, trees, s);
   } else {
     {
       TraceScope ts(K_PART_COUNT, st, points);
-      k_part_count<<<std::max<uint32_t>(1, std::min((max_tiles + 7) / 8, sms * 16u)), 256, 0, st>>>(trees, s);
+      launch_chained(k_part_count, std::max<uint32_t>(1, std::min((max_tiles + 7) / 8, sms * 16u)), 256, 0, st, trees,
+                     s);
     }
     // a cell of very many tiles: a CTA scans them, not a warp
     const bool scanned = !dev && max_tiles / nc > 64u;
     if (scanned) {
       TraceScope ts(K_PART_SCAN, st);
-      k_part_scan<<<nc, 1024, 0, st>>>(s);
+      launch_chained(k_part_scan, nc, 1024, 0, st, s);
     }
-    { TraceScope ts(K_CLASSIFY, st); k_classify<<<cells_grid(32, sms * 4u), 256, 0, st>>>(trees, s, scanned); }
+    {
+      TraceScope ts(K_CLASSIFY, st);
+      launch_chained(k_classify, cells_grid(32, sms * 4u), 256, 0, st, trees, s, scanned);
+    }
   }
   launch_scatter(trees, s, max_tiles, sms / 2, points, uniform_d, any_widest, st);
   if (any_widest && s.shards) launch_shard_minmax(trees, s, nc, st);
   if (any_widest) {
     TraceScope ts(K_CHILD_DIMS, st);
-    k_child_dims<<<cells_grid(8, sms * 8u), 256, 0, st>>>(trees, s);
+    launch_chained(k_child_dims, cells_grid(8, sms * 8u), 256, 0, st, trees, s);
   }
 }
 

@@ -241,6 +241,7 @@ template <int kShape>
 __global__ void __launch_bounds__(kShapes[kShape].threads, kShapes[kShape].ctas)
 k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t* count_dev, uint32_t reversed,
           const uint32_t* small_off, uint32_t* head, LCell* slices, uint32_t slice_cells, uint32_t probe_tries) {
+  chain_wait();
   constexpr SubtreeShape kSh = kShapes[kShape];
   constexpr int T = kSh.threads, NW = T / 32, kQ = kSh.q, kCells = kSh.cells;
   extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -887,6 +888,7 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
 // Trees that failed, or have cells left (their steps were launched ahead and
 // were too few), are left as they are.
 __global__ void k_finalize(const TreeDev* trees, SlotChunks sc) {
+  chain_wait();
   uint32_t chunk, chunks;
   const TreeDev& t = trees[pick_chunk(sc, &chunk, &chunks)];
   if (*t.status != ST_OK || *t.live > 0) return;
@@ -953,13 +955,13 @@ void launch_subtree(const SubtreeShape& sh, const TreeDev* trees, const Cell* li
     cudaMemsetAsync(head, 0, sizeof(uint32_t), st);
   const uint32_t probe = fault_take(KDT_FAULT_WAIT) ? 1024u : 0u;
   TraceScope ts(K_SUBTREE, st, points);
-  subtree_kernel(sh)<<<grid, sh.threads, sh.smem, st>>>(trees, list, count, count_dev, reversed ? 1u : 0u, small_off,
-                                               head, slices, slice_cells, probe);
+  launch_chained(subtree_kernel(sh), grid, sh.threads, sh.smem, st, trees, list, count, count_dev, reversed ? 1u : 0u,
+                 small_off, head, slices, slice_cells, probe);
 }
 
 void launch_finalize_many(const TreeDev* trees, const SlotChunks& sc, cudaStream_t st) {
   TraceScope ts(K_FINALIZE, st);
-  k_finalize<<<sc.chunks, 256, 0, st>>>(trees, sc);
+  launch_chained(k_finalize, sc.chunks, 256, 0, st, trees, sc);
 }
 
 }  // namespace kdt
