@@ -119,8 +119,8 @@ typedef struct kdt_params {
 
 /*
  * Bytes of device workspace kdt_build needs for these parameters on the
- * current device. The workspace holds two ping-pong copies of the points,
- * permutation and subset ids, a key scratch array and per-level tables.
+ * current device. The workspace holds two ping-pong copies of the points and
+ * the permutation, and per-level tables.
  * Errors: KDT_ERR_INVALID_ARG.
  */
 kdt_status kdt_workspace_size(const kdt_params *p, size_t *bytes);
@@ -253,15 +253,16 @@ kdt_status kdt_server_destroy(kdt_server *s);
  * The lower median of every (cell, subset) segment (paper, Sec. 2: the
  * medians computed independently on the r subsets) takes one of four paths by
  * the segment's size: one thread sorting it in registers; one warp with a
- * bitonic network; one warp with a radix select; one CTA with a radix select.
+ * bitonic network; one warp by brackets from a sample; one CTA with a radix
+ * select.
  * Where the paths change, the CTA's size and the width of its radix digits
  * are tunable. Every choice gives the same outputs, bit for bit: the choices
  * trade only speed, and kdt_autotune times them on the caller's own trees.
  */
 typedef struct kdt_tuning {
   int32_t tiny_max;     /* one thread per segment up to this many keys: 8 to 64 (x2)   */
-  int32_t bitonic_max;  /* a warp's bitonic network up to this many: 64, 128 or 256    */
-  int32_t warp_max;     /* a warp's radix select up to this many: 1024, 2048 or 4096   */
+  int32_t bitonic_max;  /* a warp's network up to this many: 64, 128 or 256 (as 128)   */
+  int32_t warp_max;     /* a warp's brackets up to this many: 1024, 2048 or 4096       */
   int32_t cta_threads;  /* threads of the CTA radix select: 256 or 512                 */
   int32_t digit_bits;   /* digit width of the CTA radix select: 8 (4 passes) or 11 (3) */
   int32_t reserved[3];  /* zero                                                        */
@@ -363,7 +364,7 @@ kdt_status kdt_build_sharded(const float *points, const kdt_params *p, int32_t s
  * region can reach are visited. The tree is a build's output: points (device,
  * float32 SoA [d][n], the build's input), perm, split_vals, split_dims and
  * node_offsets (device) and L = levels. Query arrays are device SoA [d][nq].
- * One CUDA thread per query; the call returns when the results are written.
+ * One warp per query; the call returns when the results are written.
  * Errors: KDT_ERR_INVALID_ARG (sizes out of range, missing pointers),
  *         KDT_ERR_CUDA. */
 

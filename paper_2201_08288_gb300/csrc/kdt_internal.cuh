@@ -180,7 +180,7 @@ struct StepDev {
   uint32_t small_off_cap;
   uint32_t bigseg_cap;
   // select paths by segment size (kdt_tuning): one thread up to tiny_max keys,
-  // a warp's bitonic network up to bitonic_max, a warp's radix select up to
+  // a warp's bitonic network up to bitonic_max (at most 128), a warp's brackets up to
   // warp_max, a CTA above
   uint32_t tiny_max, bitonic_max, warp_max;
   uint32_t midseg_cap;

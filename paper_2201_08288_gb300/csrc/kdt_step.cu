@@ -12,8 +12,8 @@
 //      moves the columns);
 //   2. per (cell, subset) segment (the subsets of Sec. 3.2 / App. C.2): its
 //      position range, from the cell's subset offsets;
-//   3. per segment: the exact lower median (8-bit MSD radix select) read in
-//      place from the key column;
+//   3. per segment: the exact lower median, read in place from the key column
+//      (by size: a network, brackets or a radix select);
 //   4. per cell: the count-weighted lower median of the segment medians;
 //   5. children sizes from per-tile counts and a per-cell scan of them; the
 //      children are classified (terminal / small / big) before the move;
@@ -672,13 +672,13 @@ __device__ __forceinline__ bool radix_start(uint32_t lo, uint32_t hi, uint32_t r
   return true;
 }
 
-// Lower median (rank (w-1)/2) of w keys by one warp: MSD radix select with
+// The key of the given rank among w by one warp: MSD radix select with
 // 8-bit digits over the bits where the keys differ (histogram of 256 words
 // owned by the warp), the keys read on every pass from global memory (raw
 // float bits, turned into order keys), 8 loads per lane issued together, or
 // from a shared-memory copy (order keys already).
 template <bool kGlobal>
-__device__ uint32_t warp_select_stream(const uint32_t* keys, uint32_t w, uint32_t* hist) {
+__device__ uint32_t warp_select_stream(const uint32_t* keys, uint32_t w, uint32_t rank, uint32_t* hist) {
   constexpr int U = 8;
   const int lane = threadIdx.x & 31;
   auto load = [&](uint32_t i) -> uint32_t { return kGlobal ? kload(keys + i) : keys[i]; };
@@ -698,7 +698,7 @@ __device__ uint32_t warp_select_stream(const uint32_t* keys, uint32_t w, uint32_
       }
   }
   RadixState st;
-  if (!radix_start(lo, hi, (w - 1) / 2, &st)) return st.prefix;
+  if (!radix_start(lo, hi, rank, &st)) return st.prefix;
   while (st.rem > 0) {
     const int bits = st.rem < 8 ? st.rem : 8, shift = st.rem - bits;
     const uint32_t nb = 1u << bits, hmask = st.rem == 32 ? 0u : ~((1u << st.rem) - 1u);
@@ -727,14 +727,155 @@ __device__ uint32_t warp_select_stream(const uint32_t* keys, uint32_t w, uint32_
   return st.prefix;
 }
 
+// Ascending sort of 32 K keys, element k * 32 + lane in register k of a lane:
+// the bitonic network of warp_bitonic_median with its last stages.
+template <int K>
+__device__ __forceinline__ void warp_sort(uint32_t (&v)[K]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int size = 2; size <= 32 * K; size <<= 1)
+#pragma unroll
+    for (int j = size >> 1; j > 0; j >>= 1)
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const bool asc = ((k * 32 + lane) & size) == 0;
+        if (j >= 32) {
+          const int kk = k ^ (j >> 5);
+          if (k < kk) {
+            const uint32_t lo = min(v[k], v[kk]), hi = max(v[k], v[kk]);
+            v[k] = asc ? lo : hi;
+            v[kk] = asc ? hi : lo;
+          }
+        } else {
+          const uint32_t o = __shfl_xor_sync(0xffffffffu, v[k], j);
+          v[k] = (((lane & j) == 0) == asc) ? min(v[k], o) : max(v[k], o);
+        }
+      }
+}
+
+// Keys between which the one of rank m of c is expected: those `under` below
+// and `over` above its place in a sorted sample of 32 K, taken at even distances.
+template <int K, class Get>
+__device__ __forceinline__ void warp_bracket(Get get, uint32_t c, uint32_t m, int under, int over, uint32_t* a,
+                                             uint32_t* b) {
+  const int lane = threadIdx.x & 31;
+  uint32_t v[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) v[k] = get(((uint32_t)(k * 32 + lane) * c) / (32u * K));
+  warp_sort<K>(v);
+  const int at = (int)((m * 32u * K) / c), i = at - under, j = at + over;
+  uint32_t x = 0u, y = 0xffffffffu;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t p = __shfl_sync(0xffffffffu, v[k], i & 31), q = __shfl_sync(0xffffffffu, v[k], j & 31);
+    if (i >= 0 && (i >> 5) == k) x = p;
+    if ((j >> 5) == k) y = q;
+  }
+  *a = x;
+  *b = y;
+}
+
+// One pass over c keys, U rows of 32 loaded together: how many lie below a, how
+// many in [a, b], and those (up to cap of them, in their order) to dst.
+template <int U, class Get>
+__device__ __forceinline__ void warp_bracket_pass(Get get, uint32_t c, uint32_t a, uint32_t b, uint32_t* dst,
+                                                  uint32_t cap, uint32_t* below, uint32_t* inside) {
+  const uint32_t lane = threadIdx.x & 31u, width = b - a;
+  const unsigned lt = (1u << lane) - 1u;
+  uint32_t l = 0, n = 0;
+  for (uint32_t b0 = 0; b0 < c; b0 += 32 * U) {
+    uint32_t x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t i = b0 + (uint32_t)(u * 32) + lane;
+      x[u] = i < c ? get(i) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool real = b0 + (uint32_t)(u * 32) + lane < c, in = real && x[u] - a <= width;
+      l += real && x[u] < a ? 1u : 0u;
+      const unsigned who = __ballot_sync(0xffffffffu, in);
+      const uint32_t pos = n + (uint32_t)__popc(who & lt);
+      if (in && pos < cap) dst[pos] = x[u];
+      n += (uint32_t)__popc(who);
+    }
+  }
+  *below = __reduce_add_sync(0xffffffffu, l);
+  *inside = n;
+  __syncwarp();
+}
+
+// A pass for the key of rank m, and where the sample misled (about one time in
+// fifty) another over the side that holds it. On return [a, b] holds it, at
+// rank m among the *inside keys there.
+template <int U, class Get>
+__device__ __forceinline__ void warp_bracket_narrow(Get get, uint32_t c, uint32_t* m, uint32_t* a, uint32_t* b,
+                                                    uint32_t* dst, uint32_t cap, uint32_t* inside) {
+  uint32_t below;
+  warp_bracket_pass<U>(get, c, *a, *b, dst, cap, &below, inside);
+  if (*m < below || *m - below >= *inside) {
+    if (*m < below) {
+      *b = *a - 1u;
+      *a = 0u;
+    } else {
+      *a = *b + 1u;
+      *b = 0xffffffffu;
+    }
+    warp_bracket_pass<U>(get, c, *a, *b, dst, cap, &below, inside);
+  }
+  *m -= below;
+}
+
+// Lower median of w > 32 keys by one warp: a small sorted sample gives two keys
+// that the median lies between, and one pass keeps what does (two fifths for a
+// sample of 32, a fifth for 128); again among those, until a sort of 32 ends it.
+// Many equal keys may not thin out: what is left then goes to the radix select,
+// as does what finds no room. (The radix select, for all segments above 256 keys,
+// took up to four passes with a shared-memory atomic per key, 92 instructions per
+// 32 keys of 1024 against 71 here; the bitonic network of 256 keys, for those
+// above 128, 28 rounds of shuffles of 8 registers. 2^27 points, 256 subsets: the
+// small selects of a build 3.75 -> 2.82 ms; 2^24 points, 64 subsets: 590 -> 497
+// us; 50,000,021 points, 64 subsets: 428 -> 284. Columns per lane instead of a
+// dense list, or a first pass that compares floats, took 519 and 530 us where
+// this takes 497. A CTA's select by brackets lost to its radix select, whose
+// later passes hit L1 and L2: 56 against 41 us for 2^24 keys in segments of 8192.)
+constexpr uint32_t kBracketA = 1024, kBracketB = 512;  // room after odd and after even passes
+template <class Get>
+__device__ uint32_t warp_bracket_median(const uint32_t* keys, Get get, uint32_t w, uint32_t* buf) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t a, b, c, m = (w - 1u) / 2u;
+  if (w > 1024u)
+    warp_bracket<4>(get, w, m, 12, 13, &a, &b);
+  else
+    warp_bracket<1>(get, w, m, 6, 7, &a, &b);
+  warp_bracket_narrow<8>(get, w, &m, &a, &b, buf, kBracketA, &c);
+  if (a == b) return a;
+  if (c > kBracketA) return warp_select_stream<true>(keys, w, (w - 1u) / 2u, buf);
+  uint32_t *src = buf, *dst = buf + kBracketA, cap = kBracketB;
+  while (c > 32u) {
+    auto kept = [&](uint32_t i) { return src[i]; };
+    warp_bracket<1>(kept, c, m, 6, 7, &a, &b);
+    const uint32_t m0 = m;
+    uint32_t n;
+    warp_bracket_narrow<4>(kept, c, &m, &a, &b, dst, cap, &n);
+    if (a == b) return a;
+    if (n > cap || 8u * n > 7u * c) return warp_select_stream<false>(src, c, m0, dst);
+    c = n;
+    uint32_t* const t = src;
+    src = dst;
+    dst = t;
+    cap = kBracketB;
+  }
+  uint32_t v[1] = {lane < c ? src[lane] : 0xffffffffu};
+  warp_sort<1>(v);
+  return __shfl_sync(0xffffffffu, v[0], (int)m);
+}
+
 // One warp per listed segment of tiny_max+1 .. warp_max points: up to
-// bitonic_max keys sorted in registers; up to 1024 keys staged once in shared
-// memory for a radix select; larger segments read from global memory on every
-// pass.
+// bitonic_max keys sorted in registers, larger ones by brackets.
 __global__ void __launch_bounds__(256) k_select_small(const TreeDev* trees, StepDev s) {
   chain_wait();
-  __shared__ uint32_t hist[8][256];
-  __shared__ uint32_t stage[8][1024];
+  __shared__ uint32_t buf[8][kBracketA + kBracketB];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t cnt = min(*s.midseg_count, s.midseg_cap);
   for (uint32_t j = blockIdx.x * 8u + (uint32_t)warp; j < cnt; j += gridDim.x * 8u) {
@@ -743,32 +884,12 @@ __global__ void __launch_bounds__(256) k_select_small(const TreeDev* trees, Step
     const uint32_t* keys = s.seg_key[g];
     auto key_of = [&](uint32_t e) { return kload(keys + e); };
     uint32_t med;
-    if (w <= s.bitonic_max && w <= 64u) {
+    if (w <= s.bitonic_max && w <= 64u)
       med = warp_bitonic_median<2>(key_of, w);
-    } else if (w <= s.bitonic_max && w <= 128u) {
+    else if (w <= s.bitonic_max && w <= 128u)
       med = warp_bitonic_median<4>(key_of, w);
-    } else if (w <= s.bitonic_max) {
-      med = warp_bitonic_median<8>(key_of, w);
-    } else if (w <= 1024u) {
-      uint32_t* st = stage[warp];
-      for (uint32_t b0 = 0; b0 < w; b0 += 256) {
-        uint32_t x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const uint32_t i = b0 + (uint32_t)(u * 32 + lane);
-          x[u] = i < w ? kload(keys + i) : 0u;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const uint32_t i = b0 + (uint32_t)(u * 32 + lane);
-          if (i < w) st[i] = x[u];
-        }
-      }
-      __syncwarp();
-      med = warp_select_stream<false>(st, w, hist[warp]);
-    } else {
-      med = warp_select_stream<true>(keys, w, hist[warp]);
-    }
+    else
+      med = warp_bracket_median(keys, key_of, w, buf[warp]);
     if (lane == 0) s.seg_med[g] = med;
     __syncwarp();
   }
