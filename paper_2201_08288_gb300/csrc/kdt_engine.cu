@@ -117,6 +117,13 @@ TreePlan plan_tree(const kdt_params& p0, bool no_subtree, bool alone) {
   const bool fourier = p.fourier_j > 0;
   t.small_max = (fourier || no_subtree) ? 0 : subtree_capacity(p.d);
   t.sub_wide = &subtree_shape(p.d) == &kSubWide;
+  const uint64_t live_min = p.depth > 0 ? 1 : (uint64_t)p.leaf_size + 1;  // points of a cell that still splits
+  // cells that one small cell of so many points can have on a level (the last
+  // has none; a small cell is the root, or lies below a big one)
+  auto slice_cells = [&](int points) {
+    const uint64_t inner = (uint64_t)1 << std::max(t.L_cap - (n > (uint64_t)points ? 2 : 1), 0);
+    return std::max<uint64_t>(32, std::min((uint64_t)points / live_min, inner));
+  };
   if (t.small_max > 0 && alone && n > (uint64_t)t.small_max) {
     // the tall shape while its cells, of half its capacity to all of it, are no
     // more than the SMs (a single cell that the other shapes hold finishes sooner
@@ -125,12 +132,16 @@ TreePlan plan_tree(const kdt_params& p0, bool no_subtree, bool alone) {
     const uint64_t sms = (uint64_t)plan_sms();
     uint64_t cells = 1;
     while (cells <= sms && cells * (uint64_t)tall < n) cells *= 2;
-    if (cells <= sms && tall > t.small_max) {
+    const uint64_t ctas = std::min<uint64_t>(sms, cells + cells / 4 + 1);
+    // (and the cell tables of its levels take no more memory)
+    if (cells <= sms && tall > t.small_max &&
+        ctas * slice_cells(tall) <= sms * (uint64_t)subtree_shape(p.d).ctas * slice_cells(t.small_max)) {
       t.small_max = tall;
       t.sub_wide = false;
-      t.sub_tall = (int)std::min<uint64_t>(sms, cells + cells / 4 + 1);
+      t.sub_tall = (int)ctas;
     }
   }
+  t.slice_cells = slice_cells(t.small_max);
   t.sid_bytes = p.subset_mode == KDT_SUBSET_EXPLICIT ? (p.subset_id16 ? 2 : 1) : 0;
   const bool root_terminal = p.depth > 0 ? (n == 0) : (n <= (uint64_t)p.leaf_size);
   t.leafsort = !root_terminal && p.subset_mode != KDT_SUBSET_CONTIGUOUS && !fourier;
@@ -142,9 +153,13 @@ TreePlan plan_tree(const kdt_params& p0, bool no_subtree, bool alone) {
   if (!root_terminal && (t.presorted || n > (uint64_t)t.small_max)) t.steps = 1;
   while (t.steps > 0 && t.steps < t.L_cap && ((n - 1) >> t.steps) + 1 > ends) ++t.steps;
   t.huge_cap = t.leafsort ? n / (uint64_t)(kLeafBlockMax + 1) + 1 : 0;
-  const uint64_t leaves = (uint64_t)1 << t.L_cap;
-  t.maxB = std::min<uint64_t>(n / (uint64_t)(t.small_max + 1) + 1, leaves);
-  t.cap_small = std::min<uint64_t>(n, leaves) + 1;
+  // cells that still split are disjoint, lie above the last level and hold more
+  // than leaf_size points (of a fixed depth: one or more)
+  const uint64_t leaves = (uint64_t)1 << t.L_cap, inner = std::max<uint64_t>(leaves / 2, 1);
+  t.maxB = std::min<uint64_t>(n / (uint64_t)(t.small_max + 1) + 1, inner);
+  // (small ones are children of big ones, two each at most; or the root)
+  const uint64_t parents = (uint64_t)t.L_cap * (n / (uint64_t)(t.small_max + 1)) + 1;
+  t.cap_small = t.small_max > 0 ? std::min({n / live_min, inner, 2 * parents}) + 1 : 1;
   t.term_cap = leaves + 1;
   size_t off = 0;
   auto take = [&](size_t b) {
@@ -175,7 +190,7 @@ void StepNeeds::add(const kdt_params& p0, const TreePlan& tp) {
   // two columns of the ids would take
   if (tp.small_max > 0) small_off += tp.n * (uint64_t)tp.sid_bytes / 2;
   max_trees += 1;
-  slice_cells = std::max<uint32_t>(slice_cells, (uint32_t)tp.small_max);
+  slice_cells = std::max<uint32_t>(slice_cells, (uint32_t)tp.slice_cells);
   sub_tall = tp.sub_tall;
   widest = widest || p.key_rule == KDT_KEY_WIDEST_SPREAD;
   max_d = std::max(max_d, (int)p.d);
@@ -217,7 +232,7 @@ StepPlan plan_step(const StepNeeds& needs) {
   s.tile_seg = take((size_t)s.max_tiles * 4);
   s.tile_left = take((size_t)s.max_tiles * 4);
   s.tile_loff = take((size_t)s.max_tiles * 4);
-  s.tile_mm = take(needs.widest || needs.fourier ? (size_t)s.max_tiles * 2 * kMaxDims * 2 * 4 : 0);
+  s.tile_mm = take(needs.widest || needs.fourier ? (size_t)s.max_tiles * kTileRecWords * 4 : 0);
   s.child_mm = take(needs.widest ? (size_t)s.maxB * 2 * kMaxDims * 2 * 4 : 0);
   s.kdim = take((size_t)s.maxB * 4);
   s.mkey = take((size_t)s.maxB * 4);

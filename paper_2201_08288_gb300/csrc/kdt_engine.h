@@ -37,6 +37,7 @@ struct TreePlan {
   uint64_t n = 0;
   uint64_t term_cap = 0;
   uint64_t huge_cap = 0;  // terminal cells larger than one CTA's leaf sort
+  uint64_t slice_cells = 0;  // a level's cells of one small cell
   uint64_t maxB = 0;      // big cells at one level
   uint64_t cap_small = 0; // small cells over the whole build
   size_t xbuf[2] = {0, 0}, pbuf[2] = {0, 0}, terms = 0, root_off = 0, root_cur = 0,

@@ -28,6 +28,7 @@ constexpr int kMaxDims = 64;          // d <= 64
 constexpr int kMaxSubsets = 4096;     // r <= 4096 on the CUDA path
 constexpr int kMaxLevels = 30;        // depth / max_levels <= 30
 constexpr int kTile = 2048;           // points per tile of the multi-CTA pipeline
+constexpr int kTileRecWords = 2 * kMaxDims + 4;  // words of a tile's record in tile_mm (16-byte aligned)
 constexpr int kTileThreads = 256;     // threads of the tile kernels
 constexpr int kSelTinyMax = 64;       // segments up to this size: one thread per segment
 constexpr int kSelSmallMax = 4096;    // largest warp-select segment (kdt_tuning warp_max)
@@ -135,7 +136,7 @@ struct StepDev {
   uint32_t* kdim;         // [ncells] key coordinate
   uint32_t* mkey;         // [ncells] split key
   uint32_t* lcount;       // [ncells] left child size
-  uint32_t* tile_mm;      // [ntiles][2][kMaxDims][2] per-tile min/max keys of a root (widest; side 0)
+  uint32_t* tile_mm;      // [ntiles][kTileRecWords] a root's min and max key per coordinate (widest), or a run's sums
   uint32_t* child_mm;     // [ncells][2][kMaxDims][2] per-child min/max keys (widest), reduced
                           // by the scatter with atomics
   uint32_t* seg_w;        // [nseg] points per (cell, subset)

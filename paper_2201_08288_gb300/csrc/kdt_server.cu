@@ -237,7 +237,7 @@ kdt_status kdt_server_create(size_t mem_budget_bytes, int32_t max_trees_in_fligh
   cap.cap_small = cap.points / 16 + 2 * (uint64_t)max_trees_in_flight;
   cap.nseg = cap.maxB * 64;
   cap.max_trees = sv->max_slots;
-  cap.slice_cells = 8192;
+  cap.slice_cells = kdt::kSubWide.q * kdt::kSubWide.threads;  // the most points of a small cell
   cap.widest = true;
   cap.max_d = KDT_MAX_DIMS;
   cap.max_r = KDT_MAX_SUBSETS;

@@ -70,7 +70,7 @@ __device__ __forceinline__ void tiles_cell(const TreeDev* trees, const StepDev& 
     for (uint32_t j = lane; j < (uint32_t)t.r; j += 32u) t.root_cur[j] = 0;
     if (t.key_rule == KEY_WIDEST && cell.dim < 0 && nt > 0u)
       for (uint32_t j = lane; j < 2u * (uint32_t)t.d; j += 32u)
-        s.tile_mm[((size_t)tb * 2 * kMaxDims + j / 2) * 2 + (j & 1)] = (j & 1) ? 0u : 0xffffffffu;
+        s.tile_mm[(size_t)tb * kTileRecWords + j] = (j & 1) ? 0u : 0xffffffffu;
   }
 }
 
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, St
   if ((tl.y / (uint32_t)kTile) % (uint32_t)kPsGroup != 0u) {  // the group's first tile runs it
     if (want_mm)
       for (int j = threadIdx.x; j < 2 * t.d; j += blockDim.x)
-        s.tile_mm[((size_t)blockIdx.x * 2 * kMaxDims + j / 2) * 2 + (j & 1)] = (j & 1) ? 0u : 0xffffffffu;
+        s.tile_mm[(size_t)blockIdx.x * kTileRecWords + j] = (j & 1) ? 0u : 0xffffffffu;
     return;
   }
   extern __shared__ __align__(16) uint32_t ps_buf[];  // a word per place, then a u16 subset per place
@@ -320,10 +320,10 @@ __global__ void __launch_bounds__(kPsThreads) k_ps_move(const TreeDev* trees, St
     // tile's own record, if another, holds the identities
     const uint32_t tb = cell.tile0;
     for (int j = threadIdx.x; j < 2 * t.d; j += kPsThreads) {
-      uint32_t* acc = &s.tile_mm[((size_t)tb * 2 * kMaxDims + j / 2) * 2 + (j & 1)];
+      uint32_t* acc = &s.tile_mm[(size_t)tb * kTileRecWords + j];
       if (j & 1) atomicMax(acc, gmm[j / 2][1]); else atomicMin(acc, gmm[j / 2][0]);
       if (blockIdx.x != tb)
-        s.tile_mm[((size_t)blockIdx.x * 2 * kMaxDims + j / 2) * 2 + (j & 1)] = (j & 1) ? 0u : 0xffffffffu;
+        s.tile_mm[(size_t)blockIdx.x * kTileRecWords + j] = (j & 1) ? 0u : 0xffffffffu;
     }
   }
   pass([&](int q) { return i0 + threadIdx.x + q * kPsThreads; },
@@ -377,8 +377,8 @@ __global__ void __launch_bounds__(kTileThreads) k_minmax(const TreeDev* trees, S
         lo = min(lo, red[0][w]);
         hi = max(hi, red[1][w]);
       }
-      s.tile_mm[((size_t)blockIdx.x * 2 * kMaxDims + l) * 2 + 0] = lo;
-      s.tile_mm[((size_t)blockIdx.x * 2 * kMaxDims + l) * 2 + 1] = hi;
+      s.tile_mm[(size_t)blockIdx.x * kTileRecWords + 2 * l + 0] = lo;
+      s.tile_mm[(size_t)blockIdx.x * kTileRecWords + 2 * l + 1] = hi;
     }
     __syncthreads();
   }
@@ -421,8 +421,8 @@ __device__ __forceinline__ void pick_dim_cell(const TreeDev* trees, const StepDe
       hi[q] = 0u;
     }
     for (uint32_t j = tb + threadIdx.x; j < te; j += blockDim.x) {
-      // 16-byte aligned: a record is 2 * kMaxDims * 2 words, c0 a multiple of 8
-      const uint4* p = (const uint4*)(s.tile_mm + ((size_t)j * 2 * kMaxDims + c0) * 2);
+      // 16-byte aligned: a record is a multiple of 4 words, c0 of 8
+      const uint4* p = (const uint4*)(s.tile_mm + (size_t)j * kTileRecWords + 2 * c0);
 #pragma unroll
       for (int h = 0; h < 4; ++h) {
         if (2 * h >= nc) break;
@@ -1207,7 +1207,6 @@ __global__ void __launch_bounds__(256, 1) k_combine_warp(const TreeDev* trees, S
 // ------------------------------------------- the paper's estimator (Sec. 3)
 
 constexpr int kFourierTerms = 2 * KDT_FOURIER_MAX_J + 1;
-constexpr int kTileRecWords = 2 * kMaxDims * 2;  // words of a tile's record in tile_mm
 static_assert(kFourierTerms * 2 <= kTileRecWords, "a tile's sums fit its record");
 
 // The sums over a cell's points of the basis terms of Lemma 1 on its key
