@@ -234,6 +234,12 @@ __device__ __forceinline__ uint32_t warp_segment_median(uint32_t w, KeyOf key_of
   return warp_wsel_bits<16, true>(w, rank, key_of, one);
 }
 
+// Most subsets whose medians a thread per segment combines: it walks its cell's
+// medians, where a warp per cell takes a chain of warp sums, a bit each. (8
+// subsets: 1000 points 49 -> 45 us in this kernel, 65,536 points 87 -> 83; 32
+// subsets are level, 72 us either way for 300,007 points.)
+constexpr int kCountMax = 16;
+
 // The shapes of kdt_launch.h.
 constexpr SubtreeShape kShapes[3] = {kSubNarrow, kSubWide, kSubTall};
 
@@ -600,8 +606,8 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
         }
         if (tid == 0) s_nbig = s_nhist = 0;
         __syncthreads();
+        uint32_t total;  // segments of the level
         {
-          uint32_t total;
           block_counts_scan<kQ, NW>(balq, s_bcnt, lane, warp, segq, &total);
 #pragma unroll
           for (int q = 0; q < kQ; ++q) {
@@ -678,7 +684,9 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
         // ---- 4. weighted lower median per cell: the smallest segment median m
         // whose segments with median <= m hold >= ceil(W/2) points, i.e. the
         // key of weighted rank (W-1)/2. A cell's segments are [pre[begin],
-        // pre[end]). One warp per cell, no block barrier: up to 256 segments
+        // pre[end]). Trees of up to kCountMax subsets: a thread per segment sums
+        // what its cell's medians below its own weigh, and those up to its own.
+        // Others: one warp per cell, no block barrier: up to 256 segments
         // are held in registers and the key is settled one bit per step by a
         // warp sum; more segments go through the warp's radix histogram.
         // (the histograms are fewer than the warps of the tall shape: its cells of
@@ -706,7 +714,25 @@ k_subtree(const TreeDev* trees, const Cell* list, uint32_t count, const uint32_t
             m = warp_weighted_select(ns, rank, S.whist + warp * 256, key_of, w_of);
           if (lane == 0) cc[k].mkey = m;
         };
-        for (uint32_t k = warp; k < ncur; k += NW) combine(k, false);
+        if (r <= kCountMax) {
+          const bool unit = t.combine_rule == 1;
+          for (uint32_t sx = tid; sx < total; sx += T) {
+            const uint32_t k = S.cellid[S.segs[sx]];
+            const uint32_t b = cc[k].begin, e = b + cc[k].count;
+            const uint32_t s0 = S.pre[b], s1 = S.pre[e];
+            const uint32_t key = S.smed[sx], rank = unit ? (s1 - s0 - 1u) / 2u : (cc[k].count - 1u) / 2u;
+            uint32_t below = 0, upto = 0, at = b;
+            for (uint32_t j = s0; j < s1; ++j) {
+              const uint32_t kj = S.smed[j], end = min((uint32_t)S.segs[j + 1], e), w = unit ? 1u : end - at;
+              below += kj < key ? w : 0u;
+              upto += kj <= key ? w : 0u;
+              at = end;
+            }
+            if (below <= rank && rank < upto) cc[k].mkey = key;  // (equal medians write the same)
+          }
+        } else {
+          for (uint32_t k = warp; k < ncur; k += NW) combine(k, false);
+        }
         if (NW > kSubtreeHists && r > 256 && warp < kSubtreeHists)
           for (uint32_t k = warp; k < ncur; k += kSubtreeHists) combine(k, true);
         __syncthreads();
