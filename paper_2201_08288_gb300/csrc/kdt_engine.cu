@@ -141,7 +141,7 @@ TreePlan plan_tree(const kdt_params& p0, bool no_subtree, bool alone) {
       t.sub_tall = (int)ctas;
     }
   }
-  t.slice_cells = slice_cells(t.small_max);
+  t.slice_cells = t.small_max > 0 ? slice_cells(t.small_max) : 0;
   t.sid_bytes = p.subset_mode == KDT_SUBSET_EXPLICIT ? (p.subset_id16 ? 2 : 1) : 0;
   const bool root_terminal = p.depth > 0 ? (n == 0) : (n <= (uint64_t)p.leaf_size);
   t.leafsort = !root_terminal && p.subset_mode != KDT_SUBSET_CONTIGUOUS && !fourier;
@@ -762,7 +762,8 @@ kdt_status Engine::run_graph() {
 }
 
 kdt_status Engine::run_to_completion() {
-  if (ahead_ > 0) return run_ahead();
+  // (a traced launch states its points, which only the host's counts tell)
+  if (ahead_ > 0 && !trace_enabled()) return run_ahead();
   for (int guard = 0; busy() || !pending_.empty(); ++guard) {
     if (guard > 2 * KDT_MAX_LEVELS + 4) return KDT_ERR_CUDA;
     const kdt_status s = tick();

@@ -53,7 +53,7 @@ TreePlan plan_tree(const kdt_params& p, bool no_subtree = false, bool alone = fa
 // at the same time.
 struct StepNeeds {
   uint64_t points = 0, maxB = 0, cap_small = 0, nseg = 0, small_off = 0;
-  uint32_t max_trees = 0, slice_cells = 32;
+  uint32_t max_trees = 0, slice_cells = 0;
   int sub_tall = 0;  // the forest's one tree uses the subtree kernel's tall shape
   bool widest = false;
   bool fourier = false;  // a tree splits by the Fourier-moment estimator
@@ -69,9 +69,10 @@ struct StepPlan {
   // or sub_tall)
   uint32_t maxB = 0, cap_small = 0, max_tiles = 0, nseg_cap = 0, bigseg_cap = 0, grid_step = 0, sms = 0, off_cap = 0,
            small_off_cap = 0;
-  size_t trees = 0, words = 0, slot_words = 0, slots_list = 0, admits = 0, big[2] = {0, 0}, small = 0, tiles = 0, tile_seg = 0, tile_left = 0, tile_loff = 0, tile_mm = 0, child_mm = 0, kdim = 0,
-         mkey = 0, lcount = 0, seg_w = 0, seg_key = 0, seg_med = 0, bigseg = 0, midseg = 0, slices = 0,
-         off[2] = {0, 0}, obase[2] = {0, 0}, small_off = 0, crow = 0;
+  size_t trees = 0, words = 0, slot_words = 0, slots_list = 0, admits = 0, big[2] = {0, 0}, small = 0, tiles = 0,
+         tile_seg = 0, tile_left = 0, tile_loff = 0, tile_mm = 0, child_mm = 0, kdim = 0, mkey = 0, lcount = 0,
+         seg_w = 0, seg_key = 0, seg_med = 0, bigseg = 0, midseg = 0, slices = 0, off[2] = {0, 0}, obase[2] = {0, 0},
+         small_off = 0, crow = 0;
   size_t bytes = 0;
 };
 StepPlan plan_step(const StepNeeds& needs);

@@ -49,6 +49,8 @@ bool capturing(cudaStream_t st) {
   return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
 }
 
+bool trace_enabled() { return tracer().on.load(std::memory_order_relaxed); }
+
 void trace_add_launches(uint64_t n) { tracer().launches.fetch_add(n, std::memory_order_relaxed); }
 
 TraceScope::TraceScope(KernelId id, cudaStream_t st, uint64_t units) : id_(id), st_(st), units_(units) {

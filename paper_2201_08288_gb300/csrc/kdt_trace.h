@@ -20,6 +20,8 @@ enum KernelId {
 
 // Launches replayed by a graph beyond the ones counted while it was captured.
 void trace_add_launches(uint64_t n);
+// True while launches are timed.
+bool trace_enabled();
 // True while `st` is being captured into a graph.
 bool capturing(cudaStream_t st);
 

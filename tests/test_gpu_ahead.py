@@ -60,3 +60,19 @@ def test_steps_ahead(kind, n, d, r, mode, rule, kw):
 def test_estimator(depth):
     x = np.clip(np.random.default_rng(5).random((3, 50_000), dtype=np.float32) ** 3, 1e-6, 1 - 1e-6)
     check_tree(x, gpu_build(x, depth=depth, fourier_j=9), 9)
+
+
+def test_a_traced_build_states_its_points():
+    from paper_2201_08288_gb300 import kdt
+    x = torch.rand(3, 70_001, device="cuda")
+    kw = dict(r=8, subset_mode=0, depth=12)
+    a = kdt.kdt_build(x, **kw)
+    kdt.kdt_trace_enable(True)
+    try:
+        kdt.kdt_trace_read(True)
+        b = kdt.kdt_build(x, **kw)
+        units = {k: v[2] for k, v in kdt.kdt_trace_read(True).items()}
+    finally:
+        kdt.kdt_trace_enable(False)
+    assert units["k_subtree"] == 70_001  # every point ends in a small cell
+    assert torch.equal(a.perm, b.perm) and torch.equal(a.split_vals, b.split_vals)
