@@ -62,9 +62,9 @@ def workload(name: str, rank: int):
 def bytes_per_point(kernel: str, d: int, sid_bytes: int, subset_mode: int) -> float:
     """Algorithmic bytes one launch moves per point it processes."""
     return {
-        "k_part_scatter": 2.0 * (4 * d + 4 + sid_bytes),   # read + write every column, perm, ids
+        "k_part_scatter": 2.0 * (4 * d + 4),               # read + write every column and perm (no ids)
         "k_subtree": 4.0 * d + 4 + sid_bytes + 4,           # stage everything once, write perm once
-        "k_ps_move": 2.0 * (4 * d + sid_bytes) + 4,         # columns and ids in and out, perm out
+        "k_ps_move": 2.0 * 4 * d + sid_bytes + 4,           # columns in and out, ids in, perm out
         "k_part_count": 4.0,
         "k_select_small": 4.0,                              # the key column, read in place
         "k_fourier_moments": 4.0,                           # the key column, read in place
