@@ -1905,10 +1905,11 @@ bool step_selects_all(uint32_t nseg, uint64_t points, uint32_t sms) {
   return nseg <= 8u * sms && points <= 8192ull * nseg;
 }
 
-// Few, large segments: several CTAs each. One CTA takes about 0.25 ns a key,
-// the four launches 40 us and 4 ps a key of the step (64 segments of 262,144
-// keys: 66 us with a CTA each, 108 here), so the line lies where 262,144 keys
-// of each of 32 segments cost the same.
+// Few, large segments: several CTAs each. A CTA takes about 0.2 ns a key, the
+// four launches 40 us and 4 ps a key of the step. Builds of one level: 32
+// segments of 262,144 keys 209 us here and 208 with a CTA each, of 524,288 keys
+// 276 and 303; 8 of 262,144 keys 156 and 173; 64 of 262,144 keys take a CTA each
+// 57 us and would take 108 here.
 bool step_selects_wide(uint32_t nseg, uint64_t points) { return nseg <= 32u && points >= 262144ull * nseg; }
 
 // One CTA per cell combines, counts, scans and classifies: while the cells'
@@ -1950,9 +1951,16 @@ static void launch_listed_selects(const TreeDev* trees, const StepDev& s, uint32
   TraceScope ts(K_SELECT_BIG, st);
   // nseg bounds the big segments too; with few of them (the first levels
   // of a large tree) a CTA's loads in flight set the rate, so they take
-  // 512 threads whatever the tuning
+  // 512 threads whatever the tuning, and 1024 while two CTAs per SM take them
+  // all (64 segments of 780,000 keys: 322 us with 512 threads, 188 with 1024;
+  // 300 of 100,000: 71 and 64; a build of 50,000,021 points 5.64 -> 5.42 ms)
   const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>(std::min(max_bigseg, nseg), sms * 4u));
-  if (tune.cta_threads == 512 || nseg <= sms * 4u) {
+  if (nseg <= sms) {
+    if (tune.digit_bits == 8)
+      launch_chained(k_select_big<1024, 8>, grid, 1024, 0, st, trees, s);
+    else
+      launch_chained(k_select_big<1024, 11>, grid, 1024, 0, st, trees, s);
+  } else if (tune.cta_threads == 512 || nseg <= sms * 4u) {
     if (tune.digit_bits == 8)
       launch_chained(k_select_big<512, 8>, grid, 512, 0, st, trees, s);
     else
