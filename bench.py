@@ -72,13 +72,12 @@ def bytes_per_point(kernel: str, d: int, sid_bytes: int, subset_mode: int) -> fl
     }.get(kernel, 0.0)
 
 
-def model_bytes_per_point_level(d: int, sid_bytes: int, subset_mode: int) -> float:
-    """Bytes each level must move per point (SoA ping-pong model): the key
-    column read for the selection, the subset-id source (explicit ids, or the
-    permutation the id is derived from), read+write of all columns and the
-    permutation, read+write of an explicit id column."""
-    s_sel = sid_bytes if subset_mode == 2 else 4
-    return 4 + s_sel + 8 * (d + 1) + 2 * (sid_bytes if subset_mode == 2 else 0)
+def model_bytes_per_point_level(d: int) -> float:
+    """Bytes each level must move per point (two copies of columns and
+    permutation in turn): the key column read once, every column and the
+    permutation read and written. Subset ids take no part: after the root is
+    put in subset order a cell's segments say them."""
+    return 4.0 + 8 * (d + 1)
 
 
 def max_over_ranks(x: float, dist, device) -> float:
@@ -541,7 +540,7 @@ def main() -> None:
                 "traffic": (traffic_pp * pts_done / max(nl, 1)) if traffic_pp is not None else None,
                 "share_of_step": tot_ms / (ms / args.steps * args.steps) if ms > 0 else None}
     kernel_table = {k: {"launches": v[0], "ms": round(v[1], 3), "points": v[2]} for k, v in stats.items()}
-    mb = model_bytes_per_point_level(spec.d, sid_bytes, spec.subset_mode)
+    mb = model_bytes_per_point_level(spec.d)
     build_model_gbs = spec.n * levels * mb / (ms / args.steps / 1e3) / 1e9
 
     e2e = None
