@@ -158,6 +158,7 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
 // Most dynamic shared memory of the staged scatter: three CTAs per SM with
 // their static part and the kilobyte that each one reserves.
 constexpr uint32_t kScatterSmemBytes = 74240;
+constexpr uint32_t kScatterLargeSmemBytes = 112640;  // and two CTAs per SM
 cudaError_t prepare_scatter_kernel(int uniform_d, bool any_widest);
 // uniform_d: the coordinate count of every tree of the step, 0 if they differ
 // (a kernel compiled for that d is used where there is one)

@@ -53,13 +53,36 @@ __host__ __device__ constexpr uint32_t col_stride(uint32_t T) { return T + 4u; }
 // Bytes of the two buffers for d coordinate columns and the permutation.
 __host__ __device__ constexpr uint32_t buf_bytes(int d, uint32_t T) { return (uint32_t)(d + 1) * col_stride(T) * 4u; }
 
-// Points of a sub-tile: a power of two, as many as two buffers of
-// kScatterSmemBytes in all hold, at most 1024.
-__host__ __device__ constexpr uint32_t sub_tile(int d) {
+// The instances: one for d = 1 to 8, 12 and 16 each, one for steps whose trees all
+// have another d, and one for trees of mixed d.
+constexpr int kMixedD = 0, kOtherD = -1;
+
+// Dynamic shared memory of two buffers at most.
+__host__ __device__ constexpr uint32_t most_smem(int kD) { return kD == kOtherD ? kScatterLargeSmemBytes : kScatterSmemBytes; }
+
+// Points of which two buffers in so many bytes have room, at most 1024.
+__host__ __device__ constexpr uint32_t sub_tile_room(int d, uint32_t smem) {
+  const uint32_t most = smem / 8u / (uint32_t)(d + 1) - 4u;
+  return most < 1024u ? most : 1024u;
+}
+// Points of a sub-tile. An instance for one d gives every consumer thread the
+// same number of them: a power of two. The others take as few equal parts of a
+// tile as have room, in whole warps: how many points are in flight bounds them,
+// and a power of two would leave up to half of the buffers empty. kdt_build of
+// 2,000,003 points, 64 subsets, leaves of 64, widest spread, at d = 9, 23, 40 and
+// 64: 1.86, 4.51, 11.6 and 18.1 ms with a power of two and three CTAs per SM, 1.70,
+// 3.81, 8.6 and 18.1 with parts of a tile, 1.54, 3.14, 6.5 and 13.8 with parts, two
+// CTAs and kScatterLargeSmemBytes each.
+__host__ __device__ constexpr uint32_t sub_tile_one(int d) {
   uint32_t T = 1024;
-  while (T > 32 && 2u * buf_bytes(d, T) > kScatterSmemBytes) T >>= 1;
+  while (T > sub_tile_room(d, kScatterSmemBytes)) T >>= 1;
   return T;
 }
+__host__ __device__ constexpr uint32_t sub_tile_any(int d, uint32_t smem) {
+  const uint32_t room = sub_tile_room(d, smem) / 32u * 32u, parts = ((uint32_t)kTile + room - 1u) / room;
+  return ((uint32_t)kTile + 32u * parts - 1u) / (32u * parts) * 32u;
+}
+static_assert(sub_tile_any(kMaxDims, kScatterSmemBytes) >= 32u, "every d has a sub-tile");
 
 // Resident CTAs per SM of an instance. A sub-tile costs its barriers, its scan
 // and a round trip to L2 whatever it holds, so what bounds a launch of few
@@ -68,11 +91,11 @@ __host__ __device__ constexpr uint32_t sub_tile(int d) {
 // 1.37 with four (0.18 per level at 6.8 TB/s would be 1.1). At d = 8 without
 // min / max two buffers of nine columns fit three times; with them the
 // accumulators take 94 registers, and three CTAs spill (28.0 against 26.8 ms
-// per build of 2^27 points). The instance for any d (forests of mixed d) takes
+// per build of 2^27 points). The instance for mixed d takes
 // 72 registers, so three CTAs too: a forest of 512 trees spent 2.38 ms in it
 // with two CTAs of 100 KB each, 1.81 with three of 72.5.
 constexpr int scatter_ctas(int kD, bool kMM) {
-  if ((kD == 7 || kD == 8) && kMM) return 2;
+  if (((kD == 7 || kD == 8) && kMM) || kD == kOtherD) return 2;
   return kD >= 2 && kD <= 5 && !kMM ? 4 : 3;
 }
 
@@ -94,16 +117,16 @@ struct SubMeta {
   uint32_t ph[kMaxDims + 1];  // alignment phase of each staged word column
 };
 
-// kD > 0: compiled for trees of kD coordinates (the column loops unroll);
-// kD = 0: any d. kMM: some tree of the step uses widest spread.
+// kD > 0: compiled for trees of kD coordinates (the column loops unroll); else
+// any d. kMM: some tree of the step uses widest spread.
 template <int kD, bool kMM>
 __global__ void __launch_bounds__(kST, scatter_ctas(kD, kMM)) k_scatter_tma(const TreeDev* trees, StepDev s) {
   chain_wait();
-  constexpr int kMaxItems = kD > 0 ? (int)(sub_tile(kD > 0 ? kD : 1) / kCT) : 4;  // points per consumer thread
-  // words of a buffer (kD = 0: trees of several d may follow one another, so
+  constexpr int kMaxItems = kD > 0 ? (int)(sub_tile_one(kD > 0 ? kD : 1) / kCT) : 4;  // points per consumer thread
+  // words of a buffer (for any d: trees of several d may follow one another, so
   // the halves are fixed)
   constexpr uint32_t kBufWords =
-      (kD > 0 ? buf_bytes(kD > 0 ? kD : 1, (uint32_t)(kMaxItems * kCT)) : kScatterSmemBytes / 2) / 4;
+      (kD > 0 ? buf_bytes(kD > 0 ? kD : 1, (uint32_t)(kMaxItems * kCT)) : most_smem(kD) / 2) / 4;
   extern __shared__ __align__(128) uint32_t sm[];
   __shared__ __align__(8) uint64_t full[2], empty[2];
   __shared__ SubMeta meta[2];
@@ -146,7 +169,7 @@ __global__ void __launch_bounds__(kST, scatter_ctas(kD, kMM)) k_scatter_tma(cons
       const bool run_more = tile + 1 < t_end && tl_next.x == tl.x;
       const TreeDev& tg = trees[c.tree];
       const int d = kD > 0 ? kD : tg.d, ncols = d + 1;
-      const uint32_t T = kD > 0 ? (uint32_t)(kMaxItems * kCT) : sub_tile(d), stride = col_stride(T);
+      const uint32_t T = kD > 0 ? (uint32_t)(kMaxItems * kCT) : sub_tile_any(d, most_smem(kD)), stride = col_stride(T);
       const uint32_t tend = min(tl.y + (uint32_t)kTile, c.count);
       const float* X = src_cols(tg, c.level);
       const uint32_t* P = src_perm(tg, c.level);
@@ -535,9 +558,8 @@ __global__ void __launch_bounds__(kST, scatter_ctas(kD, kMM)) k_scatter_tma(cons
 
 }  // namespace
 
-// Dynamic shared memory of an instance for trees of d coordinates (kD = 0:
-// the most a mix can need).
-constexpr uint32_t scatter_smem(int kD) { return kD > 0 ? 2u * buf_bytes(kD, sub_tile(kD)) : kScatterSmemBytes; }
+// Dynamic shared memory of an instance (for any d: the most a mix can need).
+constexpr uint32_t scatter_smem(int kD) { return kD > 0 ? 2u * buf_bytes(kD, sub_tile_one(kD)) : most_smem(kD); }
 
 template <int kD, bool kMM>
 cudaError_t prepare_one() {
@@ -552,12 +574,12 @@ void launch_one(const TreeDev* trees, const StepDev& s, uint32_t max_tiles, uint
   launch_chained(k_scatter_tma<kD, kMM>, grid, kST, scatter_smem(kD), st, trees, s);
 }
 
-// f(instance) for the trees' coordinate count: compiled for 1 to 8, 12 and 16.
+// f(instance) for the trees' coordinate count (0: they differ).
 // (3,000,017 points in 5 coordinates, depth rule: the scatters of a build took
 // 0.67 ms in the instance for any d and take 0.49 ms in their own.)
 template <bool kMM, class F>
-auto with_d(int d, F f) {
-  switch (d) {
+auto with_d(int uniform_d, F f) {
+  switch (uniform_d) {
     case 1: return f(std::integral_constant<int, 1>{});
     case 2: return f(std::integral_constant<int, 2>{});
     case 3: return f(std::integral_constant<int, 3>{});
@@ -568,7 +590,8 @@ auto with_d(int d, F f) {
     case 8: return f(std::integral_constant<int, 8>{});
     case 12: return f(std::integral_constant<int, 12>{});
     case 16: return f(std::integral_constant<int, 16>{});
-    default: return f(std::integral_constant<int, 0>{});
+    default:
+      return uniform_d > 0 ? f(std::integral_constant<int, kOtherD>{}) : f(std::integral_constant<int, kMixedD>{});
   }
 }
 
