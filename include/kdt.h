@@ -364,7 +364,8 @@ kdt_status kdt_build_sharded(const float *points, const kdt_params *p, int32_t s
  * region can reach are visited. The tree is a build's output: points (device,
  * float32 SoA [d][n], the build's input), perm, split_vals, split_dims and
  * node_offsets (device) and L = levels. Query arrays are device SoA [d][nq].
- * One warp per query; the call returns when the results are written.
+ * One warp per query, or one thread where many searches see few points each;
+ * the call returns when the results are written.
  * Errors: KDT_ERR_INVALID_ARG (sizes out of range, missing pointers),
  *         KDT_ERR_CUDA. */
 

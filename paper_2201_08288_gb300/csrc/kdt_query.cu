@@ -11,7 +11,8 @@
 //
 // One warp per query, depth first with an explicit stack (at most one node
 // per level: the lanes hold it, lane s entry s), a leaf's points 32 at a time,
-// one per lane.
+// one per lane. Many searches of few points each go a thread per query (see
+// "searches by a thread").
 //   Box: a point is inside when lo_j <= x_j <= hi_j for every coordinate j,
 //   compared as keys; the left child is visited when key(lo_t) <= split key,
 //   the right when key(hi_t) > split key.
@@ -131,7 +132,8 @@ __device__ __forceinline__ bool nearer(double a, uint32_t ia, double b, uint32_t
   return a < b || (a == b && ia < ib);
 }
 
-__device__ __forceinline__ double dist2(const TreeView& tv, const float* q, uint32_t i) {
+// (coordinate j of the query at q[j stride])
+__device__ __forceinline__ double dist2(const TreeView& tv, const float* q, uint32_t i, int64_t stride = 1) {
   double d2 = 0.0;
   for (int j0 = 0; j0 < tv.d; j0 += kDimChunk) {
     float x[kDimChunk];
@@ -141,7 +143,7 @@ __device__ __forceinline__ double dist2(const TreeView& tv, const float* q, uint
 #pragma unroll
     for (int j = 0; j < kDimChunk; ++j)
       if (j0 + j < tv.d) {
-        const double df = __dsub_rn((double)x[j], (double)q[j0 + j]);
+        const double df = __dsub_rn((double)x[j], (double)q[(j0 + j) * stride]);
         d2 = __dadd_rn(d2, __dmul_rn(df, df));
       }
   }
@@ -152,7 +154,8 @@ __device__ __forceinline__ double dist2(const TreeView& tv, const float* q, uint
 // Queries that meet a distance that is no number (infinities of one sign on
 // both sides, NaN in the query) go this way: such distances are in no order,
 // so which of them are kept is fixed by the sequence alone.
-__device__ void knn_serial(const TreeView& tv, const float* q, int k, uint32_t* out_idx, double* out_d2) {
+__device__ void knn_serial(const TreeView& tv, const float* q, int64_t stride, int k, uint32_t* out_idx,
+                           double* out_d2) {
   for (int j = 0; j < k; ++j) {
     out_d2[j] = __longlong_as_double(0x7ff0000000000000ll);  // +inf
     out_idx[j] = 0xffffffffu;
@@ -171,7 +174,7 @@ __device__ void knn_serial(const TreeView& tv, const float* q, int k, uint32_t* 
     const int l = level_of(h);
     const int t = l < tv.L ? (int)tv.dims[h] : -1;
     if (t >= 0) {
-      const float mv = tv.vals[h], qv = q[t];
+      const float mv = tv.vals[h], qv = q[t * stride];
       const double diff = __dsub_rn((double)qv, (double)mv);
       const bool q_left = ord_key(qv) <= ord_key(mv);
       stack_h[sp] = q_left ? 2u * h + 2u : 2u * h + 1u;  // the farther child, visited last
@@ -183,7 +186,7 @@ __device__ void knn_serial(const TreeView& tv, const float* q, int k, uint32_t* 
     const uint32_t leaf = first_leaf(tv, h, l);
     for (int64_t p = tv.offs[leaf]; p < tv.offs[leaf + 1]; ++p) {
       const uint32_t i = tv.perm[p];
-      const double d2 = dist2(tv, q, i);
+      const double d2 = dist2(tv, q, i, stride);
       if (nbest == k && !nearer(d2, i, out_d2[k - 1], out_idx[k - 1])) continue;
       int pos = nbest < k ? nbest++ : k - 1;
       for (int j = k - 1; j > 0; --j)
@@ -429,8 +432,142 @@ __global__ void __launch_bounds__(kQueryThreads) k_query_knn(TreeView tv, const 
   out_d2 += (size_t)qi * k;
   KnnResult r = knn_warp<false>(tv, q, k, lane, out_idx, out_d2);
   if (r == KNN_AGAIN) r = knn_warp<true>(tv, q, k, lane, out_idx, out_d2);
-  if (r == KNN_ODD && lane == 0) knn_serial(tv, q, k, out_idx, out_d2);
+  if (r == KNN_ODD && lane == 0) knn_serial(tv, q, 1, k, out_idx, out_d2);
 }
+
+// ----------------------------------------------- searches by a thread
+//
+// A warp spends as many instructions on a node, or on a leaf of one point, as a
+// thread does, so searches that see few points are cheaper 32 at a time, by a
+// thread each, once there are enough of them for the threads to hide their loads.
+// The lines below are drawn from n / 2^L, all that the host knows of the leaves (in
+// depth mode their points, in leaf mode a third to an eighth of them), the number of
+// queries and d. Measured, a warp's time over a thread's, among 1,000,003 points in
+// 3 coordinates, boxes of half a point to 60 points: 1,000,003 queries, leaves of 1
+// (n / 2^L 0.12) 4.8 to 4.5, of 8 (0.95) 3.2 to 2.1, of 16 (3.8) 2.2 to 1.35, of 32
+// (7.6) 1.5 to 0.92, of 64 1.1 to 0.8; 300,000 queries 3.9 to 4.4, 2.5 to 1.9, 1.8
+// to 1.2, 1.2 to 0.8; 100,000 queries 2.0, 1.3 to 1.0, 1.0 to 0.7; 50,000 queries
+// 1.3, 1.0 to 0.6. In 8 coordinates 300,000 queries in leaves of 8 (1.1) 1.4 to 1.1,
+// of 16 (4.6) 0.9 to 0.7. The nearest point of a point of the tree, and of a place
+// beside one: 1,000,003 queries, leaves of 1 3.8 and 1.6, of 4 (0.48) 2.8 and 1.2,
+// of 8 2.2 and 0.9; 300,000 queries 3.1 and 1.1, 2.4 and 0.9, 1.9 and 0.6; in 2
+// coordinates 3.5 and 2.2, 2.9 and 2.0, 2.3 and 1.65, of 16 (3.8) 1.7 and 1.2. (More
+// coordinates, more leaves around a place; and the threads measure in double. More
+// than one neighbour was never better.)
+constexpr int kEachThreads = 128;
+constexpr int32_t kEachMin = 32768;
+
+float mean_leaf(const TreeView& tv) { return std::ldexp((float)tv.n, -tv.L); }
+bool each_box(const TreeView& tv, int32_t nq) {
+  return nq >= kEachMin && mean_leaf(tv) * (float)tv.d <= std::min(24.0f, 1.1f * std::pow((float)nq / 50000.0f, 1.25f));
+}
+bool each_nearest(const TreeView& tv, int32_t nq) {
+  return nq >= kEachMin && mean_leaf(tv) * std::pow(5.0f, (float)(tv.d - 2)) <= std::min(4.0f, (float)nq / 75000.0f);
+}
+
+__global__ void __launch_bounds__(kEachThreads) k_box_each(TreeView tv, const float* lo, const float* hi, int32_t nq,
+                                                           uint32_t* count, uint32_t* list, uint32_t cap) {
+  const int64_t qi = (int64_t)blockIdx.x * kEachThreads + threadIdx.x;
+  if (qi >= nq) return;
+  lo += qi;
+  hi += qi;
+  uint32_t stack[KDT_MAX_LEVELS + 1];  // right children left for later, one per level at most
+  int sp = 0;
+  uint32_t h = 0, leaf = 0, found = 0;
+  auto next_leaf = [&]() {  // from h on; false: none is left
+    for (;;) {
+      const int l = level_of(h), t = l < tv.L ? (int)tv.dims[h] : -1;
+      if (t < 0) {
+        leaf = first_leaf(tv, h, l);
+        return true;
+      }
+      const uint32_t m = ord_key(tv.vals[h]);
+      const bool left = ord_key(lo[(int64_t)t * nq]) <= m, right = ord_key(hi[(int64_t)t * nq]) > m;
+      if (left || right) {
+        if (left && right) stack[sp++] = 2u * h + 2u;
+        h = left ? 2u * h + 1u : 2u * h + 2u;
+      } else {
+        if (sp == 0) return false;
+        h = stack[--sp];
+      }
+    }
+  };
+  // (the lanes of a warp go down together, then read their leaves together)
+  while (next_leaf()) {
+    for (int64_t p = tv.offs[leaf]; p < tv.offs[leaf + 1]; ++p) {
+      const uint32_t i = tv.perm[p];
+      bool in = true;
+      for (int j = 0; j < tv.d && in; ++j) {
+        const uint32_t kx = ord_key(tv.x[(int64_t)j * tv.n + i]);
+        in = ord_key(lo[(int64_t)j * nq]) <= kx && kx <= ord_key(hi[(int64_t)j * nq]);
+      }
+      if (in) {
+        if (list && found < cap) list[(size_t)qi * cap + found] = i;
+        ++found;
+      }
+    }
+    if (sp == 0) break;
+    h = stack[--sp];
+  }
+  count[qi] = found;
+}
+
+// The nearest point (k = 1). A search that meets a distance that is no number goes
+// the serial way.
+__global__ void __launch_bounds__(kEachThreads) k_nearest_each(TreeView tv, const float* qs, int32_t nq,
+                                                               uint32_t* out_idx, double* out_d2) {
+  const int64_t qi = (int64_t)blockIdx.x * kEachThreads + threadIdx.x;
+  if (qi >= nq) return;
+  qs += qi;
+  uint32_t stack_h[KDT_MAX_LEVELS + 1];
+  float stack_b[KDT_MAX_LEVELS + 1];  // at most the squared distance of any point below the node
+  int sp = 0;
+  double best = __longlong_as_double(0x7ff0000000000000ll);  // +inf
+  uint32_t best_i = 0xffffffffu, h = 0;
+  float bound = 0.0f;
+  bool odd = false;
+  auto descend = [&]() {  // from h to the leaf on the query's side
+    for (;;) {
+      const int l = level_of(h), t = l < tv.L ? (int)tv.dims[h] : -1;
+      if (t < 0) return first_leaf(tv, h, l);
+      const float mv = tv.vals[h], qv = qs[(int64_t)t * nq], diff = __fsub_rz(qv, mv);
+      const float fb = fmaxf(bound, __fmul_rd(diff, diff));
+      const bool q_left = ord_key(qv) <= ord_key(mv);
+      if (!((double)fb > best)) {  // the farther child waits
+        stack_h[sp] = q_left ? 2u * h + 2u : 2u * h + 1u;
+        stack_b[sp++] = fb;
+      }
+      h = q_left ? 2u * h + 1u : 2u * h + 2u;
+    }
+  };
+  for (bool more = true; more && !odd;) {
+    const uint32_t leaf = descend();
+    for (int64_t p = tv.offs[leaf]; p < tv.offs[leaf + 1]; ++p) {
+      const uint32_t i = tv.perm[p];
+      double d2 = 0.0;
+      for (int j = 0; j < tv.d; ++j) {
+        const double df = __dsub_rn((double)tv.x[(int64_t)j * tv.n + i], (double)qs[(int64_t)j * nq]);
+        d2 = __dadd_rn(d2, __dmul_rn(df, df));
+      }
+      odd |= d2 != d2;
+      if (nearer(d2, i, best, best_i)) {
+        best = d2;
+        best_i = i;
+      }
+    }
+    more = false;
+    while (sp > 0 && !more) {
+      bound = stack_b[--sp];
+      more = !((double)bound > best);
+      h = stack_h[sp];
+    }
+  }
+  out_idx[qi] = best_i;
+  out_d2[qi] = best;
+  if (odd) knn_serial(tv, qs, nq, 1, out_idx + qi, out_d2 + qi);
+}
+
+uint32_t blocks_of(int32_t nq, int per) { return ((uint32_t)nq + (uint32_t)per - 1u) / (uint32_t)per; }
 
 kdt_status check_tree(const float* points, int64_t n, int32_t d, const uint32_t* perm, const float* vals,
                       const int8_t* dims, const int64_t* offs, int32_t L) {
@@ -461,8 +598,10 @@ kdt_status kdt_query_box(const float* points, int64_t n, int32_t d, const uint32
   cudaStream_t st = (cudaStream_t)stream;
   {
     TraceScope ts(K_QUERY, st, (uint64_t)nq);
-    k_query_box<<<((uint32_t)nq + kQueryWarps - 1) / kQueryWarps, kQueryThreads, 0, st>>>(tv, lo, hi, nq, out_count,
-                                                                                          out_list, list_cap);
+    if (each_box(tv, nq))
+      k_box_each<<<blocks_of(nq, kEachThreads), kEachThreads, 0, st>>>(tv, lo, hi, nq, out_count, out_list, list_cap);
+    else
+      k_query_box<<<blocks_of(nq, kQueryWarps), kQueryThreads, 0, st>>>(tv, lo, hi, nq, out_count, out_list, list_cap);
   }
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
     (void)cudaGetLastError();
@@ -484,8 +623,10 @@ kdt_status kdt_query_knn(const float* points, int64_t n, int32_t d, const uint32
   cudaStream_t st = (cudaStream_t)stream;
   {
     TraceScope ts(K_QUERY, st, (uint64_t)nq);
-    k_query_knn<<<((uint32_t)nq + kQueryWarps - 1) / kQueryWarps, kQueryThreads, 0, st>>>(tv, queries, nq, k, out_idx,
-                                                                                          out_dist2);
+    if (k == 1 && each_nearest(tv, nq))
+      k_nearest_each<<<blocks_of(nq, kEachThreads), kEachThreads, 0, st>>>(tv, queries, nq, out_idx, out_dist2);
+    else
+      k_query_knn<<<blocks_of(nq, kQueryWarps), kQueryThreads, 0, st>>>(tv, queries, nq, k, out_idx, out_dist2);
   }
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
     (void)cudaGetLastError();
