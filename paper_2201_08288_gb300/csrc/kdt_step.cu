@@ -28,6 +28,7 @@
 #include "kdt_internal.cuh"
 #include "kdt_launch.h"
 #include "kdt_ptx.cuh"
+#include "kdt_runs.h"
 #include "kdt_trace.h"
 
 namespace kdt {
@@ -619,7 +620,7 @@ __device__ __forceinline__ uint32_t thread_lower_median(const uint32_t* keys, ui
   return med;
 }
 
-// One thread per segment of at most tiny_max <= kSelTinyMax points (the
+// One thread per segment of at most tiny_max <= 64 points (the
 // threads stride over the segments of the step). The network's size is
 // chosen per warp, by the warp's largest segment, so a warp never runs two.
 // Five CTAs per SM by a register bound (48 registers): the path waits on its
@@ -1211,30 +1212,35 @@ static_assert(kFourierTerms * 2 <= kTileRecWords, "a tile's sums fit its record"
 
 // The sums over a cell's points of the basis terms of Lemma 1 on its key
 // coordinate, c_0 = 1, c_{2j-1} = cos((2j-1)x), c_{2j} = sin((2j-1)x) for
-// j = 1..J (the additive statistics of Sec. 3.2). The kernel is persistent:
-// CTA k takes the tiles [k T / G, (k+1) T / G) of the step (T tiles, G
-// CTAs). Each thread holds 8 points of a tile and runs the odd harmonics
-// for all of them at once (h(k+2) = 2 cos(2x) h(k) - h(k-2), from one sincosf
-// per point), adding each harmonic's terms in float, then over the warp by
-// a shuffle tree in float (double arithmetic is scarce on this GPU); the CTA
-// adds the warps' sums in double in a fixed order into a running total per
-// term, written to the record of the run's first tile when the
-// CTA's run of the cell's tiles ends. The split kernel adds a cell's run
-// records in order, so the result does not depend on scheduling. A
-// coordinate outside (0,1) is reported.
+// j = 1..J (the additive statistics of Sec. 3.2). The kernel is persistent: CTA k
+// takes the runs (kdt_runs.h) that start among the tiles [k T / G, (k+1) T / G) of
+// the step (T tiles, G CTAs). Each thread holds 8 points of a tile and runs the odd
+// harmonics for all of them at once (h(k+2) = 2 cos(2x) h(k) - h(k-2), from one
+// sincosf per point), adding each harmonic's terms in float, then over the warp by
+// a shuffle tree in float (double arithmetic is scarce on this GPU); the CTA adds
+// the warps' sums in double in a fixed order into a running total per term,
+// written to the record of the run's first tile when the run ends. The split
+// kernel adds a cell's run records in an order that their number fixes, so the
+// result does not depend on scheduling. A coordinate outside (0,1) is reported.
 __global__ void __launch_bounds__(256, 2) k_fourier_moments(const TreeDev* trees, StepDev s) {
   chain_wait();
   constexpr int kPer = kTile / 256;
   __shared__ float red[8][kFourierTerms];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t ntiles = ntiles_of(s);
-  const uint32_t t_begin = (uint32_t)(((uint64_t)blockIdx.x * ntiles) / gridDim.x);
-  const uint32_t t_end = (uint32_t)(((uint64_t)(blockIdx.x + 1) * ntiles) / gridDim.x);
+  auto start_from = [&](uint32_t tile) {
+    if (tile >= ntiles) return ntiles;
+    const uint2 tl = s.tiles[tile];
+    const Cell cell = s.cells[tl.x];
+    return run_start(tile, tl.y / (uint32_t)kTile, tiles_of(cell.count), run_tiles(tiles_of((uint32_t)trees[cell.tree].n)));
+  };
+  const uint32_t t_begin = start_from((uint32_t)(((uint64_t)blockIdx.x * ntiles) / gridDim.x));
+  const uint32_t t_end = start_from((uint32_t)(((uint64_t)(blockIdx.x + 1) * ntiles) / gridDim.x));
   // a tile's record, cell and this thread's points (loaded one tile ahead)
   struct Ahead {
     uint2 tl;
     int32_t tree;
-    uint32_t end;
+    uint32_t end, run;
     float x[kPer];
   };
   auto fetch = [&](uint32_t tile, Ahead& a) {
@@ -1243,6 +1249,7 @@ __global__ void __launch_bounds__(256, 2) k_fourier_moments(const TreeDev* trees
     const TreeDev& t = trees[cell.tree];
     const float* X = (const float*)key_column(t, cell, s.kdim[a.tl.x]) + cell.begin;
     a.tree = cell.tree;
+    a.run = run_tiles(tiles_of((uint32_t)t.n));
     a.end = min(a.tl.y + (uint32_t)kTile, cell.count);
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
@@ -1310,8 +1317,9 @@ __global__ void __launch_bounds__(256, 2) k_fourier_moments(const TreeDev* trees
       for (int w = 0; w < 8; ++w) v += (double)red[w][threadIdx.x];
       run += v;
     }
-    // the CTA's run of this cell's tiles ends here: write its record
-    if (tile + 1 == t_end || nxt.tl.x != cur.tl.x) {
+    // the run ends here: write its record
+    if (tile + 1 == t_end || nxt.tl.x != cur.tl.x ||
+        (cur.tl.y / (uint32_t)kTile + 1u) % cur.run == 0u) {
       if ((int)threadIdx.x <= 2 * J) ((double*)(s.tile_mm + (size_t)run_first * kTileRecWords))[threadIdx.x] = run;
       run = 0.0;
       run_first = tile + 1;
@@ -1321,8 +1329,8 @@ __global__ void __launch_bounds__(256, 2) k_fourier_moments(const TreeDev* trees
   }
 }
 
-// Per cell, one CTA: the cell's sums C_j (its run records added in order,
-// thread j term j), its bounds (a, b) on its key coordinate (the splits of its
+// Per cell, one CTA: the cell's sums C_j (its run records, every G-th by one of G
+// threads per term, then the G partial sums in order), its bounds (a, b) on its key coordinate (the splits of its
 // ancestors on that coordinate, (0,1) at the root), and the root of Eq.
 // (kd:eq:b) by 60 bisection steps in double on (a, b) of F(m) = 1_J(a, m) -
 // 1_J(m, b) = sum_j C_j (g_j(a, m) - g_j(m, b)), with g_j of Lemma 1: the term
@@ -1349,13 +1357,14 @@ __global__ void __launch_bounds__(256, 2) k_fourier_moments(const TreeDev* trees
 //   half a warp per candidate adds its terms, in the order and tree of the
 //     one-warp form, so the splits are the same bits; the signs are the round's
 //     outcome.
-// The start of every run record comes from a 64-bit division: formed once per
-// chunk of them, by a lane each (a thread that formed its own spent 347,000
-// cycles on the root's 304). 4,000,037 points, J = 16, ten levels: 0.60 ms per
-// build; 1.86 with a warp per cell.
+// The records are loaded eight at a time per thread, so that a root's thousands
+// wait for few round trips; their sums are split over as many threads as there are,
+// since a double addition occupies a quarter of an SM for 64 cycles. 4,000,037
+// points, J = 16, ten levels: 0.50 ms per build; 0.58 with the records staged 32 at
+// a time and one thread per term, 1.86 with a warp per cell.
 constexpr int kFsSteps = 3, kFsCand = 1 << kFsSteps;  // candidates 1 .. kFsCand - 1
 constexpr int kFsThreads = 256;
-constexpr int kFsChunk = 32;  // run records staged at a time
+constexpr int kFsParts = 8;  // partial sums of a term at most
 static_assert((kFsCand - 1) * KDT_FOURIER_MAX_J <= kFsThreads, "a thread per candidate and harmonic");
 static_assert((kFsCand - 1) * 16 <= kFsThreads && 4 * KDT_FOURIER_MAX_J <= kFsThreads, "threads for the other parts");
 
@@ -1391,62 +1400,47 @@ __device__ __forceinline__ double widen(float x) {
   return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu)), (int)(u << 29));
 }
 
-__global__ void __launch_bounds__(kFsThreads) k_fourier_split(const TreeDev* trees, StepDev s, uint32_t mgrid) {
+__global__ void __launch_bounds__(kFsThreads) k_fourier_split(const TreeDev* trees, StepDev s) {
   chain_wait();
-  __shared__ double rec[kFsChunk][kFourierTerms];
+  __shared__ double s_part[kFsParts][kFourierTerms];
   __shared__ double s_base[kFourierTerms], s_slope[kFourierTerms];
   __shared__ double s_wave[4][KDT_FOURIER_MAX_J];  // sin K a, sin K b, cos K a, cos K b
   __shared__ double s_mid[2][kFsCand][kFsCand];  // by round's parity, outcome of the round before, candidate
   __shared__ double s_end[2][kFsCand][2];        // and each outcome's (lo, hi)
   __shared__ double s_term[kFsCand][96];
   __shared__ uint32_t s_neg[2];  // by round's parity; bit w: F < 0 at candidate w's midpoint
-  __shared__ uint32_t s_run[kFsChunk], s_nrun;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t nc = ncells_of(s);
-  const uint32_t ntiles = ntiles_of(s);
-  auto range_start = [&](uint32_t k) { return (uint32_t)(((uint64_t)k * ntiles) / mgrid); };
   for (int i = tid; i < kFsCand * 96; i += kFsThreads) (&s_term[0][0])[i] = 0.0;  // terms that no tree here has
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
     const Cell cell = s.cells[c];
     const TreeDev& t = trees[cell.tree];
     const int J = t.fourier_j, nt = 2 * J + 1;
-    const uint32_t tb = cell.tile0, te = tb + tiles_of(cell.count);
-    // The moments kernel's runs of this cell start at tb and at every start of
-    // a CTA's tile range inside (tb, te): with at least as many tiles as CTAs
-    // the starts of ranges k0 + 1, k0 + 2, ... (k0: the range that holds tb),
-    // with fewer every tile.
-    uint32_t k0 = 0;
-    const bool dense = ntiles < mgrid;
-    if (!dense) {
-      const uint64_t kk = ((uint64_t)tb * mgrid) / (ntiles > 0u ? ntiles : 1u);
-      k0 = (uint32_t)(kk < (uint64_t)mgrid ? kk : (uint64_t)(mgrid - 1u));
-      while (k0 > 0u && range_start(k0) > tb) --k0;
-      while (k0 + 1u < mgrid && range_start(k0 + 1u) <= tb) ++k0;
-    }
-    auto run_start = [&](uint32_t m) -> uint32_t {  // te: no such run
-      if (m == 0u) return tb;
-      if (dense) return min(tb + m, te);
-      return k0 + m < mgrid ? min(range_start(k0 + m), te) : te;
-    };
-    double C = 0.0;  // thread j: the sum of term j
-    for (uint32_t m0 = 0;; m0 += kFsChunk) {
-      if (warp == 0) {
-        const uint32_t r0 = run_start(m0 + (uint32_t)lane);
-        s_run[lane] = r0;
-        const unsigned some = __ballot_sync(0xffffffffu, r0 < te);
-        if (lane == 0) s_nrun = (uint32_t)__popc(some);
+    // thread (part, term): the sum of every parts-th run record
+    const uint32_t len = run_tiles(tiles_of((uint32_t)t.n)), nrun = (tiles_of(cell.count) + len - 1u) / len;
+    const int parts = min(kFsParts, kFsThreads / nt), part = tid / nt;
+    if (part < parts) {
+      const int j = tid % nt;
+      const double* first = (const double*)(s.tile_mm + (size_t)cell.tile0 * kTileRecWords) + j;
+      const size_t step = (size_t)len * (kTileRecWords / 2);
+      double sum = 0.0;
+      for (uint32_t m0 = (uint32_t)part; m0 < nrun; m0 += 8u * (uint32_t)parts) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const uint32_t m = m0 + (uint32_t)(u * parts);
+          v[u] = m < nrun ? first[m * step] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (m0 + (uint32_t)(u * parts) < nrun) sum += v[u];
       }
-      __syncthreads();
-      const uint32_t nrun = s_nrun;
-      for (uint32_t m = warp; m < nrun; m += kFsThreads / 32)
-        for (int j = lane; j < nt; j += 32)
-          rec[m][j] = ((const double*)(s.tile_mm + (size_t)s_run[m] * kTileRecWords))[j];
-      __syncthreads();
-      if (tid < nt)
-        for (uint32_t m = 0; m < nrun; ++m) C += rec[m][tid];
-      __syncthreads();
-      if (nrun < (uint32_t)kFsChunk) break;
+      s_part[part][j] = sum;
     }
+    __syncthreads();
+    double C = 0.0;  // thread j: the sum of term j
+    if (tid < nt)
+      for (uint32_t p = 0; p < min((uint32_t)parts, nrun); ++p) C += s_part[p][tid];
     // bounds: lane i of every warp takes the i-th ancestor (splits are in
     // [0, 1], where floats order like their bits)
     const uint32_t dim = s.kdim[c];
@@ -2083,7 +2077,7 @@ void launch_big_step(const TreeDev* trees, const StepDev& s, uint32_t max_tiles,
     }
     {
       TraceScope ts(K_FOURIER_SPLIT, st);
-      launch_chained(k_fourier_split, cells_grid(1, sms * 4u), kFsThreads, 0, st, trees, s, mgrid);
+      launch_chained(k_fourier_split, cells_grid(1, sms * 4u), kFsThreads, 0, st, trees, s);
     }
   } else {
     if (s.few_segs) {
