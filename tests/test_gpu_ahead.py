@@ -14,6 +14,7 @@ from test_gpu_fourier import check_tree
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+KDT_ERR_LEVEL_CAP = 7
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -42,13 +43,16 @@ def test_steps_ahead(kind, n, d, r, mode, rule, kw):
     from paper_2201_08288_gb300 import kdt
     x = _points(kind, n, d)
     kw = dict(kw, r=r, subset_mode=mode, key_rule=rule)
+    X = torch.from_numpy(x).cuda()
     try:
         o = oracle.build_tree(x, **kw)
-    except oracle.OracleError:
-        with pytest.raises(kdt.KdtError):
-            kdt.kdt_build(torch.from_numpy(x).cuda(), **kw)
-        return
-    g = kdt.kdt_build(torch.from_numpy(x).cuda(), **kw)
+    except oracle.OracleError:  # more levels than the cap: refused for that, and a build with room works after it
+        with pytest.raises(kdt.KdtError) as err:
+            kdt.kdt_build(X, **kw)
+        assert err.value.status == KDT_ERR_LEVEL_CAP
+        kw.update(max_levels=25, leaf_size=max(kw["leaf_size"], 200))
+        o = oracle.build_tree(x, **kw)
+    g = kdt.kdt_build(X, **kw)
     assert g.levels == o.levels
     assert np.array_equal(g.perm.cpu().numpy().view(np.uint32), o.perm)
     assert np.array_equal(g.split_vals.cpu().numpy().view(np.uint32), o.split_vals.view(np.uint32))

@@ -1,7 +1,8 @@
 """GPU: the tuning of the select paths changes only speed. Under every choice
-of every kdt_tuning field (and all four shapes of the CTA radix select) the
-build is bit-identical to the default tuning's, which is checked against the
-oracle; the autotuner returns and installs one of the choices."""
+of every kdt_tuning field the build is bit-identical to the default tuning's,
+which is checked against the oracle, also where the steps list segments of
+every size and are too many for the untuned forms; the autotuner returns and
+installs one of the choices."""
 from __future__ import annotations
 
 import numpy as np
@@ -25,11 +26,12 @@ def _gpu():
 
 
 def _cases():
-    """Segments of every select path: config 3's recipe (r = 256 explicit,
-    widest; root segments of 4096 keys), a cyclic r = 8 tree whose root
-    segments hold 2^17 keys, and a clustered one: uniform on [1, 2), where
-    every key shares its sign and exponent and the CTA select's first digit
-    leaves 2^15 keys in each of four bins."""
+    """Config 3's recipe (r = 256 explicit, widest; root segments of 4096
+    keys), a cyclic r = 8 tree whose root segments hold 2^17 keys, and a
+    clustered one: uniform on [1, 2), where every key shares its sign and
+    exponent and the CTA select's first digit leaves 2^15 keys in each of four
+    bins. (Their first steps have few segments: of the tuning those use the
+    digit width alone, or nothing. test_listed_segments has many.)"""
     s3 = workloads.config3(n=1 << 20, depth=13)
     pts1 = np.random.default_rng(21).standard_normal((3, 1 << 20)).astype(np.float32)
     pts2 = (1.0 + np.random.default_rng(22).random((3, 1 << 18))).astype(np.float32)
@@ -48,10 +50,38 @@ def _tunings():
                 t = dict(d)
                 t[f] = v
                 out.append(t)
-    for th in (256, 512):  # the four shapes of the CTA select, on segments above 1024 keys
+    for th in (256, 512):
         for bits in (8, 11):
             out.append(dict(d, warp_max=1024, cta_threads=th, digit_bits=bits))
     return out
+
+
+@pytest.fixture(scope="module")
+def listed():
+    """A tree whose steps have more segments than the untuned forms take (8 per
+    SM and fewer): 100 to 9000 keys in the root's, so that each warp_max puts others
+    of them on the CTA select, which then has the threads of the tuning."""
+    r = 8 * torch.cuda.get_device_properties(0).multi_processor_count + 61
+    rng = np.random.default_rng(31)
+    sid = np.repeat(np.arange(r, dtype=np.uint16), rng.integers(100, 9000, r))
+    rng.shuffle(sid)
+    pts = rng.standard_normal((2, len(sid))).astype(np.float32)
+    pts[:, rng.random(len(sid)) < 0.1] = 0.25
+    kw = dict(r=r, subset_mode=2, depth=2, key_rule=0)
+    return pts, sid, kw, oracle.build_tree(pts, sid=sid, **kw)
+
+
+@pytest.mark.parametrize("bits", [8, 11])
+@pytest.mark.parametrize("threads", [256, 512])
+@pytest.mark.parametrize("warp_max", [1024, 2048, 4096])
+def test_listed_segments(listed, warp_max, threads, bits):
+    from paper_2201_08288_gb300 import kdt
+    pts, sid, kw, ref = listed
+    kdt.set_tuning(dict(kdt.tuning_default(), warp_max=warp_max, cta_threads=threads, digit_bits=bits))
+    try:
+        assert_same_tree(gpu_build(pts, sid=sid, **kw), ref, f"{warp_max} {threads} {bits}")
+    finally:
+        kdt.set_tuning(None)
 
 
 def test_every_tuning_gives_the_default_bits():
