@@ -26,12 +26,9 @@ namespace kdt {
 
 constexpr int kMaxDims = 64;          // d <= 64
 constexpr int kMaxSubsets = 4096;     // r <= 4096 on the CUDA path
-constexpr int kMaxLevels = 30;        // depth / max_levels <= 30
 constexpr int kTile = 2048;           // points per tile of the multi-CTA pipeline
 constexpr int kTileRecWords = 2 * kMaxDims + 4;  // words of a tile's record in tile_mm (16-byte aligned)
 constexpr int kTileThreads = 256;     // threads of the tile kernels
-constexpr int kSelTinyMax = 64;       // segments up to this size: one thread per segment
-constexpr int kSelSmallMax = 4096;    // largest warp-select segment (kdt_tuning warp_max)
 constexpr int kSelWarpMin = 1024;     // smallest warp_max: sizes the list of CTA-select segments
 
 // status codes (mirror include/kdt.h)
@@ -142,10 +139,10 @@ struct StepDev {
   uint32_t* seg_w;        // [nseg] points per (cell, subset)
   const uint32_t** seg_key; // [nseg] first key of the segment (raw float bits, key column)
   uint32_t* seg_med;      // [nseg] lower median key
-  uint32_t* bigseg;       // [bigseg_cap] segments larger than kSelSmallMax
+  uint32_t* bigseg;       // [bigseg_cap] segments above warp_max keys
   uint32_t* bigseg_count; // device word
   uint32_t* bigseg_count_next;  // the next step's, cleared by this one
-  uint32_t* midseg;       // [midseg_cap] segments of kSelTinyMax+1 .. kSelSmallMax points
+  uint32_t* midseg;       // [midseg_cap] segments of tiny_max+1 .. warp_max keys
   uint32_t* midseg_count; // device word
   uint32_t* midseg_count_next;
   uint32_t few_segs;      // every segment gets a CTA: no lists
@@ -185,7 +182,6 @@ struct StepDev {
   // warp_max, a CTA above
   uint32_t tiny_max, bitonic_max, warp_max;
   uint32_t midseg_cap;
-  uint32_t pad4;
   uint2* crow;                // [ncells][2] (slot, row of off_next) of each big child; (kNoRow, slot in
                               // small) of a child queued for the subtree kernel; else (kNoRow, kNoRow)
   // Sharded build (0 shards: off). The forest's trees 0..shards-1 are the
@@ -261,8 +257,6 @@ __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Terminal test for a cell about to be processed at `level` (reading R8 in
-// leaf mode; empty cells and the last level in depth mode).
 // Cells of a step: the host's count, or the device word a graph-driven step
 // reads (clamped to the capacity of the cell lists).
 __device__ __forceinline__ uint32_t ncells_of(const StepDev& s) {
@@ -285,6 +279,8 @@ __device__ __forceinline__ uint32_t cell_weight(const StepDev& s, uint32_t c, co
   return s.shards ? s.wcount[c] : cell.count;
 }
 
+// Terminal test for a cell about to be processed at `level` (reading R8 in
+// leaf mode; empty cells and the last level in depth mode).
 __device__ __forceinline__ bool is_terminal(const TreeDev& t, uint32_t count, int level, int stall) {
   if (t.depth > 0) return count == 0 || level >= t.depth;
   return count <= (uint32_t)t.leaf_size || stall >= t.stall_limit;
@@ -316,18 +312,6 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
 __device__ __forceinline__ uint32_t warp_sum(uint32_t v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __forceinline__ uint32_t warp_min(uint32_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
-__device__ __forceinline__ uint32_t warp_max(uint32_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
 

@@ -228,7 +228,6 @@ struct TreeHost {
   const TermRec* terms = nullptr;   // device
   uint32_t term_cap = 0;
 };
-size_t leaf_huge_tiles_cap(uint64_t n);
 cudaError_t leaf_sort_huge(const TreeHost& th, const std::vector<TermRec>& recs, cudaStream_t st);
 
 }  // namespace kdt

@@ -441,8 +441,6 @@ void launch_leaf_sort(const TreeDev* trees, const SlotChunks& sc, cudaStream_t s
   launch_chained(k_leaf_sort, sc.chunks, kLsThreads, 0, st, trees, sc);
 }
 
-size_t leaf_huge_tiles_cap(uint64_t n) { return (size_t)(2 * (n / kLeafBlockMax) + 2); }
-
 namespace {
 
 // Leaves of at most kBucketPoints points; those it could not sort go to *rest.

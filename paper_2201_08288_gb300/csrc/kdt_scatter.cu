@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(kST, scatter_ctas(kD, kMM)) k_scatter_tma(cons
       }
       // ---- release the buffer: each warp's reads of it precede the next bulk
       // writes; the "empty" barrier counts the consumer warps (the next
-      // sub-tile's first barrier orders the reuse of wcnt and sedge)
+      // sub-tile's first barrier orders the reuse of wcnt and wbal)
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[b]);

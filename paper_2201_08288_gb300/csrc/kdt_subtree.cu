@@ -22,8 +22,8 @@
 //   6. children: terminal cells are recorded, the others form the next level.
 // The permutation is written once, at the end, gathered from the cell's
 // incoming permutation in global memory. The kernel is persistent: each CTA
-// pulls cells from a queue. It is compiled for the two shapes of
-// kdt_launch.h (positions per thread, CTAs per SM, cell-table size).
+// pulls cells from a queue. It is compiled for the three shapes of
+// kdt_launch.h (threads, positions per thread, CTAs per SM, cell-table size).
 #include <algorithm>
 #include <type_traits>
 
