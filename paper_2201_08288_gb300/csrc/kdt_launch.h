@@ -59,10 +59,11 @@ inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
 // In the first two several CTAs share an SM, each finishing its own cell, so
 // that one CTA's barriers and copies overlap the others' work: that is best
 // while there are more cells than CTAs. With fewer, what a build waits for is
-// the levels above, a chain of launches each (about 35 us a level with its
-// wait), so the tall shape takes cells two levels larger. (65,536 points, d = 3:
-// 427 us in the narrow shape, 382 in the tall one; 300,007 points, d = 16: 829
-// in the wide shape, 675 in the tall one.)
+// the levels above, a chain of launches each (about 25 us a level), so the tall
+// shape takes cells two levels larger. (kdt_build, the shape by d and the tall one:
+// 65,536 points, d = 3 291 and 282 us; 150,001, d = 8 488 and 369; 300,007, d = 16,
+// its 128 cells the most that the rule allows, 528 and 450; 250,001, d = 8, widest
+// spread 467 and 479.)
 struct SubtreeShape {
   int threads;
   int q;        // positions per thread

@@ -1887,7 +1887,10 @@ __global__ void __launch_bounds__(kSplitThreads) k_split(const TreeDev* trees, S
 
 // ------------------------------------------------------------ launcher
 
-constexpr uint32_t kManyCells = 1024;  // from here on: a warp per cell in combine
+// From here on a warp per cell in combine (a line of 256, 1024 and 4096 cells: 1,000,003
+// points, 4096 subsets 1097, 1098 and 1091 us, 3,000,017, 1000 subsets 1.90, 1.90 and
+// 1.87 ms, trees of fewer subsets the same).
+constexpr uint32_t kManyCells = 1024;
 
 // Steps whose launches weigh more than their work: while all segments fit the
 // SMs at once (8 CTAs of 256 threads each) and are of at most 8192 keys on
@@ -1906,11 +1909,16 @@ bool step_selects_all(uint32_t nseg, uint64_t points, uint32_t sms) {
 // 57 us and would take 108 here.
 bool step_selects_wide(uint32_t nseg, uint64_t points) { return nseg <= 32u && points >= 262144ull * nseg; }
 
-// One CTA per cell combines, counts, scans and classifies: while the cells'
-// CTAs fit the SMs at once (4 each) and a cell has at most 64 tiles on average
-// (a warp reads 4).
+// One CTA per cell combines, counts, scans and classifies: in steps of at most two
+// cells per SM, of at most 64 tiles on average (a warp reads 4). (kdt_build of
+// 1,000,003 and 3,000,017 points in 3 coordinates, 16 subsets, and of 2^24, 64: up
+// to four cells per SM 680, 1354 and 3490 us, two 660, 1339 and 3467, one 668, 1342
+// and 3459, half of one 669, 1342 and 3468; with 16 tiles 684, 1362 and 3480, with
+// 256 708, 1366 and 3496, at four cells per SM. In a step ahead both are bounds: a
+// cell with most of the points has one CTA all the same. 16,000,057 points, 95% of
+// them at one place: 20.6 ms, 22.5 with four launches and a wait per step.)
 static bool step_splits(const StepDev& s, uint32_t sms2) {
-  return (!s.ncells_dev || s.bounded) && s.ncells <= 2u * sms2 && s.ntiles <= 64u * s.ncells;
+  return (!s.ncells_dev || s.bounded) && s.ncells <= sms2 && s.ntiles <= 64u * s.ncells;
 }
 
 // The selects by segment size: one thread, one warp, one CTA per segment.
