@@ -256,8 +256,13 @@ kdt_status kdt_server_destroy(kdt_server *s);
  * bitonic network; one warp by brackets from a sample; one CTA with a radix
  * select.
  * Where the paths change, the CTA's size and the width of its radix digits
- * are tunable. Every choice gives the same outputs, bit for bit: the choices
- * trade only speed, and kdt_autotune times them on the caller's own trees.
+ * are tunable. Level steps of few segments settle more of it themselves: up to
+ * 8 per SM, of 8192 keys or fewer on average, take a CTA of 256 threads with
+ * 11-bit digits each, whatever the tuning; a CTA select has 512 threads in steps
+ * of up to 8 segments per SM and 1024 up to 2; up to 32 segments of 262,144 keys
+ * or more on average (above warp_max) take several CTAs each. Every choice gives
+ * the same outputs, bit for bit: the choices trade only speed, and kdt_autotune
+ * times them on the caller's own trees.
  */
 typedef struct kdt_tuning {
   int32_t tiny_max;     /* one thread per segment up to this many keys: 8 to 64 (x2)   */
@@ -296,7 +301,13 @@ kdt_status kdt_autotune(const kdt_tree_desc *trees, int32_t num_trees, void *wor
  * Every kernel launch of the library is counted. With tracing enabled, each
  * launch is also bracketed by two CUDA events recorded on its stream;
  * kdt_trace_read waits for them and reports, per kernel, the number of
- * launches, their summed device time and the points they processed. */
+ * launches, their summed device time and the points they processed. (kdt_build
+ * launches the level steps that are sure to have cells without waiting for
+ * their counts, with grids for the most that there can be. A traced build waits
+ * after every step, since only its counts tell the points: the same kernels on
+ * the same data, but the launches' shapes, the forms that a step takes by its
+ * bounds, and the gaps are those of the waiting build. The smaller the tree, the
+ * more the two differ.) */
 typedef struct kdt_kernel_stat {
   const char *name;   /* kernel name (static string)                       */
   uint64_t launches;  /* timed launches                                    */

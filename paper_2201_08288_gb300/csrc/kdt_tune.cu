@@ -135,6 +135,7 @@ kdt_status kdt_autotune(const kdt_tree_desc* trees, int32_t num_trees, void* wor
   for (const Field& fd : fields)
     for (int k = 0; k < fd.n; ++k) {
       if (fd.choices[k] == b.*(fd.f)) continue;
+      if (fd.f == &kdt_tuning::bitonic_max && fd.choices[k] >= 128 && b.bitonic_max >= 128) continue;  // the same
       kdt_tuning c = b;
       c.*(fd.f) = fd.choices[k];
       float ms = 0.f;
