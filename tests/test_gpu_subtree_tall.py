@@ -13,6 +13,7 @@ from gpu_util import require_gpu
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+KDT_ERR_LEVEL_CAP = 7
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -24,9 +25,10 @@ def _check(x, gsid, sid, **kw):
     from paper_2201_08288_gb300 import kdt
     try:
         o = oracle.build_tree(x, sid=sid, **kw)
-    except oracle.OracleError:  # ties beyond the level cap: refused here too
-        with pytest.raises(kdt.KdtError):
+    except oracle.OracleError:  # ties beyond the level cap: refused here too, for that
+        with pytest.raises(kdt.KdtError) as err:
             kdt.kdt_build(torch.from_numpy(x).cuda(), sid=gsid, **kw)
+        assert err.value.status == KDT_ERR_LEVEL_CAP
         return
     g = kdt.kdt_build(torch.from_numpy(x).cuda(), sid=gsid, **kw)
     assert g.levels == o.levels
