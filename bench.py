@@ -43,6 +43,8 @@ def workload(name: str, rank: int):
         spec = W.config1()
     elif name == "c3s":  # profiling case: config 3's recipe at n=2^22 (larger than L2, small for ncu)
         spec = W.config3(n=1 << 22, depth=15)
+    elif name == "c3m":  # the same at n=2^25 (eight times L2, 5 GB with its workspace): DRAM bytes per launch
+        spec = W.config3(n=1 << 25, depth=18)
     elif name == "w6":  # Sec. 5's simulation shape: trivariate normal, correlation 0.5, n=2^27, depth 10
         spec = W.paper_mvn(1 << 27, 0.5, 10)
     elif name == "w6f":  # the same shape through the normal CDF, split by the paper's estimator (J = 16)
@@ -429,7 +431,7 @@ def main() -> None:
     ap.add_argument("--steps", type=int, default=10)
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
-    ap.add_argument("--workload", default="c3", choices=["c3", "c2", "c1", "c3s", "w6", "w6f", "w6fs", "c4", "c5"])
+    ap.add_argument("--workload", default="c3", choices=["c3", "c2", "c1", "c3s", "c3m", "w6", "w6f", "w6fs", "c4", "c5"])
     ap.add_argument("--trees", type=int, default=4096, help="c4: number of trees")
     ap.add_argument("--requests", type=int, default=20000, help="c5: number of requests")
     ap.add_argument("--load", type=float, default=0.7, help="c5: arrival rate / solo capacity")
